@@ -134,7 +134,7 @@ def measured_peaks() -> tuple[float, str]:
         return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("bn_kernels.cu", "bn_tile13.cu", "bn_levels.cu", "bn_device.cuh")
+KERNEL_SOURCES = ("bn_scores.cu", "bn_kernels.cu", "bn_tile13.cu", "bn_levels.cu", "bn_device.cuh")
 
 
 def kernel_source_sha(files=KERNEL_SOURCES) -> str:

@@ -30,8 +30,8 @@ LIB_TESTING = os.path.join(OUTDIR, "libbnedge_testing.so")
 LIB_PEAKS = os.path.join(OUTDIR, "libbnpeaks.so")
 LIB_CHECKED = os.path.join(OUTDIR, "libbnedge_checked.so")
 LIB_ASAN = os.path.join(OUTDIR, "libbnedge_asan.so")
-SOURCES = ["bn_kernels.cu", "bn_tile13.cu", "bn_levels.cu", "bn_runtime.cu", "bn_noalloc.cu",
-           "bn_mega.cu"]
+SOURCES = ["bn_scores.cu", "bn_kernels.cu", "bn_tile13.cu", "bn_levels.cu", "bn_runtime.cu",
+           "bn_noalloc.cu", "bn_mega.cu"]
 # extra nvcc flags per translation unit
 UNIT_FLAGS: dict = {}
 PEAKS_SOURCE = "bn_peaks.cu"

@@ -1,6 +1,6 @@
-// bn_kernels.cu -- sm_103a kernels of the five steps of Algorithm 1.
+// bn_kernels.cu -- sm_103a kernels of steps 2 to 5 of Algorithm 1 (step 1 is in
+// bn_scores.cu).
 //
-// Step 1  k_pack_planes, k_lgamma_table, k_scores, k_node_max, k_shift_scores
 // Step 2  k_upzeta         truncated upward zeta (Eq. 7, Definition 1)
 // Step 3  k_forward_level, k_backward_level   F (Eq. 9) and R (Eq. 10)
 // Step 4  k_gamma_p1, k_gamma_p2              truncated downward zeta (Eq. 12)
@@ -21,104 +21,6 @@ namespace bn {
 
 static constexpr unsigned FULL = 0xffffffffu;
 
-// ===========================================================================
-// Step 1: local scores.
-// ===========================================================================
-
-// planes[(v*rmax + x)*W + w] bit b  <=>  data[(64w + b)*n + v] == x.
-// mj (may be null) holds the job's own sample count at the job stride; m
-// then only bounds the padded group layout.
-__global__ void k_pack_planes(const uint8_t* __restrict__ data, int n, int m, int rmax, int W,
-                              uint64_t* __restrict__ planes, const int* __restrict__ mj, size_t js)
-{
-    data = job_ptr(data, js);
-    planes = job_ptr(planes, js);
-    if (mj) m = *job_ptr(mj, js);
-    const int64_t total = (int64_t)n * rmax * W;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int w = (int)(t % W);
-        const int64_t vx = t / W;
-        const int x = (int)(vx % rmax);
-        const int v = (int)(vx / rmax);
-        uint64_t word = 0;
-        const int s0 = w * 64;
-        const int cnt = min(64, m - s0);
-        for (int b = 0; b < cnt; ++b)
-            word |= (uint64_t)(data[(size_t)(s0 + b) * n + v] == x) << b;
-        planes[t] = word;
-    }
-}
-
-// err |= 1 when some data value is not below its variable's arity.
-__global__ void k_check_data(const uint8_t* __restrict__ data, const uint8_t* __restrict__ arity,
-                             int n, int m, int* err)
-{
-    const int64_t total = (int64_t)n * m;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        if (data[t] >= arity[t % n]) atomicOr(err, 1);
-    }
-}
-
-// T[row*(m+1) + N] = [lgamma(alpha_row + N) - lgamma(alpha_row)] * scale,
-// N = 0..m, rounded to an integer: the fixed-point table (scale = 2^S) the
-// score kernels sum exactly in int64.
-// In a batch group fxj holds each job's (scale, 1/scale) and mj its own m:
-// entries past the job's m stay 0 (no count reaches them).
-__global__ void k_lgamma_table(const double* __restrict__ alpha, int rows, int m,
-                               long long* __restrict__ T, size_t js, double scale,
-                               const double* __restrict__ fxj, const int* __restrict__ mj)
-{
-    alpha = job_ptr(alpha, js);
-    T = job_ptr(T, js);
-    if (fxj) scale = job_ptr(fxj, js)[0];
-    const int mown = mj ? *job_ptr(mj, js) : m;
-    const int64_t total = (int64_t)rows * (m + 1);
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int row = (int)(t / (m + 1));
-        const int N = (int)(t % (m + 1));
-        const double a = alpha[row];
-        T[t] = (N == 0 || N > mown) ? 0ll
-                                    : __double2ll_rn((lgamma(a + (double)N) - lgamma(a)) * scale);
-    }
-}
-
-// Bit pattern of the double equal to the integer q >= 1, by integer
-// operations only.
-__device__ __forceinline__ long long double_bits(uint32_t q)
-{
-    const int e = 31 - __clz(q);
-    return ((long long)(1023 + e) << 52) | (long long)(((uint64_t)q << (52 - e)) & ((1ull << 52) - 1));
-}
-
-// Row of the denominator D in the sorted table of denominators.  Positive
-// doubles are ordered like their bit patterns, so the search compares
-// integers: the FP64 pipe, narrow on this GPU, is not used.
-__device__ __forceinline__ int find_row(const double* Dvals, int rows, uint32_t D)
-{
-    const long long key = double_bits(D);
-    int lo = 0, hi = rows - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__double_as_longlong(Dvals[mid]) < key) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ double warp_sum(double x)
-{
-    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-    return x;
-}
-
-__device__ __forceinline__ long long warp_sum(long long x)
-{
-    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-    return x;
-}
-
 __device__ __forceinline__ unsigned long long to_fixed(double x) { return __double2ull_rn(x); }
 __device__ __forceinline__ unsigned long long to_fixed(float x) { return __float2ull_rn(x); }
 template <typename T> __device__ __forceinline__ T from_fixed(unsigned long long u);
@@ -129,659 +31,6 @@ template <> __device__ __forceinline__ double from_fixed<double>(unsigned long l
 template <> __device__ __forceinline__ float from_fixed<float>(unsigned long long u)
 {
     return __ull2float_rn(u);
-}
-
-// Step-1 kernels of a batch group run for every job of the group at once:
-// job blockIdx.y finds its arrays js bytes after those of job blockIdx.y - 1.
-#define BN_JOB_SCORES()                                                                   \
-    do {                                                                                  \
-        planes = job_ptr(planes, js);                                                     \
-        Dvals = job_ptr(Dvals, js);                                                       \
-        T = job_ptr(T, js);                                                               \
-        if (log_rho) log_rho = job_ptr(log_rho, js);                                      \
-        masks = job_ptr(masks, js);                                                       \
-        cmasks = job_ptr(cmasks, js);                                                     \
-        logB = job_ptr(logB, js);                                                         \
-        if (fxj) tinv = job_ptr(fxj, js)[1];                                              \
-    } while (0)
-
-// One warp per family x = i*K + f.  Counts N_jk = popc(AND of bit planes),
-// lanes split the words of a plane and the cells of the table lookups.
-//   log B_i(G) = log rho(|G|) + sum_j [ -T_q(N_j) + sum_k T_qr(N_jk) ]
-// with T_a(N) = lgamma(a+N) - lgamma(a), a = ess/q and ess/(q r_i).
-__global__ void __launch_bounds__(256)
-k_scores(int n, int d, int m, int W, int rmax, int64_t K, const uint8_t* __restrict__ arity,
-         const uint64_t* __restrict__ planes, const double* __restrict__ Dvals, int rows,
-         const long long* __restrict__ T, const double* __restrict__ log_rho, int64_t x_begin,
-         int64_t x_count, uint32_t* __restrict__ masks, uint32_t* __restrict__ cmasks,
-         double* __restrict__ logB, int64_t* __restrict__ debug_counts, size_t js, double tinv,
-         const double* __restrict__ fxj)
-{
-    BN_JOB_SCORES();
-    arity = job_ptr(arity, js);
-    const int lane = threadIdx.x & 31;
-    const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t xi = warp0; xi < x_count; xi += nwarps) {
-        const int64_t x = x_begin + xi;
-        const int i = (int)(x / K);
-        uint32_t f = (uint32_t)(x % K);
-        int k = 0;
-        while (f >= binom(n - 1, k)) { f -= binom(n - 1, k); ++k; }
-        const uint32_t cm = colex_unrank(f, k, n - 1);
-        const uint32_t G = expand(cm, i);
-        int par[32];
-        int rad[32];
-        int np = 0;
-        uint32_t q = 1;                             // at most 65536 cells
-        for (uint32_t g = G; g; g &= g - 1) {
-            const int p = __ffs(g) - 1;
-            par[np] = p;
-            rad[np] = arity[p];
-            q *= arity[p];
-            ++np;
-        }
-        const int ri = arity[i];
-        const int row_q = find_row(Dvals, rows, q);
-        const int row_qr = find_row(Dvals, rows, q * (uint32_t)ri);
-        const long long* Tq = T + (size_t)row_q * (m + 1);
-        const long long* Tqr = T + (size_t)row_qr * (m + 1);
-        const int64_t qi = (int64_t)q;
-        int dig[32];
-        for (int t = 0; t < np; ++t) dig[t] = 0;
-        long long acc = 0;
-        for (int64_t cfg = 0; cfg < qi; ++cfg) {
-            uint32_t Nj = 0;
-            for (int xv = 0; xv < ri; ++xv) {
-                uint32_t part = 0;
-                for (int w = lane; w < W; w += 32) {
-                    uint64_t M = planes[((size_t)i * rmax + xv) * W + w];
-                    for (int t = 0; t < np; ++t)
-                        M &= planes[((size_t)par[t] * rmax + dig[t]) * W + w];
-                    part += (uint32_t)__popcll(M);
-                }
-                const uint32_t N = __reduce_add_sync(FULL, part);
-                Nj += N;
-                const int64_t cell = cfg * ri + xv;
-                if (lane == (int)(cell & 31)) {
-                    acc += Tqr[N];
-                    if (debug_counts) debug_counts[cell] = N;
-                }
-            }
-            if (lane == (int)(cfg & 31)) acc -= Tq[Nj];
-            for (int t = 0; t < np; ++t) {          // mixed-radix increment
-                if (++dig[t] < rad[t]) break;
-                dig[t] = 0;
-            }
-        }
-        acc = warp_sum(acc);
-        if (lane == 0) {
-            {
-                const size_t xc = BN_AT(x, 1, (size_t)n * K);
-                logB[xc] = (double)acc * tinv + (log_rho ? log_rho[k] : 0.0);
-                masks[xc] = G;
-                cmasks[xc] = cm;
-            }
-        }
-    }
-    (void)d;
-}
-
-// Scores with one thread per family, for binary data (every arity 2) and
-// families of at most 4 parents: at most 16 parent configurations and 32
-// cells.  The launch covers the first Kc families of every node (those of
-// at most 4 parents; Kc = K when d <= 4); thread index xc stands for family
-// (xc / Kc) * K + xc % Kc.  Word by
-// word the thread builds the masks of all 16 configurations as a product
-// tree of the parent planes (configuration index: digit t = value of parent
-// t, parent 0 least significant; a missing parent t >= |G| contributes the
-// planes (all ones, none), so the configurations with digit 1 there stay
-// empty), counts every cell with popc, and adds the BDeu terms in FP64 in
-// the order (configuration, child value).  Empty cells add
-// lgamma(a) - lgamma(a) = 0 exactly, so the padding changes nothing.
-// The bit planes (n * 2 * W words) stay in L1.
-__global__ void __launch_bounds__(128)
-k_scores_bin(int n, int m, int W, int64_t K, int64_t Kc, const uint64_t* __restrict__ planes,
-             const double* __restrict__ Dvals, int rows, const long long* __restrict__ T,
-             const double* __restrict__ log_rho, int64_t x_begin, int64_t x_count,
-             uint32_t* __restrict__ masks, uint32_t* __restrict__ cmasks,
-             double* __restrict__ logB, int64_t* __restrict__ debug_counts, size_t js, double tinv,
-         const double* __restrict__ fxj)
-{
-    BN_JOB_SCORES();
-    __shared__ uint32_t bt[32][5];                  // C(a, b), b <= 4, for the unrank
-    for (int e = threadIdx.x; e < 32 * 5; e += blockDim.x) bt[e / 5][e % 5] = binom(e / 5, e % 5);
-    __syncthreads();
-    const int64_t xi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (xi >= x_count) return;
-    const int64_t xc = x_begin + xi;
-    const int i = (int)(xc / Kc);
-    uint32_t f = (uint32_t)(xc % Kc);
-    const int64_t x = (int64_t)i * K + f;
-    int k = 0;
-    while (f >= bt[n - 1][k]) { f -= bt[n - 1][k]; ++k; }
-    uint32_t cm = 0;                                // colex unrank of f among k-subsets
-    {
-        int c = n - 2;
-        for (int t = k; t >= 1; --t) {
-            while (bt[c][t] > f) --c;
-            cm |= 1u << c;
-            f -= bt[c][t];
-            --c;
-        }
-    }
-    const uint32_t G = expand(cm, i);
-    int par[4];
-    {
-        uint32_t g = G;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            par[t] = g ? __ffs(g) - 1 : -1;
-            g &= g - 1;
-        }
-    }
-    uint32_t cnt[32];
-#pragma unroll
-    for (int c = 0; c < 32; ++c) cnt[c] = 0;
-    for (int w = 0; w < W; ++w) {
-        uint64_t E[16];
-        E[0] = ~0ull;
-#pragma unroll
-        for (int t = 3; t >= 0; --t) {              // most significant digit first
-            const uint64_t p0 = par[t] >= 0 ? planes[((size_t)par[t] * 2) * W + w] : ~0ull;
-            const uint64_t p1 = par[t] >= 0 ? planes[((size_t)par[t] * 2 + 1) * W + w] : 0ull;
-            const int size = 1 << (3 - t);
-#pragma unroll
-            for (int j = size - 1; j >= 0; --j) {
-                const uint64_t e = E[j];
-                E[2 * j] = e & p0;
-                E[2 * j + 1] = e & p1;
-            }
-        }
-        const uint64_t c0 = planes[((size_t)i * 2) * W + w];
-        const uint64_t c1 = planes[((size_t)i * 2 + 1) * W + w];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            cnt[2 * j] += (uint32_t)__popcll(E[j] & c0);
-            cnt[2 * j + 1] += (uint32_t)__popcll(E[j] & c1);
-        }
-    }
-    const uint32_t q = 1u << k;
-    const long long* Tq = T + (size_t)find_row(Dvals, rows, q) * (m + 1);
-    const long long* Tqr = T + (size_t)find_row(Dvals, rows, 2u * q) * (m + 1);
-    long long acc = 0;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        acc -= Tq[cnt[2 * j] + cnt[2 * j + 1]];
-        acc += Tqr[cnt[2 * j]];
-        acc += Tqr[cnt[2 * j + 1]];
-    }
-    if (debug_counts) {
-        const int cells = 2 << k;
-#pragma unroll
-        for (int c = 0; c < 32; ++c)
-            if (c < cells) debug_counts[c] = cnt[c];
-    }
-    {
-        const size_t xc = BN_AT(x, 1, (size_t)n * K);
-        logB[xc] = (double)acc * tinv + (log_rho ? log_rho[k] : 0.0);
-        masks[xc] = G;
-        cmasks[xc] = cm;
-    }
-}
-
-// Scores of the families with exactly k = 4 + HB parents (5 <= k <= 8), for
-// binary data.  A family takes 2^HB adjacent threads of a warp; thread h
-// owns the 16 configurations whose digits of parents 4..k-1 spell h.  Word
-// by word it ANDs the planes of those high digits into one mask, splits the
-// mask over the four low parents with the product tree of k_scores_bin and
-// counts the 32 cells with popc.  Its FP64 sum of BDeu terms meets those of
-// the family's other threads in an xor butterfly (every lane ends with the
-// same sum, so the order is fixed).  The launch covers families f_begin ..
-// f_begin + f_count - 1 of the n * C(n-1, k) families of this size, family
-// g being rank g % C(n-1, k) of node g / C(n-1, k); off is the index of the
-// first k-parent family inside a node's block of K.
-template <int HB>
-__global__ void __launch_bounds__(128)
-k_scores_bin_hi(int n, int m, int W, int64_t K, int64_t off, int64_t Ck,
-                const uint64_t* __restrict__ planes, const double* __restrict__ Dvals, int rows,
-                const long long* __restrict__ T, const double* __restrict__ log_rho, int64_t f_begin,
-                int64_t f_count, uint32_t* __restrict__ masks, uint32_t* __restrict__ cmasks,
-                double* __restrict__ logB, int64_t* __restrict__ debug_counts, size_t js, double tinv,
-         const double* __restrict__ fxj)
-{
-    BN_JOB_SCORES();
-    constexpr int k = 4 + HB;
-    constexpr int NH = 1 << HB;
-    __shared__ uint32_t bt[32][k + 1];
-    for (int e = threadIdx.x; e < 32 * (k + 1); e += blockDim.x)
-        bt[e / (k + 1)][e % (k + 1)] = binom(e / (k + 1), e % (k + 1));
-    __syncthreads();
-    const int64_t gt = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int h = (int)(gt & (NH - 1));
-    const bool live = (gt >> HB) < f_count;
-    // a thread past the end works on the last family (all lanes stay in the
-    // butterfly) and writes nothing
-    const int64_t g = f_begin + (live ? (gt >> HB) : f_count - 1);
-    const int i = (int)(g / Ck);
-    uint32_t r = (uint32_t)(g % Ck);
-    uint32_t cm = 0;                                // colex unrank of r among k-subsets
-    {
-        int c = n - 2;
-        for (int t = k; t >= 1; --t) {
-            while (bt[c][t] > r) --c;
-            cm |= 1u << c;
-            r -= bt[c][t];
-            --c;
-        }
-    }
-    const uint32_t G = expand(cm, i);
-    int par[k];
-    {
-        uint32_t gg = G;
-#pragma unroll
-        for (int t = 0; t < k; ++t) {
-            par[t] = __ffs(gg) - 1;
-            gg &= gg - 1;
-        }
-    }
-    // plane rows of the high digits of configuration block h
-    int hrow[HB];
-#pragma unroll
-    for (int t = 0; t < HB; ++t) hrow[t] = (par[4 + t] * 2 + ((h >> t) & 1)) * W;
-    uint32_t cnt[32];
-#pragma unroll
-    for (int c = 0; c < 32; ++c) cnt[c] = 0;
-    for (int w = 0; w < W; ++w) {
-        uint64_t E[16];
-        E[0] = planes[hrow[0] + w];
-#pragma unroll
-        for (int t = 1; t < HB; ++t) E[0] &= planes[hrow[t] + w];
-#pragma unroll
-        for (int t = 3; t >= 0; --t) {              // most significant digit first
-            const uint64_t p0 = planes[((size_t)par[t] * 2) * W + w];
-            const uint64_t p1 = planes[((size_t)par[t] * 2 + 1) * W + w];
-            const int size = 1 << (3 - t);
-#pragma unroll
-            for (int j = size - 1; j >= 0; --j) {
-                const uint64_t e = E[j];
-                E[2 * j] = e & p0;
-                E[2 * j + 1] = e & p1;
-            }
-        }
-        const uint64_t c0 = planes[((size_t)i * 2) * W + w];
-        const uint64_t c1 = planes[((size_t)i * 2 + 1) * W + w];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            cnt[2 * j] += (uint32_t)__popcll(E[j] & c0);
-            cnt[2 * j + 1] += (uint32_t)__popcll(E[j] & c1);
-        }
-    }
-    const uint32_t q = 1u << k;
-    const long long* Tq = T + (size_t)find_row(Dvals, rows, q) * (m + 1);
-    const long long* Tqr = T + (size_t)find_row(Dvals, rows, 2u * q) * (m + 1);
-    long long acc = 0;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        acc -= Tq[cnt[2 * j] + cnt[2 * j + 1]];
-        acc += Tqr[cnt[2 * j]];
-        acc += Tqr[cnt[2 * j + 1]];
-    }
-#pragma unroll
-    for (int o = 1; o < NH; o <<= 1) acc += __shfl_xor_sync(FULL, acc, o);
-    if (!live) return;
-    if (debug_counts) {
-#pragma unroll
-        for (int c = 0; c < 32; ++c) debug_counts[32 * h + c] = cnt[c];
-    }
-    if (h == 0) {
-        const int64_t x = (int64_t)i * K + off + (int64_t)(g % Ck);
-        {
-            const size_t xc = BN_AT(x, 1, (size_t)n * K);
-            logB[xc] = (double)acc * tinv + (log_rho ? log_rho[k] : 0.0);
-            masks[xc] = G;
-            cmasks[xc] = cm;
-        }
-    }
-}
-
-// Scores of the families with exactly KP parents (5 <= KP <= 8), binary
-// data, from a histogram of the samples' cells: one warp per family.  A lane
-// takes runs of 16 samples; for each valid sample it forms the cell key
-// (parent t's value in bit t, the child's value in bit KP) from the bit
-// planes with shifts and masks, and adds 1 to the warp's histogram of
-// 2^(KP+1) cells in shared memory.  The BDeu terms follow configuration by
-// configuration (cell = 2 * configuration + child value, the canonical
-// order) in 64-bit fixed point, so the sum equals the per-cell kernels' bit
-// for bit.  The work is O(m) per family instead of O(2^KP m / 64) popcs:
-// the better choice once 2^KP cells outnumber the words.
-template <int KP>
-__global__ void __launch_bounds__(256)
-k_scores_bin_hist(int n, int m, int W, int64_t K, int64_t off, int64_t Ck,
-                  const uint64_t* __restrict__ planes, const double* __restrict__ Dvals, int rows,
-                  const long long* __restrict__ T, const double* __restrict__ log_rho,
-                  int64_t f_begin, int64_t f_count, uint32_t* __restrict__ masks,
-                  uint32_t* __restrict__ cmasks, double* __restrict__ logB,
-                  int64_t* __restrict__ debug_counts, size_t js, double tinv,
-                  const double* __restrict__ fxj)
-{
-    BN_JOB_SCORES();
-    constexpr int NCFG = 1 << KP;
-    __shared__ uint32_t hist[8][2 * NCFG];
-    __shared__ uint32_t bt[32][KP + 1];
-    for (int e = threadIdx.x; e < 32 * (KP + 1); e += blockDim.x)
-        bt[e / (KP + 1)][e % (KP + 1)] = binom(e / (KP + 1), e % (KP + 1));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t* hw = hist[warp];
-    for (int c = lane; c < 2 * NCFG; c += 32) hw[c] = 0u;
-    __syncthreads();
-    const long long* Tq = T + (size_t)find_row(Dvals, rows, (uint32_t)NCFG) * (m + 1);
-    const long long* Tqr = T + (size_t)find_row(Dvals, rows, 2u * NCFG) * (m + 1);
-    const int64_t nwarps = (int64_t)gridDim.x * 8;
-    for (int64_t fi = (int64_t)blockIdx.x * 8 + warp; fi < f_count; fi += nwarps) {
-        const int64_t g = f_begin + fi;
-        const int i = (int)(g / Ck);
-        uint32_t r = (uint32_t)(g % Ck);
-        const uint32_t rank = r;
-        uint32_t cm = 0;                            // colex unrank of r among KP-subsets
-        {
-            int c = n - 2;
-            for (int t = KP; t >= 1; --t) {
-                while (bt[c][t] > r) --c;
-                cm |= 1u << c;
-                r -= bt[c][t];
-                --c;
-            }
-        }
-        const uint32_t G = expand(cm, i);
-        const uint64_t* pr[KP];                     // the value-1 plane of each parent
-        {
-            uint32_t gg = G;
-#pragma unroll
-            for (int t = 0; t < KP; ++t) {
-                pr[t] = planes + ((size_t)(__ffs(gg) - 1) * 2 + 1) * W;
-                gg &= gg - 1;
-            }
-        }
-        const uint64_t* c0 = planes + (size_t)i * 2 * W;
-        const uint64_t* c1 = c0 + W;
-        for (int ch = lane; ch < 4 * W; ch += 32) {
-            const int w = ch >> 2, sh = (ch & 3) * 16;
-            const uint64_t x1w = c1[w];
-            uint32_t valid = (uint32_t)((c0[w] | x1w) >> sh) & 0xFFFFu;
-            const uint32_t x1 = (uint32_t)(x1w >> sh);
-            uint32_t pb[KP];
-#pragma unroll
-            for (int t = 0; t < KP; ++t) pb[t] = (uint32_t)(pr[t][w] >> sh);
-            while (valid) {
-                const int b = __ffs(valid) - 1;
-                valid &= valid - 1;
-                uint32_t key = (x1 >> b & 1u) << KP;
-#pragma unroll
-                for (int t = 0; t < KP; ++t) key |= (pb[t] >> b & 1u) << t;
-                atomicAdd(&hw[key], 1u);
-            }
-        }
-        __syncwarp();
-        long long acc = 0;
-        for (int j = lane; j < NCFG; j += 32) {
-            const uint32_t N0 = hw[j], N1 = hw[j | NCFG];
-            acc += Tqr[N0] + Tqr[N1] - Tq[N0 + N1];
-            if (debug_counts) {
-                debug_counts[2 * j] = N0;
-                debug_counts[2 * j + 1] = N1;
-            }
-            hw[j] = 0u;
-            hw[j | NCFG] = 0u;
-        }
-        __syncwarp();
-        acc = warp_sum(acc);
-        if (lane == 0) {
-            const int64_t x = (int64_t)i * K + off + rank;
-            {
-                const size_t xc = BN_AT(x, 1, (size_t)n * K);
-                logB[xc] = (double)acc * tinv + (log_rho ? log_rho[KP] : 0.0);
-                masks[xc] = G;
-                cmasks[xc] = cm;
-            }
-        }
-    }
-}
-
-// Scores with one warp per family and one lane per 64-sample word (m <= 2048):
-// every lane keeps its word of each parent plane and child plane in
-// registers, so a cell costs an AND chain, a popc and one warp reduction.
-// Lane c % 32 keeps the count of cell c and adds its lgamma-table term when a
-// run of 32 cells is complete (FP64 adds in a fixed order).
-template <int MP, int MR>
-__global__ void __launch_bounds__(256)
-k_scores_w(int n, int m, int W, int rmax, int64_t K, const uint8_t* __restrict__ arity,
-           const uint64_t* __restrict__ planes, const double* __restrict__ Dvals, int rows,
-           const long long* __restrict__ T, const double* __restrict__ log_rho, int64_t x_begin,
-           int64_t x_count, uint32_t* __restrict__ masks, uint32_t* __restrict__ cmasks,
-           double* __restrict__ logB, int64_t* __restrict__ debug_counts, size_t js, double tinv,
-         const double* __restrict__ fxj)
-{
-    BN_JOB_SCORES();
-    arity = job_ptr(arity, js);
-    const int lane = threadIdx.x & 31;
-    const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const bool has_word = lane < W;
-    for (int64_t xi = warp0; xi < x_count; xi += nwarps) {
-        const int64_t x = x_begin + xi;
-        const int i = (int)(x / K);
-        uint32_t f = (uint32_t)(x % K);
-        int k = 0;
-        while (f >= binom(n - 1, k)) { f -= binom(n - 1, k); ++k; }
-        const uint32_t cm = colex_unrank(f, k, n - 1);
-        const uint32_t G = expand(cm, i);
-        uint64_t pw[MP][MR];
-        int rad[MP];
-        uint32_t g = G;
-        int q = 1;
-#pragma unroll
-        for (int t = 0; t < MP; ++t) {
-            rad[t] = 1;
-#pragma unroll
-            for (int v = 0; v < MR; ++v) pw[t][v] = (v == 0) ? ~0ull : 0ull;
-            if (t < k) {
-                const int p = __ffs(g) - 1;
-                g &= g - 1;
-                rad[t] = arity[p];
-                q *= rad[t];
-#pragma unroll
-                for (int v = 0; v < MR; ++v)
-                    pw[t][v] = (v < rad[t] && has_word) ? planes[((size_t)p * rmax + v) * W + lane] : 0ull;
-            }
-        }
-        const int ri = arity[i];
-        uint64_t cw[MR];
-#pragma unroll
-        for (int v = 0; v < MR; ++v)
-            cw[v] = (v < ri && has_word) ? planes[((size_t)i * rmax + v) * W + lane] : 0ull;
-        const long long* Tq = T + (size_t)find_row(Dvals, rows, (uint32_t)q) * (m + 1);
-        const long long* Tqr = T + (size_t)find_row(Dvals, rows, (uint32_t)(q * ri)) * (m + 1);
-        int dig[MP];
-#pragma unroll
-        for (int t = 0; t < MP; ++t) dig[t] = 0;
-        long long acc = 0;
-        uint32_t cur = 0, curj = 0;
-        int cell = 0;
-        for (int cfg = 0; cfg < q; ++cfg) {
-            uint64_t M = ~0ull;
-#pragma unroll
-            for (int t = 0; t < MP; ++t) {
-                uint64_t w = pw[t][0];
-#pragma unroll
-                for (int v = 1; v < MR; ++v)
-                    if (dig[t] == v) w = pw[t][v];
-                M &= w;
-            }
-            uint32_t Nj = 0;
-#pragma unroll
-            for (int v = 0; v < MR; ++v) {
-                if (v < ri) {
-                    const uint32_t N = __reduce_add_sync(FULL, (uint32_t)__popcll(M & cw[v]));
-                    Nj += N;
-                    if (lane == (cell & 31)) {
-                        cur = N;
-                        if (debug_counts) debug_counts[cell] = N;
-                    }
-                    if ((cell & 31) == 31) acc += Tqr[cur];
-                    ++cell;
-                }
-            }
-            if (lane == (cfg & 31)) curj = Nj;
-            if ((cfg & 31) == 31) acc -= Tq[curj];
-            bool carry = true;
-#pragma unroll
-            for (int t = 0; t < MP; ++t) {
-                if (carry) {
-                    if (++dig[t] < rad[t]) carry = false;
-                    else dig[t] = 0;
-                }
-            }
-        }
-        if ((cell & 31) != 0 && lane < (cell & 31)) acc += Tqr[cur];
-        if ((q & 31) != 0 && lane < (q & 31)) acc -= Tq[curj];
-        acc = warp_sum(acc);
-        if (lane == 0) {
-            {
-                const size_t xc = BN_AT(x, 1, (size_t)n * K);
-                logB[xc] = (double)acc * tinv + (log_rho ? log_rho[k] : 0.0);
-                masks[xc] = G;
-                cmasks[xc] = cm;
-            }
-        }
-    }
-}
-
-// Register version of k_scores for at most MP parents and child arity at
-// most MR: one warp per family, one lane per parent configuration j.  The
-// lane ANDs the planes of its configuration's parent values word by word and
-// counts each child value with popc, then adds its own BDeu terms
-//   -T_q(N_j) + sum_k T_qr(N_jk);
-// the warp sum gives log B.  No cross-lane step per cell.
-constexpr int SC_MP = 8, SC_MR = 8;
-template <int MP, int MR>
-__global__ void __launch_bounds__(256)
-k_scores_cfg(int n, int m, int W, int rmax, int64_t K, const uint8_t* __restrict__ arity,
-             const uint64_t* __restrict__ planes, const double* __restrict__ Dvals, int rows,
-             const long long* __restrict__ T, const double* __restrict__ log_rho, int64_t x_begin,
-             int64_t x_count, uint32_t* __restrict__ masks, uint32_t* __restrict__ cmasks,
-             double* __restrict__ logB, int64_t* __restrict__ debug_counts, size_t js, double tinv,
-         const double* __restrict__ fxj)
-{
-    BN_JOB_SCORES();
-    arity = job_ptr(arity, js);
-    const int lane = threadIdx.x & 31;
-    const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t xi = warp0; xi < x_count; xi += nwarps) {
-        const int64_t x = x_begin + xi;
-        const int i = (int)(x / K);
-        uint32_t f = (uint32_t)(x % K);
-        int k = 0;
-        while (f >= binom(n - 1, k)) { f -= binom(n - 1, k); ++k; }
-        const uint32_t cm = colex_unrank(f, k, n - 1);
-        const uint32_t G = expand(cm, i);
-        int par[MP], rad[MP];
-        uint32_t g = G;
-        int q = 1;
-#pragma unroll
-        for (int t = 0; t < MP; ++t) {
-            par[t] = 0;
-            rad[t] = 1;
-            if (g) {
-                par[t] = __ffs(g) - 1;
-                g &= g - 1;
-                rad[t] = arity[par[t]];
-                q *= rad[t];
-            }
-        }
-        const int ri = arity[i];
-        const long long* Tq = T + (size_t)find_row(Dvals, rows, (uint32_t)q) * (m + 1);
-        const long long* Tqr = T + (size_t)find_row(Dvals, rows, (uint32_t)(q * ri)) * (m + 1);
-        const uint64_t* cp = planes + (size_t)i * rmax * W;
-        long long acc = 0;
-        for (int j0 = 0; j0 < q; j0 += 32) {
-            const int j = j0 + lane;
-            if (j < q) {
-                const uint64_t* pp[MP];
-                int jj = j;
-#pragma unroll
-                for (int t = 0; t < MP; ++t) {
-                    const int dg = jj % rad[t];
-                    jj /= rad[t];
-                    pp[t] = planes + ((size_t)par[t] * rmax + dg) * W;
-                }
-                uint32_t N[MR];
-#pragma unroll
-                for (int xv = 0; xv < MR; ++xv) N[xv] = 0;
-                for (int w = 0; w < W; ++w) {
-                    uint64_t M = ~0ull;
-#pragma unroll
-                    for (int t = 0; t < MP; ++t)
-                        if (t < k) M &= pp[t][w];
-#pragma unroll
-                    for (int xv = 0; xv < MR; ++xv)
-                        if (xv < ri) N[xv] += (uint32_t)__popcll(M & cp[(size_t)xv * W + w]);
-                }
-                uint32_t Nj = 0;
-#pragma unroll
-                for (int xv = 0; xv < MR; ++xv) {
-                    if (xv < ri) {
-                        acc += Tqr[N[xv]];
-                        Nj += N[xv];
-                        if (debug_counts) debug_counts[(int64_t)j * ri + xv] = N[xv];
-                    }
-                }
-                acc -= Tq[Nj];
-            }
-        }
-        acc = warp_sum(acc);
-        if (lane == 0) {
-            {
-                const size_t xc = BN_AT(x, 1, (size_t)n * K);
-                logB[xc] = (double)acc * tinv + (log_rho ? log_rho[k] : 0.0);
-                masks[xc] = G;
-                cmasks[xc] = cm;
-            }
-        }
-    }
-}
-
-// cmax[i] = max_f logB[i*K + f]; one block per node.
-__global__ void k_node_max(int64_t K, const double* __restrict__ logB, double* __restrict__ cmax,
-                           size_t js)
-{
-    logB = job_ptr(logB, js);
-    cmax = job_ptr(cmax, js);
-    __shared__ double red[32];
-    const int i = blockIdx.x;
-    double mx = -INFINITY;
-    for (int64_t f = threadIdx.x; f < K; f += blockDim.x) mx = fmax(mx, logB[(size_t)i * K + f]);
-    for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(FULL, mx, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        mx = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : -INFINITY;
-        for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(FULL, mx, o));
-        if (threadIdx.x == 0) cmax[i] = mx;
-    }
-}
-
-template <typename T>
-__global__ void k_shift_scores(int64_t total, int64_t K, const double* __restrict__ logB,
-                               const double* __restrict__ cmax, T* __restrict__ lbs, size_t js)
-{
-    logB = job_ptr(logB, js);
-    cmax = job_ptr(cmax, js);
-    lbs = job_ptr(lbs, js);
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < total;
-         x += (int64_t)gridDim.x * blockDim.x)
-        lbs[x] = (T)LogOps<T>::from_ln(logB[x] - cmax[x / K]);
 }
 
 // ===========================================================================
@@ -1369,14 +618,6 @@ __global__ void k_edges_fin(int n, int use_z, int qbits, const double* __restric
 // Priors beyond the defaults and single features (Eqs. 4-9).
 // ===========================================================================
 
-// log B_i(G) += log w_i(G): a per-family weight (a general rho_i(G), Eq. 4).
-__global__ void k_add_weights(double* __restrict__ logB, const double* __restrict__ w, int64_t nK)
-{
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < nK;
-         x += (int64_t)gridDim.x * blockDim.x)
-        logB[x] += w[x];
-}
-
 // A_i(S) += log q_i(S), q_i a function of |S| (Eq. 7): lq[i * n + |S|] in
 // the working precision and log base; A is [i * 2^(n-1) + c], c = S with
 // bit i removed, so |S| = popc(c).
@@ -1453,184 +694,7 @@ static int grid_for(int64_t work, int threads, int cap = 152 * 32)
     return (int)g;
 }
 
-cudaError_t launch_pack_planes(const uint8_t* data, int n, int m, int rmax, int W,
-                               uint64_t* planes, cudaStream_t s, const int* mj, int nj, size_t js)
-{
-    const int64_t total = (int64_t)n * rmax * W;
-    launch_or_record(KID_PACK_PLANES, k_pack_planes, dim3(grid_for(total, 256), nj), 256, 0, s, data, n, m, rmax, W, planes, mj,
-                                                                 js);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_check_data(const uint8_t* data, const uint8_t* arity, int n, int m,
-                              int* err, cudaStream_t s)
-{
-    if ((int64_t)n * m == 0) return cudaSuccess;
-    launch_or_record(KID_CHECK_DATA, k_check_data, grid_for((int64_t)n * m, 256), 256, 0, s, data, arity, n, m, err);
-    return cudaGetLastError();
-}
-
-int fixed_shift(int m, double ess, const double* Dvals, int rows)
-{
-    double L = std::log1p((double)m);
-    for (int r = 0; r < rows; ++r) {
-        const double a = ess / Dvals[r];
-        L = std::max(L, std::max(std::fabs(std::log(a)), std::log(a + (double)m)));
-    }
-    const double B = 2.0 * (double)m * L + 1.0;
-    const int S = 61 - (int)std::ceil(std::log2(B));
-    return std::min(52, std::max(8, S));
-}
-
-cudaError_t launch_lgamma_table(const double* alpha, int rows, int m, int fxs, void* T,
-                                cudaStream_t s, int nj, size_t js, const double* fxj,
-                                const int* mj)
-{
-    const int64_t total = (int64_t)rows * (m + 1);
-    launch_or_record(KID_LGAMMA_TABLE, k_lgamma_table, dim3(grid_for(total, 256), nj), 256, 0, s, 
-        alpha, rows, m, (long long*)T, js, std::ldexp(1.0, fxs), fxj, mj);
-    return cudaGetLastError();
-}
-
 static uint32_t host_binom(int n, int k);
-
-// Binary data, d <= 8: k_scores_bin for the families of at most 4 parents
-// and one launch per larger family size: k_scores_bin_hi (per-cell popc)
-// below kHistFrom parents, k_scores_bin_hist (per-sample histogram) from
-// there.  The range is all families or a single one.
-static constexpr int kHistFrom = 7;
-static cudaError_t launch_scores_bin(const Plan& P, const uint64_t* planes, const double* Dvals,
-                                     const void* Tv, const double* log_rho, int64_t x_begin,
-                                     int64_t x_count, uint32_t* masks, uint32_t* cmasks,
-                                     double* logB, int64_t* debug_counts, cudaStream_t s,
-                                     const double* fxj)
-{
-    const long long* T = static_cast<const long long*>(Tv);
-    const double tinv = std::ldexp(1.0, -P.fxs);
-    int64_t off[10] = {0};
-    for (int k = 0; k <= P.d; ++k) off[k + 1] = off[k] + host_binom(P.n - 1, k);
-    const int dl = P.d < 4 ? P.d : 4;
-    const int64_t Kc = off[dl + 1];
-    int k1 = 0, klo = 0, khi = P.d;                 // single family: its size only
-    int64_t i1 = 0, f1 = 0;
-    if (x_count == 1) {
-        i1 = x_begin / P.K;
-        f1 = x_begin % P.K;
-        while (f1 >= off[k1 + 1]) ++k1;
-        klo = khi = k1;
-    }
-    if (klo <= 4) {
-        const int64_t xb = x_count == 1 ? i1 * Kc + f1 : 0;
-        const int64_t xn = x_count == 1 ? 1 : (int64_t)P.n * Kc;
-        const unsigned tbb = rec_block(128);
-        launch_or_record(KID_SCORES_BIN, k_scores_bin, dim3((unsigned)((xn + tbb - 1) / tbb), P.nj), tbb, 0, s, 
-            P.n, P.m, P.W, P.K, Kc, planes, Dvals, P.rows, T, log_rho, xb, xn, masks, cmasks, logB,
-            debug_counts, P.js, tinv, fxj);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    for (int k = klo > 5 ? klo : 5; k <= khi; ++k) {
-        const int64_t Ck = host_binom(P.n - 1, k);
-        const int64_t fb = x_count == 1 ? i1 * Ck + (f1 - off[k]) : 0;
-        const int64_t fn = x_count == 1 ? 1 : (int64_t)P.n * Ck;
-        if (k >= kHistFrom) {                       // histogram of the samples' cells
-            const unsigned grid = (unsigned)std::min<int64_t>((fn + 7) / 8, 152 * 32);
-#define BN_BIN_HIST(KP)                                                                           \
-    launch_or_record((int)KID_SCORES_BIN_HIST5 + (KP) - 5, k_scores_bin_hist<KP>, dim3(grid, P.nj), 256, 0, s,                                     \
-        P.n, P.m, P.W, P.K, off[k], Ck, planes, Dvals, P.rows, T, log_rho, fb, fn, masks, cmasks, \
-        logB, debug_counts, P.js, tinv, fxj)
-            switch (k) {
-            case 5: BN_BIN_HIST(5); break;
-            case 6: BN_BIN_HIST(6); break;
-            case 7: BN_BIN_HIST(7); break;
-            default: BN_BIN_HIST(8); break;
-            }
-#undef BN_BIN_HIST
-            cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            continue;
-        }
-        const int64_t threads = fn << (k - 4);
-        const unsigned tbh = rec_block(128);
-        const unsigned grid = (unsigned)((threads + tbh - 1) / tbh);
-#define BN_BIN_HI(HB)                                                                             \
-    launch_or_record((int)KID_SCORES_BIN_HI1 + (HB) - 1, k_scores_bin_hi<HB>, dim3(grid, P.nj), tbh, 0, s,                                       \
-        P.n, P.m, P.W, P.K, off[k], Ck, planes, Dvals, P.rows, T, log_rho, fb, fn, masks, cmasks, \
-        logB, debug_counts, P.js, tinv, fxj)
-        switch (k) {
-        case 5: BN_BIN_HI(1); break;
-        case 6: BN_BIN_HI(2); break;
-        case 7: BN_BIN_HI(3); break;
-        default: BN_BIN_HI(4); break;
-        }
-#undef BN_BIN_HI
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
-bool scores_cfg_fits(const Plan& P)
-{
-    return !P.allbin && P.d <= SC_MP && P.rmax <= SC_MR;
-}
-
-int scores_launches(const Plan& P)
-{
-    return P.allbin && P.d > 4 && P.d <= 8 ? P.d - 3 : 1;
-}
-
-cudaError_t launch_scores(const Plan& P, const uint8_t* arity, const uint64_t* planes,
-                          const double* Dvals, const void* Tv, const double* log_rho,
-                          int64_t x_begin, int64_t x_count, uint32_t* masks, uint32_t* cmasks,
-                          double* logB, int64_t* debug_counts, cudaStream_t s,
-                          const double* fxj)
-{
-    const long long* T = static_cast<const long long*>(Tv);
-    const double tinv = std::ldexp(1.0, -P.fxs);
-    const int threads = 256;
-    const int64_t warps_wanted = x_count;
-    int grid = grid_for(warps_wanted * 32, threads, 152 * 64);
-    if (P.allbin && P.d <= 8 && (x_count == 1 || (x_begin == 0 && x_count == (int64_t)P.n * P.K)))
-        return launch_scores_bin(P, planes, Dvals, Tv, log_rho, x_begin, x_count, masks, cmasks,
-                                 logB, debug_counts, s, fxj);
-    if (P.scfg && scores_cfg_fits(P) && P.d <= 4 && P.rmax <= 4)
-        launch_or_record(KID_SCORES_CFG44, k_scores_cfg<4, 4>, dim3(grid, P.nj), threads, 0, s, 
-            P.n, P.m, P.W, P.rmax, P.K, arity, planes, Dvals, P.rows, T, log_rho, x_begin, x_count,
-            masks, cmasks, logB, debug_counts, P.js, tinv, fxj);
-    else if (P.scfg && scores_cfg_fits(P))
-        launch_or_record(KID_SCORES_CFG, k_scores_cfg<SC_MP, SC_MR>, dim3(grid, P.nj), threads, 0, s, 
-            P.n, P.m, P.W, P.rmax, P.K, arity, planes, Dvals, P.rows, T, log_rho, x_begin, x_count,
-            masks, cmasks, logB, debug_counts, P.js, tinv, fxj);
-    else if (P.W <= 32 && P.d <= 4 && P.rmax <= 2)
-        launch_or_record(KID_SCORES_W42, k_scores_w<4, 2>, dim3(grid, P.nj), threads, 0, s, P.n, P.m, P.W, P.rmax, P.K, arity, planes, Dvals,
-                                                  P.rows, T, log_rho, x_begin, x_count, masks,
-                                                  cmasks, logB, debug_counts, P.js, tinv, fxj);
-    else if (P.W <= 32 && P.d <= 4 && P.rmax <= 4)
-        launch_or_record(KID_SCORES_W44, k_scores_w<4, 4>, dim3(grid, P.nj), threads, 0, s, P.n, P.m, P.W, P.rmax, P.K, arity, planes, Dvals,
-                                                  P.rows, T, log_rho, x_begin, x_count, masks,
-                                                  cmasks, logB, debug_counts, P.js, tinv, fxj);
-    else if (P.W <= 32 && P.d <= 8 && P.rmax <= 4)
-        launch_or_record(KID_SCORES_W84, k_scores_w<8, 4>, dim3(grid, P.nj), threads, 0, s, P.n, P.m, P.W, P.rmax, P.K, arity, planes, Dvals,
-                                                  P.rows, T, log_rho, x_begin, x_count, masks,
-                                                  cmasks, logB, debug_counts, P.js, tinv, fxj);
-    else if (P.d <= SC_MP && P.rmax <= SC_MR)
-        launch_or_record(KID_SCORES_CFG, k_scores_cfg<SC_MP, SC_MR>, dim3(grid, P.nj), threads, 0, s, P.n, P.m, P.W, P.rmax, P.K, arity, planes, Dvals,
-                                              P.rows, T, log_rho, x_begin, x_count, masks,
-                                              cmasks, logB, debug_counts, P.js, tinv, fxj);
-    else
-        launch_or_record(KID_SCORES, k_scores, dim3(grid, P.nj), threads, 0, s, P.n, P.d, P.m, P.W, P.rmax, P.K, arity, planes, Dvals,
-                                          P.rows, T, log_rho, x_begin, x_count, masks, cmasks,
-                                          logB, debug_counts, P.js, tinv, fxj);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_add_weights(const Plan& P, double* logB, const double* w, cudaStream_t s)
-{
-    const int64_t nK = (int64_t)P.n * P.K;
-    launch_or_record(KID_ADD_WEIGHTS, k_add_weights, grid_for(nK, 256), 256, 0, s, logB, w, nK);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_apply_q(const Plan& P, const void* lq, void* A, cudaStream_t s)
 {
@@ -1657,24 +721,6 @@ cudaError_t launch_add_feature(const Plan& P, const void* lbs, const void* lf, v
     return cudaGetLastError();
 }
 
-cudaError_t launch_node_max(const Plan& P, const double* logB, double* cmax, cudaStream_t s)
-{
-    launch_or_record(KID_NODE_MAX, k_node_max, dim3(P.n, P.nj), 256, 0, s, P.K, logB, cmax, P.js);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_shift_scores(const Plan& P, const double* logB, const double* cmax, void* lbs,
-                                cudaStream_t s)
-{
-    const int64_t total = (int64_t)P.n * P.K;
-    const dim3 grid(grid_for(total, 256), P.nj);
-    if (P.prec == 0)
-        launch_or_record(KID_SHIFT_D, k_shift_scores<double>, grid, 256, 0, s, total, P.K, logB, cmax, (double*)lbs, P.js);
-    else
-        launch_or_record(KID_SHIFT_F, k_shift_scores<float>, grid, 256, 0, s, total, P.K, logB, cmax, (float*)lbs, P.js);
-    return cudaGetLastError();
-}
-
 size_t upzeta_smem_bytes(const Plan& P)
 {
     const size_t es = P.prec == 0 ? 8 : 4;
@@ -1690,11 +736,14 @@ static int fixed_bits(int64_t terms)
 }
 
 cudaError_t launch_upzeta(const Plan& P, const uint32_t* cmasks, const void* lbs, void* tab,
-                          const uint16_t* rk13, void* A, cudaStream_t s, cudaEvent_t sums_done, int* err)
+                          const uint16_t* rk13, void* A, cudaStream_t s, cudaEvent_t sums_done, int* err,
+                          bool reordered)
 {
     if (use_tile13_up(P)) {
-        cudaError_t e = launch_reorder_up(P, lbs, tab, s);
-        if (e != cudaSuccess) return e;
+        if (!reordered) {
+            const cudaError_t e = launch_reorder_up(P, lbs, tab, s);
+            if (e != cudaSuccess) return e;
+        }
         return launch_upzeta13(P, tab, rk13 + 8192, A, s, sums_done, err);
     }
     const int h = P.n - 1 - P.b_up;
@@ -1912,6 +961,8 @@ cudaError_t set_kernel_attributes()
     SETA(k_gamma_p2<double>)
     SETA(k_gamma_p2<float>)
 #undef SETA
+    e = set_scores_attributes();
+    if (e != cudaSuccess) return e;
     return set_tile13_attributes();
 }
 

@@ -22,16 +22,13 @@ constexpr int kErrDeviceTimeout = 2;
 
 enum KernelId : int32_t {
     KID_NONE = 0,
-    KID_PACK_PLANES, KID_CHECK_DATA, KID_LGAMMA_TABLE,
-    KID_SCORES_BIN, KID_SCORES_BIN_HIST5, KID_SCORES_BIN_HIST6, KID_SCORES_BIN_HIST7,
-    KID_SCORES_BIN_HIST8, KID_SCORES_BIN_HI1, KID_SCORES_BIN_HI2, KID_SCORES_BIN_HI3,
-    KID_SCORES_BIN_HI4, KID_SCORES_CFG44, KID_SCORES_CFG, KID_SCORES_W42, KID_SCORES_W44,
-    KID_SCORES_W84, KID_SCORES, KID_ADD_WEIGHTS, KID_APPLY_Q_D, KID_APPLY_Q_F,
-    KID_ADD_FEATURE_D, KID_ADD_FEATURE_F, KID_NODE_MAX, KID_SHIFT_D, KID_SHIFT_F,
+    KID_STEP1_PREP, KID_CHECK_DATA, KID_SET_ONES, KID_SET_MOEBIUS, KID_SET_HIST_WARP,
+    KID_SET_HIST_BLOCK, KID_SET_ANY, KID_FAMILIES, KID_APPLY_Q_D, KID_APPLY_Q_F,
+    KID_ADD_FEATURE_D, KID_ADD_FEATURE_F, KID_SHIFT_D, KID_SHIFT_F,
     KID_UPZETA_D, KID_UPZETA_F, KID_FWD_LEVEL_D, KID_FWD_LEVEL_F, KID_BWD_LEVEL_D,
     KID_BWD_LEVEL_F, KID_GAMMA_TABLE, KID_GAMMA_P1_D, KID_GAMMA_P1_F, KID_GAMMA_P2_D,
     KID_GAMMA_P2_F, KID_GAMMA_P2S_D, KID_GAMMA_P2S_F, KID_EDGES_ZERO, KID_EDGES_ACC_D,
-    KID_EDGES_ACC_F, KID_EDGES_FIN_D, KID_EDGES_FIN_F, KID_RANK13, KID_REORDER_D,
+    KID_EDGES_ACC_F, KID_EDGES_FIN_D, KID_EDGES_FIN_F, KID_REORDER_D,
     KID_REORDER_F, KID_COLB8, KID_COLB4, KID_COLB2, KID_COLW_D, KID_COLW_F, KID_COLS_D,
     KID_COLS_F, KID_UP13_D, KID_UP13_F_TLO, KID_UP13_F, KID_G13_D_Q, KID_G13_D, KID_G13_F_Q,
     KID_G13_F, KID_FROWS_D, KID_FROWS_F_TLO, KID_FROWS_F, KID_BROWS_D, KID_BROWS_F_TLO,
@@ -142,6 +139,9 @@ struct Plan {
     int wb;               // in-warp bits of the F / R' tiles
     int prec;             // 0 = FP64, 1 = FP32
     int allbin = 0;       // every variable has arity 2
+    // Joint states of the largest set of k variables: the product of the k
+    // largest arities, capped at 65537 (a batch group's largest).
+    uint32_t states[33] = {};
     int fxs = 40;         // fixed-point shift of the lgamma table (fixed_shift)
     int hasq = 0;         // an order prior q_i(S) by |S| is given (Eq. 4, 7, 12)
     int hasw = 0;         // per-family log weights are given (Eq. 4)
@@ -149,7 +149,6 @@ struct Plan {
     int up13 = 0;         // step 2 by the 13-dimension tiles (n >= 14)
     int g13 = 0;          // step 4 phase 1 by the 13-dimension tiles (n >= 14)
     int frows = 0;        // FP32 step 3 by the 16-subset row kernels
-    int scfg = 0;         // step 1 by one lane per parent configuration (non-binary data)
     int frc = 0;          // FP32 step 3 of a batch group by the persistent cluster kernel
     // Batch groups: nj jobs with equal plans, their arrays js bytes apart;
     // the launches of steps 2-5 cover all of them (gridDim.y = nj).
@@ -179,6 +178,17 @@ struct Plan {
 };
 inline int up_nodes(const Plan& P) { return P.nodes ? P.nodes : P.n; }
 
+// Plan::states from the arities in descending order.
+inline void set_states(Plan& P, const uint32_t* sorted)
+{
+    uint64_t q = 1;
+    P.states[0] = 1;
+    for (int k = 1; k <= 32; ++k) {
+        if (k <= P.n && q <= 65536u) q *= sorted[k - 1];
+        P.states[k] = (uint32_t)(q < 65537u ? q : 65537u);
+    }
+}
+
 // Host check of m x n row-major data: every value below its variable's
 // arity.  Column maxima first (a loop the compiler vectorises), then one
 // comparison per variable.
@@ -193,57 +203,73 @@ inline bool data_below_arity(const uint8_t* data, int m, int n, const uint8_t* a
     return true;
 }
 
-// Step 1.  A batch group passes nj jobs js bytes apart (mj: each job's own
-// sample count, at the same stride); a single job leaves the defaults.
-cudaError_t launch_pack_planes(const uint8_t* data, int n, int m, int rmax, int W,
-                               uint64_t* planes, cudaStream_t s, const int* mj = nullptr,
-                               int nj = 1, size_t js = 0);
+// Step 1 (bn_scores.cu).  A batch group's launches cover nj jobs js bytes
+// apart (mj: each job's own sample count, fxj: its table scale 2^S and 2^-S,
+// at the same stride); a single job leaves the defaults.
+//
+// Scratch of step 1: H(X) per set and, for binary data, the all-ones counts
+// (score_sets(P) entries each), and the nodes' encoded maxima (n entries).
+// They lie in arrays the later steps fill: H in F and R', the counts in lbs,
+// the maxima in the edge accumulators.
+struct SetScratch {
+    long long* H;
+    uint32_t* cnt;
+    unsigned long long* enc;
+};
+uint32_t score_sets(const Plan& P);       // sets of at most d + 1 variables
+// Bit planes, the lgamma table T (rows x (m+1) int64: lgamma(alpha + N) -
+// lgamma(alpha) in fixed point, scaled by 2^fxs; the scores sum it exactly),
+// the 13-bit rank tables, the maxima and the error word (each when given).
+cudaError_t launch_step1_prep(const Plan& P, const uint8_t* data, uint64_t* planes,
+                              const double* alpha, void* T, uint16_t* rank13,
+                              unsigned long long* enc, int* err, cudaStream_t s,
+                              const int* mj = nullptr, const double* fxj = nullptr);
 cudaError_t launch_check_data(const uint8_t* data, const uint8_t* arity, int n, int m,
                               int* err, cudaStream_t s);
-// The lgamma table T (rows x (m+1) int64) holds lgamma(alpha + N) - lgamma(alpha)
-// in fixed point, scaled by 2^fxs (fixed_shift); the scores sum it exactly.
-// A batch group passes fxj (each job's scale 2^S and 2^-S) and mj (each
-// job's m) at the job stride; fxs then is not used.
-cudaError_t launch_lgamma_table(const double* alpha, int rows, int m, int fxs, void* T,
-                                cudaStream_t s, int nj = 1, size_t js = 0,
-                                const double* fxj = nullptr, const int* mj = nullptr);
+// H(X) for every set; the joint-state counts of set dbg_set to dbg (states in
+// mixed-radix order, the lowest variable least significant) when given.
+cudaError_t launch_set_scores(const Plan& P, const uint8_t* data, const uint8_t* arity,
+                              const uint64_t* planes, const double* Dvals, const void* T,
+                              const SetScratch& x, cudaStream_t s, const int* mj = nullptr,
+                              int64_t* dbg = nullptr, uint32_t dbg_set = 0);
+// The sets, then log B (with log rho and the family weights log_w, either may
+// be null), the parent masks and the maxima (x.enc may be null).
+cudaError_t launch_scores(const Plan& P, const uint8_t* data, const uint8_t* arity,
+                          const uint64_t* planes, const double* Dvals, const void* T,
+                          const double* log_rho, const double* log_w, const SetScratch& x,
+                          uint32_t* masks, uint32_t* cmasks, double* logB, cudaStream_t s,
+                          const int* mj = nullptr, const double* fxj = nullptr);
+// Kernels one launch_scores call starts.
+int scores_launches(const Plan& P);
+// lbs = log B - c_i, the shifts c_i from enc to cmax, and the reordered table
+// of the 13-dimension tiles (tab, may be null).
+cudaError_t launch_shift_scores(const Plan& P, const double* logB, const unsigned long long* enc,
+                                const uint32_t* cmasks, double* cmax, void* lbs, void* tab,
+                                cudaStream_t s);
+cudaError_t set_scores_attributes();
 // The fixed-point shift S of the lgamma table: every partial sum of one
 // family's score, at most sum_j |T_q(N_j)| + sum_jk |T_qr(N_jk)| <= 2 m L
 // with L = max |ln(alpha + t)| over the rows (alpha = 1 included) and
 // 0 <= t < m, stays below 2^61 after scaling by 2^S; each term's rounding
 // error is at most 2^-(S+1).
 int fixed_shift(int m, double ess, const double* Dvals, int rows);
-cudaError_t launch_scores(const Plan& P, const uint8_t* arity, const uint64_t* planes,
-                          const double* Dvals, const void* T, const double* log_rho,
-                          int64_t x_begin, int64_t x_count, uint32_t* masks,
-                          uint32_t* cmasks, double* logB, int64_t* debug_counts,
-                          cudaStream_t s, const double* fxj = nullptr);
-// Step 1 has the lane-per-configuration alternative (Plan::scfg): data not
-// all binary, at most 8 parents and arity at most 8.
-bool scores_cfg_fits(const Plan& P);
-// Kernels one launch_scores call over all n * K families starts.
-int scores_launches(const Plan& P);
 // Priors beyond the defaults and single features (Eqs. 4-9):
-// log B += w (n*K doubles, natural log); A_i(S) += lq[i*n + |S|] (lq in the
-// working precision and log base); out = lbs + lf (shifted scores times a
-// feature, working precision).
-cudaError_t launch_add_weights(const Plan& P, double* logB, const double* w, cudaStream_t s);
+// A_i(S) += lq[i*n + |S|] (lq in the working precision and log base);
+// out = lbs + lf (shifted scores times a feature, working precision).
 cudaError_t launch_apply_q(const Plan& P, const void* lq, void* A, cudaStream_t s);
 cudaError_t launch_add_feature(const Plan& P, const void* lbs, const void* lf, void* out,
                                cudaStream_t s);
-cudaError_t launch_node_max(const Plan& P, const double* logB, double* cmax, cudaStream_t s);
-cudaError_t launch_shift_scores(const Plan& P, const double* logB, const double* cmax,
-                                void* lbs, cudaStream_t s);
 // Step 2.  n >= 14 uses the 13-dimension register tiles and needs `tab`
-// (n*K values, the scores reordered by high and low parts); smaller n use
-// one shared-memory tile per node slice and ignore `tab`.
+// (n*K values, the scores reordered by high and low parts; reordered: the
+// shift wrote it already); smaller n use one shared-memory tile per node
+// slice and ignore `tab`.
 // `rk13` points at the two 8192-entry uint16 subset-rank tables (rank, then
 // inverse) of the 13-dimension tiles, filled by launch_rank13_tables.  `err`
 // (the job's error word) lets an FP32 single job use the persistent tile
 // kernel, which reports a bulk copy that never landed there.
 cudaError_t launch_upzeta(const Plan& P, const uint32_t* cmasks, const void* lbs, void* tab,
                           const uint16_t* rk13, void* A, cudaStream_t s, cudaEvent_t sums_done = nullptr,
-                          int* err = nullptr);
+                          int* err = nullptr, bool reordered = false);
 // Step 3 in FP32 with one thread per 16-subset tile (bn_levels.cu).
 bool rows_levels_fit(const Plan& P);      // FP32 and 5 <= n < 32
 bool rows64_fit(const Plan& P);           // FP64 and 4 <= n < 31: 8-subset row tiles
@@ -259,6 +285,7 @@ uint32_t shard_rows_count(const Plan& P, uint32_t r, int hl);
 #ifdef BN_CHECK_BOUNDS
 // The first failing index check of each translation unit (0: none), cleared
 // by the read (bn_device.cuh).
+unsigned int bounds_line_scores();
 unsigned int bounds_line_kernels();
 unsigned int bounds_line_tile13();
 unsigned int bounds_line_levels();
@@ -306,7 +333,6 @@ cudaError_t launch_edges(const Plan& P, const double* logB, const double* cmax,
 size_t upzeta_smem_bytes(const Plan& P);
 // bn_tile13.cu
 cudaError_t launch_reorder_up(const Plan& P, const void* lbs, void* tab, cudaStream_t s);
-cudaError_t launch_rank13_tables(const Plan& P, uint16_t* rank13, uint16_t* unrank13, cudaStream_t s);
 cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unrank13, void* A,
                             cudaStream_t s, cudaEvent_t sums_done = nullptr, int* err = nullptr);
 cudaError_t launch_upzeta13p_withheld(float* A, uint16_t* rank13, uint16_t* unrank13, int* err,
@@ -333,8 +359,6 @@ inline bool use_tlo(const Plan& P) { return P.prec != 0 && P.up13 && P.frows && 
 // The default schedule: every specialised kernel that fits.
 inline void default_schedule(Plan& P)
 {
-    // lane per configuration where the 4-parent, arity-4 instance applies
-    P.scfg = scores_cfg_fits(P) && P.d <= 4 && P.rmax <= 4;
     P.up13 = tile13_up_fits(P);
     P.g13 = tile13_gamma_fits(P);
     P.frows = rows_levels_fit(P);

@@ -18,7 +18,7 @@
 // the abort flag every block checks, and the kernel returns.
 //
 // The kernels are compiled here a second time, as device functions: this
-// file includes the three kernel sources with __global__ turned into
+// file includes the kernel sources with __global__ turned into
 // __device__ __noinline__ and blockIdx / gridDim redirected to the virtual
 // block being run.  Values one block writes are read by other blocks within
 // the same launch.  A producer's writes are ordered before its count by a
@@ -57,6 +57,7 @@ __shared__ uint3 bn_mega_gdim;
 #define __ldcs(p) __ldcg(p)
 #define __ldg(p) __ldcg(p)
 #define BN_MEGA 1
+#include "bn_scores.cu"
 #include "bn_kernels.cu"
 #include "bn_tile13.cu"
 #include "bn_levels.cu"
@@ -92,28 +93,22 @@ __device__ __forceinline__ void run(void (*f)(P...), const unsigned char* a)
 // One virtual block of launch record `kid`.  PREC 1: FP32 kernels and those
 // of either precision; PREC 0: FP64 kernels and those of either precision
 // (two instances, so that the FP32 one is not held to the FP64 tiles'
-// register count).  The binary score kernels for families of 5-8 parents
-// are left out: the static shared memory of every kernel called here adds up
-// in the persistent kernel, and theirs (38 KB) would cost it its second
-// block per SM; batches that need them run as a graph of launches.  Returns
-// false for a kernel this instance does not run.
+// register count).  The static shared memory of every kernel called here adds
+// up in the persistent kernel.  Returns false for a kernel this instance does
+// not run.
 template <int PREC>
 __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
 {
     switch (kid) {
-    case KID_PACK_PLANES: run(k_pack_planes, a); return true;
+    case KID_STEP1_PREP: run(k_step1_prep, a); return true;
     case KID_CHECK_DATA: run(k_check_data, a); return true;
-    case KID_LGAMMA_TABLE: run(k_lgamma_table, a); return true;
-    case KID_SCORES_BIN: run(k_scores_bin, a); return true;
-    case KID_SCORES_CFG44: run(k_scores_cfg<4, 4>, a); return true;
-    case KID_SCORES_CFG: run(k_scores_cfg<SC_MP, SC_MR>, a); return true;
-    case KID_SCORES_W42: run(k_scores_w<4, 2>, a); return true;
-    case KID_SCORES_W44: run(k_scores_w<4, 4>, a); return true;
-    case KID_SCORES_W84: run(k_scores_w<8, 4>, a); return true;
-    case KID_SCORES: run(k_scores, a); return true;
-    case KID_NODE_MAX: run(k_node_max, a); return true;
+    case KID_SET_ONES: run(k_set_ones, a); return true;
+    case KID_SET_MOEBIUS: run(k_set_moebius, a); return true;
+    case KID_SET_HIST_WARP: run(k_set_hist<32>, a); return true;
+    case KID_SET_HIST_BLOCK: run(k_set_hist<256>, a); return true;
+    case KID_SET_ANY: run(k_set_any, a); return true;
+    case KID_FAMILIES: run(k_family_scores, a); return true;
     case KID_EDGES_ZERO: run(k_edges_zero, a); return true;
-    case KID_RANK13: run(k_rank13_tables, a); return true;
     default: break;
     }
     if constexpr (PREC == 1) {
@@ -274,10 +269,9 @@ BN_BOUNDS_READER(bounds_line_mega)
 bool persistent_runs(int prec, int kid)
 {
     switch (kid) {
-    case KID_PACK_PLANES: case KID_CHECK_DATA: case KID_LGAMMA_TABLE: case KID_SCORES_BIN:
-    case KID_SCORES_CFG44: case KID_SCORES_CFG:
-    case KID_SCORES_W42: case KID_SCORES_W44: case KID_SCORES_W84: case KID_SCORES:
-    case KID_NODE_MAX: case KID_EDGES_ZERO: case KID_RANK13:
+    case KID_STEP1_PREP: case KID_CHECK_DATA: case KID_SET_ONES: case KID_SET_MOEBIUS:
+    case KID_SET_HIST_WARP: case KID_SET_HIST_BLOCK: case KID_SET_ANY: case KID_FAMILIES:
+    case KID_EDGES_ZERO:
         return true;
     case KID_SHIFT_F: case KID_UPZETA_F: case KID_FWD_LEVEL_F: case KID_BWD_LEVEL_F:
     case KID_GAMMA_TABLE: case KID_GAMMA_P1_F: case KID_GAMMA_P2_F: case KID_GAMMA_P2S_F:

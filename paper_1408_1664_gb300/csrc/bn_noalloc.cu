@@ -162,6 +162,7 @@ try {
     uint64_t cells = 1;
     for (int t = 0; t <= P.d && t < P.n; ++t) cells *= sorted[t];
     if (cells > 65536u) return BN_EINVAL;
+    bn::set_states(P, sorted);
     double log_rho[32] = {};
     if (j->log_q || j->log_w) return BN_EINVAL;        // not in this entry point
     if (j->log_rho)
@@ -227,7 +228,6 @@ try {
     CKS(cudaMemcpyAsync(base + o_ar, arity, P.n, cudaMemcpyHostToDevice, s));
     CKS(cudaMemcpyAsync(base + o_lr, log_rho, (size_t)(P.d + 1) * 8, cudaMemcpyHostToDevice, s));
     CKS(cudaMemcpyAsync(base + o_tab, tables, (size_t)2 * rows * 8, cudaMemcpyHostToDevice, s));
-    CKS(cudaMemsetAsync(base + o_err, 0, 4, s));        // the one value that must start at 0
     int* err = reinterpret_cast<int*>(base + o_err);
     const uint8_t* ar = base + o_ar;
     const double* Dvals = reinterpret_cast<const double*>(base + o_tab);
@@ -238,17 +238,20 @@ try {
     uint32_t* cm = reinterpret_cast<uint32_t*>(base + o_cm);
     double* logB = reinterpret_cast<double*>(base + o_logB);
     double* cmax = reinterpret_cast<double*>(base + o_cmax);
-    if (j->data_on_device) CKS(bn::launch_check_data(data_dev, ar, P.n, P.m, err, s));
-    CKS(bn::launch_pack_planes(data_dev, P.n, P.m, P.rmax, P.W, planes, s));
-    CKS(bn::launch_lgamma_table(alpha, P.rows, P.m, P.fxs, lgT, s));
-    CKS(bn::launch_scores(P, ar, planes, Dvals, lgT,
-                          j->log_rho ? reinterpret_cast<const double*>(base + o_lr) : nullptr, 0,
-                          (int64_t)P.n * P.K, masks, cm, logB, nullptr, s));
-    CKS(bn::launch_node_max(P, logB, cmax, s));
-    CKS(bn::launch_shift_scores(P, logB, cmax, base + o_lbs, s));
     uint16_t* rk13 = reinterpret_cast<uint16_t*>(base + o_rk);
-    if (bn::needs_rank13(P)) CKS(bn::launch_rank13_tables(P, rk13, rk13 + 8192, s));
-    CKS(bn::launch_upzeta(P, cm, base + o_lbs, base + o_reo, rk13, base + o_A, s));
+    // step 1's scratch in arrays the later steps fill (8 bytes per set in F
+    // and R', 4 in lbs, the maxima in the edge accumulators)
+    const bn::SetScratch x{reinterpret_cast<long long*>(base + o_F), reinterpret_cast<uint32_t*>(base + o_lbs),
+                           reinterpret_cast<unsigned long long*>(base + o_ea)};
+    CKS(bn::launch_step1_prep(P, data_dev, planes, alpha, lgT, bn::needs_rank13(P) ? rk13 : nullptr, x.enc,
+                              err, s));
+    if (j->data_on_device) CKS(bn::launch_check_data(data_dev, ar, P.n, P.m, err, s));
+    CKS(bn::launch_scores(P, data_dev, ar, planes, Dvals, lgT,
+                          j->log_rho ? reinterpret_cast<const double*>(base + o_lr) : nullptr, nullptr, x,
+                          masks, cm, logB, s));
+    CKS(bn::launch_shift_scores(P, logB, x.enc, cm, cmax, base + o_lbs,
+                                bn::use_tile13_up(P) ? base + o_reo : nullptr, s));
+    CKS(bn::launch_upzeta(P, cm, base + o_lbs, base + o_reo, rk13, base + o_A, s, nullptr, nullptr, true));
     CKS(bn::launch_forward(P, base + o_A, base + o_F, s, nullptr));
     CKS(bn::launch_backward(P, base + o_A, base + o_Rc, s, nullptr));
     CKS(bn::launch_gamma_p1(P, base + o_F, base + o_Rc, rk13, base + o_W, s, nullptr, base + o_A));

@@ -195,6 +195,7 @@ int validate_and_plan(const bn_job_desc* j, HostJob& hj)
     uint64_t cells = 1;
     for (int t = 0; t <= P.d && t < P.n; ++t) cells *= sorted[t];
     if (cells > 65536u) return BN_EINVAL;
+    bn::set_states(P, sorted.data());
     if (j->log_rho) {
         hj.log_rho.assign(j->log_rho, j->log_rho + (j->d + 1));
         hj.log_rho.resize(P.d + 1);
@@ -296,6 +297,13 @@ struct Bufs {
     char* A_ext = nullptr;           // A outside the layout (a job whose A is spilled)
     template <typename T> T* at(size_t off) const { return reinterpret_cast<T*>(base + off); }
     void* A() const { return A_ext ? (void*)A_ext : (void*)(base + L.A); }
+    // Step 1's scratch in arrays the later steps fill: 8 bytes per set fit
+    // F and R' (at most 2^n sets), 4 per set lbs (n*K values, at least the
+    // nonempty sets' number)
+    bn::SetScratch set_scratch() const
+    {
+        return {at<long long>(L.F), at<uint32_t>(L.lbs), at<unsigned long long>(L.eacc)};
+    }
 };
 
 int enqueue_kernels(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, double* post_dev,
@@ -365,44 +373,40 @@ int enqueue(const HostJob& hj, const Bufs& B, double* post_dev, double* logPD_de
     return enqueue_kernels(hj, B, data_dev, post_dev, logPD_dev, s, ev, launches, side);
 }
 
-// Step 1 on stream s (inputs on the device): scores, the family weights,
-// the per-node maximum and the shifted scores; the rank tables of the
-// 13-dimension tiles.
+// Step 1 on stream s (inputs on the device): scores with the family weights,
+// the per-node maximum and the shifted scores (also reordered for the
+// 13-dimension up-zeta tiles); the rank tables of those tiles.
 int enqueue_step1(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, cudaStream_t s,
                   int* nl)
 {
     const Plan& P = hj.P;
     const Layout& L = B.L;
-    CK(cudaMemsetAsync(B.at<int>(L.err), 0, 4, s));
     int* err = B.at<int>(L.err);
     const uint8_t* ar = B.at<uint8_t>(L.arity);
+    const bn::SetScratch x = B.set_scratch();
+    CK(bn::launch_step1_prep(P, data_dev, B.at<uint64_t>(L.planes), B.at<double>(L.alpha), B.at<void>(L.lgT),
+                             bn::needs_rank13(P) ? B.at<uint16_t>(L.rk13) : nullptr, x.enc, err, s)); ++*nl;
     if (hj.data_on_device) { CK(bn::launch_check_data(data_dev, ar, P.n, P.m, err, s)); ++*nl; }
-    CK(bn::launch_pack_planes(data_dev, P.n, P.m, P.rmax, P.W, B.at<uint64_t>(L.planes), s)); ++*nl;
-    CK(bn::launch_lgamma_table(B.at<double>(L.alpha), P.rows, P.m, P.fxs, B.at<void>(L.lgT), s)); ++*nl;
-    CK(bn::launch_scores(P, ar, B.at<uint64_t>(L.planes), B.at<double>(L.Dvals),
-                         B.at<void>(L.lgT), hj.log_rho.empty() ? nullptr : B.at<double>(L.log_rho),
-                         0, (int64_t)P.n * P.K, B.at<uint32_t>(L.masks), B.at<uint32_t>(L.cmasks),
-                         B.at<double>(L.logB), nullptr, s));
+    CK(bn::launch_scores(P, data_dev, ar, B.at<uint64_t>(L.planes), B.at<double>(L.Dvals), B.at<void>(L.lgT),
+                         hj.log_rho.empty() ? nullptr : B.at<double>(L.log_rho),
+                         P.hasw ? B.at<double>(L.logw) : nullptr, x, B.at<uint32_t>(L.masks),
+                         B.at<uint32_t>(L.cmasks), B.at<double>(L.logB), s));
     *nl += bn::scores_launches(P);
-    if (P.hasw) { CK(bn::launch_add_weights(P, B.at<double>(L.logB), B.at<double>(L.logw), s)); ++*nl; }
-    CK(bn::launch_node_max(P, B.at<double>(L.logB), B.at<double>(L.cmax), s)); ++*nl;
-    CK(bn::launch_shift_scores(P, B.at<double>(L.logB), B.at<double>(L.cmax), B.at<void>(L.lbs), s)); ++*nl;
-    if (bn::needs_rank13(P)) {
-        uint16_t* rk = B.at<uint16_t>(L.rk13);
-        CK(bn::launch_rank13_tables(P, rk, rk + 8192, s));
-        ++*nl;
-    }
+    CK(bn::launch_shift_scores(P, B.at<double>(L.logB), x.enc, B.at<uint32_t>(L.cmasks), B.at<double>(L.cmax),
+                               B.at<void>(L.lbs), bn::use_tile13_up(P) ? B.at<void>(L.tab) : nullptr, s)); ++*nl;
     return BN_OK;
 }
 
 // Step 2 from the shifted scores lbs into A, then the order prior q.
+// reordered: the tiles' table already holds these scores (step 1 wrote it).
 int enqueue_upzeta(const Plan& P, const Bufs& B, const void* lbs, cudaStream_t s, int* nl,
-                   cudaEvent_t sums_done)
+                   cudaEvent_t sums_done, bool reordered)
 {
     const Layout& L = B.L;
     CK(bn::launch_upzeta(P, B.at<uint32_t>(L.cmasks), lbs, B.at<void>(L.tab),
-                         B.at<uint16_t>(L.rk13), B.A(), s, sums_done, B.at<int>(L.err)));
-    *nl += bn::use_tile13_up(P) ? 3 : 1;
+                         B.at<uint16_t>(L.rk13), B.A(), s, sums_done, B.at<int>(L.err),
+                         reordered));
+    *nl += bn::use_tile13_up(P) ? (reordered ? 2 : 3) : 1;
     if (P.hasq) { CK(bn::launch_apply_q(P, B.at<void>(L.logq), B.A(), s)); ++*nl; }
     return BN_OK;
 }
@@ -418,7 +422,7 @@ int enqueue_kernels(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, d
     if (rc) return rc;
     if (ev) CK(cudaEventRecord(ev->ev[1], s));
     rc = enqueue_upzeta(P, B, B.at<void>(L.lbs), s, &nl,
-                        ev && bn::use_tile13_up(P) ? ev->ev[kEvSums] : nullptr);
+                        ev && bn::use_tile13_up(P) ? ev->ev[kEvSums] : nullptr, true);
     if (rc) return rc;
     int* err = B.at<int>(L.err);
     if (ev) CK(cudaEventRecord(ev->ev[2], s));
@@ -572,8 +576,8 @@ struct bn_ctx {
     uint64_t reserved = 0;
     // batches
     int flags = 0;
-    // (n, d, prec, binary, jobs) -> schedule (scfg, up13, frows, frc, g13)
-    std::map<std::array<int, 5>, std::array<int, 5>> tuned;
+    // (n, d, prec, binary, jobs) -> schedule (up13, frows, frc, g13)
+    std::map<std::array<int, 5>, std::array<int, 4>> tuned;
 };
 
 // Jobs of a batch with equal n, d and precision: their arrays lie js bytes
@@ -992,7 +996,11 @@ try {
     Plan P = hj.P;
     Layout L = make_layout(P, 0);
     const size_t need = L.cmax;   // everything up to and including logB
-    rc = ensure_ws(c, need + al((size_t)P.n * 8) + (P.hasw ? al((size_t)P.n * P.K * 8) : 0));
+    const size_t o_w = need + al((size_t)P.n * 8);
+    const size_t o_H = o_w + (P.hasw ? al((size_t)P.n * P.K * 8) : 0);
+    const size_t sets = bn::score_sets(P);
+    const size_t o_cnt = o_H + al(sets * 8);
+    rc = ensure_ws(c, o_cnt + al(sets * 4));
     if (rc) return rc;
     rc = ensure_pin(&c->pin, &c->pin_bytes, small_bytes(P) + 64);
     if (rc) return rc;
@@ -1012,21 +1020,21 @@ try {
     CK(cudaMemcpyAsync(B.at<char>(L.log_rho), lr.data(), lr.size() * 8, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(B.at<char>(L.Dvals), hj.Dvals.data(), hj.Dvals.size() * 8, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(B.at<char>(L.alpha), alpha.data(), alpha.size() * 8, cudaMemcpyHostToDevice, s));
-    CK(cudaMemsetAsync(B.at<int>(L.err), 0, 4, s));
     const uint8_t* ar = B.at<uint8_t>(L.arity);
+    CK(bn::launch_step1_prep(P, data_dev, B.at<uint64_t>(L.planes), B.at<double>(L.alpha), B.at<void>(L.lgT),
+                             nullptr, nullptr, B.at<int>(L.err), s));
     if (hj.data_on_device) CK(bn::launch_check_data(data_dev, ar, P.n, P.m, B.at<int>(L.err), s));
-    CK(bn::launch_pack_planes(data_dev, P.n, P.m, P.rmax, P.W, B.at<uint64_t>(L.planes), s));
-    CK(bn::launch_lgamma_table(B.at<double>(L.alpha), P.rows, P.m, P.fxs, B.at<void>(L.lgT), s));
-    CK(bn::launch_scores(P, ar, B.at<uint64_t>(L.planes), B.at<double>(L.Dvals), B.at<void>(L.lgT),
-                         hj.log_rho.empty() ? nullptr : B.at<double>(L.log_rho), 0,
-                         (int64_t)P.n * P.K, B.at<uint32_t>(L.masks), B.at<uint32_t>(L.cmasks),
-                         B.at<double>(L.logB), nullptr, s));
+    // the weights and the sets' scratch sit past logB in the layout
+    double* w = nullptr;
     if (P.hasw) {
-        // the weights sit past logB in the layout: a scratch copy right after it
-        double* w = reinterpret_cast<double*>(c->ws + need + al((size_t)P.n * 8));
+        w = reinterpret_cast<double*>(c->ws + o_w);
         CK(cudaMemcpyAsync(w, hj.log_w.data(), hj.log_w.size() * 8, cudaMemcpyHostToDevice, s));
-        CK(bn::launch_add_weights(P, B.at<double>(L.logB), w, s));
     }
+    const bn::SetScratch x{reinterpret_cast<long long*>(c->ws + o_H),
+                           reinterpret_cast<uint32_t*>(c->ws + o_cnt), nullptr};
+    CK(bn::launch_scores(P, data_dev, ar, B.at<uint64_t>(L.planes), B.at<double>(L.Dvals), B.at<void>(L.lgT),
+                         hj.log_rho.empty() ? nullptr : B.at<double>(L.log_rho), w, x,
+                         B.at<uint32_t>(L.masks), B.at<uint32_t>(L.cmasks), B.at<double>(L.logB), s));
     int err = 0;
     CK(cudaMemcpyAsync(parent_mask, B.at<char>(L.masks), (size_t)P.n * P.K * 4, cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(log_B, B.at<char>(L.logB), (size_t)P.n * P.K * 8, cudaMemcpyDeviceToHost, s));
@@ -1086,7 +1094,7 @@ try {
     int nl = 0;
     rc = enqueue_step1(hj, B, data_dev, s, &nl);
     if (rc) return rc;
-    rc = enqueue_upzeta(P, B, B.at<void>(L.lbs), s, &nl, nullptr);
+    rc = enqueue_upzeta(P, B, B.at<void>(L.lbs), s, &nl, nullptr, true);
     if (rc) return rc;
     CK(bn::launch_forward(P, B.at<void>(L.A), B.at<void>(L.F), s, &nl));
     double fv[2] = {0.0, 0.0};
@@ -1097,7 +1105,7 @@ try {
         CK(cudaMemcpyAsync(lw[0], B.at<char>(L.F) + (full + 1) * es, sizeof(lw[0]),
                            cudaMemcpyDeviceToHost, s));
     CK(bn::launch_add_feature(P, B.at<void>(L.lbs), B.at<void>(L.logf), B.at<void>(L.lbsf), s));
-    rc = enqueue_upzeta(P, B, B.at<void>(L.lbsf), s, &nl, nullptr);
+    rc = enqueue_upzeta(P, B, B.at<void>(L.lbsf), s, &nl, nullptr, false);
     if (rc) return rc;
     CK(bn::launch_forward(P, B.at<void>(L.A), B.at<void>(L.F), s, &nl));
     CK(cudaMemcpyAsync(raw[1], B.at<char>(L.F) + full * es, es, cudaMemcpyDeviceToHost, s));
@@ -1151,13 +1159,12 @@ try {
     for (int p = 0; p < P.n; ++p)
         if (mask >> p & 1u) want *= hj.arity[p];
     if (want != cells) return BN_EINVAL;
-    // family index in canonical order
-    const uint32_t low = (1u << i) - 1u;
-    const uint32_t cm = (mask & low) | ((mask >> 1) & ~low);
-    int64_t f = 0;
-    for (int s = 0; s < k; ++s) f += host_binom(P.n - 1, s);
+    // the counts of the set mask + {i}, in the set's own state order
+    const uint32_t set = mask | (1u << i);
+    uint32_t rank = 0;
+    for (int s = 0; s < k + 1; ++s) rank += (uint32_t)host_binom(P.n, s);
     int t = 1;
-    for (uint32_t x = cm; x; x &= x - 1, ++t) f += host_binom(__builtin_ctz(x), t);
+    for (uint32_t x = set; x; x &= x - 1, ++t) rank += (uint32_t)host_binom(__builtin_ctz(x), t);
     if (cudaSetDevice(c->device) != cudaSuccess) return BN_ECUDA;
     Layout L = make_layout(P, (size_t)cells);
     rc = ensure_ws(c, L.total);
@@ -1175,14 +1182,30 @@ try {
     CK(cudaMemcpyAsync(B.at<char>(L.arity), hj.arity.data(), P.n, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(B.at<char>(L.Dvals), hj.Dvals.data(), hj.Dvals.size() * 8, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(B.at<char>(L.alpha), alpha.data(), alpha.size() * 8, cudaMemcpyHostToDevice, s));
-    CK(bn::launch_pack_planes(data_dev, P.n, P.m, P.rmax, P.W, B.at<uint64_t>(L.planes), s));
-    CK(bn::launch_lgamma_table(B.at<double>(L.alpha), P.rows, P.m, P.fxs, B.at<void>(L.lgT), s));
-    CK(bn::launch_scores(P, B.at<uint8_t>(L.arity), B.at<uint64_t>(L.planes), B.at<double>(L.Dvals),
-                         B.at<void>(L.lgT), nullptr, (int64_t)i * P.K + f, 1,
-                         B.at<uint32_t>(L.masks), B.at<uint32_t>(L.cmasks), B.at<double>(L.logB),
-                         B.at<int64_t>(L.dbg), s));
-    CK(cudaMemcpyAsync(counts, B.at<char>(L.dbg), (size_t)cells * 8, cudaMemcpyDeviceToHost, s));
+    CK(bn::launch_step1_prep(P, data_dev, B.at<uint64_t>(L.planes), B.at<double>(L.alpha), B.at<void>(L.lgT),
+                             nullptr, nullptr, nullptr, s));
+    CK(bn::launch_set_scores(P, data_dev, B.at<uint8_t>(L.arity), B.at<uint64_t>(L.planes),
+                             B.at<double>(L.Dvals), B.at<void>(L.lgT), B.set_scratch(), s, nullptr,
+                             B.at<int64_t>(L.dbg), rank));
+    std::vector<int64_t> own((size_t)cells);
+    CK(cudaMemcpyAsync(own.data(), B.at<char>(L.dbg), (size_t)cells * 8, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    // to the family's order: parents' configuration times r_i plus x_i
+    for (int64_t c0 = 0; c0 < cells; ++c0) {
+        int64_t rest = c0, cfg = 0, stride = 1, xi = 0;
+        for (int p = 0; p < P.n; ++p) {
+            if (!(set >> p & 1u)) continue;
+            const int64_t r = hj.arity[p], dig = rest % r;
+            rest /= r;
+            if (p == i) {
+                xi = dig;
+            } else {
+                cfg += dig * stride;
+                stride *= r;
+            }
+        }
+        counts[cfg * hj.arity[i] + xi] = own[(size_t)c0];
+    }
     c->have_last = false;
     c->tables_sig.clear();
     return BN_OK;
@@ -1319,34 +1342,29 @@ int enqueue_steps(const Plan& G, const Layout& L, char* base, cudaStream_t s, un
         // one launch per kernel for the whole group, on the padded tables:
         // words past a job's m are empty and count nothing, rows past its
         // own are never looked up
-        CK(bn::launch_pack_planes(reinterpret_cast<const uint8_t*>(at(L.data)), G.n, G.m, G.rmax,
-                                  G.W, reinterpret_cast<uint64_t*>(at(L.planes)), s,
-                                  reinterpret_cast<const int*>(at(L.mj)), G.nj, G.js));
-        CK(bn::launch_lgamma_table(reinterpret_cast<const double*>(at(L.alpha)), G.rows, G.m,
-                                   G.fxs, at(L.lgT), s, G.nj, G.js,
-                                   reinterpret_cast<const double*>(at(L.fx)),
-                                   reinterpret_cast<const int*>(at(L.mj))));
-        CK(bn::launch_scores(G, reinterpret_cast<const uint8_t*>(at(L.arity)),
-                             reinterpret_cast<const uint64_t*>(at(L.planes)),
-                             reinterpret_cast<const double*>(at(L.Dvals)),
-                             at(L.lgT),
-                             reinterpret_cast<const double*>(at(L.log_rho)), 0,
-                             (int64_t)G.n * G.K, reinterpret_cast<uint32_t*>(at(L.masks)),
-                             reinterpret_cast<uint32_t*>(at(L.cmasks)),
-                             reinterpret_cast<double*>(at(L.logB)), nullptr, s,
-                             reinterpret_cast<const double*>(at(L.fx))));
-        CK(bn::launch_node_max(G, reinterpret_cast<const double*>(at(L.logB)),
-                               reinterpret_cast<double*>(at(L.cmax)), s));
-        CK(bn::launch_shift_scores(G, reinterpret_cast<const double*>(at(L.logB)),
-                                   reinterpret_cast<const double*>(at(L.cmax)), at(L.lbs), s));
-        if (bn::tile13_gamma_fits(G)) {
-            uint16_t* rk = reinterpret_cast<uint16_t*>(at(L.rk13));
-            CK(bn::launch_rank13_tables(G, rk, rk + 8192, s));
-        }
+        const bn::SetScratch x{reinterpret_cast<long long*>(at(L.F)), reinterpret_cast<uint32_t*>(at(L.lbs)),
+                               reinterpret_cast<unsigned long long*>(at(L.eacc))};
+        const uint8_t* data = reinterpret_cast<const uint8_t*>(at(L.data));
+        const int* mj = reinterpret_cast<const int*>(at(L.mj));
+        const double* fx = reinterpret_cast<const double*>(at(L.fx));
+        uint64_t* planes = reinterpret_cast<uint64_t*>(at(L.planes));
+        CK(bn::launch_step1_prep(G, data, planes, reinterpret_cast<const double*>(at(L.alpha)), at(L.lgT),
+                                 bn::tile13_gamma_fits(G) ? reinterpret_cast<uint16_t*>(at(L.rk13)) : nullptr,
+                                 x.enc, nullptr, s, mj, fx));
+        CK(bn::launch_scores(G, data, reinterpret_cast<const uint8_t*>(at(L.arity)), planes,
+                             reinterpret_cast<const double*>(at(L.Dvals)), at(L.lgT),
+                             reinterpret_cast<const double*>(at(L.log_rho)), nullptr, x,
+                             reinterpret_cast<uint32_t*>(at(L.masks)), reinterpret_cast<uint32_t*>(at(L.cmasks)),
+                             reinterpret_cast<double*>(at(L.logB)), s, mj, fx));
+        CK(bn::launch_shift_scores(G, reinterpret_cast<const double*>(at(L.logB)), x.enc,
+                                   reinterpret_cast<const uint32_t*>(at(L.cmasks)),
+                                   reinterpret_cast<double*>(at(L.cmax)), at(L.lbs),
+                                   bn::use_tile13_up(G) ? at(L.tab) : nullptr, s));
     }
     if (stages & 2u)
         CK(bn::launch_upzeta(G, reinterpret_cast<const uint32_t*>(at(L.cmasks)), at(L.lbs),
-                             at(L.tab), reinterpret_cast<const uint16_t*>(at(L.rk13)), at(L.A), s));
+                             at(L.tab), reinterpret_cast<const uint16_t*>(at(L.rk13)), at(L.A), s, nullptr,
+                             nullptr, true));
     if (stages & 4u) {
         if (G.frc) {
             CK(bn::launch_rows_cluster(G, at(L.A), at(L.F), at(L.Rc), s, nullptr));
@@ -1478,9 +1496,8 @@ int record_groups(bn_batch* b)
                     !(x.block == 256 || (x.kid == bn::KID_GAMMA_TABLE && x.block == 32)))
                     return BN_EINVAL;
                 switch (x.kid) {                   // kernels that loop grid-stride in x
-                case bn::KID_PACK_PLANES: case bn::KID_CHECK_DATA: case bn::KID_LGAMMA_TABLE:
-                case bn::KID_SCORES: case bn::KID_SCORES_W42: case bn::KID_SCORES_W44:
-                case bn::KID_SCORES_W84: case bn::KID_SCORES_CFG44: case bn::KID_SCORES_CFG:
+                case bn::KID_STEP1_PREP: case bn::KID_CHECK_DATA: case bn::KID_SET_HIST_WARP:
+                case bn::KID_SET_HIST_BLOCK: case bn::KID_SET_ANY: case bn::KID_FAMILIES:
                 case bn::KID_SHIFT_F: case bn::KID_SHIFT_D: case bn::KID_EDGES_ACC_F:
                 case bn::KID_EDGES_ACC_D: case bn::KID_REORDER_F: case bn::KID_REORDER_D:
                 case bn::KID_COLW_F: case bn::KID_COLW_D:
@@ -1669,9 +1686,8 @@ int tune_persistent(bn_batch* b, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1)
 // The autotuner.  The groups of a batch run at the same time, so a kernel
 // that wins alone (by spreading over the whole GPU) can lose in the mix; the
 // objective is therefore the time of the whole batch, on its own data.
-// Starting from the default schedules, each knob in turn -- step 1 score
-// kernel, step 2 tiles, step 3 rows, step 3 cluster kernel, step 4 tiles --
-// is switched to its alternative for three sets of groups where it fits
+// Starting from the default schedules, each knob in turn -- step 2 tiles,
+// step 3 rows, step 3 cluster kernel, step 4 tiles -- is switched to its alternative for three sets of groups where it fits
 // (all, those with n <= 14, those with n > 14); the fastest batch is kept
 // when it beats the current one by more than 1%.
 int tune_batch(bn_batch* b, cudaStream_t s)
@@ -1682,14 +1698,13 @@ int tune_batch(bn_batch* b, cudaStream_t s)
         return BN_ECUDA;
     }
     struct Knob { int Plan::*flag; bool (*fits)(const Plan&); };
-    const Knob knobs[5] = {{&Plan::scfg, bn::scores_cfg_fits}, {&Plan::up13, bn::tile13_up_fits},
-                           {&Plan::frows, bn::rows_levels_fit}, {&Plan::frc, bn::rows_levels_fit},
+    const Knob knobs[4] = {{&Plan::up13, bn::tile13_up_fits}, {&Plan::frows, bn::rows_levels_fit}, {&Plan::frc, bn::rows_levels_fit},
                            {&Plan::g13, bn::tile13_gamma_fits}};
     const bool forced_frc = (b->ctx->flags & BN_CTX_CLUSTER_STEP3) != 0;
     float best = 0.0f;
     int rc = time_batch(b, s, e0, e1, &best);
     b->ms_default = best;
-    for (int k = 0; rc == BN_OK && k < 5; ++k) {
+    for (int k = 0; rc == BN_OK && k < 4; ++k) {
         if (knobs[k].flag == &Plan::frc && forced_frc) continue;
         std::vector<Plan> keep;
         for (auto& g : b->groups) keep.push_back(g.P);
@@ -1766,6 +1781,7 @@ try {
         g.P.W = std::max(g.P.W, P.W);
         g.P.rmax = std::max(g.P.rmax, P.rmax);
         g.P.rows = std::max(g.P.rows, P.rows);
+        for (int s = 0; s < 33; ++s) g.P.states[s] = std::max(g.P.states[s], P.states[s]);
     }
     size_t total = 0;
     for (auto& g : b->groups) {
@@ -1833,16 +1849,15 @@ try {
         if (all_cached) {
             for (auto& g : b->groups) {
                 const auto& v = c->tuned[key_of(g.P)];
-                g.P.scfg = v[0];
-                g.P.up13 = v[1];
-                g.P.frows = v[2];
-                g.P.frc = v[3];
-                g.P.g13 = v[4];
+                g.P.up13 = v[0];
+                g.P.frows = v[1];
+                g.P.frc = v[2];
+                g.P.g13 = v[3];
             }
         } else {
             ok = tune_batch(b, cap) == BN_OK;
             for (const auto& g : b->groups)
-                if (ok) c->tuned[key_of(g.P)] = {g.P.scfg, g.P.up13, g.P.frows, g.P.frc, g.P.g13};
+                if (ok) c->tuned[key_of(g.P)] = {g.P.up13, g.P.frows, g.P.frc, g.P.g13};
         }
     }
     ok = ok && cudaStreamSynchronize(cap) == cudaSuccess;
@@ -1928,10 +1943,10 @@ try {
     char line[256];
     for (const auto& g : b->groups) {
         std::snprintf(line, sizeof line,
-                      "n=%d d=%d %s %s jobs=%d scfg=%d up13=%d frows=%d frc=%d g13=%d %s"
+                      "n=%d d=%d %s %s jobs=%d up13=%d frows=%d frc=%d g13=%d %s"
                       " batch_ms(default %.3f tuned %.3f)\n",
                       g.P.n, g.P.d, g.P.prec == 0 ? "fp64" : "fp32",
-                      g.P.allbin ? "binary" : "general", g.P.nj, g.P.scfg, g.P.up13, g.P.frows,
+                      g.P.allbin ? "binary" : "general", g.P.nj, g.P.up13, g.P.frows,
                       g.P.frc, g.P.g13, g.timed ? "timed" : "default-or-cached", b->ms_default,
                       b->ms_tuned);
         s += line;
@@ -2180,10 +2195,10 @@ try {
     *unit = 0;
 #ifdef BN_CHECK_BOUNDS
     CK(cudaDeviceSynchronize());
-    const unsigned int v[4] = {bn::bounds_line_kernels(), bn::bounds_line_tile13(),
+    const unsigned int v[5] = {bn::bounds_line_scores(), bn::bounds_line_kernels(), bn::bounds_line_tile13(),
                                bn::bounds_line_levels(), bn::bounds_line_mega()};
     *line = 0;
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 5; ++k) {
         if (v[k] == ~0u) return BN_ECUDA;
         if (v[k] && *unit == 0) {
             *line = (int32_t)v[k];
@@ -2328,7 +2343,7 @@ try {
                              B.at<uint16_t>(L.rk13), sh->slab + sh->o_A, s, nullptr, B.at<int>(L.err)));
         CK(bn::launch_top_slabs(V, P.shard_k, sh->slab + sh->o_A, sh->slab + sh->o_top, s));
     } else {
-        rc = enqueue_upzeta(P, B, B.at<void>(L.lbs), s, &nl, nullptr);
+        rc = enqueue_upzeta(P, B, B.at<void>(L.lbs), s, &nl, nullptr, true);
         if (rc) return rc;
     }
     if (P.prec != 0) {                        // every rank starts both sweeps' level words

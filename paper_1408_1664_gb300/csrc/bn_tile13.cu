@@ -1548,12 +1548,6 @@ size_t gamma13_smem_bytes(const Plan& P)
     return (size_t)TN * (2 * es) + 16;
 }
 
-cudaError_t launch_rank13_tables(const Plan& P, uint16_t* rank13, uint16_t* unrank13, cudaStream_t s)
-{
-    launch_or_record(KID_RANK13, k_rank13_tables, dim3(TN / 256, P.nj), 256, 0, s, rank13, unrank13, P.js);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_reorder_up(const Plan& P, const void* lbs, void* tab, cudaStream_t s)
 {
     const int64_t total = (int64_t)up_nodes(P) * P.K;
