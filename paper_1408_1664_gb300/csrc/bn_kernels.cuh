@@ -149,7 +149,7 @@ struct Plan {
     int up13 = 0;         // step 2 by the 13-dimension tiles (n >= 14)
     int g13 = 0;          // step 4 phase 1 by the 13-dimension tiles (n >= 14)
     int frows = 0;        // FP32 step 3 by the 16-subset row kernels
-    int frc = 0;          // FP32 step 3 of a batch group by the persistent cluster kernel
+    int frc = 0;          // FP32 step 3 of a batch group by k_sweeps (one launch)
     // Batch groups: nj jobs with equal plans, their arrays js bytes apart;
     // the launches of steps 2-5 cover all of them (gridDim.y = nj).
     int nj = 1;
@@ -303,10 +303,14 @@ cudaError_t launch_fold_scores(const Plan& P, int nl, int64_t Kv, uint32_t r, co
 cudaError_t launch_top_slabs(const Plan& V, int k, const void* Av, void* Atop, cudaStream_t s);
 cudaError_t launch_level_rows(const Plan& P, uint32_t r, int hl, void* X, void* buf, int dir,
                               cudaStream_t s);
-// F and R' of every job of a batch group in one persistent launch of
-// thread-block clusters (FP32, rows_levels_fit); one launch.
-cudaError_t launch_rows_cluster(const Plan& P, const void* A, void* F, void* Rc, cudaStream_t s,
-                                int* launches);
+// F and R' in one launch (k_sweeps): FP32 plans with the row schedule, whole
+// jobs with A in device memory.  use_sweeps: whether a single job's direct
+// launches take it; err is the job's error word, the first of 256 bytes that
+// also hold the sweeps' counters.  Rc null: F alone.
+bool sweeps_fit(const Plan& P);
+bool use_sweeps(const Plan& P, const int* err);
+cudaError_t launch_sweeps(const Plan& P, const void* A, void* F, void* Rc, cudaStream_t s, int* err,
+                          int* launches);
 cudaError_t launch_backward_rows(const Plan& P, const void* A, void* Rc, cudaStream_t s,
                                  int* launches);
 cudaError_t launch_forward(const Plan& P, const void* A, void* F, cudaStream_t s, int* launches);
@@ -354,8 +358,8 @@ inline bool use_tile13_gamma(const Plan& P) { return P.g13 != 0; }
 inline bool use_rows_levels(const Plan& P) { return P.frows != 0; }
 inline bool needs_rank13(const Plan& P) { return P.up13 || P.g13; }
 // A in tile-level row order (see bn_device.cuh): FP32 with the 13-dimension
-// up-zeta tiles and the step-3 row kernels (not the cluster kernel).
-inline bool use_tlo(const Plan& P) { return P.prec != 0 && P.up13 && P.frows && !P.frc; }
+// up-zeta tiles and the step-3 row kernels or k_sweeps.
+inline bool use_tlo(const Plan& P) { return P.prec != 0 && P.up13 && P.frows; }
 // The default schedule: every specialised kernel that fits.
 inline void default_schedule(Plan& P)
 {

@@ -29,6 +29,11 @@ namespace {
 constexpr int LB = 4;             // low bits of an FP32 tile
 constexpr int LB64 = 3;           // low bits of an FP64 tile
 constexpr int BT = 29;            // binomial table rows (n - B < 29: n <= 32 in FP32)
+// k_sweeps: single jobs up to this n; levels wider than kSweepGrid tiles run
+// on the whole GPU; polls before a block gives up a wait (about 1 us each).
+constexpr int kSweepMaxN = 21;
+constexpr uint64_t kSweepGrid = 400;
+constexpr uint32_t kSweepSpinCap = 1u << 22;
 
 __device__ const BinomTable g_binom_lanes = make_binom_table();
 
@@ -293,27 +298,6 @@ __device__ __forceinline__ void level_words_start(int* lw, int level, float mx)
     lw[level] = level_floor(mx);
 }
 
-__device__ __forceinline__ void cluster_barrier()
-{
-    // every thread of every block of the cluster; release/acquire at cluster
-    // scope orders the tiles written before it against the reads after it
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ uint32_t cluster_blocks()
-{
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-
 }  // namespace
 
 // FP32: 16-subset tiles at three blocks per SM (80 registers); FP64:
@@ -387,55 +371,217 @@ k_backward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __re
     }
 }
 
-// Step 3 of a whole batch group in one persistent launch of thread-block
-// clusters (1 to 8 blocks, by the width of the widest level).  Work item it is F (it even) or R' (it odd) of job it / 2; the
-// clusters take the items in turn (item = cluster id, + clusters, ...).  A
-// cluster runs every popcount level of its item: its blocks' threads split
-// the level's tiles, then meet at a cluster barrier before the next level.
-// The blocks of a cluster are resident together by construction, and no
-// cluster waits for another, so every barrier completes.  Every thread
-// reaches every barrier: the item loop and the level loop are uniform
-// across the cluster.  F and R' tiles written in the launch are read
-// through L2 (another block, on another SM, wrote them).
-__global__ void __launch_bounds__(256, 2)
-k_rows_cluster(int n, int items, const float* __restrict__ A, float* __restrict__ F,
-               float* __restrict__ Rc, size_t js)
+// F and R' of one or more jobs in one launch, every popcount level of a sweep
+// separated by a barrier of the blocks that share it, instead of a launch per
+// level.  A level launch of a job up to n of about 20 took 9 to 12 us, nearly
+// all of it latency: the launch itself and one thread walking a tile's terms,
+// each a dependent pair of row loads.  Here a tile's 16 subsets take 16 lanes
+// (one value each), a lane issues the loads of up to eight terms together,
+// and the first tile's index and A values for the next level are fetched
+// between arriving at the barrier and waiting on it.  The sums run in the
+// order of forward_tile / backward_tile, so the results are the same bits.
+//
+// Item it (2 per job: F, then R') is shared by nb blocks.  R' is F's recursion
+// read from the full set down: with bits = the elements of S (F) or the
+// missing ones (R'), step st takes the tiles with st of them, a term per
+// element j reads A_j at S without j and the neighbour tile S ^ {j}.
+//
+// SYNC 0: nb = 1, the block's own barrier.  SYNC 1: the item's blocks are one
+// thread-block cluster (co-resident by construction; hardware barrier).
+// SYNC 2: a cooperative launch (all blocks resident); a block arrives by an
+// atomic on its sweep's counter and polls it, at most `cap` times: past that
+// it sets kErrDeviceTimeout in *err and returns, and so does every other block
+// of the sweep when its own wait runs out.  sync[0] / sync[16] count the
+// arrivals of F / R', sync[8] / sync[24] the blocks done (the last resets
+// both); they start at zero (k_step1_prep).
+enum { SYNC_BLOCK = 0, SYNC_CLUSTER = 1, SYNC_GRID = 2 };
+constexpr int kSweepThreads = 512;
+
+template <typename T, bool TLO, int SYNC>
+__global__ void __launch_bounds__(kSweepThreads, 2)
+k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restrict__ Rc, size_t js,
+         unsigned* __restrict__ sync, int* __restrict__ err, uint32_t cap)
 {
+    constexpr int LN = 1 << LB, CH = 8;
+    constexpr bool kBases = sizeof(T) == 4;
+    using L = LogOps<T>;
     __shared__ uint32_t bt[BT][BT];
+    __shared__ int wm[kSweepThreads / 32];
+    __shared__ int ok_s;
     fill_table(bt);
     __syncthreads();
+    // the empty accumulator: far enough below any value that the first term
+    // replaces it, finite so that a left-out term (x = -inf) changes nothing
+    const T none = (T)-3.0e38f;
+    const int it = (int)(blockIdx.x / (unsigned)nb);
+    const uint32_t rank = blockIdx.x % (unsigned)nb;
+    const bool fwd = (it & 1) == 0;
+    const size_t off = (size_t)(it >> 1) * js;
+    A = reinterpret_cast<const T*>(reinterpret_cast<const char*>(A) + off);
+    T* X = reinterpret_cast<T*>(reinterpret_cast<char*>(fwd ? F : Rc) + off);
     const int nh = n - LB;
-    const uint32_t cs = cluster_blocks();
-    const uint32_t cid = blockIdx.x / cs;
-    const uint32_t ncl = gridDim.x / cs;
-    const uint32_t t0 = cluster_rank() * blockDim.x + threadIdx.x;
-    const uint32_t stride = cs * blockDim.x;
-    for (int it = (int)cid; it < items; it += (int)ncl) {
-        const size_t off = (size_t)(it >> 1) * js;
-        const float* Aj = reinterpret_cast<const float*>(reinterpret_cast<const char*>(A) + off);
-        const bool fwd = (it & 1) == 0;
-        float* X = reinterpret_cast<float*>(reinterpret_cast<char*>(fwd ? F : Rc) + off);
-        // the per-level bases of the level kernels, with the level words
-        // read after the cluster barrier that ends the level before
-        int* lw = level_words(X, n);
-        for (int st = 0; st <= nh; ++st) {
-            const int hl = fwd ? st : nh - st;
-            const uint32_t nt = bt[nh][hl];
-            const float rebase = st == 0 ? 0.f : (float)level_delta(lw, fwd ? hl - 1 : hl + 1);
-            float mx = LogOps<float>::ninf();
-            for (uint32_t g = t0; g < nt; g += stride) {
-                const uint32_t Ht = tile_of(g, hl, nh, bt);
-                const float m1 = fwd ? forward_tile<float, LD_L2, LB>(n, Ht, Aj, X, rebase)
-                                     : backward_tile<float, LD_L2, LB>(n, Ht, Aj, X, rebase);
-                mx = m1 > mx ? m1 : mx;
+    const uint32_t hmask = (1u << nh) - 1u;
+    const size_t half = (size_t)1 << (n - 1), full = (size_t)1 << n;
+    const int l = threadIdx.x & (LN - 1);
+    const uint32_t own = fwd ? (uint32_t)l : (uint32_t)l ^ (LN - 1);   // the lane's in-tile elements
+    const int size = __popc(own);
+    // half warps number across the blocks: a narrow level spreads over them
+    const uint32_t hw = (threadIdx.x >> LB) * (uint32_t)nb + rank;
+    const uint32_t nhw = (blockDim.x >> LB) * (uint32_t)nb;
+    int* lw = kBases ? level_words(reinterpret_cast<float*>(X), n) : nullptr;
+    unsigned* arr = SYNC == SYNC_GRID ? sync + (fwd ? 0 : 16) : nullptr;
+
+    // place of element l of row S-without-j of A_{LB + j}, and of the row of
+    // A_i (i < LB) that the tile's in-tile terms read
+    auto a_at = [&](uint32_t H, int j) {
+        const uint32_t R = squeeze(H, j);
+        return BN_AT((size_t)(LB + j) * half + ((size_t)(TLO ? tlo_row(R, 9) : R) << LB) + l, 1, n * half);
+    };
+    auto in_at = [&](uint32_t H, int i) {
+        return BN_AT((size_t)i * half + ((size_t)(TLO ? tlo_row(H, 10) : H) << (LB - 1)) + squeeze4(l, i), 1,
+                     n * half);
+    };
+    // a half warp's run of tiles in step st: consecutive in colex order, so
+    // only the first is unranked.  Its bits, the A values of its first terms
+    // and of its in-tile terms are fetched ahead of the step.
+    uint32_t bits = 0, g0 = 0, g1 = 0;
+    T pa[CH], pi[LB];
+    auto load_a = [&](uint32_t H, uint32_t& rest, int st, T (&a)[CH]) {
+#pragma unroll
+        for (int q = 0; q < CH; ++q) {
+            if (q < st) {
+                a[q] = __ldcs(A + a_at(H, __ffs(rest) - 1));
+                rest &= rest - 1;
             }
-            if (st == 0) {
-                if (t0 == 0) level_words_start(lw, hl, mx);   // the level's one tile
-            } else {
-                block_level_max(lw + hl, mx);
-            }
-            cluster_barrier();
         }
+    };
+    auto ahead = [&](int st) {
+        const uint32_t nt = bt[nh][st], run = (nt + nhw - 1) / nhw;
+        g0 = hw * run;
+        g1 = min(nt, g0 + run);
+        if (g0 >= g1) return;
+        bits = tile_of(g0, st, nh, bt);
+        const uint32_t H = fwd ? bits : hmask ^ bits;
+        uint32_t rest = bits;
+        load_a(H, rest, st, pa);
+#pragma unroll
+        for (int i = 0; i < LB; ++i) pi[i] = __ldcs(A + in_at(H, i));
+    };
+    ahead(0);
+    for (int st = 0; st <= nh; ++st) {
+        T mx = L::ninf();
+        T rebase = T(0);
+        if constexpr (kBases)
+            if (st > 0) {
+                const int w = SYNC == SYNC_BLOCK ? *(volatile int*)(lw + (fwd ? st - 1 : nh - st + 1))
+                                                 : __ldcg(lw + (fwd ? st - 1 : nh - st + 1));
+                rebase = w == kLevelUnset ? T(0) : (T)w;
+            }
+        for (uint32_t g = g0; g < g1; ++g) {
+            const uint32_t H = fwd ? bits : hmask ^ bits;
+            uint32_t ra = bits, rf = bits;
+            T m = none, s = T(0);
+            for (int c0 = 0; c0 < st; c0 += CH) {
+                T a[CH], f[CH];
+#pragma unroll
+                for (int q = 0; q < CH; ++q) {
+                    f[q] = L::ninf();
+                    if (c0 + q < st) {
+                        const T* p = X + BN_AT(((size_t)(H ^ (rf & (0u - rf))) << LB) + l, 1, full);
+                        rf &= rf - 1;
+                        f[q] = SYNC == SYNC_BLOCK ? *p : __ldcg(p);
+                    }
+                }
+                if (g == g0 && c0 == 0) {
+#pragma unroll
+                    for (int q = 0; q < CH; ++q) {
+                        a[q] = pa[q];
+                        ra &= ra - 1;
+                    }
+                } else {
+                    load_a(H, ra, st - c0, a);
+                }
+#pragma unroll
+                for (int q = 0; q < CH; ++q) lazy_add(m, s, c0 + q < st ? a[q] + f[q] : L::ninf());
+            }
+            m -= rebase;
+            T ai[LB];
+#pragma unroll
+            for (int i = 0; i < LB; ++i) ai[i] = g == g0 ? pi[i] : __ldcs(A + in_at(H, i));
+            // the in-tile terms, in popcount order of the lane's elements: in
+            // round k the lanes with k elements add theirs (the others a left-out
+            // term, so the lanes of a warp stay together)
+            T v = st == 0 ? T(0) : m + L::lg(s);
+#pragma unroll
+            for (int k = 1; k <= LB; ++k) {
+#pragma unroll
+                for (int i = 0; i < LB; ++i) {
+                    const T y = __shfl_xor_sync(0xffffu << (threadIdx.x & 16), v, 1 << i);
+                    lazy_add(m, s, size == k && (own >> i & 1) ? ai[i] + y : L::ninf());
+                }
+                v = size == k ? m + L::lg(s) : v;
+            }
+            X[BN_AT(((size_t)H << LB) + l, 1, full)] = v;
+            mx = v > mx ? v : mx;
+            if (g + 1 < g1) {                       // the next tile of the run
+                const uint32_t u = bits & (0u - bits), w = bits + u;
+                bits = w | (((w ^ bits) >> 2) >> (__ffs(u) - 1));
+            }
+        }
+        // the level's largest value, for the next level's base
+        if constexpr (kBases) {
+            const int lv = fwd ? st : nh - st;
+            if (st == 0) {
+                // the one tile of the first level: its lanes' maximum
+                if (hw == 0) {
+                    for (int o = LN / 2; o; o >>= 1) {
+                        const T y = __shfl_xor_sync(0xffffu, mx, o);
+                        mx = y > mx ? y : mx;
+                    }
+                    if (l == 0) level_words_start(lw, lv, mx);
+                }
+            } else {
+                int v = __reduce_max_sync(0xffffffffu, level_floor(mx));
+                if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = v;
+                __syncthreads();
+                if (threadIdx.x < 32) {
+                    v = threadIdx.x < (blockDim.x >> 5) ? wm[threadIdx.x] : kLevelUnset;
+                    v = __reduce_max_sync(0xffffffffu, v);
+                    if (threadIdx.x == 0 && v != kLevelUnset) atomicMax(lw + lv, v);
+                }
+            }
+        }
+        if (st == nh) break;
+        if constexpr (SYNC == SYNC_CLUSTER) {
+            asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+            ahead(st + 1);
+            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        } else {
+            __syncthreads();
+            if (SYNC == SYNC_GRID && threadIdx.x == 0) {
+                __threadfence();
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arr) : "memory");
+            }
+            ahead(st + 1);
+            if constexpr (SYNC == SYNC_GRID) {
+                if (threadIdx.x == 0) {
+                    const unsigned need = (unsigned)nb * (unsigned)(st + 1);
+                    uint32_t k = 0;
+                    unsigned v;
+                    do {
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arr) : "memory");
+                    } while (v < need && ++k < cap);
+                    if (v < need) atomicOr(err, kErrDeviceTimeout);
+                    ok_s = v >= need;
+                }
+                __syncthreads();
+                if (!ok_s) return;
+            }
+        }
+    }
+    if (SYNC == SYNC_GRID && threadIdx.x == 0 && atomicAdd(arr + 8, 1u) == (unsigned)nb - 1u) {
+        arr[0] = 0u;                                // every block has passed its last wait
+        arr[8] = 0u;
     }
 }
 
@@ -745,31 +891,62 @@ cudaError_t launch_backward_rows(const Plan& P, const void* A, void* Rc, cudaStr
     return cudaSuccess;
 }
 
-cudaError_t launch_rows_cluster(const Plan& P, const void* A, void* F, void* Rc, cudaStream_t s,
-                                int* launches)
+// Blocks that share one item of k_sweeps and how they meet.  One block of 512
+// threads holds 32 tiles at a time: levels of up to 64 tiles (n <= 11) gain
+// nothing from a second one.  Clusters (at most 8 blocks, the portable size)
+// serve the middle and every batch group; from kSweepGrid tiles in the widest
+// level on the whole GPU shares the two sweeps of a single job (err given).
+static int sweep_blocks(uint64_t widest, const int* err)
 {
-    // blocks per cluster: one 256-thread block per 256 tiles of the largest
-    // level, at most 8 (the portable cluster size)
-    const int nh = P.n - LB;
-    const uint64_t widest = choose(nh, nh / 2);
-    const unsigned kCluster = (unsigned)std::min<uint64_t>(8, (widest + 255) / 256);
-    const int items = 2 * P.nj;
-    // at most two blocks per SM: 152 * 2 blocks at once
-    const unsigned clusters = (unsigned)std::min(items, 152 * 2 / (int)kCluster);
+    // the whole-GPU form needs the counters beside the job's error word
+    const uint64_t most = err && widest > kSweepGrid ? 152 : 8;
+    return (int)std::max<uint64_t>(1, std::min<uint64_t>((widest + 31) / 32, most));
+}
+
+bool sweeps_fit(const Plan& P)
+{
+    return rows_levels_fit(P) && P.frows && P.shard_k == 0 && !P.slab && !P.spill;
+}
+
+bool use_sweeps(const Plan& P, const int* err)
+{
+    return sweeps_fit(P) && P.n <= kSweepMaxN && err && !recording();
+}
+
+template <typename T, bool TLO>
+static cudaError_t sweeps(const Plan& P, const T* A, T* F, T* Rc, int items, cudaStream_t s, int* err)
+{
+    const uint64_t widest = choose(P.n - LB, (P.n - LB) / 2);
+    const int nb = sweep_blocks(widest, err);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(clusters * kCluster, 1, 1);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = 0;
+    cfg.gridDim = dim3((unsigned)(items * nb), 1, 1);
+    cfg.blockDim = dim3(kSweepThreads, 1, 1);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kCluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_rows_cluster, P.n, items, (const float*)A, (float*)F,
-                                       (float*)Rc, P.js);
+    cfg.numAttrs = nb > 1 ? 1 : 0;
+    unsigned* sync = err ? reinterpret_cast<unsigned*>(err) + 16 : nullptr;
+    if (nb == 1)
+        return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_BLOCK>, P.n, nb, A, F, Rc, P.js, sync, err, 0u);
+    if (nb <= 8) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = nb;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_CLUSTER>, P.n, nb, A, F, Rc, P.js, sync, err, 0u);
+    }
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_GRID>, P.n, nb, A, F, Rc, P.js, sync, err,
+                              kSweepSpinCap);
+}
+
+cudaError_t launch_sweeps(const Plan& P, const void* A, void* F, void* Rc, cudaStream_t s, int* err,
+                          int* launches)
+{
+    const int items = Rc ? 2 * P.nj : 1;            // a feature's job: F alone
+    const cudaError_t e = use_tlo(P) ? sweeps<float, true>(P, (const float*)A, (float*)F, (float*)Rc, items, s, err)
+                                     : sweeps<float, false>(P, (const float*)A, (float*)F, (float*)Rc, items, s, err);
     if (e == cudaSuccess && launches) ++*launches;
     return e;
 }

@@ -201,7 +201,7 @@ try {
     const size_t o_data = take((size_t)P.m * P.n), o_ar = take(P.n),
                  o_lr = take((size_t)(P.d + 1) * 8), o_tab = take((size_t)2 * rows * 8),
                  o_lgT = take((size_t)rows * (P.m + 1) * 8),
-                 o_pl = take((size_t)P.n * P.rmax * P.W * 8), o_err = take(4),
+                 o_pl = take((size_t)P.n * P.rmax * P.W * 8), o_err = take(256),
                  o_masks = take(nK * 4), o_cm = take(nK * 4), o_logB = take(nK * 8),
                  o_cmax = take((size_t)P.n * 8), o_lbs = take(nK * es),
                  o_reo = take(bn::use_tile13_up(P) ? nK * es : 0),
@@ -252,8 +252,12 @@ try {
     CKS(bn::launch_shift_scores(P, logB, x.enc, cm, cmax, base + o_lbs,
                                 bn::use_tile13_up(P) ? base + o_reo : nullptr, s));
     CKS(bn::launch_upzeta(P, cm, base + o_lbs, base + o_reo, rk13, base + o_A, s, nullptr, nullptr, true));
-    CKS(bn::launch_forward(P, base + o_A, base + o_F, s, nullptr));
-    CKS(bn::launch_backward(P, base + o_A, base + o_Rc, s, nullptr));
+    if (bn::use_sweeps(P, err)) {
+        CKS(bn::launch_sweeps(P, base + o_A, base + o_F, base + o_Rc, s, err, nullptr));
+    } else {
+        CKS(bn::launch_forward(P, base + o_A, base + o_F, s, nullptr));
+        CKS(bn::launch_backward(P, base + o_A, base + o_Rc, s, nullptr));
+    }
     CKS(bn::launch_gamma_p1(P, base + o_F, base + o_Rc, rk13, base + o_W, s, nullptr, base + o_A));
     CKS(bn::launch_gamma_p2(P, base + o_W, base + o_G, s));
     CKS(bn::launch_edges(P, logB, cmax, masks, base + o_G, base + o_F, err,

@@ -87,7 +87,7 @@ Layout make_layout(const Plan& P, size_t dbg_cells, bool feature = false)
     L.alpha = take((size_t)P.rows * 8);
     L.lgT = take((size_t)P.rows * (P.m + 1) * 8);
     L.planes = take((size_t)P.n * P.rmax * P.W * 8);
-    L.err = take(4);
+    L.err = take(256);               // the error word, then the counters of k_sweeps
     L.masks = take(nK * 4);
     L.cmasks = take(nK * 4);
     L.logB = take(nK * 8);
@@ -426,7 +426,14 @@ int enqueue_kernels(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, d
     if (rc) return rc;
     int* err = B.at<int>(L.err);
     if (ev) CK(cudaEventRecord(ev->ev[2], s));
-    if (side && side->s) {
+    const bool one = bn::use_sweeps(P, err);        // F and R' in one launch
+    if (one) {
+        CK(bn::launch_sweeps(P, B.A(), B.at<void>(L.F), B.at<void>(L.Rc), s, err, &nl));
+        if (ev) {
+            CK(cudaEventRecord(ev->ev[3], s));
+            CK(cudaEventRecord(ev->ev[kEvR], s));
+        }
+    } else if (side && side->s) {
         CK(cudaEventRecord(side->fork, s));
         CK(cudaStreamWaitEvent(side->s, side->fork, 0));
         CK(bn::launch_backward(P, B.A(), B.at<void>(L.Rc), side->s, &nl));
@@ -443,7 +450,7 @@ int enqueue_kernels(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, d
     }
     if (ev) {
         CK(cudaEventRecord(ev->ev[4], s));
-        ev->overlap = side && side->s;
+        ev->overlap = one || (side && side->s);
     }
     if (P.vgroup) {
         // step 4 a group of endpoints at a time through one group's W (the
@@ -1092,11 +1099,17 @@ try {
     const size_t es = P.prec == 0 ? 8 : 4;
     const size_t full = ((size_t)1 << P.n) - 1;
     int nl = 0;
+    auto forward = [&] {
+        int* err = B.at<int>(L.err);
+        return bn::use_sweeps(P, err)
+                   ? bn::launch_sweeps(P, B.at<void>(L.A), B.at<void>(L.F), nullptr, s, err, &nl)
+                   : bn::launch_forward(P, B.at<void>(L.A), B.at<void>(L.F), s, &nl);
+    };
     rc = enqueue_step1(hj, B, data_dev, s, &nl);
     if (rc) return rc;
     rc = enqueue_upzeta(P, B, B.at<void>(L.lbs), s, &nl, nullptr, true);
     if (rc) return rc;
-    CK(bn::launch_forward(P, B.at<void>(L.A), B.at<void>(L.F), s, &nl));
+    CK(forward());
     double fv[2] = {0.0, 0.0};
     char raw[2][8];
     int lw[2][bn::kLevelWords];                  // FP32: the level words of each run's F
@@ -1107,7 +1120,7 @@ try {
     CK(bn::launch_add_feature(P, B.at<void>(L.lbs), B.at<void>(L.logf), B.at<void>(L.lbsf), s));
     rc = enqueue_upzeta(P, B, B.at<void>(L.lbsf), s, &nl, nullptr, false);
     if (rc) return rc;
-    CK(bn::launch_forward(P, B.at<void>(L.A), B.at<void>(L.F), s, &nl));
+    CK(forward());
     CK(cudaMemcpyAsync(raw[1], B.at<char>(L.F) + full * es, es, cudaMemcpyDeviceToHost, s));
     if (P.prec != 0)
         CK(cudaMemcpyAsync(lw[1], B.at<char>(L.F) + (full + 1) * es, sizeof(lw[1]),
@@ -1367,7 +1380,7 @@ int enqueue_steps(const Plan& G, const Layout& L, char* base, cudaStream_t s, un
                              nullptr, true));
     if (stages & 4u) {
         if (G.frc) {
-            CK(bn::launch_rows_cluster(G, at(L.A), at(L.F), at(L.Rc), s, nullptr));
+            CK(bn::launch_sweeps(G, at(L.A), at(L.F), at(L.Rc), s, nullptr, nullptr));
         } else if (side && side->s) {
             CK(cudaEventRecord(side->fork, s));
             CK(cudaStreamWaitEvent(side->s, side->fork, 0));
@@ -1687,7 +1700,7 @@ int tune_persistent(bn_batch* b, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1)
 // that wins alone (by spreading over the whole GPU) can lose in the mix; the
 // objective is therefore the time of the whole batch, on its own data.
 // Starting from the default schedules, each knob in turn -- step 2 tiles,
-// step 3 rows, step 3 cluster kernel, step 4 tiles -- is switched to its alternative for three sets of groups where it fits
+// step 3 rows, step 3 in one launch, step 4 tiles -- is switched to its alternative for three sets of groups where it fits
 // (all, those with n <= 14, those with n > 14); the fastest batch is kept
 // when it beats the current one by more than 1%.
 int tune_batch(bn_batch* b, cudaStream_t s)
@@ -1698,7 +1711,7 @@ int tune_batch(bn_batch* b, cudaStream_t s)
         return BN_ECUDA;
     }
     struct Knob { int Plan::*flag; bool (*fits)(const Plan&); };
-    const Knob knobs[4] = {{&Plan::up13, bn::tile13_up_fits}, {&Plan::frows, bn::rows_levels_fit}, {&Plan::frc, bn::rows_levels_fit},
+    const Knob knobs[4] = {{&Plan::up13, bn::tile13_up_fits}, {&Plan::frows, bn::rows_levels_fit}, {&Plan::frc, bn::sweeps_fit},
                            {&Plan::g13, bn::tile13_gamma_fits}};
     const bool forced_frc = (b->ctx->flags & BN_CTX_CLUSTER_STEP3) != 0;
     float best = 0.0f;
@@ -1838,7 +1851,7 @@ try {
     // schedules: the default, forced, cached (when every group's shape is in
     // the context's cache) or timed
     for (auto& g : b->groups)
-        if (c->flags & BN_CTX_CLUSTER_STEP3) g.P.frc = bn::rows_levels_fit(g.P);
+        if (c->flags & BN_CTX_CLUSTER_STEP3) g.P.frc = bn::sweeps_fit(g.P);
     auto key_of = [](const Plan& P) {
         return std::array<int, 5>{P.n, P.d, P.prec, P.allbin, P.nj};
     };

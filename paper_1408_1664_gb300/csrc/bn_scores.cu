@@ -148,7 +148,8 @@ k_step1_prep(const uint8_t* __restrict__ data, int n, int m, int rmax, int W,
             rk[8192 + r] = (uint16_t)L;
         } else {
             if (enc && lane < n) job_ptr(enc, js)[lane] = 0ull;
-            if (err && lane == 0) *job_ptr(err, js) = 0;
+            // the error word and the counters of k_sweeps after it (256 bytes)
+            if (err) reinterpret_cast<int2*>(job_ptr(err, js))[lane] = make_int2(0, 0);
         }
     }
 }
