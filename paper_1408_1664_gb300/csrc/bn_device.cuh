@@ -462,6 +462,122 @@ template <typename T> struct LseAcc {
     }
 };
 
+// ---------------------------------------------------------------------------
+// The linear FP64 form (Plan::lin).  A value v >= 0 of the FP64 path is kept
+// itself, not its logarithm: 64 bits hold an exponent of 64 - FB bits and a
+// fraction of FB bits.  Every sum over logarithms costs an FP64 exponential
+// per term and a logarithm per result, on a pipe that retires two lanes per
+// clock and SM; here a term costs one multiplication and one fused
+// multiply-add there and integer operations on the exponents.  Values compare
+// like their bits; 0 is all zeros; anything below the smallest kept exponent
+// is 0.  Sums run in double, relative to an integer exponent.
+//   X64: FB = 46, values in 2^+-131072 (90000 nats), rounding 2^-47 = 7e-15.
+//     Used from n = 14: a stored logarithm of a few hundred nats is no more
+//     exact (its unit in the last place is 6e-14 from 256 nats on).
+//   X64S: FB = 49, values in 2^+-16384, rounding 2^-50.  Used below n = 14,
+//     where logarithms stay short and the wider fraction is needed to lose
+//     nothing against them.
+// The planner keeps the logarithms when the job's values could leave the
+// range (lin_range in bn_kernels.cuh).
+// ---------------------------------------------------------------------------
+template <int FB> struct XValue {
+    static constexpr int frac = FB;
+    static constexpr int bias = 1 << (63 - FB);
+    static constexpr int min = (FB == 46 ? 4096 : 2048) - bias;   // smallest exponent kept
+    unsigned long long u;
+};
+using X64 = XValue<46>;
+using X64S = XValue<49>;
+constexpr int kXBias = X64::bias, kXMin = X64::min;
+
+template <typename X> __host__ __device__ __forceinline__ X x_one() { return X{(unsigned long long)X::bias << X::frac}; }
+// The exponent (that of 0 is -bias: far below every sum it enters) and the
+// fraction with its leading one, in [1, 2).
+template <int FB> __device__ __forceinline__ int x_exp(XValue<FB> x) { return (int)(x.u >> FB) - XValue<FB>::bias; }
+template <int FB> __device__ __forceinline__ double x_mant(XValue<FB> x)
+{
+    return __longlong_as_double((long long)(((x.u << (52 - FB)) & 0x000fffffffffffffull) | 0x3ff0000000000000ull));
+}
+// x * 2^-ref as a double: 0 below 2^-1000, +inf above 2^1010.
+template <int FB> __device__ __forceinline__ double x_scaled(XValue<FB> x, int ref)
+{
+    const int e = x_exp(x) - ref;
+    const unsigned long long b =
+        ((x.u << (52 - FB)) & 0x000fffffffffffffull) | ((unsigned long long)(unsigned)(e + 1023) << 52);
+    return __longlong_as_double(e < -1000 ? 0ll : e > 1010 ? 0x7ff0000000000000ll : (long long)b);
+}
+// s * 2^ref (s >= 0, finite) rounded to the nearest stored value.
+template <typename X> __device__ __forceinline__ X x_pack(double s, int ref)
+{
+    constexpr int drop = 52 - X::frac;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(s) + (1ull << (drop - 1));
+    const int ex = (int)(b >> 52);
+    const int e = ex - 1023 + ref;
+    if (ex == 0 || e < X::min) return X{0ull};
+    return X{((unsigned long long)(unsigned)(e + X::bias) << X::frac) | ((b & 0x000fffffffffffffull) >> drop)};
+}
+// 2^e for an integer e <= 1023 (0 below 2^-1022).
+__device__ __forceinline__ double pow2d(int e)
+{
+    return __longlong_as_double(e < -1022 ? 0ll : (long long)(e + 1023) << 52);
+}
+template <int FB> __device__ __forceinline__ XValue<FB> x_mul(XValue<FB> a, XValue<FB> b)
+{
+    return x_pack<XValue<FB>>(x_mant(a) * x_mant(b), x_exp(a) + x_exp(b));
+}
+template <int FB> __device__ __forceinline__ XValue<FB> x_add(XValue<FB> a, XValue<FB> b)
+{
+    const XValue<FB> hi = a.u > b.u ? a : b, lo = a.u > b.u ? b : a;
+    const int e = x_exp(hi);
+    return x_pack<XValue<FB>>(fma(x_mant(lo), pow2d(x_exp(lo) - e), x_mant(hi)), e);
+}
+// exp(x) for a natural logarithm x: x = k ln 2 + r in two parts, so that the
+// fraction is as exact as x.
+template <typename X> __device__ __forceinline__ X x_from_ln(double x)
+{
+    if (!(x > -91000.0)) return X{0ull};
+    const double k = rint(x * 1.4426950408889634074);
+    double r = fma(-k, explog::kLn2Hi, x);
+    r = fma(-k, explog::kLn2Lo, r);
+    return x_pack<X>(exp_t(r), (int)k);
+}
+
+// A lazy sum: add() takes one term, value() gives the result in the array's
+// own form.  float / double: (m, s) stands for m + log(s), s rescaled only
+// when a term exceeds m by more than 64 log units, so a term costs one
+// exponential (the values are finite).  XValue: s 2^e, rescaled only when a term
+// exceeds 2^e by more than 2^500.
+template <typename T> struct LazySum {
+    T m, s;
+    __device__ __forceinline__ LazySum() : m(LogOps<T>::ninf()), s(T(0)) {}
+    __device__ __forceinline__ void add(T x)
+    {
+        const T dd = x - m;                         // +inf while the sum is empty
+        const bool big = dd > T(64);
+        const T e = LogOps<T>::ex(big ? -dd : dd);
+        if constexpr (sizeof(T) == 4) s = big ? __fmaf_rn(s, e, 1.0f) : s + e;
+        else s = big ? __fma_rn(s, e, 1.0) : s + e;
+        m = big ? x : m;
+    }
+    __device__ __forceinline__ T value() const { return m + LogOps<T>::lg(s); }
+};
+template <int FB> struct LazySum<XValue<FB>> {
+    using X = XValue<FB>;
+    int e;
+    double s;
+    __device__ __forceinline__ LazySum() : e(-(1 << 28)), s(0.0) {}
+    // p * 2^ep, p in [1, 8)
+    __device__ __forceinline__ void add(double p, int ep)
+    {
+        const int d = ep - e;
+        const bool big = d > 500;
+        s = fma(big ? s : p, pow2d(big ? -d : d), big ? p : s);
+        e = big ? ep : e;
+    }
+    __device__ __forceinline__ void add(X x) { add(x_mant(x), x_exp(x)); }
+    __device__ __forceinline__ X value() const { return x_pack<X>(s, e); }
+};
+
 // Order-preserving integer encodings for atomicMax on shared memory.
 __device__ __forceinline__ uint32_t ord_enc(float x)
 {

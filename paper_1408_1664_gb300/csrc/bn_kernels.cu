@@ -347,6 +347,13 @@ __global__ void k_gamma_table(int n, const float* __restrict__ F, float* __restr
     tab[l] = l < 30 ? off[l] : l == 30 ? __int_as_float(sh) : fvrel;
 }
 
+__device__ __forceinline__ float p2_add(float a, float b) { return LogOps<float>::lse(a, b); }
+__device__ __forceinline__ double p2_add(double a, double b) { return LogOps<double>::lse(a, b); }
+template <int FB> __device__ __forceinline__ XValue<FB> p2_add(XValue<FB> a, XValue<FB> b) { return x_add(a, b); }
+__device__ __forceinline__ void p2_zero(float& a) { a = LogOps<float>::ninf(); }
+__device__ __forceinline__ void p2_zero(double& a) { a = LogOps<double>::ninf(); }
+template <int FB> __device__ __forceinline__ void p2_zero(XValue<FB>& a) { a.u = 0ull; }
+
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_gamma_p2(int n, int d, int b, int hc, uint32_t nlow, int64_t K, const T* __restrict__ W,
@@ -356,7 +363,6 @@ k_gamma_p2(int n, int d, int b, int hc, uint32_t nlow, int64_t K, const T* __res
     if (!(vsel >> v & 1u)) return;
     W = job_ptr(W, js) + ((size_t)endpoint_slot(vsel, v) << (n - 1 - b)) * nlow;
     Gam = job_ptr(Gam, js) + (size_t)v * K;
-    using L = LogOps<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int h = n - 1 - b;
     const int hh = h - hc;
@@ -377,7 +383,7 @@ k_gamma_p2(int n, int d, int b, int hc, uint32_t nlow, int64_t K, const T* __res
         int k = 0;
         while (ro >= binom(h, k)) { ro -= binom(h, k); ++k; }
         gh[o] = colex_unrank(ro, k, h);
-        acc[o] = L::ninf();
+        p2_zero(acc[o]);
     }
     const uint32_t lowc = chunkN - 1u;
     for (uint32_t Hhi = 0; Hhi < (1u << hh); ++Hhi) {
@@ -389,13 +395,13 @@ k_gamma_p2(int n, int d, int b, int hc, uint32_t nlow, int64_t K, const T* __res
             const uint32_t jm = (1u << j) - 1u;
             for (uint32_t p = threadIdx.x; p < (chunkN >> 1); p += blockDim.x) {
                 const uint32_t lo = ((p & ~jm) << 1) | (p & jm);
-                if (__popc(lo & jm) <= dp) vals[lo] = L::lse(vals[lo], vals[lo | (1u << j)]);
+                if (__popc(lo & jm) <= dp) vals[lo] = p2_add(vals[lo], vals[lo | (1u << j)]);
             }
             __syncthreads();
         }
         for (uint32_t o = threadIdx.x; o < nout; o += blockDim.x) {
             const uint32_t G = gh[o];
-            if (((G >> hc) & ~Hhi) == 0u) acc[o] = L::lse(acc[o], vals[G & lowc]);
+            if (((G >> hc) & ~Hhi) == 0u) acc[o] = p2_add(acc[o], vals[G & lowc]);
         }
     }
     __syncthreads();
@@ -580,6 +586,20 @@ k_edges_acc(int n, int64_t K, int qbits, const double* __restrict__ logB,
     if (tid == 0) atomicAdd(&acc[(size_t)n * n + v], Nz);
 }
 
+// ln F(V) of the shifted scores.
+__device__ __forceinline__ double ln_full(const float* F, int n)
+{
+    // FP32: add the level base of F(V)
+    return LogOps<float>::to_ln((double)F[((size_t)1 << n) - 1] +
+                                level_base_fwd(level_words(F, n), n - kLevelShift));
+}
+__device__ __forceinline__ double ln_full(const double* F, int n) { return F[((size_t)1 << n) - 1]; }
+template <int FB> __device__ __forceinline__ double ln_full(const XValue<FB>* F, int n)
+{
+    const XValue<FB> f = F[((size_t)1 << n) - 1];
+    return f.u ? (double)x_exp(f) * 0.69314718055994530942 + log(x_mant(f)) : -INFINITY;
+}
+
 template <typename T>
 __global__ void k_edges_fin(int n, int use_z, int qbits, const double* __restrict__ cmax,
                             const T* __restrict__ F, const int* __restrict__ err,
@@ -607,16 +627,17 @@ __global__ void k_edges_fin(int n, int use_z, int qbits, const double* __restric
     if (threadIdx.x == 0 && log_PD) {
         double c = 0.0;
         for (int i = 0; i < n; ++i) c += cmax[i];
-        double fv = (double)F[((size_t)1 << n) - 1];
-        if (sizeof(T) == 4)                       // FP32: add the level base of F(V)
-            fv += level_base_fwd(level_words(reinterpret_cast<const float*>(F), n), n - kLevelShift);
-        *log_PD = bad ? NAN : LogOps<T>::to_ln(fv) + c;
+        *log_PD = bad ? NAN : ln_full(F, n) + c;
     }
 }
 
 // ===========================================================================
 // Priors beyond the defaults and single features (Eqs. 4-9).
 // ===========================================================================
+
+__device__ __forceinline__ void apply_weight(float& a, float w) { a += w; }
+__device__ __forceinline__ void apply_weight(double& a, double w) { a += w; }
+template <int FB> __device__ __forceinline__ void apply_weight(XValue<FB>& a, XValue<FB> w) { a = x_mul(a, w); }
 
 // A_i(S) += log q_i(S), q_i a function of |S| (Eq. 7): lq[i * n + |S|] in
 // the working precision and log base; A is [i * 2^(n-1) + c], c = S with
@@ -640,8 +661,186 @@ __global__ void k_apply_q(int n, const T* __restrict__ lq, T* __restrict__ A, in
             for (uint32_t end = 1; end <= p; end += binom(rb, k)) ++k;
             size = __popc(c >> 13) + k + __popc(c & ((1u << lw) - 1u));
         }
-        A[t] += lq[i * n + size];
+        apply_weight(A[t], lq[i * n + size]);
     }
+}
+
+// ===========================================================================
+// The linear FP64 form (XValue, bn_device.cuh) of steps 2 (n < 14),
+// 4 and 5.
+// ===========================================================================
+
+// Step 2 for n < 14: one block per node, every family in its slot of the
+// 2^(n-1) values in shared memory, then the butterflies of Algorithm 2.
+__global__ void __launch_bounds__(256)
+k_upzeta_x(int n, int64_t K, const uint32_t* __restrict__ cmasks, const X64S* __restrict__ lbs,
+           X64S* __restrict__ A, size_t js)
+{
+    cmasks = job_ptr(cmasks, js);
+    lbs = job_ptr(lbs, js);
+    A = job_ptr(A, js);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    X64S* v = reinterpret_cast<X64S*>(smem_raw);
+    const uint32_t N = 1u << (n - 1);
+    const int i = (int)blockIdx.x;
+    for (uint32_t t = threadIdx.x; t < N; t += blockDim.x) v[t] = X64S{0ull};
+    __syncthreads();
+    for (int64_t f = threadIdx.x; f < K; f += blockDim.x)
+        v[BN_AT(cmasks[(size_t)i * K + f], 1, N)] = lbs[(size_t)i * K + f];
+    __syncthreads();
+    for (int j = 0; j < n - 1; ++j) {
+        const uint32_t jm = (1u << j) - 1u;
+        for (uint32_t p = threadIdx.x; p < (N >> 1); p += blockDim.x) {
+            const uint32_t lo = ((p & ~jm) << 1) | (p & jm), hi = lo | (1u << j);
+            v[hi] = x_add(v[hi], v[lo]);
+        }
+        __syncthreads();
+    }
+    for (uint32_t t = threadIdx.x; t < N; t += blockDim.x) A[BN_AT((size_t)i * N + t, 1, (size_t)n * N)] = v[t];
+}
+
+// Step 4 phase 1 for n < 14 (k_gamma_p1): one tile per endpoint.
+__global__ void __launch_bounds__(256)
+k_gamma_p1_x(int n, int d, int b, uint32_t nlow, const X64S* __restrict__ F, const X64S* __restrict__ Rc,
+             X64S* __restrict__ W, size_t js, const X64S* __restrict__ lq, uint32_t vsel)
+{
+    const int v = blockIdx.z;
+    if (!(vsel >> v & 1u)) return;
+    F = job_ptr(F, js);
+    Rc = job_ptr(Rc, js);
+    W = job_ptr(W, js) + (size_t)endpoint_slot(vsel, v) * gridDim.x * nlow;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    X64S* vals = reinterpret_cast<X64S*>(smem_raw);
+    const uint32_t tileN = 1u << b;
+    const uint32_t H = blockIdx.x;
+    for (uint32_t t = threadIdx.x; t < tileN; t += blockDim.x) {
+        const uint32_t S = expand((H << b) | t, v);
+        X64S y = x_mul(F[BN_AT(S, 1, (size_t)1 << n)], Rc[BN_AT(S | (1u << v), 1, (size_t)1 << n)]);
+        if (lq) y = x_mul(y, lq[v * n + __popc(S)]);
+        vals[t] = y;
+    }
+    __syncthreads();
+    for (int j = 0; j < b; ++j) {
+        const uint32_t jm = (1u << j) - 1u;
+        for (uint32_t p = threadIdx.x; p < (tileN >> 1); p += blockDim.x) {
+            const uint32_t lo = ((p & ~jm) << 1) | (p & jm);
+            if (__popc(lo & jm) <= d) vals[lo] = x_add(vals[lo], vals[lo | (1u << j)]);
+        }
+        __syncthreads();
+    }
+    X64S* row = W + (size_t)H * nlow;
+    for (uint32_t t = threadIdx.x; t < tileN; t += blockDim.x)
+        if (__popc(t) <= d) row[BN_AT(small_subset_rank(t, b), 1, nlow)] = vals[t];
+}
+
+// Warp-wide sum of the lanes' LazySums, in a fixed tree order.
+template <typename X> __device__ __forceinline__ X warp_sum_x(LazySum<X> a)
+{
+    for (int o = 16; o; o >>= 1) {
+        const int e2 = __shfl_xor_sync(FULL, a.e, o);
+        const double s2 = __shfl_xor_sync(FULL, a.s, o);
+        const int m = max(a.e, e2);
+        // both lanes of a pair form the same sum (the operands swap)
+        a.s = a.s * pow2d(a.e - m) + s2 * pow2d(e2 - m);
+        a.e = m;
+    }
+    return a.value();
+}
+
+// Phase 2 for the columns with at most one high element left (k_gamma_p2s).
+// One unpacking per value of W; each sum it enters costs an aligned addition.
+template <typename X>
+__global__ void __launch_bounds__(256)
+k_gamma_p2s_x(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const X* __restrict__ W,
+              X* __restrict__ Gam, size_t js, uint32_t vsel)
+{
+    constexpr int MB = 14;                          // high bits from 5 up (h <= 18)
+    const int v = blockIdx.z;
+    if (!(vsel >> v & 1u)) return;
+    W = job_ptr(W, js) + ((size_t)endpoint_slot(vsel, v) << (n - 1 - b)) * nlow;
+    Gam = job_ptr(Gam, js) + (size_t)v * K;
+    const int h = n - 1 - b;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t col = c0 + blockIdx.x * 8 + warp;
+    if (col >= nlow) return;                        // whole warps leave
+    int kg = 0;
+    uint32_t r = col;
+    while (r >= binom(b, kg)) { r -= binom(b, kg); ++kg; }
+    const uint32_t g = colex_unrank(r, kg, b);
+    const bool one = d - kg == 1;
+    LazySum<X> s0, sb[MB];
+    const uint32_t nH = 1u << h;
+    const size_t wsize = (size_t)nlow << h;
+    X wa = lane < nH ? W[BN_AT((size_t)lane * nlow + col, 1, wsize)] : X{0ull};
+    X wb = lane + 32 < nH ? W[BN_AT((size_t)(lane + 32) * nlow + col, 1, wsize)] : X{0ull};
+    for (uint32_t H = lane; H < nH; H += 32) {
+        const double p = x_mant(wa);
+        const int e = x_exp(wa);
+        wa = wb;
+        if (H + 64 < nH) wb = W[BN_AT((size_t)(H + 64) * nlow + col, 1, wsize)];
+        s0.add(p, e);
+        if (one) {
+#pragma unroll
+            for (int q = 0; q < MB; ++q)
+                if (5 + q < h && (H >> (5 + q) & 1u)) sb[q].add(p, e);
+        }
+    }
+    const X all = warp_sum_x(s0);
+    if (lane == 0) Gam[BN_AT(family_index(g, n), 1, K)] = all;
+    if (!one) return;
+    for (int bb = 0; bb < h && bb < 5; ++bb) {
+        LazySum<X> s = s0;
+        if (!(lane >> bb & 1)) s = LazySum<X>();
+        const X x = warp_sum_x(s);
+        if (lane == 0) Gam[BN_AT(family_index(g | (1u << (b + bb)), n), 1, K)] = x;
+    }
+#pragma unroll
+    for (int q = 0; q < MB; ++q) {
+        if (5 + q >= h) break;
+        const X x = warp_sum_x(sb[q]);
+        if (lane == 0) Gam[BN_AT(family_index(g | (1u << (b + 5 + q)), n), 1, K)] = x;
+    }
+}
+
+// Step 5: e(G) = B_v(G) Gamma_v(G) / F(V) in fixed point (k_edges_acc), from
+// the shifted scores themselves.
+template <typename X>
+__global__ void __launch_bounds__(256)
+k_edges_acc_x(int n, int64_t K, int qbits, const X* __restrict__ lbs, const uint32_t* __restrict__ masks,
+              const X* __restrict__ Gam, const X* __restrict__ F, unsigned long long* __restrict__ acc,
+              size_t js, uint32_t vsel)
+{
+    if (!(vsel >> blockIdx.z & 1u)) return;
+    lbs = job_ptr(lbs, js);
+    masks = job_ptr(masks, js);
+    Gam = job_ptr(Gam, js);
+    F = job_ptr(F, js);
+    acc = job_ptr(acc, js);
+    __shared__ unsigned long long Nu[32], Nz;
+    const int v = blockIdx.z;
+    const int tid = threadIdx.x;
+    if (tid < 32) Nu[tid] = 0ull;
+    if (tid == 0) Nz = 0ull;
+    __syncthreads();
+    const X fv = F[(uint32_t)(((uint64_t)1 << n) - 1)];
+    const double inv = 1.0 / x_mant(fv);
+    const int eq = qbits - x_exp(fv);
+    unsigned long long z = 0ull;
+    for (int64_t f = blockIdx.x * (int64_t)blockDim.x + tid; f < K;
+         f += (int64_t)gridDim.x * blockDim.x) {
+        const size_t x = (size_t)v * K + f;
+        const X b = lbs[x], g = Gam[x];
+        const int e = x_exp(b) + x_exp(g) + eq;      // the term is at most 2^qbits
+        const unsigned long long q =
+            e < -8 ? 0ull : __double2ull_rn(x_mant(b) * x_mant(g) * inv * pow2d(min(e, 64)));
+        z += q;
+        for (uint32_t y = masks[x]; y; y &= y - 1) atomicAdd(&Nu[BN_AT(__ffs(y) - 1, 1, 32)], q);
+    }
+    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(FULL, z, o);
+    if ((tid & 31) == 0) atomicAdd(&Nz, z);
+    __syncthreads();
+    if (tid < n && Nu[tid]) atomicAdd(&acc[(size_t)v * n + tid], Nu[tid]);
+    if (tid == 0) atomicAdd(&acc[(size_t)n * n + v], Nz);
 }
 
 // out = lbs + lf: the shifted scores of B_i(G) f_i(G) (Eq. 6 with a feature).
@@ -651,7 +850,11 @@ __global__ void k_add_feature(const T* __restrict__ lbs, const T* __restrict__ l
 {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < nK;
          x += (int64_t)gridDim.x * blockDim.x)
-        out[x] = lbs[x] + lf[x];
+    {
+        T y = lbs[x];
+        apply_weight(y, lf[x]);
+        out[x] = y;
+    }
 }
 
 // Byte copies between scattered device regions, one block per segment: the
@@ -700,7 +903,11 @@ cudaError_t launch_apply_q(const Plan& P, const void* lq, void* A, cudaStream_t 
 {
     const int64_t total = (int64_t)P.n << (P.n - 1);
     const int grid = grid_for(total, 256, 152 * 16);
-    if (P.prec == 0)
+    if (P.lin == 2)
+        launch_or_record(KID_APPLY_Q_XS, k_apply_q<X64S>, grid, 256, 0, s, P.n, (const X64S*)lq, (X64S*)A, 0);
+    else if (P.lin)
+        launch_or_record(KID_APPLY_Q_X, k_apply_q<X64>, grid, 256, 0, s, P.n, (const X64*)lq, (X64*)A, 0);
+    else if (P.prec == 0)
         launch_or_record(KID_APPLY_Q_D, k_apply_q<double>, grid, 256, 0, s, P.n, (const double*)lq, (double*)A, 0);
     else
         launch_or_record(KID_APPLY_Q_F, k_apply_q<float>, grid, 256, 0, s, P.n, (const float*)lq, (float*)A,
@@ -712,7 +919,13 @@ cudaError_t launch_add_feature(const Plan& P, const void* lbs, const void* lf, v
                                cudaStream_t s)
 {
     const int64_t nK = (int64_t)P.n * P.K;
-    if (P.prec == 0)
+    if (P.lin == 2)
+        launch_or_record(KID_ADD_FEATURE_XS, k_add_feature<X64S>, grid_for(nK, 256), 256, 0, s,
+            (const X64S*)lbs, (const X64S*)lf, (X64S*)out, nK);
+    else if (P.lin)
+        launch_or_record(KID_ADD_FEATURE_X, k_add_feature<X64>, grid_for(nK, 256), 256, 0, s,
+            (const X64*)lbs, (const X64*)lf, (X64*)out, nK);
+    else if (P.prec == 0)
         launch_or_record(KID_ADD_FEATURE_D, k_add_feature<double>, grid_for(nK, 256), 256, 0, s, 
             (const double*)lbs, (const double*)lf, (double*)out, nK);
     else
@@ -746,6 +959,9 @@ cudaError_t launch_upzeta(const Plan& P, const uint32_t* cmasks, const void* lbs
         }
         return launch_upzeta13(P, tab, rk13 + 8192, A, s, sums_done, err);
     }
+    if (P.lin)                                      // n < 14: a node per block
+        return launch_or_record(KID_UPZETA_XS, k_upzeta_x, dim3(P.n, P.nj), 256, (size_t)8 << (P.n - 1), s, P.n,
+                                P.K, cmasks, (const X64S*)lbs, (X64S*)A, P.js);
     const int h = P.n - 1 - P.b_up;
     const dim3 grid((unsigned)P.n << h, P.nj);
     const size_t sm = upzeta_smem_bytes(P);
@@ -850,7 +1066,10 @@ cudaError_t launch_gamma_p1(const Plan& P, const void* F, const void* Rc, const 
     const int h = P.n - 1 - P.b_g;
     const size_t sm1 = gamma_p1_smem_bytes(P);
     const dim3 grid(1u << h, P.nj, P.n);
-    if (P.prec == 0)
+    if (P.lin)
+        launch_or_record(KID_GAMMA_P1_XS, k_gamma_p1_x, grid, 256, sm1, s, P.n, P.d, P.b_g, P.nlow_g, (const X64S*)F,
+                         (const X64S*)Rc, (X64S*)W, P.js, (const X64S*)lq, P.vsel);
+    else if (P.prec == 0)
         launch_or_record(KID_GAMMA_P1_D, k_gamma_p1<double>, grid, 256, sm1, s, P.n, P.d, P.b_g, P.nlow_g,
                                                   (const double*)F, (const double*)Rc,
                                                   (double*)W, P.js, (const double*)lq, P.vsel);
@@ -885,7 +1104,13 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_
     if (c0 > 0) {
         const size_t sm2 = gamma_p2_smem_bytes(P);
         const dim3 grid(c0, P.nj, P.n);
-        if (P.prec == 0)
+        if (P.lin == 2)
+            launch_or_record(KID_GAMMA_P2_XS, k_gamma_p2<X64S>, grid, 256, sm2, s, P.n, P.d, P.b_g, P.hc_g, P.nlow_g,
+                             P.K, (const X64S*)W, (X64S*)Gam, P.js, P.vsel);
+        else if (P.lin)
+            launch_or_record(KID_GAMMA_P2_X, k_gamma_p2<X64>, grid, 256, sm2, s, P.n, P.d, P.b_g, P.hc_g, P.nlow_g,
+                             P.K, (const X64*)W, (X64*)Gam, P.js, P.vsel);
+        else if (P.prec == 0)
             launch_or_record(KID_GAMMA_P2_D, k_gamma_p2<double>, grid, 256, sm2, s, P.n, P.d, P.b_g, P.hc_g, P.nlow_g, P.K,
                                                       (const double*)W, (double*)Gam, P.js, P.vsel);
         else
@@ -896,7 +1121,13 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_
     }
     if (c0 < P.nlow_g) {
         const dim3 grid((P.nlow_g - c0 + 7) / 8, P.nj, P.n);
-        if (P.prec == 0)
+        if (P.lin == 2)
+            launch_or_record(KID_GAMMA_P2S_XS, k_gamma_p2s_x<X64S>, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0,
+                             P.K, (const X64S*)W, (X64S*)Gam, P.js, P.vsel);
+        else if (P.lin)
+            launch_or_record(KID_GAMMA_P2S_X, k_gamma_p2s_x<X64>, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
+                             (const X64*)W, (X64*)Gam, P.js, P.vsel);
+        else if (P.prec == 0)
             launch_or_record(KID_GAMMA_P2S_D, k_gamma_p2s<double>, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
                                                      (const double*)W, (double*)Gam, P.js, P.vsel);
         else
@@ -906,7 +1137,7 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t launch_edges(const Plan& P, const double* logB, const double* cmax,
+cudaError_t launch_edges(const Plan& P, const double* logB, const void* lbs, const double* cmax,
                          const uint32_t* masks, const void* Gam, const void* F, const int* err,
                          unsigned long long* acc, double* post, double* log_PD, cudaStream_t s)
 {
@@ -915,7 +1146,13 @@ cudaError_t launch_edges(const Plan& P, const double* logB, const double* cmax,
     if (e != cudaSuccess) return e;
     const unsigned chunks = (unsigned)std::min<int64_t>((P.K + 1023) / 1024, 64);
     const dim3 grid(chunks, P.nj, P.n);
-    if (P.prec == 0)
+    if (P.lin == 2)
+        launch_or_record(KID_EDGES_ACC_XS, k_edges_acc_x<X64S>, grid, 256, 0, s, P.n, P.K, fixed_bits(P.K),
+                         (const X64S*)lbs, masks, (const X64S*)Gam, (const X64S*)F, acc, P.js, P.vsel);
+    else if (P.lin)
+        launch_or_record(KID_EDGES_ACC_X, k_edges_acc_x<X64>, grid, 256, 0, s, P.n, P.K, fixed_bits(P.K), (const X64*)lbs,
+                         masks, (const X64*)Gam, (const X64*)F, acc, P.js, P.vsel);
+    else if (P.prec == 0)
         launch_or_record(KID_EDGES_ACC_D, k_edges_acc<double>, grid, 256, 0, s, P.n, P.K, fixed_bits(P.K), logB, cmax, masks,
                                                  (const double*)Gam, (const double*)F, acc, P.js, P.vsel);
     else
@@ -923,7 +1160,13 @@ cudaError_t launch_edges(const Plan& P, const double* logB, const double* cmax,
                                                 (const float*)Gam, (const float*)F, acc, P.js, P.vsel);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (P.prec == 0)
+    if (P.lin == 2)
+        launch_or_record(KID_EDGES_FIN_XS, k_edges_fin<X64S>, dim3(1, P.nj), rec_block(1024), 0, s, P.n, 0,
+                         fixed_bits(P.K), cmax, (const X64S*)F, err, acc, post, log_PD, P.js, P.vsel);
+    else if (P.lin)
+        launch_or_record(KID_EDGES_FIN_X, k_edges_fin<X64>, dim3(1, P.nj), rec_block(1024), 0, s, P.n, 0,
+                         fixed_bits(P.K), cmax, (const X64*)F, err, acc, post, log_PD, P.js, P.vsel);
+    else if (P.prec == 0)
         launch_or_record(KID_EDGES_FIN_D, k_edges_fin<double>, dim3(1, P.nj), rec_block(1024), 0, s, P.n, 0, fixed_bits(P.K), cmax,
                                                            (const double*)F, err, acc, post,
                                                            log_PD, P.js, P.vsel);
@@ -960,6 +1203,10 @@ cudaError_t set_kernel_attributes()
     SETA(k_gamma_p1<float>)
     SETA(k_gamma_p2<double>)
     SETA(k_gamma_p2<float>)
+    SETA(k_upzeta_x)
+    SETA(k_gamma_p1_x)
+    SETA(k_gamma_p2<X64>)
+    SETA(k_gamma_p2<X64S>)
 #undef SETA
     e = set_scores_attributes();
     if (e != cudaSuccess) return e;

@@ -1,6 +1,7 @@
 // bn_kernels.cuh -- host-side launch interface of the device kernels.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <cuda_runtime.h>
@@ -32,7 +33,13 @@ enum KernelId : int32_t {
     KID_REORDER_F, KID_COLB8, KID_COLB4, KID_COLB2, KID_COLW_D, KID_COLW_F, KID_COLS_D,
     KID_COLS_F, KID_UP13_D, KID_UP13_F_TLO, KID_UP13_F, KID_G13_D_Q, KID_G13_D, KID_G13_F_Q,
     KID_G13_F, KID_FROWS_D, KID_FROWS_F_TLO, KID_FROWS_F, KID_BROWS_D, KID_BROWS_F_TLO,
-    KID_BROWS_F, KID_COLB4_D, KID_COLB2_D, KID_COLB1_D, KID_COLB1, KID_COUNT
+    KID_BROWS_F, KID_COLB4_D, KID_COLB2_D, KID_COLB1_D, KID_COLB1,
+    // the linear FP64 form
+    KID_SHIFT_XS, KID_APPLY_Q_XS, KID_ADD_FEATURE_XS, KID_UPZETA_XS, KID_FROWS_XS, KID_BROWS_XS,
+    KID_GAMMA_P1_XS, KID_GAMMA_P2_XS, KID_GAMMA_P2S_XS, KID_EDGES_ACC_XS, KID_EDGES_FIN_XS,
+    KID_SHIFT_X, KID_APPLY_Q_X, KID_ADD_FEATURE_X, KID_REORDER_X, KID_COLB4_X, KID_COLB2_X,
+    KID_COLB1_X, KID_COLW_X, KID_UP13_X, KID_FROWS_X, KID_BROWS_X, KID_G13_X_Q, KID_G13_X,
+    KID_GAMMA_P2_X, KID_GAMMA_P2S_X, KID_EDGES_ACC_X, KID_EDGES_FIN_X, KID_COUNT
 };
 
 // Arguments as one trivially copyable structure whose members have the
@@ -138,6 +145,7 @@ struct Plan {
     uint32_t nlow_g;      // subsets of b_g dims with at most d elements
     int wb;               // in-warp bits of the F / R' tiles
     int prec;             // 0 = FP64, 1 = FP32
+    int lin = 0;          // FP64 values kept linear (bn_device.cuh; see lin_range), not as logarithms
     int allbin = 0;       // every variable has arity 2
     // Joint states of the largest set of k variables: the product of the k
     // largest arities, capped at 65537 (a batch group's largest).
@@ -187,6 +195,28 @@ inline void set_states(Plan& P, const uint32_t* sorted)
         if (k <= P.n && q <= 65536u) q *= sorted[k - 1];
         P.states[k] = (uint32_t)(q < 65537u ? q : 65537u);
     }
+}
+
+// Whether an FP64 job may keep its values linear (Plan::lin): 1 in X64 (n >=
+// 14), 2 in X64S (n < 14), 0 as logarithms.  With the nodes' scores shifted
+// by their maxima the values lie below 2^1000, and only those within reach of
+// F(V) matter; F(V) is at least the weight of the empty parent sets, Prod_i
+// B_i(empty) / c_i, and that is bounded per node by m log2 r + r log2(r (1 +
+// m / ess)) bits of score and by `logs`, the largest magnitude of the job's own
+// (finite) log weights per node in nats.  118000 (12500) bits leave 9000
+// (1800) for the products beside F(V).  Lattices whose tiles do not fit keep
+// the logarithms.
+inline int lin_range(const Plan& P, const uint8_t* arity, double ess, double logs)
+{
+    if (P.prec != 0 || P.n < 5 || P.n > 31) return 0;
+    if (P.n >= 14 && !(P.up13 && P.g13)) return 0;
+    double bits = 0.0;
+    for (int i = 0; i < P.n; ++i) {
+        const double r = arity[i];
+        bits += P.m * std::log2(r) + r * std::log2(r * (1.0 + P.m / ess) + 2.0) + 2.8854 * logs;
+    }
+    if (P.n >= 14) return bits < 118000.0 ? 1 : 0;
+    return bits < 12500.0 ? 2 : 0;
 }
 
 // Host check of m x n row-major data: every value below its variable's
@@ -303,8 +333,8 @@ cudaError_t launch_fold_scores(const Plan& P, int nl, int64_t Kv, uint32_t r, co
 cudaError_t launch_top_slabs(const Plan& V, int k, const void* Av, void* Atop, cudaStream_t s);
 cudaError_t launch_level_rows(const Plan& P, uint32_t r, int hl, void* X, void* buf, int dir,
                               cudaStream_t s);
-// F and R' in one launch (k_sweeps): FP32 plans with the row schedule, whole
-// jobs with A in device memory.  use_sweeps: whether a single job's direct
+// F and R' in one launch (k_sweeps): FP32 plans with the row schedule and
+// linear FP64 plans, whole jobs with A in device memory.  use_sweeps: whether a single job's direct
 // launches take it; err is the job's error word, the first of 256 bytes that
 // also hold the sweeps' counters.  Rc null: F alone.
 bool sweeps_fit(const Plan& P);
@@ -329,7 +359,7 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_
 // made by launch_gamma_p1 itself; stored after the level words of Rc).
 cudaError_t launch_gamma_table(const Plan& P, const void* F, const void* Rc, cudaStream_t s);
 // Step 5 (three launches); acc: n * (n + 1) scratch words.
-cudaError_t launch_edges(const Plan& P, const double* logB, const double* cmax,
+cudaError_t launch_edges(const Plan& P, const double* logB, const void* lbs, const double* cmax,
                          const uint32_t* masks, const void* Gam, const void* F,
                          const int* err, unsigned long long* acc, double* post, double* log_PD,
                          cudaStream_t s);
@@ -348,6 +378,7 @@ constexpr size_t kRank13Bytes = 2 * 8192 * sizeof(uint16_t);
 size_t upzeta13_smem_bytes(const Plan& P);
 size_t gamma13_smem_bytes(const Plan& P);
 cudaError_t set_tile13_attributes();
+bool lin_tiles_fit(const Plan& P);    // the tiles of the linear FP64 form
 bool tile13_up_fits(const Plan& P);   // n >= 14 and the column kernel's shared memory fits
 inline bool tile13_gamma_fits(const Plan& P) { return P.n >= 14; }
 

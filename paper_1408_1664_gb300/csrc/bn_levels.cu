@@ -29,10 +29,11 @@ namespace {
 constexpr int LB = 4;             // low bits of an FP32 tile
 constexpr int LB64 = 3;           // low bits of an FP64 tile
 constexpr int BT = 29;            // binomial table rows (n - B < 29: n <= 32 in FP32)
-// k_sweeps: single jobs up to this n; levels wider than kSweepGrid tiles run
-// on the whole GPU; polls before a block gives up a wait (about 1 us each).
+// k_sweeps: single jobs up to this n (FP32; linear FP64); levels that fill
+// more than kSweepGrid blocks run on the whole GPU; polls before a block gives up a wait (about 1 us each).
 constexpr int kSweepMaxN = 21;
-constexpr uint64_t kSweepGrid = 400;
+constexpr int kSweepMaxNX = 20;
+constexpr uint64_t kSweepGrid = 12;
 constexpr uint32_t kSweepSpinCap = 1u << 22;
 
 __device__ const BinomTable g_binom_lanes = make_binom_table();
@@ -54,6 +55,33 @@ __device__ __forceinline__ void lazy_add(double& m, double& s, double x)
     s = big ? fma(s, e, 1.0) : s + e;
     m = big ? x : m;
 }
+
+// The sum of one subset's terms A * F: (m, s) as above for logarithms (an
+// empty sum has m far below any value, finite so that a left-out term of -inf
+// changes nothing), LazySum for XValue.  add() takes a term or leaves it out.
+template <typename T> struct TileSum {
+    T m = (T)-3.0e38f, s = T(0);
+    __device__ __forceinline__ void add(T a, T f, bool take = true)
+    {
+        lazy_add(m, s, take ? a + f : LogOps<T>::ninf());
+    }
+    __device__ __forceinline__ void rebase(T r) { m -= r; }
+    __device__ __forceinline__ T value() const { return m + LogOps<T>::lg(s); }
+};
+template <int FB> struct TileSum<XValue<FB>> {
+    using X = XValue<FB>;
+    LazySum<X> v;
+    __device__ __forceinline__ void add(X a, X f, bool take = true)
+    {
+        const double p = x_mant(a) * x_mant(f);
+        v.add(take ? p : 0.0, take ? x_exp(a) + x_exp(f) : -(1 << 28));
+    }
+    __device__ __forceinline__ void rebase(X) {}
+    __device__ __forceinline__ X value() const { return v.value(); }
+};
+template <typename T> __device__ __forceinline__ T unit() { return T(0); }         // log 1
+template <> __device__ __forceinline__ X64 unit<X64>() { return x_one<X64>(); }
+template <> __device__ __forceinline__ X64S unit<X64S>() { return x_one<X64S>(); }
 
 // x with bit i (i < B) removed: an index among the 2^(B-1) B-bit patterns
 // without bit i.
@@ -93,6 +121,34 @@ __device__ __forceinline__ void load_row(const double* p, double (&v)[N], int mo
     }
 }
 
+template <int N, int FB>
+__device__ __forceinline__ void load_row(const XValue<FB>* p, XValue<FB> (&v)[N], int mode)
+{
+    const ulonglong2* q = reinterpret_cast<const ulonglong2*>(p);
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+        const ulonglong2 x = mode == LD_STREAM ? __ldcs(q + k) : mode == LD_L2 ? __ldcg(q + k) : q[k];
+        v[2 * k].u = x.x;
+        v[2 * k + 1].u = x.y;
+    }
+}
+
+// One value by load mode.
+__device__ __forceinline__ float load_one(const float* p, int mode)
+{
+    return mode == LD_STREAM ? __ldcs(p) : mode == LD_L2 ? __ldcg(p) : *p;
+}
+template <int FB> __device__ __forceinline__ XValue<FB> load_one(const XValue<FB>* p, int mode)
+{
+    const unsigned long long* q = &p->u;
+    return XValue<FB>{mode == LD_STREAM ? __ldcs(q) : mode == LD_L2 ? __ldcg(q) : *q};
+}
+__device__ __forceinline__ float shfl_one(unsigned mask, float v, int o) { return __shfl_xor_sync(mask, v, o); }
+template <int FB> __device__ __forceinline__ XValue<FB> shfl_one(unsigned mask, XValue<FB> v, int o)
+{
+    return XValue<FB>{__shfl_xor_sync(mask, v.u, o)};
+}
+
 template <int N>
 __device__ __forceinline__ void store_row(float* p, const float (&v)[N])
 {
@@ -107,6 +163,14 @@ __device__ __forceinline__ void store_row(double* p, const double (&v)[N])
     double2* q = reinterpret_cast<double2*>(p);
 #pragma unroll
     for (int k = 0; k < N / 2; ++k) q[k] = make_double2(v[2 * k], v[2 * k + 1]);
+}
+
+template <int N, int FB>
+__device__ __forceinline__ void store_row(XValue<FB>* p, const XValue<FB> (&v)[N])
+{
+    ulonglong2* q = reinterpret_cast<ulonglong2*>(p);
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) q[k] = make_ulonglong2(v[2 * k].u, v[2 * k + 1].u);
 }
 
 // Tile g of the level: the g-th hl-element subset of nh bits in colex order.
@@ -157,19 +221,16 @@ __device__ __forceinline__ void fill_table(uint32_t (*bt)[BT])
 // bits of the row index dropped; a term of a top variable reads Atop.
 template <typename T, int FMODE, int B, bool TLO = false, bool SLAB = false>
 __device__ __forceinline__ T forward_tile(int n, uint32_t Ht, const T* __restrict__ A,
-                                          T* __restrict__ F, T rebase = T(0), int nl = 0,
+                                          T* __restrict__ F, T rebase = T{}, int nl = 0,
                                           const T* __restrict__ Atop = nullptr)
 {
     constexpr int LN = 1 << B;
-    const size_t full = (size_t)1 << n;
+    [[maybe_unused]] const size_t full = (size_t)1 << n;
     const size_t half = (size_t)1 << ((SLAB ? nl : n) - 1);
     const uint32_t rmask = SLAB ? (1u << (nl - 1 - B)) - 1u : ~0u;   // slab row bits
     const uint32_t lmask = SLAB ? (1u << (nl - B)) - 1u : ~0u;       // low tile bits
-    using L = LogOps<T>;
 
-    T m[LN], s[LN];
-#pragma unroll
-    for (int l = 0; l < LN; ++l) { m[l] = L::ninf(); s[l] = T(0); }
+    TileSum<T> s[LN];
     // terms across tiles: i = B + j for the set bits j of Ht
     for (uint32_t rest = Ht; rest; rest &= rest - 1) {
         const int j = __ffs(rest) - 1;
@@ -187,12 +248,11 @@ __device__ __forceinline__ T forward_tile(int n, uint32_t Ht, const T* __restric
         }
         load_row(F + BN_AT((size_t)Hm << B, LN, full), f, FMODE);
 #pragma unroll
-        for (int l = 0; l < LN; ++l) lazy_add(m[l], s[l], a[l] + f[l]);
+        for (int l = 0; l < LN; ++l) s[l].add(a[l], f[l]);
     }
-    // (m, s) stands for m + lg(s): moving the cross-tile sums to this level's
-    // base moves m
+    // the cross-tile sums moved to this level's base
 #pragma unroll
-    for (int l = 0; l < LN; ++l) m[l] -= rebase;
+    for (int l = 0; l < LN; ++l) s[l].rebase(rebase);
     // terms inside the tile: A_i(S - {i}) for i < B, 2^(B-1) values per i
     T ai[B][LN / 2];
 #pragma unroll
@@ -201,18 +261,20 @@ __device__ __forceinline__ T forward_tile(int n, uint32_t Ht, const T* __restric
                            LN / 2, (SLAB ? nl : n) * half),
                  ai[i], LD_STREAM);
     T Fv[LN];
-    Fv[0] = Ht == 0u ? T(0) : m[0] + L::lg(s[0]);
+    Fv[0] = Ht == 0u ? unit<T>() : s[0].value();
 #pragma unroll
     for (int l = 1; l < LN; ++l) {
 #pragma unroll
         for (int i = 0; i < B; ++i)
-            if (l >> i & 1) lazy_add(m[l], s[l], ai[i][squeeze4(l ^ (1 << i), i)] + Fv[l ^ (1 << i)]);
-        Fv[l] = m[l] + L::lg(s[l]);
+            if (l >> i & 1) s[l].add(ai[i][squeeze4(l ^ (1 << i), i)], Fv[l ^ (1 << i)]);
+        Fv[l] = s[l].value();
     }
     store_row(F + BN_AT((size_t)Ht << B, LN, full), Fv);
     T mx = Fv[0];
+    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-    for (int l = 1; l < LN; ++l) mx = Fv[l] > mx ? Fv[l] : mx;
+        for (int l = 1; l < LN; ++l) mx = Fv[l] > mx ? Fv[l] : mx;
+    }
     return mx;
 }
 
@@ -220,7 +282,7 @@ __device__ __forceinline__ T forward_tile(int n, uint32_t Ht, const T* __restric
 //   R'(T) = sum_{i not in T} A_i(T) R'(T + {i}),  R'(V) = 1
 template <typename T, int FMODE, int B, bool TLO = false, bool SLAB = false>
 __device__ __forceinline__ T backward_tile(int n, uint32_t Ht, const T* __restrict__ A,
-                                           T* __restrict__ Rc, T rebase = T(0), int nl = 0,
+                                           T* __restrict__ Rc, T rebase = T{}, int nl = 0,
                                            const T* __restrict__ Atop = nullptr)
 {
     constexpr int LN = 1 << B;
@@ -230,11 +292,8 @@ __device__ __forceinline__ T backward_tile(int n, uint32_t Ht, const T* __restri
     const size_t half = (size_t)1 << ((SLAB ? nl : n) - 1);
     const uint32_t rmask = SLAB ? (1u << (nl - 1 - B)) - 1u : ~0u;
     const uint32_t lmask = SLAB ? (1u << (nl - B)) - 1u : ~0u;
-    using L = LogOps<T>;
 
-    T m[LN], s[LN];
-#pragma unroll
-    for (int l = 0; l < LN; ++l) { m[l] = L::ninf(); s[l] = T(0); }
+    TileSum<T> s[LN];
     for (uint32_t rest = ~Ht & hmask; rest; rest &= rest - 1) {
         const int j = __ffs(rest) - 1;
         T a[LN], r[LN];
@@ -250,10 +309,10 @@ __device__ __forceinline__ T backward_tile(int n, uint32_t Ht, const T* __restri
         }
         load_row(Rc + BN_AT((size_t)(Ht | (1u << j)) << B, LN, full), r, FMODE);
 #pragma unroll
-        for (int l = 0; l < LN; ++l) lazy_add(m[l], s[l], a[l] + r[l]);
+        for (int l = 0; l < LN; ++l) s[l].add(a[l], r[l]);
     }
 #pragma unroll
-    for (int l = 0; l < LN; ++l) m[l] -= rebase;
+    for (int l = 0; l < LN; ++l) s[l].rebase(rebase);
     // A_i(T) for i < B not in T, 2^(B-1) values per i
     T ai[B][LN / 2];
 #pragma unroll
@@ -262,18 +321,20 @@ __device__ __forceinline__ T backward_tile(int n, uint32_t Ht, const T* __restri
                            LN / 2, (SLAB ? nl : n) * half),
                  ai[i], LD_STREAM);
     T Rv[LN];
-    Rv[LN - 1] = Ht == hmask ? T(0) : m[LN - 1] + L::lg(s[LN - 1]);
+    Rv[LN - 1] = Ht == hmask ? unit<T>() : s[LN - 1].value();
 #pragma unroll
     for (int l = LN - 2; l >= 0; --l) {
 #pragma unroll
         for (int i = 0; i < B; ++i)
-            if (!(l >> i & 1)) lazy_add(m[l], s[l], ai[i][squeeze4(l, i)] + Rv[l | (1 << i)]);
-        Rv[l] = m[l] + L::lg(s[l]);
+            if (!(l >> i & 1)) s[l].add(ai[i][squeeze4(l, i)], Rv[l | (1 << i)]);
+        Rv[l] = s[l].value();
     }
     store_row(Rc + BN_AT((size_t)Ht << B, LN, full), Rv);
     T mx = Rv[0];
+    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-    for (int l = 1; l < LN; ++l) mx = Rv[l] > mx ? Rv[l] : mx;
+        for (int l = 1; l < LN; ++l) mx = Rv[l] > mx ? Rv[l] : mx;
+    }
     return mx;
 }
 
@@ -333,7 +394,7 @@ k_forward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __res
         }
     } else {
         if (g >= ntiles) return;
-        forward_tile<T, LD_PLAIN, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, F, T(0),
+        forward_tile<T, LD_PLAIN, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, F, T{},
                                                 n - kfix, Atop);
     }
 }
@@ -366,7 +427,7 @@ k_backward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __re
         }
     } else {
         if (g >= ntiles) return;
-        backward_tile<T, LD_PLAIN, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, Rc, T(0),
+        backward_tile<T, LD_PLAIN, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, Rc, T{},
                                                  n - kfix, Atop);
     }
 }
@@ -375,8 +436,8 @@ k_backward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __re
 // separated by a barrier of the blocks that share it, instead of a launch per
 // level.  A level launch of a job up to n of about 20 took 9 to 12 us, nearly
 // all of it latency: the launch itself and one thread walking a tile's terms,
-// each a dependent pair of row loads.  Here a tile's 16 subsets take 16 lanes
-// (one value each), a lane issues the loads of up to eight terms together,
+// each a dependent pair of row loads.  Here a tile's 16 (FP64: 8) subsets take as many lanes
+// (one value each), a lane issues the loads of up to eight (four) terms together,
 // and the first tile's index and A values for the next level are fetched
 // between arriving at the barrier and waiting on it.  The sums run in the
 // order of forward_tile / backward_tile, so the results are the same bits.
@@ -402,55 +463,55 @@ __global__ void __launch_bounds__(kSweepThreads, 2)
 k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restrict__ Rc, size_t js,
          unsigned* __restrict__ sync, int* __restrict__ err, uint32_t cap)
 {
-    constexpr int LN = 1 << LB, CH = 8;
+    constexpr int B = sizeof(T) == 4 ? LB : LB64;
+    constexpr int LN = 1 << B;                      // lanes per tile
+    constexpr int CH = sizeof(T) == 4 ? 8 : 4;      // terms loaded together (64 registers)
     constexpr bool kBases = sizeof(T) == 4;
-    using L = LogOps<T>;
+    constexpr int XMODE = SYNC == SYNC_BLOCK ? LD_PLAIN : LD_L2;
     __shared__ uint32_t bt[BT][BT];
     __shared__ int wm[kSweepThreads / 32];
     __shared__ int ok_s;
     fill_table(bt);
     __syncthreads();
-    // the empty accumulator: far enough below any value that the first term
-    // replaces it, finite so that a left-out term (x = -inf) changes nothing
-    const T none = (T)-3.0e38f;
     const int it = (int)(blockIdx.x / (unsigned)nb);
     const uint32_t rank = blockIdx.x % (unsigned)nb;
     const bool fwd = (it & 1) == 0;
     const size_t off = (size_t)(it >> 1) * js;
     A = reinterpret_cast<const T*>(reinterpret_cast<const char*>(A) + off);
     T* X = reinterpret_cast<T*>(reinterpret_cast<char*>(fwd ? F : Rc) + off);
-    const int nh = n - LB;
+    const int nh = n - B;
     const uint32_t hmask = (1u << nh) - 1u;
     const size_t half = (size_t)1 << (n - 1), full = (size_t)1 << n;
     const int l = threadIdx.x & (LN - 1);
     const uint32_t own = fwd ? (uint32_t)l : (uint32_t)l ^ (LN - 1);   // the lane's in-tile elements
     const int size = __popc(own);
-    // half warps number across the blocks: a narrow level spreads over them
-    const uint32_t hw = (threadIdx.x >> LB) * (uint32_t)nb + rank;
-    const uint32_t nhw = (blockDim.x >> LB) * (uint32_t)nb;
+    const unsigned tmask = ((1u << LN) - 1u) << (threadIdx.x & 31 & ~(LN - 1));   // the tile's lanes
+    // the groups of LN lanes number across the blocks: a narrow level spreads over them
+    const uint32_t hw = (threadIdx.x >> B) * (uint32_t)nb + rank;
+    const uint32_t nhw = (blockDim.x >> B) * (uint32_t)nb;
     int* lw = kBases ? level_words(reinterpret_cast<float*>(X), n) : nullptr;
     unsigned* arr = SYNC == SYNC_GRID ? sync + (fwd ? 0 : 16) : nullptr;
 
-    // place of element l of row S-without-j of A_{LB + j}, and of the row of
-    // A_i (i < LB) that the tile's in-tile terms read
+    // place of element l of row S-without-j of A_{B + j}, and of the row of
+    // A_i (i < B) that the tile's in-tile terms read
     auto a_at = [&](uint32_t H, int j) {
         const uint32_t R = squeeze(H, j);
-        return BN_AT((size_t)(LB + j) * half + ((size_t)(TLO ? tlo_row(R, 9) : R) << LB) + l, 1, n * half);
+        return BN_AT((size_t)(B + j) * half + ((size_t)(TLO ? tlo_row(R, 9) : R) << B) + l, 1, n * half);
     };
     auto in_at = [&](uint32_t H, int i) {
-        return BN_AT((size_t)i * half + ((size_t)(TLO ? tlo_row(H, 10) : H) << (LB - 1)) + squeeze4(l, i), 1,
+        return BN_AT((size_t)i * half + ((size_t)(TLO ? tlo_row(H, 10) : H) << (B - 1)) + squeeze4(l, i), 1,
                      n * half);
     };
-    // a half warp's run of tiles in step st: consecutive in colex order, so
+    // a group's run of tiles in step st: consecutive in colex order, so
     // only the first is unranked.  Its bits, the A values of its first terms
     // and of its in-tile terms are fetched ahead of the step.
     uint32_t bits = 0, g0 = 0, g1 = 0;
-    T pa[CH], pi[LB];
+    T pa[CH], pi[B];
     auto load_a = [&](uint32_t H, uint32_t& rest, int st, T (&a)[CH]) {
 #pragma unroll
         for (int q = 0; q < CH; ++q) {
             if (q < st) {
-                a[q] = __ldcs(A + a_at(H, __ffs(rest) - 1));
+                a[q] = load_one(A + a_at(H, __ffs(rest) - 1), LD_STREAM);
                 rest &= rest - 1;
             }
         }
@@ -465,12 +526,12 @@ k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restric
         uint32_t rest = bits;
         load_a(H, rest, st, pa);
 #pragma unroll
-        for (int i = 0; i < LB; ++i) pi[i] = __ldcs(A + in_at(H, i));
+        for (int i = 0; i < B; ++i) pi[i] = load_one(A + in_at(H, i), LD_STREAM);
     };
     ahead(0);
     for (int st = 0; st <= nh; ++st) {
-        T mx = L::ninf();
-        T rebase = T(0);
+        float mx = LogOps<float>::ninf();
+        T rebase{};
         if constexpr (kBases)
             if (st > 0) {
                 const int w = SYNC == SYNC_BLOCK ? *(volatile int*)(lw + (fwd ? st - 1 : nh - st + 1))
@@ -480,16 +541,16 @@ k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restric
         for (uint32_t g = g0; g < g1; ++g) {
             const uint32_t H = fwd ? bits : hmask ^ bits;
             uint32_t ra = bits, rf = bits;
-            T m = none, s = T(0);
+            TileSum<T> s;
             for (int c0 = 0; c0 < st; c0 += CH) {
                 T a[CH], f[CH];
 #pragma unroll
                 for (int q = 0; q < CH; ++q) {
-                    f[q] = L::ninf();
+                    f[q] = T{};
                     if (c0 + q < st) {
-                        const T* p = X + BN_AT(((size_t)(H ^ (rf & (0u - rf))) << LB) + l, 1, full);
+                        const T* p = X + BN_AT(((size_t)(H ^ (rf & (0u - rf))) << B) + l, 1, full);
                         rf &= rf - 1;
-                        f[q] = SYNC == SYNC_BLOCK ? *p : __ldcg(p);
+                        f[q] = load_one(p, XMODE);
                     }
                 }
                 if (g == g0 && c0 == 0) {
@@ -502,27 +563,27 @@ k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restric
                     load_a(H, ra, st - c0, a);
                 }
 #pragma unroll
-                for (int q = 0; q < CH; ++q) lazy_add(m, s, c0 + q < st ? a[q] + f[q] : L::ninf());
+                for (int q = 0; q < CH; ++q) s.add(a[q], f[q], c0 + q < st);
             }
-            m -= rebase;
-            T ai[LB];
+            s.rebase(rebase);
+            T ai[B];
 #pragma unroll
-            for (int i = 0; i < LB; ++i) ai[i] = g == g0 ? pi[i] : __ldcs(A + in_at(H, i));
+            for (int i = 0; i < B; ++i) ai[i] = g == g0 ? pi[i] : load_one(A + in_at(H, i), LD_STREAM);
             // the in-tile terms, in popcount order of the lane's elements: in
             // round k the lanes with k elements add theirs (the others a left-out
             // term, so the lanes of a warp stay together)
-            T v = st == 0 ? T(0) : m + L::lg(s);
+            T v = st == 0 ? unit<T>() : s.value();
 #pragma unroll
-            for (int k = 1; k <= LB; ++k) {
+            for (int k = 1; k <= B; ++k) {
 #pragma unroll
-                for (int i = 0; i < LB; ++i) {
-                    const T y = __shfl_xor_sync(0xffffu << (threadIdx.x & 16), v, 1 << i);
-                    lazy_add(m, s, size == k && (own >> i & 1) ? ai[i] + y : L::ninf());
+                for (int i = 0; i < B; ++i) {
+                    const T y = shfl_one(tmask, v, 1 << i);
+                    s.add(ai[i], y, size == k && (own >> i & 1));
                 }
-                v = size == k ? m + L::lg(s) : v;
+                if (size == k) v = s.value();
             }
-            X[BN_AT(((size_t)H << LB) + l, 1, full)] = v;
-            mx = v > mx ? v : mx;
+            X[BN_AT(((size_t)H << B) + l, 1, full)] = v;
+            if constexpr (kBases) mx = v > mx ? v : mx;
             if (g + 1 < g1) {                       // the next tile of the run
                 const uint32_t u = bits & (0u - bits), w = bits + u;
                 bits = w | (((w ^ bits) >> 2) >> (__ffs(u) - 1));
@@ -535,7 +596,7 @@ k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restric
                 // the one tile of the first level: its lanes' maximum
                 if (hw == 0) {
                     for (int o = LN / 2; o; o >>= 1) {
-                        const T y = __shfl_xor_sync(0xffffu, mx, o);
+                        const float y = __shfl_xor_sync(0xffffu, mx, o);
                         mx = y > mx ? y : mx;
                     }
                     if (l == 0) level_words_start(lw, lv, mx);
@@ -630,11 +691,27 @@ __global__ void k_level_rows(int n, int hl, uint32_t ntiles, uint32_t rsrc, int 
 
 // The folded tables, in the virtual job's canonical family order (Kv per
 // table), from the job's shifted scores lbs (K per node, the same shift).
+template <typename T> struct FoldSum {
+    using L = LogOps<T>;
+    T m = L::ninf(), s = T(0);
+    __device__ __forceinline__ void add(T v)
+    {
+        if (v == L::ninf()) return;
+        if (v > m) {
+            s = s * L::ex(m - v) + T(1);
+            m = v;
+        } else {
+            s += L::ex(v - m);
+        }
+    }
+    __device__ __forceinline__ T value() const { return m == L::ninf() ? m : m + L::lg(s); }
+};
+template <> struct FoldSum<X64> : LazySum<X64> {};
+
 template <typename T>
 __global__ void k_fold_scores(int n, int nl, int d, int64_t K, int64_t Kv, uint32_t r,
                               const T* __restrict__ lbs, T* __restrict__ out)
 {
-    using L = LogOps<T>;
     const int k = n - nl;
     const int64_t total = (int64_t)(nl + 2 * k) * Kv;
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < total;
@@ -657,27 +734,23 @@ __global__ void k_fold_scores(int n, int nl, int d, int64_t K, int64_t Kv, uint3
             tops = r & ~(1u << q);
         }
         const int g = __popc(G);
-        T m = L::ninf(), s = T(0);
+        FoldSum<T> sum;
         if (g <= d) {
             for (uint32_t t = tops;; t = (t - 1) & tops) {
                 if (g + __popc(t) <= d) {
                     const uint32_t c = squeeze(G | (t << nl), node);   // node's own index
-                    const T v = lbs[BN_AT((size_t)node * K + small_subset_rank(c, n - 1), 1, (size_t)n * K)];
-                    if (v != L::ninf()) {
-                        if (v > m) {
-                            s = s * L::ex(m - v) + T(1);
-                            m = v;
-                        } else {
-                            s += L::ex(v - m);
-                        }
-                    }
+                    sum.add(lbs[BN_AT((size_t)node * K + small_subset_rank(c, n - 1), 1, (size_t)n * K)]);
                 }
                 if (t == 0) break;
             }
         }
-        out[x] = m == L::ninf() ? m : m + L::lg(s);
+        out[x] = sum.value();
     }
 }
+
+__device__ __forceinline__ float add_logs(float a, float b) { return LogOps<float>::lse(a, b); }
+__device__ __forceinline__ double add_logs(double a, double b) { return LogOps<double>::lse(a, b); }
+__device__ __forceinline__ X64 add_logs(X64 a, X64 b) { return x_add(a, b); }
 
 // The top variables' slabs (plain order over the nl low variables) from the
 // X1 and X2 tables of the virtual job's A (its own layout: tile-level row
@@ -685,7 +758,6 @@ __global__ void k_fold_scores(int n, int nl, int d, int64_t K, int64_t Kv, uint3
 template <typename T, bool TLO>
 __global__ void k_top_slabs(int nl, int k, const T* __restrict__ Av, T* __restrict__ Atop)
 {
-    using L = LogOps<T>;
     const size_t per = (size_t)1 << nl;
     const size_t half = per >> 1;
     for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < per * (size_t)k;
@@ -696,7 +768,7 @@ __global__ void k_top_slabs(int nl, int k, const T* __restrict__ Av, T* __restri
         const uint32_t pos = TLO ? (tlo_row(c >> 4, 9) << 4) | (c & 15u) : c;
         const T* X1 = Av + (size_t)(nl + 2 * q) * half;
         T v = X1[BN_AT(pos, 1, half)];
-        if (Lw & 1u) v = L::lse(v, X1[half + BN_AT(pos, 1, half)]);
+        if (Lw & 1u) v = add_logs(v, X1[half + BN_AT(pos, 1, half)]);
         Atop[x] = v;
     }
 }
@@ -769,7 +841,9 @@ static cudaError_t rows_level(const Plan& P, int sweep, int hl, uint32_t nt, uns
             k_backward_rows<T, TLO, true><<<grid, tb, 0, s>>>(P.n, hl, nt, a, (T*)X, P.js, rf, kf, at);
         return cudaGetLastError();
     }
-    const int kid = sizeof(T) == 8 ? (sweep == 0 ? KID_FROWS_D : KID_BROWS_D)
+    const int kid = std::is_same<T, X64>::value ? (sweep == 0 ? KID_FROWS_X : KID_BROWS_X)
+                    : std::is_same<T, X64S>::value ? (sweep == 0 ? KID_FROWS_XS : KID_BROWS_XS)
+                    : sizeof(T) == 8 ? (sweep == 0 ? KID_FROWS_D : KID_BROWS_D)
                     : TLO ? (sweep == 0 ? KID_FROWS_F_TLO : KID_BROWS_F_TLO)
                           : (sweep == 0 ? KID_FROWS_F : KID_BROWS_F);
     if (sweep == 0)
@@ -786,6 +860,8 @@ cudaError_t launch_rows_level(const Plan& P, int sweep, int hl, const void* A, v
     if (nt == 0) return cudaSuccess;
     const unsigned tb = rec_block(level_block(nt));
     const dim3 grid((nt + tb - 1) / tb, P.nj);
+    if (P.lin == 2) return rows_level<X64S, false>(P, sweep, hl, nt, tb, grid, A, X, Atop, s);
+    if (P.lin) return rows_level<X64, false>(P, sweep, hl, nt, tb, grid, A, X, Atop, s);
     if (P.prec == 0) return rows_level<double, false>(P, sweep, hl, nt, tb, grid, A, X, Atop, s);
     if (use_tlo(P)) return rows_level<float, true>(P, sweep, hl, nt, tb, grid, A, X, Atop, s);
     return rows_level<float, false>(P, sweep, hl, nt, tb, grid, A, X, Atop, s);
@@ -796,7 +872,9 @@ cudaError_t launch_fold_scores(const Plan& P, int nl, int64_t Kv, uint32_t r, co
 {
     const int64_t total = (int64_t)(nl + 2 * (P.n - nl)) * Kv;
     const unsigned grid = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 16);
-    if (P.prec == 0)
+    if (P.lin)
+        k_fold_scores<X64><<<grid, 256, 0, s>>>(P.n, nl, P.d, P.K, Kv, r, (const X64*)lbs, (X64*)out);
+    else if (P.prec == 0)
         k_fold_scores<double><<<grid, 256, 0, s>>>(P.n, nl, P.d, P.K, Kv, r, (const double*)lbs, (double*)out);
     else
         k_fold_scores<float><<<grid, 256, 0, s>>>(P.n, nl, P.d, P.K, Kv, r, (const float*)lbs, (float*)out);
@@ -809,7 +887,9 @@ cudaError_t launch_top_slabs(const Plan& V, int k, const void* Av, void* Atop, c
     const uint64_t total = (uint64_t)k << nl;
     if (total == 0) return cudaSuccess;                 // no top variables (one rank)
     const unsigned grid = (unsigned)std::min<uint64_t>((total + 255) / 256, 152 * 16);
-    if (V.prec == 0)
+    if (V.lin)
+        k_top_slabs<X64, false><<<grid, 256, 0, s>>>(nl, k, (const X64*)Av, (X64*)Atop);
+    else if (V.prec == 0)
         k_top_slabs<double, false><<<grid, 256, 0, s>>>(nl, k, (const double*)Av, (double*)Atop);
     else if (use_tlo(V))
         k_top_slabs<float, true><<<grid, 256, 0, s>>>(nl, k, (const float*)Av, (float*)Atop);
@@ -844,80 +924,55 @@ cudaError_t launch_level_rows(const Plan& P, uint32_t r, int hl, void* X, void* 
     return cudaGetLastError();
 }
 
+// Every level of one sweep (0 F, 1 R'), a launch each.
+static cudaError_t rows_sweep(const Plan& P, int sweep, const void* A, void* X, cudaStream_t s, int* launches)
+{
+    const int nh = P.n - (P.prec == 0 ? LB64 : LB);
+    for (int st = 0; st <= nh; ++st) {
+        const cudaError_t e = launch_rows_level(P, sweep, sweep == 0 ? st : nh - st, A, X, s);
+        if (e != cudaSuccess) return e;
+        if (launches) ++*launches;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t launch_forward_rows(const Plan& P, const void* A, void* F, cudaStream_t s, int* launches)
 {
-    const int nh = P.n - (P.prec == 0 ? LB64 : LB);
-    for (int hl = 0; hl <= nh; ++hl) {
-        const uint32_t nt = (uint32_t)choose(nh, hl);
-        const unsigned tb = rec_block(level_block(nt));
-        const dim3 grid((nt + tb - 1) / tb, P.nj);
-        if (P.prec == 0)
-            launch_or_record(KID_FROWS_D, k_forward_rows<double, false>, grid, tb, 0, s, P.n, hl, nt, (const double*)A,
-                                                               (double*)F, P.js, 0u, 0, (const double*)nullptr);
-        else if (use_tlo(P))
-            launch_or_record(KID_FROWS_F_TLO, k_forward_rows<float, true>, grid, tb, 0, s, P.n, hl, nt, (const float*)A,
-                                                             (float*)F, P.js, 0u, 0, (const float*)nullptr);
-        else
-            launch_or_record(KID_FROWS_F, k_forward_rows<float, false>, grid, tb, 0, s, P.n, hl, nt, (const float*)A,
-                                                              (float*)F, P.js, 0u, 0, (const float*)nullptr);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        if (launches) ++*launches;
-    }
-    return cudaSuccess;
+    return rows_sweep(P, 0, A, F, s, launches);
 }
 
-cudaError_t launch_backward_rows(const Plan& P, const void* A, void* Rc, cudaStream_t s,
-                                 int* launches)
+cudaError_t launch_backward_rows(const Plan& P, const void* A, void* Rc, cudaStream_t s, int* launches)
 {
-    const int nh = P.n - (P.prec == 0 ? LB64 : LB);
-    for (int hl = nh; hl >= 0; --hl) {
-        const uint32_t nt = (uint32_t)choose(nh, hl);
-        const unsigned tb = rec_block(level_block(nt));
-        const dim3 grid((nt + tb - 1) / tb, P.nj);
-        if (P.prec == 0)
-            launch_or_record(KID_BROWS_D, k_backward_rows<double, false>, grid, tb, 0, s, P.n, hl, nt, (const double*)A,
-                                                                (double*)Rc, P.js, 0u, 0, (const double*)nullptr);
-        else if (use_tlo(P))
-            launch_or_record(KID_BROWS_F_TLO, k_backward_rows<float, true>, grid, tb, 0, s, P.n, hl, nt, (const float*)A,
-                                                              (float*)Rc, P.js, 0u, 0, (const float*)nullptr);
-        else
-            launch_or_record(KID_BROWS_F, k_backward_rows<float, false>, grid, tb, 0, s, P.n, hl, nt, (const float*)A,
-                                                               (float*)Rc, P.js, 0u, 0, (const float*)nullptr);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        if (launches) ++*launches;
-    }
-    return cudaSuccess;
+    return rows_sweep(P, 1, A, Rc, s, launches);
 }
 
-// Blocks that share one item of k_sweeps and how they meet.  One block of 512
-// threads holds 32 tiles at a time: levels of up to 64 tiles (n <= 11) gain
-// nothing from a second one.  Clusters (at most 8 blocks, the portable size)
-// serve the middle and every batch group; from kSweepGrid tiles in the widest
-// level on the whole GPU shares the two sweeps of a single job (err given).
-static int sweep_blocks(uint64_t widest, const int* err)
+// Blocks that share one item of k_sweeps: enough that every tile of the
+// widest level has its own lanes.  Clusters (at most 8 blocks, the portable
+// size) serve the small jobs and every batch group; past kSweepGrid blocks
+// the whole GPU shares the two sweeps of a single job (err given).
+static int sweep_blocks(const Plan& P, const int* err)
 {
+    const int B = P.prec == 0 ? LB64 : LB;
+    const uint64_t widest = choose(P.n - B, (P.n - B) / 2), per = kSweepThreads >> B;
     // the whole-GPU form needs the counters beside the job's error word
-    const uint64_t most = err && widest > kSweepGrid ? 152 : 8;
-    return (int)std::max<uint64_t>(1, std::min<uint64_t>((widest + 31) / 32, most));
+    const uint64_t most = err && widest > kSweepGrid * per ? 152 : 8;
+    return (int)std::max<uint64_t>(1, std::min<uint64_t>((widest + per - 1) / per, most));
 }
 
 bool sweeps_fit(const Plan& P)
 {
-    return rows_levels_fit(P) && P.frows && P.shard_k == 0 && !P.slab && !P.spill;
+    return ((rows_levels_fit(P) && P.frows) || P.lin) && P.shard_k == 0 && !P.slab && !P.spill;
 }
 
 bool use_sweeps(const Plan& P, const int* err)
 {
-    return sweeps_fit(P) && P.n <= kSweepMaxN && err && !recording();
+    return sweeps_fit(P) && P.n <= (P.lin ? kSweepMaxNX : kSweepMaxN) && err && !recording();
 }
 
 template <typename T, bool TLO>
 static cudaError_t sweeps(const Plan& P, const T* A, T* F, T* Rc, int items, cudaStream_t s, int* err)
 {
-    const uint64_t widest = choose(P.n - LB, (P.n - LB) / 2);
-    const int nb = sweep_blocks(widest, err);
+    const int nb = sweep_blocks(P, err);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(items * nb), 1, 1);
     cfg.blockDim = dim3(kSweepThreads, 1, 1);
@@ -945,7 +1000,9 @@ cudaError_t launch_sweeps(const Plan& P, const void* A, void* F, void* Rc, cudaS
                           int* launches)
 {
     const int items = Rc ? 2 * P.nj : 1;            // a feature's job: F alone
-    const cudaError_t e = use_tlo(P) ? sweeps<float, true>(P, (const float*)A, (float*)F, (float*)Rc, items, s, err)
+    const cudaError_t e = P.lin == 2 ? sweeps<X64S, false>(P, (const X64S*)A, (X64S*)F, (X64S*)Rc, items, s, err)
+                          : P.lin ? sweeps<X64, false>(P, (const X64*)A, (X64*)F, (X64*)Rc, items, s, err)
+                          : use_tlo(P) ? sweeps<float, true>(P, (const float*)A, (float*)F, (float*)Rc, items, s, err)
                                      : sweeps<float, false>(P, (const float*)A, (float*)F, (float*)Rc, items, s, err);
     if (e == cudaSuccess && launches) ++*launches;
     return e;

@@ -141,6 +141,29 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
         }
     } else {
         switch (kid) {
+        case KID_SHIFT_X: run(k_shift_scores<X64>, a); return true;
+        case KID_SHIFT_XS: run(k_shift_scores<X64S>, a); return true;
+        case KID_UPZETA_XS: run(k_upzeta_x, a); return true;
+        case KID_FROWS_XS: run(k_forward_rows<X64S, false>, a); return true;
+        case KID_BROWS_XS: run(k_backward_rows<X64S, false>, a); return true;
+        case KID_GAMMA_P1_XS: run(k_gamma_p1_x, a); return true;
+        case KID_GAMMA_P2_XS: run(k_gamma_p2<X64S>, a); return true;
+        case KID_GAMMA_P2S_XS: run(k_gamma_p2s_x<X64S>, a); return true;
+        case KID_EDGES_ACC_XS: run(k_edges_acc_x<X64S>, a); return true;
+        case KID_EDGES_FIN_XS: run(k_edges_fin<X64S>, a); return true;
+        case KID_REORDER_X: run(k_reorder_up<X64>, a); return true;
+        case KID_COLB4_X: run(k_colb_x<4>, a); return true;
+        case KID_COLB2_X: run(k_colb_x<2>, a); return true;
+        case KID_COLB1_X: run(k_colb_x<1>, a); return true;
+        case KID_COLW_X: run(k_upzeta13_colw<X64>, a); return true;
+        case KID_UP13_X: run(k_up13_x, a); return true;
+        case KID_FROWS_X: run(k_forward_rows<X64, false>, a); return true;
+        case KID_BROWS_X: run(k_backward_rows<X64, false>, a); return true;
+        case KID_G13_X: run(k_g13_x<false>, a); return true;
+        case KID_GAMMA_P2_X: run(k_gamma_p2<X64>, a); return true;
+        case KID_GAMMA_P2S_X: run(k_gamma_p2s_x<X64>, a); return true;
+        case KID_EDGES_ACC_X: run(k_edges_acc_x<X64>, a); return true;
+        case KID_EDGES_FIN_X: run(k_edges_fin<X64>, a); return true;
         case KID_SHIFT_D: run(k_shift_scores<double>, a); return true;
         case KID_UPZETA_D: run(k_upzeta<double>, a); return true;
         case KID_FWD_LEVEL_D: run(k_forward_level<double>, a); return true;
@@ -284,6 +307,12 @@ bool persistent_runs(int prec, int kid)
     case KID_EDGES_FIN_D: case KID_REORDER_D: case KID_COLW_D: case KID_COLS_D: case KID_UP13_D:
     case KID_COLB4_D: case KID_COLB2_D: case KID_COLB1_D:
     case KID_G13_D: case KID_FROWS_D: case KID_BROWS_D:
+    case KID_SHIFT_XS: case KID_UPZETA_XS: case KID_FROWS_XS: case KID_BROWS_XS: case KID_GAMMA_P1_XS:
+    case KID_GAMMA_P2_XS: case KID_GAMMA_P2S_XS: case KID_EDGES_ACC_XS: case KID_EDGES_FIN_XS:
+    case KID_SHIFT_X: case KID_REORDER_X: case KID_COLB4_X: case KID_COLB2_X:
+    case KID_COLB1_X: case KID_COLW_X: case KID_UP13_X: case KID_FROWS_X: case KID_BROWS_X:
+    case KID_G13_X: case KID_GAMMA_P2_X: case KID_GAMMA_P2S_X:
+    case KID_EDGES_ACC_X: case KID_EDGES_FIN_X:
         return prec == 0;
     default:
         return false;

@@ -192,6 +192,9 @@ try {
     P.nlow_g = (uint32_t)nl;
     P.wb = P.n < 5 ? P.n : 5;
     bn::default_schedule(P);
+    double rho_max = 0.0;
+    for (int k = 0; k <= P.d; ++k) rho_max = std::fmax(rho_max, std::fabs(log_rho[k]));
+    P.lin = bn::lin_tiles_fit(P) ? bn::lin_range(P, arity, j->ess, rho_max) : 0;
 
     // layout inside the static array
     const size_t es = P.prec == 0 ? 8 : 4;
@@ -260,7 +263,7 @@ try {
     }
     CKS(bn::launch_gamma_p1(P, base + o_F, base + o_Rc, rk13, base + o_W, s, nullptr, base + o_A));
     CKS(bn::launch_gamma_p2(P, base + o_W, base + o_G, s));
-    CKS(bn::launch_edges(P, logB, cmax, masks, base + o_G, base + o_F, err,
+    CKS(bn::launch_edges(P, logB, base + o_lbs, cmax, masks, base + o_G, base + o_F, err,
                          reinterpret_cast<unsigned long long*>(base + o_ea), post_dev,
                          log_PD_dev, s));
 #undef CKS

@@ -161,17 +161,67 @@ int log_weights(const double* src, size_t count, std::vector<double>& dst)
     return BN_OK;
 }
 
-// In the working precision and log base (FP32: base 2).
-std::vector<char> working_logs(const std::vector<double>& v, int prec)
+// exp(x) of a natural log as an XValue (bn_device.cuh), and back (host).
+template <typename X> unsigned long long x_from_ln(double x)
 {
-    std::vector<char> out(v.size() * (prec == 0 ? 8 : 4));
-    if (prec == 0) {
+    if (!(x > -91000.0)) return 0ull;
+    int e = (int)std::lround(x * 1.4426950408889634074);
+    const double r = (x - e * bn::explog::kLn2Hi) - e * bn::explog::kLn2Lo;
+    int e2 = 0;
+    const double m = std::frexp(std::exp(r), &e2) * 2.0;    // [1, 2)
+    e += e2 - 1;
+    unsigned long long f = (unsigned long long)std::llround(std::ldexp(m, X::frac));
+    if (f >> (X::frac + 1)) { f >>= 1; ++e; }
+    if (e < X::min) return 0ull;
+    return ((unsigned long long)(e + X::bias) << X::frac) | (f & ((1ull << X::frac) - 1));
+}
+template <typename X> double x_to_ln(unsigned long long u)
+{
+    if (!u) return -INFINITY;
+    const double m = 1.0 + std::ldexp((double)(u & ((1ull << X::frac) - 1)), -X::frac);
+    return ((double)((int)(u >> X::frac) - X::bias)) * 0.69314718055994530942 + std::log(m);
+}
+double lin_to_ln(const Plan& P, unsigned long long u)
+{
+    return P.lin == 2 ? x_to_ln<bn::X64S>(u) : x_to_ln<bn::X64>(u);
+}
+
+// In the form of the plan's values: FP32 base-2 logs, FP64 natural logs or
+// the values themselves.
+std::vector<char> working_logs(const std::vector<double>& v, const Plan& P)
+{
+    std::vector<char> out(v.size() * (P.prec == 0 ? 8 : 4));
+    if (P.lin) {
+        unsigned long long* u = reinterpret_cast<unsigned long long*>(out.data());
+        for (size_t t = 0; t < v.size(); ++t) u[t] = P.lin == 2 ? x_from_ln<bn::X64S>(v[t]) : x_from_ln<bn::X64>(v[t]);
+    } else if (P.prec == 0) {
         std::memcpy(out.data(), v.data(), out.size());
     } else {
         float* f = reinterpret_cast<float*>(out.data());
         for (size_t t = 0; t < v.size(); ++t) f[t] = (float)(v[t] * 1.4426950408889634);
     }
     return out;
+}
+
+// The largest magnitude of the weights that are not zero.
+double largest_log(const std::vector<double>& v)
+{
+    double x = 0.0;
+    for (double y : v)
+        if (y > 0.5 * kLogZero) x = std::max(x, std::fabs(y));
+    return x;
+}
+
+// Whether the job's values stay linear (FP64; more: a feature's log weights).
+// A zero weight on an empty parent set leaves F(V) without its lower bound.
+void plan_lin(HostJob& hj, double more)
+{
+    Plan& P = hj.P;
+    const double logs = largest_log(hj.log_rho) + largest_log(hj.log_q) + largest_log(hj.log_w) + more;
+    P.lin = bn::lin_tiles_fit(P) ? bn::lin_range(P, hj.arity.data(), hj.ess, logs) : 0;
+    if (P.hasw)
+        for (int i = 0; i < P.n; ++i)
+            if (hj.log_w[(size_t)i * P.K] < 0.5 * kLogZero) P.lin = 0;
 }
 
 int validate_and_plan(const bn_job_desc* j, HostJob& hj)
@@ -232,6 +282,7 @@ int validate_and_plan(const bn_job_desc* j, HostJob& hj)
     P.nlow_g = (uint32_t)nl;
     P.wb = std::min(P.n, 5);
     bn::default_schedule(P);
+    plan_lin(hj, 0.0);
     return BN_OK;
 }
 
@@ -316,7 +367,7 @@ int upload_priors(const HostJob& hj, const Bufs& B, cudaStream_t s)
 {
     const Plan& P = hj.P;
     if (P.hasq) {
-        const std::vector<char> q = working_logs(hj.log_q, P.prec);
+        const std::vector<char> q = working_logs(hj.log_q, P);
         CK(cudaMemcpyAsync(B.at<char>(B.L.logq), q.data(), q.size(), cudaMemcpyHostToDevice, s));
     }
     if (P.hasw)
@@ -474,7 +525,7 @@ int enqueue_kernels(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, d
         if (ev) CK(cudaEventRecord(ev->ev[6], s));
         nl += bn::gamma_launches(P);
     }
-    CK(bn::launch_edges(P, B.at<double>(L.logB), B.at<double>(L.cmax), B.at<uint32_t>(L.masks),
+    CK(bn::launch_edges(P, B.at<double>(L.logB), B.at<void>(L.lbs), B.at<double>(L.cmax), B.at<uint32_t>(L.masks),
                         B.at<void>(L.Gam), B.at<void>(L.F), err,
                         B.at<unsigned long long>(L.eacc), post_dev, logPD_dev, s));
     nl += 3;
@@ -583,8 +634,8 @@ struct bn_ctx {
     uint64_t reserved = 0;
     // batches
     int flags = 0;
-    // (n, d, prec, binary, jobs) -> schedule (up13, frows, frc, g13)
-    std::map<std::array<int, 5>, std::array<int, 4>> tuned;
+    // (n, d, prec, binary, jobs, linear) -> schedule (up13, frows, frc, g13)
+    std::map<std::array<int, 6>, std::array<int, 4>> tuned;
 };
 
 // Jobs of a batch with equal n, d and precision: their arrays lie js bytes
@@ -1064,6 +1115,7 @@ try {
     const Plan& P = hj.P;
     std::vector<double> lf;
     if (log_weights(log_f, (size_t)P.n * P.K, lf)) return BN_EINVAL;
+    plan_lin(hj, largest_log(lf));
     if (cudaSetDevice(c->device) != cudaSuccess) return BN_ECUDA;
     const Layout L = make_layout(P, 0, true);
     rc = ensure_ws(c, L.total);
@@ -1091,7 +1143,7 @@ try {
     CK(cudaMemcpyAsync(B.at<char>(L.alpha), alpha.data(), alpha.size() * 8, cudaMemcpyHostToDevice, s));
     rc = upload_priors(hj, B, s);
     if (rc) return rc;
-    const std::vector<char> lfw = working_logs(lf, P.prec);
+    const std::vector<char> lfw = working_logs(lf, P);
     CK(cudaMemcpyAsync(B.at<char>(L.logf), lfw.data(), lfw.size(), cudaMemcpyHostToDevice, s));
 
     // P(D): steps 1-3 with f = 1 (F only); then P(f, D) from the same
@@ -1132,7 +1184,11 @@ try {
     CK(cudaStreamSynchronize(s));
     if (err) return err_word_status(err);
     for (int k = 0; k < 2; ++k) {
-        if (P.prec == 0) {
+        if (P.lin) {
+            unsigned long long u;
+            std::memcpy(&u, raw[k], 8);
+            fv[k] = lin_to_ln(P, u);
+        } else if (P.prec == 0) {
             std::memcpy(&fv[k], raw[k], 8);
         } else {
             float x;
@@ -1299,6 +1355,14 @@ try {
     const char* src = (stage == BN_STAGE_A && P.spill) ? c->spill : c->ws + off;   // a spilled A
     CK(cudaMemcpy(host_out, src, want, cudaMemcpyDeviceToHost));
     if (stage == BN_STAGE_A && bn::use_tlo(P)) tlo_to_plain(P.n, static_cast<float*>(host_out));
+    if (P.lin && (stage == BN_STAGE_A || stage == BN_STAGE_F || stage == BN_STAGE_RC || stage == BN_STAGE_GAMMA)) {
+        double* x = static_cast<double*>(host_out);
+        for (size_t t = 0; t < want / 8; ++t) {
+            unsigned long long u;
+            std::memcpy(&u, x + t, 8);
+            x[t] = lin_to_ln(P, u);
+        }
+    }
     if (P.prec != 0 && (stage == BN_STAGE_F || stage == BN_STAGE_RC || stage == BN_STAGE_GAMMA))
         undo_level_bases(c, P, L, stage, static_cast<float*>(host_out));
     return BN_OK;
@@ -1399,7 +1463,7 @@ int enqueue_steps(const Plan& G, const Layout& L, char* base, cudaStream_t s, un
         CK(bn::launch_gamma_p2(G, at(L.W), at(L.Gam), s));
     }
     if (stages & 16u)
-        CK(bn::launch_edges(G, reinterpret_cast<const double*>(at(L.logB)),
+        CK(bn::launch_edges(G, reinterpret_cast<const double*>(at(L.logB)), at(L.lbs),
                             reinterpret_cast<const double*>(at(L.cmax)),
                             reinterpret_cast<const uint32_t*>(at(L.masks)), at(L.Gam), at(L.F),
                             reinterpret_cast<const int*>(at(L.err)),
@@ -1511,7 +1575,9 @@ int record_groups(bn_batch* b)
                 switch (x.kid) {                   // kernels that loop grid-stride in x
                 case bn::KID_STEP1_PREP: case bn::KID_CHECK_DATA: case bn::KID_SET_HIST_WARP:
                 case bn::KID_SET_HIST_BLOCK: case bn::KID_SET_ANY: case bn::KID_FAMILIES:
-                case bn::KID_SHIFT_F: case bn::KID_SHIFT_D: case bn::KID_EDGES_ACC_F:
+                case bn::KID_SHIFT_F: case bn::KID_SHIFT_D: case bn::KID_SHIFT_X: case bn::KID_EDGES_ACC_X:
+                case bn::KID_SHIFT_XS: case bn::KID_EDGES_ACC_XS:
+                case bn::KID_REORDER_X: case bn::KID_COLW_X: case bn::KID_EDGES_ACC_F:
                 case bn::KID_EDGES_ACC_D: case bn::KID_REORDER_F: case bn::KID_REORDER_D:
                 case bn::KID_COLW_F: case bn::KID_COLW_D:
                     x.pad[0] |= bn::kRecStrideX;
@@ -1521,10 +1587,12 @@ int record_groups(bn_batch* b)
                 }
                 pp.smem = std::max<size_t>(pp.smem, x.smem);
                 const bool f = x.kid == bn::KID_FROWS_F || x.kid == bn::KID_FROWS_F_TLO ||
-                               x.kid == bn::KID_FROWS_D || x.kid == bn::KID_FWD_LEVEL_F ||
+                               x.kid == bn::KID_FROWS_D || x.kid == bn::KID_FROWS_X ||
+                               x.kid == bn::KID_FROWS_XS || x.kid == bn::KID_FWD_LEVEL_F ||
                                x.kid == bn::KID_FWD_LEVEL_D;
                 const bool r = x.kid == bn::KID_BROWS_F || x.kid == bn::KID_BROWS_F_TLO ||
-                               x.kid == bn::KID_BROWS_D || x.kid == bn::KID_BWD_LEVEL_F ||
+                               x.kid == bn::KID_BROWS_D || x.kid == bn::KID_BROWS_X ||
+                               x.kid == bn::KID_BROWS_XS || x.kid == bn::KID_BWD_LEVEL_F ||
                                x.kid == bn::KID_BWD_LEVEL_D;
                 if (f || r) {
                     if (level_at == SIZE_MAX) level_at = stages.size();
@@ -1711,8 +1779,9 @@ int tune_batch(bn_batch* b, cudaStream_t s)
         return BN_ECUDA;
     }
     struct Knob { int Plan::*flag; bool (*fits)(const Plan&); };
-    const Knob knobs[4] = {{&Plan::up13, bn::tile13_up_fits}, {&Plan::frows, bn::rows_levels_fit}, {&Plan::frc, bn::sweeps_fit},
-                           {&Plan::g13, bn::tile13_gamma_fits}};
+    // (the linear FP64 form has the tile kernels only)
+    const Knob knobs[4] = {{&Plan::up13, [](const Plan& P) { return !P.lin && bn::tile13_up_fits(P); }}, {&Plan::frows, bn::rows_levels_fit}, {&Plan::frc, bn::sweeps_fit},
+                           {&Plan::g13, [](const Plan& P) { return !P.lin && bn::tile13_gamma_fits(P); }}};
     const bool forced_frc = (b->ctx->flags & BN_CTX_CLUSTER_STEP3) != 0;
     float best = 0.0f;
     int rc = time_batch(b, s, e0, e1, &best);
@@ -1766,7 +1835,7 @@ try {
     b->jobs.resize(count);
     b->group_of.assign(count, -1);
     b->slot_of.assign(count, -1);
-    std::map<std::array<int, 4>, int> key_to_group;
+    std::map<std::array<int, 5>, int> key_to_group;
     for (int k = 0; k < count; ++k) {
         HostJob& hj = b->jobs[k];
         int rc = jobs[k].data_on_device ? BN_EINVAL : validate_and_plan(&jobs[k], hj);
@@ -1778,7 +1847,7 @@ try {
         hj.data = hj.data_copy.data();
         // step 1 of a group is one launch per kernel, so its jobs also share
         // the choice of score kernel (binary data or not)
-        const std::array<int, 4> key{P.n, P.d, P.prec, P.allbin};
+        const std::array<int, 5> key{P.n, P.d, P.prec, P.allbin, P.lin};
         auto it = key_to_group.find(key);
         if (it == key_to_group.end()) {
             it = key_to_group.emplace(key, (int)b->groups.size()).first;
@@ -1853,7 +1922,7 @@ try {
     for (auto& g : b->groups)
         if (c->flags & BN_CTX_CLUSTER_STEP3) g.P.frc = bn::sweeps_fit(g.P);
     auto key_of = [](const Plan& P) {
-        return std::array<int, 5>{P.n, P.d, P.prec, P.allbin, P.nj};
+        return std::array<int, 6>{P.n, P.d, P.prec, P.allbin, P.nj, P.lin};
     };
     const bool want_persistent = !(c->flags & (BN_CTX_GRAPH_BATCH | BN_CTX_CLUSTER_STEP3));
     if (ok && !(c->flags & BN_CTX_NO_AUTOTUNE)) {
@@ -2450,7 +2519,7 @@ try {
                            B.at<void>(L.W), s, P.hasq ? B.at<void>(L.logq) : nullptr,
                            P.slab ? nullptr : B.at<void>(L.A)));
     CK(bn::launch_gamma_p2(P, B.at<void>(L.W), B.at<void>(L.Gam), s));
-    CK(bn::launch_edges(P, B.at<double>(L.logB), B.at<double>(L.cmax), B.at<uint32_t>(L.masks),
+    CK(bn::launch_edges(P, B.at<double>(L.logB), B.at<void>(L.lbs), B.at<double>(L.cmax), B.at<uint32_t>(L.masks),
                         B.at<void>(L.Gam), B.at<void>(L.F), B.at<int>(L.err),
                         B.at<unsigned long long>(L.eacc), post_dev,
                         log_PD_dev ? log_PD_dev : B.at<double>(L.logPD), s));

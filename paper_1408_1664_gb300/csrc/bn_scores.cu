@@ -588,7 +588,12 @@ k_family_scores(int n, int64_t K, const long long* __restrict__ H, uint32_t nset
     if (enc && threadIdx.x < n && top[threadIdx.x]) atomicMax(job_ptr(enc, js) + threadIdx.x, top[threadIdx.x]);
 }
 
-// The shifted scores lbs = log B - c_i in the working precision and base,
+__device__ __forceinline__ void from_ln(double x, float& y) { y = (float)LogOps<float>::from_ln(x); }
+__device__ __forceinline__ void from_ln(double x, double& y) { y = x; }
+template <int FB> __device__ __forceinline__ void from_ln(double x, XValue<FB>& y) { y = x_from_ln<XValue<FB>>(x); }
+
+// The shifted scores lbs = log B - c_i in the working precision and base
+// (XValue: B / exp(c_i)),
 // the shifts cmax themselves (from their encodings), and, for the
 // 13-dimension up-zeta tiles (tab not null), the same scores reordered by
 // high and low part of the parent set (see k_reorder_up).
@@ -626,7 +631,8 @@ k_shift_scores(int n, int d, int64_t K, const double* __restrict__ logB,
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < total;
          x += (int64_t)gridDim.x * blockDim.x) {
         const int i = (int)(x / K);
-        const T y = (T)LogOps<T>::from_ln(logB[x] - ord_dec(enc[i]));
+        T y;
+        from_ln(logB[x] - ord_dec(enc[i]), y);
         lbs[x] = y;
         if (tab) {
             const uint32_t cm = cmasks[x];
@@ -810,6 +816,12 @@ cudaError_t launch_shift_scores(const Plan& P, const double* logB, const unsigne
                                 const uint32_t* cmasks, double* cmax, void* lbs, void* tab, cudaStream_t s)
 {
     const dim3 grid(grid_for((int64_t)P.n * P.K, 256, 152 * 16), P.nj);
+    if (P.lin == 2)
+        return launch_or_record(KID_SHIFT_XS, k_shift_scores<X64S>, grid, 256, 0, s, P.n, P.d, P.K, logB, enc,
+                                cmasks, cmax, (X64S*)lbs, (X64S*)nullptr, P.js);
+    if (P.lin)
+        return launch_or_record(KID_SHIFT_X, k_shift_scores<X64>, grid, 256, 0, s, P.n, P.d, P.K, logB, enc,
+                                cmasks, cmax, (X64*)lbs, (X64*)tab, P.js);
     if (P.prec == 0)
         return launch_or_record(KID_SHIFT_D, k_shift_scores<double>, grid, 256, 0, s, P.n, P.d, P.K, logB, enc,
                                 cmasks, cmax, (double*)lbs, (double*)tab, P.js);

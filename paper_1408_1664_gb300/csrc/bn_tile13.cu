@@ -611,20 +611,6 @@ k_upzeta13_cols(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
     for (uint32_t c = ncopy + t; c < ncol; c += TT) out[c] = tb[c];
 }
 
-// Log-sum-exp kept lazily: (m, s) stands for m + log(s); s is rescaled only
-// when a term exceeds m by more than 64 log units, so a term costs one
-// exponential (the values are finite).
-template <typename T>
-__device__ __forceinline__ void lse_lazy(T& m, T& s, T x)
-{
-    using Lg = LogOps<T>;
-    const T dd = x - m;                           // +inf while the accumulator is empty
-    const bool big = dd > T(64);
-    const T e = Lg::ex(big ? -dd : dd);
-    s = big ? madd(s, e, T(1)) : s + e;
-    m = big ? x : m;
-}
-
 // Part 1 with one warp per tile: each warp enumerates its tile's rows into
 // its own list and sums the columns lane by lane (consecutive columns:
 // coalesced reads of a row); no block barrier after the tables are filled.
@@ -815,11 +801,14 @@ k_upzeta13_colb(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
 // of tile (i, (q << hl) | L) holds the sum over the rows inside chunk q
 // alone; the upward zeta over the hc chunk bits, a thread per (i, L, c) with
 // c fastest (coalesced), leaves the full column sums.
+__device__ __forceinline__ float sum_of(float a, float b) { return LogOps<float>::lse(a, b); }
+__device__ __forceinline__ double sum_of(double a, double b) { return LogOps<double>::lse(a, b); }
+__device__ __forceinline__ X64 sum_of(X64 a, X64 b) { return x_add(a, b); }
+
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_upzeta13_colt(int n, T* __restrict__ A, int nodes, uint32_t ncb, int hc)
 {
-    using Lg = LogOps<T>;
     const int h = n - 1 - TB, hl = h - hc;
     const uint64_t total = ((uint64_t)nodes << hl) * ncb;
     const size_t asize = (size_t)nodes << (n - 1);
@@ -839,7 +828,7 @@ k_upzeta13_colt(int n, T* __restrict__ A, int nodes, uint32_t ncb, int hc)
             if (b >= hc) continue;
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-                if (k < (1 << hc) && (k >> b & 1)) q[k] = Lg::lse(q[k], q[k ^ (1 << b)]);
+                if (k < (1 << hc) && (k >> b & 1)) q[k] = sum_of(q[k], q[k ^ (1 << b)]);
         }
 #pragma unroll
         for (int k = 1; k < 8; ++k)
@@ -854,7 +843,6 @@ k_upzeta13_colw(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
 {
     tab = job_ptr(tab, js);
     A = job_ptr(A, js);
-    using Lg = LogOps<T>;
     __shared__ SBinom sb;
     __shared__ uint32_t off13[16];
     __shared__ uint32_t rowoff_k[32];            // offset of the first size-k row in a node's table
@@ -909,17 +897,17 @@ k_upzeta13_colw(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
             while (off13[j + 1] <= c) ++j;
             uint32_t rend = 0;
             for (int k = 0; k <= d - j && k <= hc; ++k) rend += sb_binom(sb, hc, k);
-            T m = Lg::ninf(), s = T(0);
+            LazySum<T> s;
 #pragma unroll 4
-            for (uint32_t rp = 0; rp < rend; ++rp) lse_lazy(m, s, tb[BN_AT(rowbase[rp] + c, 1, K)]);
-            out[c] = m + Lg::lg(s);
+            for (uint32_t rp = 0; rp < rend; ++rp) s.add(tb[BN_AT(rowbase[rp] + c, 1, K)]);
+            out[c] = s.value();
         }
         const uint32_t rmid = 1u + (uint32_t)hc;               // d - 1 low elements
         for (uint32_t c = nlong + lane; c < ncopy; c += 32) {
-            T m = Lg::ninf(), s = T(0);
+            LazySum<T> s;
 #pragma unroll 4
-            for (uint32_t rp = 0; rp < rmid; ++rp) lse_lazy(m, s, tb[BN_AT(rowbase[rp] + c, 1, K)]);
-            out[c] = m + Lg::lg(s);
+            for (uint32_t rp = 0; rp < rmid; ++rp) s.add(tb[BN_AT(rowbase[rp] + c, 1, K)]);
+            out[c] = s.value();
         }
         for (uint32_t c = ncopy + lane; c < ncol; c += 32) out[c] = tb[c];   // d low elements
         __syncwarp();                                          // rowbase is reused
@@ -1455,6 +1443,324 @@ k_gamma13_p1(int n, int d, uint32_t nlow, const T* __restrict__ F,
     }
 }
 
+// ===========================================================================
+// The 13-dimension tiles of the linear FP64 form (X64, bn_device.cuh): the
+// same transforms with the values themselves.  A pass takes the tile's values
+// relative to one exponent `ref` as doubles (2^-1000 .. 2^1010: integer
+// operations, no exponential), runs the butterflies as additions, and packs
+// what it resolves (no logarithm): an output of at least 2^-900 there has lost
+// at most 8192 terms below 2^-1000, under 2^-87 of it.  Later passes move ref
+// down by 1900 bits until every output is resolved; values above 2^1010 are
+// +inf there and belong to outputs already written.  Nearly every tile takes
+// one pass.  What bounds it: the FP64 additions of the butterflies (6.5 per
+// value, two lanes per clock and SM).
+// ===========================================================================
+constexpr int kXTop = 1010, kXKeep = -900, kXStep = 1900;
+
+// Largest exponent of a block of TT threads (every thread gets it).
+__device__ __forceinline__ int block_max(int e, int* red, int t)
+{
+    e = __reduce_max_sync(FULLMASK, e);
+    if ((t & 31) == 0) red[t >> 5] = e;
+    __syncthreads();
+    int m = red[0];
+#pragma unroll
+    for (int w = 1; w < TT / 32; ++w) m = max(m, red[w]);
+    return m;
+}
+
+// Column sums by butterflies over the high dimensions (k_upzeta13_colb).
+__device__ __forceinline__ void colb_steps_x(X64* v, uint32_t H2, int h, int CPB)
+{
+    for (int j = 0; j < h; ++j) {
+        const uint32_t lowm = (1u << j) - 1u, np = H2 >> 1;
+        for (uint32_t g = threadIdx.x; g < np * CPB; g += blockDim.x) {
+            const uint32_t cc = g / np, p = g % np;
+            const uint32_t lo = cc * H2 + (((p & ~lowm) << 1) | (p & lowm)), hi = lo | (1u << j);
+            v[hi] = x_add(v[hi], v[lo]);
+        }
+        __syncthreads();
+    }
+}
+
+template <int CPB>
+__global__ void __launch_bounds__(256)
+k_colb_x(int n, int d, int64_t K, const X64* __restrict__ tab, X64* __restrict__ A, size_t js, int nodes,
+         uint32_t ncb, int hc)
+{
+    tab = job_ptr(tab, js);
+    A = job_ptr(A, js);
+    __shared__ SBinom sb;
+    __shared__ uint32_t off13[16];
+    __shared__ uint32_t rowoff_k[32];
+    __shared__ int wred[8][CPB];                     // the warps' column maxima (exponents)
+    __shared__ int ref_s[CPB];                       // a column's reference exponent
+    __shared__ int lin_s;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    X64* v = reinterpret_cast<X64*>(smem_raw);       // [column of the run][H]
+    double* vd = reinterpret_cast<double*>(smem_raw);
+    const int h = n - 1 - TB;
+    const int hl = h - hc;                           // hc: chunk bits (see k_upzeta13_colb)
+    const uint32_t H2 = 1u << hl;
+    const uint32_t ncol = num_small_subsets(TB, d);
+    const uint32_t nrun = (ncb + CPB - 1) / CPB;
+    const uint32_t nbb = ((uint32_t)nodes * nrun) << hc;
+    const size_t asize = (size_t)nodes << (n - 1);
+    if (blockIdx.x >= nbb) {                         // copies: a warp per tile
+        const uint32_t tile = (blockIdx.x - nbb) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+        if (tile >= ((uint32_t)nodes << h)) return;
+        const X64* tb = tab + (size_t)(tile >> h) * K;
+        X64* out = A + BN_AT((size_t)tile << TB, TN, asize);
+        for (uint32_t c = ncb + (threadIdx.x & 31); c < ncol; c += 32) out[c] = tb[BN_AT(c, 1, K)];
+        return;
+    }
+    fill_sbinom(sb);
+    if (threadIdx.x < 16) {
+        uint32_t o = 0;
+        for (int k = 0; k < (int)threadIdx.x && k <= TB; ++k) o += binom(TB, k);
+        off13[threadIdx.x] = o;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        uint32_t o = 0;
+        for (int k = 0; k < (int)threadIdx.x && k <= min(d, h); ++k)
+            o += binom(h, k) * off13[min(d - k, TB) + 1];
+        rowoff_k[threadIdx.x] = o;
+    }
+    __syncthreads();
+    const uint32_t chunk = blockIdx.x & ((1u << hc) - 1u);
+    const int i = (int)((blockIdx.x >> hc) / nrun);
+    const uint32_t c0 = ((blockIdx.x >> hc) % nrun) * CPB;
+    const uint32_t Hc = chunk << hl;
+    const X64* tb = tab + (size_t)i * K;
+    int kl[CPB], mx[CPB];
+#pragma unroll
+    for (int cc = 0; cc < CPB; ++cc) {
+        const uint32_t c = c0 + cc;
+        int k = 0;
+        while (k < TB && off13[k + 1] <= c) ++k;
+        kl[cc] = c < ncb ? k : -1;
+        mx[cc] = -kXBias;
+    }
+    for (uint32_t H = threadIdx.x; H < H2; H += blockDim.x) {
+        const uint32_t Hf = Hc | H;
+        const int kh = __popc(Hf);
+        uint32_t r = 0;
+        int t = 1;
+        for (uint32_t x = Hf; x; x &= x - 1, ++t) r += sb_binom(sb, __ffs(x) - 1, t);
+        const uint32_t row = kh <= d ? rowoff_k[kh] + r * off13[min(d - kh, TB) + 1] : 0u;
+#pragma unroll
+        for (int cc = 0; cc < CPB; ++cc) {
+            const bool in = kl[cc] >= 0 && kh <= d - kl[cc];
+            const X64 val = in ? tb[BN_AT(row + c0 + cc, 1, K)] : X64{0ull};
+            v[cc * H2 + H] = val;
+            mx[cc] = max(mx[cc], x_exp(val));
+        }
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int cc = 0; cc < CPB; ++cc) {
+        mx[cc] = __reduce_max_sync(FULLMASK, mx[cc]);
+        if (lane == 0) wred[warp][cc] = mx[cc];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        // a column's outputs lie between its H = {} value and its largest
+        // input times 2^h: one pass when both fit
+        int lin = 1;
+        for (int cc = 0; cc < CPB; ++cc) {
+            int m = wred[0][cc];
+            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max(m, wred[w][cc]);
+            ref_s[cc] = m + hl + 1 - kXTop;
+            if (kl[cc] >= 0 && x_exp(v[cc * H2]) - ref_s[cc] < kXKeep) lin = 0;
+        }
+        lin_s = lin;
+    }
+    __syncthreads();
+    const bool lin = lin_s != 0;
+    if (lin) {
+        for (uint32_t e = threadIdx.x; e < H2 * CPB; e += blockDim.x) vd[e] = x_scaled(v[e], ref_s[e / H2]);
+        __syncthreads();
+        colb_steps<true>(vd, H2, hl, CPB);
+    } else {
+        colb_steps_x(v, H2, hl, CPB);
+    }
+    X64* Ai = A + ((size_t)i << (n - 1));
+    for (uint32_t H = threadIdx.x; H < H2; H += blockDim.x) {
+        X64* o = Ai + BN_AT(((size_t)(Hc | H) << TB) + c0, CPB, (size_t)1 << (n - 1));
+#pragma unroll
+        for (int cc = 0; cc < CPB; ++cc)
+            if (c0 + cc < ncb) o[cc] = lin ? x_pack<X64>(vd[cc * H2 + H], ref_s[cc]) : v[cc * H2 + H];
+    }
+}
+
+// Up-zeta tile (k_upzeta13): the tile's column sums are staged in shared
+// memory (the outputs overwrite their slots), a thread reads its layout-1
+// inputs by the rank of their patterns.  64 KB for the exchanges and 8 ncol
+// bytes of columns: two blocks per SM.
+__global__ void __launch_bounds__(TT, 2)
+k_up13_x(int n, int d, const uint16_t* __restrict__ rank13, X64* __restrict__ A, size_t js)
+{
+    rank13 = job_ptr(rank13, js);
+    A = job_ptr(A, js);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double* A0 = reinterpret_cast<double*>(smem_raw);
+    X64* col = reinterpret_cast<X64*>(A0 + TN);
+    __shared__ int red[TT / 32];
+    const uint32_t ncol = num_small_subsets(TB, d);
+    const int h = n - 1 - TB;
+    const int t = threadIdx.x;
+    const int i = (int)(blockIdx.x >> h);
+    const uint32_t H = blockIdx.x & ((1u << h) - 1u);
+    X64* out = A + BN_AT(((size_t)i << (n - 1)) + ((size_t)H << TB), TN, (size_t)gridDim.x << TB);
+    int e = -kXBias;
+    for (uint32_t c = t; c < ncol; c += TT) {
+        const X64 v = out[c];
+        col[c] = v;
+        e = max(e, x_exp(v));
+    }
+    const int M = block_max(e, red, t) + TB + 1;     // every output is below 2^M
+    const int low = max(x_exp(col[0]), kXMin);       // and at least C(empty)
+    const int pt = __popc(t);                        // |el1(r, t)| = |r| + |t|
+    uint32_t done = 0u;                              // bit r: output el3(r, t) written
+    for (int ref = M - kXTop;; ref -= kXStep) {
+        const bool last = low - ref >= kXKeep;
+        double x[TR];
+#pragma unroll
+        for (int r = 0; r < TR; ++r)
+            x[r] = __popc(r) + pt <= d ? x_scaled(col[BN_AT(rank13[el1(r, t)], 1, ncol)], ref) : 0.0;
+        bfly_plain<true>(x, 0, 5);
+        st1(A0, x, t);
+        __syncthreads();
+        ld2(A0, x, t);
+        bfly_plain<true>(x, 0, 5);
+        st2(A0, x, t);
+        __syncthreads();
+        ld3(A0, x, t);
+        bfly_plain<true>(x, 0, 3);
+        if (last && done == 0u) {                    // one pass: whole runs of 8
+#pragma unroll
+            for (int q = 0; q < TR / 8; ++q) {
+                ulonglong2* p = reinterpret_cast<ulonglong2*>(out + el3(8 * q, t));
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    p[k] = make_ulonglong2(x_pack<X64>(x[8 * q + 2 * k], ref).u, x_pack<X64>(x[8 * q + 2 * k + 1], ref).u);
+            }
+            return;
+        }
+#pragma unroll
+        for (int r = 0; r < TR; ++r)
+            if (!(done >> r & 1u) && (last || x[r] >= pow2d(kXKeep))) {
+                out[el3(r, t)] = x_pack<X64>(x[r], ref);
+                done |= 1u << r;
+            }
+        if (last) return;
+        __syncthreads();                             // A0 is reused
+    }
+}
+
+// Down-zeta tile (k_gamma13_p1).  The relevance cut works on exponents: an
+// output below 2^L moves no posterior (L = log2 F(V) - margin - log2 A_v(S_H),
+// rounded down), so a tile whose bound M is below L is all zeros and a pass is
+// the last once it resolves max(L, s(full)).
+template <bool Q>
+__global__ void __launch_bounds__(TT, 2)
+k_g13_x(int n, int d, uint32_t nlow, const X64* __restrict__ F, const X64* __restrict__ Rc,
+        const uint16_t* __restrict__ rank13, X64* __restrict__ W, size_t js, const X64* __restrict__ lq,
+        const X64* __restrict__ Aup, int margin, uint32_t vsel)
+{
+    const int v = (int)(blockIdx.x % (unsigned)n);   // the endpoint fastest (k_gamma13_p1)
+    const uint32_t ntile = gridDim.x / (unsigned)n;
+    if (!(vsel >> v & 1u)) return;
+    F = job_ptr(F, js);
+    Rc = job_ptr(Rc, js);
+    const uint16_t* unrank13 = job_ptr(rank13, js) + TN;
+    W = job_ptr(W, js) + (size_t)endpoint_slot(vsel, v) * ntile * nlow;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double* A0 = reinterpret_cast<double*>(smem_raw);
+    __shared__ int red[TT / 32];
+    const int t = threadIdx.x;
+    const uint32_t H = blockIdx.x / (unsigned)n;
+    const uint32_t bv = 1u << v;
+    X64* row = W + (size_t)H * nlow;
+    int L = kXMin;
+    if (Aup) {
+        const X64 at = job_ptr(Aup, js)[BN_AT(((size_t)v << (n - 1)) + (((size_t)H << TB) | (TN - 1)), 1,
+                                              (size_t)n << (n - 1))];
+        L = max(L, x_exp(F[((size_t)1 << n) - 1]) - x_exp(at) - 1 - margin);
+    }
+    // s of the full tile set, the smallest output, is a load of its own: the
+    // first reference puts the smallest output that matters at 2^kXKeep, and
+    // the values are scaled as they arrive
+    int efull;
+    {
+        const uint32_t S = expand((H << TB) | (TN - 1), v);
+        efull = x_exp(F[BN_AT(S, 1, (size_t)1 << n)]) + x_exp(Rc[BN_AT(S | bv, 1, (size_t)1 << n)]);
+        if (Q) efull += x_exp(lq[v * n + __popc(S)]);
+    }
+    const int low = max(L, efull);
+    double x[TR];
+    auto load = [&](int ref) {                       // s relative to ref; the largest exponent
+        int mx = -2 * kXBias;
+#pragma unroll
+        for (int r = 0; r < TR; ++r) {
+            const uint32_t S = expand((H << TB) | el1(r, t), v);
+            const X64 f = F[BN_AT(S, 1, (size_t)1 << n)], g = Rc[BN_AT(S | bv, 1, (size_t)1 << n)];
+            double p = x_mant(f) * x_mant(g);
+            int e = x_exp(f) + x_exp(g);
+            if (Q) {                                 // q_v(S) of Eq. 12
+                const X64 q = lq[v * n + __popc(S)];
+                p *= x_mant(q);
+                e += x_exp(q);
+            }
+            mx = max(mx, e);
+            const int k = e - ref;
+            x[r] = k > 1000 ? __longlong_as_double(0x7ff0000000000000ll) : k < -1000 ? 0.0 : p * pow2d(k);
+            // sixteen values' loads in flight: more would spill
+            if ((r & 15) == 15) asm volatile("" ::: "memory");
+        }
+        return mx;
+    };
+    int ref = low - kXKeep;
+    const int M = block_max(load(ref), red, t) + TB + 3;    // every output is below 2^M
+    if (M < L) {                                     // nothing in the tile matters
+        for (uint32_t c = t; c < nlow; c += TT) row[BN_AT(c, 1, nlow)] = X64{0ull};
+        return;
+    }
+    if (M > ref + kXTop) {                           // wider than one pass: from the top
+        ref = M - kXTop;
+        load(ref);
+    }
+    uint32_t done = 0u;                              // bit k: output row[t + k TT] written
+    for (;;) {
+        const bool last = low - ref >= kXKeep;
+        bfly_plain<false>(x, 0, 5);
+        st1(A0, x, t);
+        __syncthreads();
+        ld2(A0, x, t);
+        bfly_plain<false>(x, 0, 5);
+        st2(A0, x, t);
+        __syncthreads();
+        ld3(A0, x, t);
+        bfly_plain<false>(x, 0, 3);
+        st3(A0, x, t);                               // each thread rewrites the slots it read
+        __syncthreads();
+        // the kept outputs (at most d elements) in rank order
+        uint32_t k = 0;
+        for (uint32_t c = t; c < nlow; c += TT, ++k) {
+            const double o = A0[swz(BN_AT(unrank13[c], 1, TN))];
+            if (!(done >> k & 1u) && (last || o >= pow2d(kXKeep))) {
+                row[BN_AT(c, 1, nlow)] = x_pack<X64>(o, ref);
+                done |= 1u << k;
+            }
+        }
+        if (last) return;
+        ref -= kXStep;
+        load(ref);
+        __syncthreads();                             // A0 is reused
+    }
+}
+
 // rank13[L] = position of L among the subsets of 13 bits ordered by size then
 // value; unrank13 is its inverse.
 __global__ void k_rank13_tables(uint16_t* __restrict__ rank13, uint16_t* __restrict__ unrank13,
@@ -1552,7 +1858,10 @@ cudaError_t launch_reorder_up(const Plan& P, const void* lbs, void* tab, cudaStr
 {
     const int64_t total = (int64_t)up_nodes(P) * P.K;
     const dim3 grid((unsigned)std::min<int64_t>((total + 255) / 256, 152 * 16), P.nj);
-    if (P.prec == 0)
+    if (P.lin)
+        launch_or_record(KID_REORDER_X, k_reorder_up<X64>, grid, 256, 0, s, P.n, P.d, P.K, (const X64*)lbs, (X64*)tab,
+                                                  P.js, up_nodes(P));
+    else if (P.prec == 0)
         launch_or_record(KID_REORDER_D, k_reorder_up<double>, grid, 256, 0, s, P.n, P.d, P.K, (const double*)lbs, (double*)tab,
                                                   P.js, up_nodes(P));
     else
@@ -1591,6 +1900,24 @@ static bool upzeta_table_copies(const Plan& P, const void* tab, const int* err)
            P.K % 4 == 0 && ((uintptr_t)tab & 15u) == 0 && h >= 1 && P.d >= 1;
 }
 
+// The per-tile column sums by a warp: its row list fits shared memory.
+static bool colw_fits(const Plan& P)
+{
+    const int h = P.n - 1 - TB;
+    uint64_t nrow = 0;
+    for (int k = 0; k <= P.d && k <= h; ++k) nrow += binom_host(h, k);
+    return nrow * 4 * 8 <= 160 * 1024;
+}
+
+// The linear FP64 form has the column butterflies and the warp's sums, and
+// stages a tile's columns beside its 64 KB exchange array.
+static size_t up13_x_smem(const Plan& P) { return (size_t)TN * 8 + (size_t)num_small_subsets_host(P.d) * 8; }
+bool lin_tiles_fit(const Plan& P)
+{
+    if (P.n < 14) return true;
+    return colw_fits(P) && up13_x_smem(P) <= 220 * 1024;
+}
+
 cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unrank13, void* A,
                             cudaStream_t s, cudaEvent_t sums_done, int* err)
 {
@@ -1617,7 +1944,17 @@ cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unra
                                          (copies ? (ntiles + 7) / 8 : 0));
         const size_t smb = ((size_t)cpb << (h - hc)) * es;
         const dim3 gb(nblk, P.nj);
-        if (P.prec == 0) {
+        if (P.lin) {
+            if (cpb >= 4)
+                launch_or_record(KID_COLB4_X, k_colb_x<4>, gb, 256, smb, s, P.n, P.d, P.K, (const X64*)tab,
+                                 (X64*)A, P.js, nodes, ncb, hc);
+            else if (cpb == 2)
+                launch_or_record(KID_COLB2_X, k_colb_x<2>, gb, 256, smb, s, P.n, P.d, P.K, (const X64*)tab,
+                                 (X64*)A, P.js, nodes, ncb, hc);
+            else
+                launch_or_record(KID_COLB1_X, k_colb_x<1>, gb, 256, smb, s, P.n, P.d, P.K, (const X64*)tab,
+                                 (X64*)A, P.js, nodes, ncb, hc);
+        } else if (P.prec == 0) {
             if (cpb >= 4)
                 launch_or_record(KID_COLB4_D, k_upzeta13_colb<double, 4>, gb, 256, smb, s, P.n, P.d, P.K,
                                  (const double*)tab, (double*)A, P.js, nodes, ncb, hc);
@@ -1645,16 +1982,21 @@ cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unra
             if (ec != cudaSuccess) return ec;
             const uint64_t total = ((uint64_t)nodes << (h - hc)) * ncb;
             const unsigned gt = (unsigned)std::min<uint64_t>((total + 255) / 256, 152 * 64);
-            if (P.prec == 0)
+            if (P.lin)
+                k_upzeta13_colt<X64><<<gt, 256, 0, s>>>(P.n, (X64*)A, nodes, ncb, hc);
+            else if (P.prec == 0)
                 k_upzeta13_colt<double><<<gt, 256, 0, s>>>(P.n, (double*)A, nodes, ncb, hc);
             else
                 k_upzeta13_colt<float><<<gt, 256, 0, s>>>(P.n, (float*)A, nodes, ncb, hc);
         }
-    } else if (nrow * 4 * 8 <= 160 * 1024) {          // warp per tile, 8 tiles per block
+    } else if (colw_fits(P)) {                        // warp per tile, 8 tiles per block
         const uint64_t ntiles = (uint64_t)nodes << h;
         const dim3 gw((unsigned)std::min<uint64_t>((ntiles + 7) / 8, 152 * 16), P.nj);
         const size_t sw = (size_t)nrow * 4 * 8;
-        if (P.prec == 0)
+        if (P.lin)
+            launch_or_record(KID_COLW_X, k_upzeta13_colw<X64>, gw, 256, sw, s, P.n, P.d, P.K, (const X64*)tab,
+                                                        (X64*)A, P.js, nodes);
+        else if (P.prec == 0)
             launch_or_record(KID_COLW_D, k_upzeta13_colw<double>, gw, 256, sw, s, P.n, P.d, P.K, (const double*)tab,
                                                         (double*)A, P.js, nodes);
         else
@@ -1693,6 +2035,9 @@ cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unra
                                                        (const float*)tab, P.K, ncb);
         return cudaGetLastError();
     }
+    if (P.lin)
+        return launch_or_record(KID_UP13_X, k_up13_x, grid, TT, up13_x_smem(P), s, P.n, P.d, unrank13 - TN,
+                                (X64*)A, P.js);
     if (P.prec == 0)
         launch_or_record(KID_UP13_D, k_upzeta13<double, false>, grid, TT, sm, s, P.n, P.d, unrank13, (double*)A, P.js);
     else if (use_tlo(P))
@@ -1737,7 +2082,15 @@ cudaError_t launch_gamma13_p1(const Plan& P, const void* F, const void* Rc,
     const double mbits = (P.prec == 0 ? 64.0 : 24.0) + std::ceil(std::log2((double)P.K)) + h;
     const double margin = P.prec == 0 ? mbits * 0.69314718055994531 : mbits;
     // the order prior is a separate instance: the plain kernel has no trace of it
-    if (P.prec == 0) {
+    if (P.lin) {
+        const size_t sx = (size_t)TN * 8;
+        if (lq)
+            launch_or_record(KID_G13_X_Q, k_g13_x<true>, grid, TT, sx, s, P.n, P.d, P.nlow_g, (const X64*)F,
+                             (const X64*)Rc, rank13, (X64*)W, P.js, (const X64*)lq, (const X64*)A, (int)mbits, P.vsel);
+        else
+            launch_or_record(KID_G13_X, k_g13_x<false>, grid, TT, sx, s, P.n, P.d, P.nlow_g, (const X64*)F,
+                             (const X64*)Rc, rank13, (X64*)W, P.js, nullptr, (const X64*)A, (int)mbits, P.vsel);
+    } else if (P.prec == 0) {
         if (lq)
             launch_or_record(KID_G13_D_Q, k_gamma13_p1<double, true>, grid, TT, sm, s, 
                 P.n, P.d, P.nlow_g, (const double*)F, (const double*)Rc, rank13, (double*)W, P.js,
@@ -1785,6 +2138,13 @@ cudaError_t set_tile13_attributes()
     SETA((k_gamma13_p1<float, false>))
     SETA((k_gamma13_p1<double, true>))
     SETA((k_gamma13_p1<float, true>))
+    SETA(k_upzeta13_colw<X64>)
+    SETA(k_colb_x<4>)
+    SETA(k_colb_x<2>)
+    SETA(k_colb_x<1>)
+    SETA(k_up13_x)
+    SETA(k_g13_x<false>)
+    SETA(k_g13_x<true>)
 #undef SETA
     return cudaSuccess;
 }
