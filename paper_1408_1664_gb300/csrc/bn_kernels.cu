@@ -525,65 +525,62 @@ k_gamma_p2s(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const T*
 
 // ===========================================================================
 // Step 5: P(u->v, D) = sum_{G: u in G} B_v(G) Gamma_v(G)  (Eq. 11) and
-// P(u->v | D) = P(u->v, D) / P(D), in FP64, in three launches.
+// P(u->v | D) = P(u->v, D) / P(D), in FP64, in one launch.
 // Every term B_v(G) Gamma_v(G) is at most their sum over G, which is F(V)
 // (Eq. 11 summed over all G), so e(G) = B_v(G) Gamma_v(G) / F(V) <= 1 (up to
 // rounding) needs no maximum pass.  Blocks over (families of v, v) add e(G)
 // in fixed point (2^qbits, integer atomics: the sums do not depend on the
 // order of arrival) into acc[v*n + u] for every u in G and into acc[n*n + v]
-// for all G.  The FP64 path divides by F(V) (Algorithm 1), i.e. takes
-// acc[v*n + u] / 2^qbits; the FP32 path divides by Z_v = acc[n*n + v]
-// (the same quantity from the same Gamma_v, so rounding common to numerator
-// and denominator cancels).  log P(D) = F~(V) + sum_i c_i.
+// for all G; the last block to finish divides.  The FP64 path divides by F(V)
+// (Algorithm 1), i.e. takes acc[v*n + u] / 2^qbits; the FP32 path divides by
+// Z_v = acc[n*n + v] (the same quantity from the same Gamma_v, so rounding
+// common to numerator and denominator cancels).  log P(D) = F~(V) + sum_i c_i.
+// Most families weigh less than half a unit of the fixed point: they are
+// left out by a comparison in the working precision, before the FP64
+// exponential and the atomics (n = 25, d = 8: 31.8 M families, 2.06 -> 0.28 ms).
 // ===========================================================================
-__global__ void k_edges_zero(int n, unsigned long long* __restrict__ acc, size_t js)
+// The weight e(G) 2^qbits of family x, rounded: 0 without an exponential when
+// it is certainly below one half.
+struct EdgeScale {
+    double cv, lnfv, qscale, inv;                   // logs: c_v, ln F(V), 2^qbits; XValue: 1 / F(V)'s fraction
+    float cut;                                      // FP32: log2 of a weight that rounds to 0
+    int eq;                                         // XValue: qbits - F(V)'s exponent
+};
+__device__ __forceinline__ EdgeScale edge_scale(const float* F, int n, int qbits, double cv)
 {
-    acc = job_ptr(acc, js);
-    for (int t = threadIdx.x; t < n * (n + 1); t += blockDim.x) acc[t] = 0ull;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256)
-k_edges_acc(int n, int64_t K, int qbits, const double* __restrict__ logB,
-            const double* __restrict__ cmax, const uint32_t* __restrict__ masks,
-            const T* __restrict__ Gam, const T* __restrict__ F,
-            unsigned long long* __restrict__ acc, size_t js, uint32_t vsel)
-{
-    if (!(vsel >> blockIdx.z & 1u)) return;         // an endpoint another rank computes
-    logB = job_ptr(logB, js);
-    cmax = job_ptr(cmax, js);
-    masks = job_ptr(masks, js);
-    Gam = job_ptr(Gam, js);
-    F = job_ptr(F, js);
-    acc = job_ptr(acc, js);
-    using L = LogOps<T>;
-    __shared__ unsigned long long Nu[32], Nz;
-    const int v = blockIdx.z;
-    const int tid = threadIdx.x;
-    if (tid < 32) Nu[tid] = 0ull;
-    if (tid == 0) Nz = 0ull;
-    __syncthreads();
-    const uint32_t full = (uint32_t)(((uint64_t)1 << n) - 1);   // n <= 32
-    // FP32: Gamma is relative to the integer Z = floor of log P(D) in the
+    // Gamma is relative to the integer Z = floor of log P(D) in the
     // level-based units (see gamma_offsets), so P(D) enters as F(V) - Z
-    const double fv = (double)F[full];
-    const double lnFV = L::to_ln(sizeof(T) == 4 ? fv - floor(fv) : fv);
-    const double qscale = ldexp(1.0, qbits);
-    const double cv = cmax[v];
-    unsigned long long z = 0ull;
-    for (int64_t f = blockIdx.x * (int64_t)blockDim.x + tid; f < K;
-         f += (int64_t)gridDim.x * blockDim.x) {
-        const size_t x = (size_t)v * K + f;
-        const double e = exp(logB[x] - cv + L::to_ln((double)Gam[x]) - lnFV);
-        const unsigned long long q = __double2ull_rn(e * qscale);
-        z += q;
-        for (uint32_t g = masks[x]; g; g &= g - 1) atomicAdd(&Nu[BN_AT(__ffs(g) - 1, 1, 32)], q);
-    }
-    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(FULL, z, o);
-    if ((tid & 31) == 0) atomicAdd(&Nz, z);
-    __syncthreads();
-    if (tid < n && Nu[tid]) atomicAdd(&acc[(size_t)v * n + tid], Nu[tid]);
-    if (tid == 0) atomicAdd(&acc[(size_t)n * n + v], Nz);
+    const double fv = (double)F[(uint32_t)(((uint64_t)1 << n) - 1)];   // n <= 32
+    const double rel = fv - floor(fv);
+    return {cv, LogOps<float>::to_ln(rel), ldexp(1.0, qbits), 0.0, (float)rel - (float)(qbits + 3), 0};
+}
+__device__ __forceinline__ EdgeScale edge_scale(const double* F, int n, int qbits, double cv)
+{
+    const double fv = F[(uint32_t)(((uint64_t)1 << n) - 1)];
+    return {cv, fv, ldexp(1.0, qbits), 0.0, -0.69314718f * (float)(qbits + 3), 0};
+}
+template <int FB> __device__ __forceinline__ EdgeScale edge_scale(const XValue<FB>* F, int n, int qbits, double)
+{
+    const XValue<FB> fv = F[(uint32_t)(((uint64_t)1 << n) - 1)];
+    return {0.0, 0.0, 0.0, 1.0 / x_mant(fv), 0.f, qbits - x_exp(fv)};
+}
+__device__ __forceinline__ unsigned long long edge_weight(const EdgeScale& s, double logB, float lb, float g)
+{
+    // lb is log B - c_v in log2 units to a few 1e-4: three bits of margin
+    if (lb + g < s.cut) return 0ull;
+    return __double2ull_rn(exp(logB - s.cv + LogOps<float>::to_ln((double)g) - s.lnfv) * s.qscale);
+}
+__device__ __forceinline__ unsigned long long edge_weight(const EdgeScale& s, double logB, double, double g)
+{
+    const double x = logB - s.cv + g - s.lnfv;
+    if (x < (double)s.cut) return 0ull;
+    return __double2ull_rn(exp(x) * s.qscale);
+}
+template <int FB>
+__device__ __forceinline__ unsigned long long edge_weight(const EdgeScale& s, double, XValue<FB> b, XValue<FB> g)
+{
+    const int e = x_exp(b) + x_exp(g) + s.eq;       // the weight is at most 2^qbits
+    return e < -8 ? 0ull : __double2ull_rn(x_mant(b) * x_mant(g) * s.inv * pow2d(min(e, 64)));
 }
 
 // ln F(V) of the shifted scores.
@@ -599,45 +596,205 @@ template <int FB> __device__ __forceinline__ double ln_full(const XValue<FB>* F,
     const XValue<FB> f = F[((size_t)1 << n) - 1];
     return f.u ? (double)x_exp(f) * 0.69314718055994530942 + log(x_mant(f)) : -INFINITY;
 }
-
 template <typename T>
-__global__ void k_edges_fin(int n, int use_z, int qbits, const double* __restrict__ cmax,
-                            const T* __restrict__ F, const int* __restrict__ err,
-                            const unsigned long long* __restrict__ acc,
-                            double* __restrict__ post, double* __restrict__ log_PD, size_t js,
-                            uint32_t vsel)
+__device__ __forceinline__ double log_evidence(int n, const double* cmax, const T* F)
 {
+    double c = 0.0;
+    for (int i = 0; i < n; ++i) c += cmax[i];
+    return ln_full(F, n) + c;
+}
+
+// acc: n * (n + 1) sums, zero before the launch and left zero by it; acc[0]
+// (no edge 0 -> 0) counts the finished blocks.
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_edges(int n, int64_t K, int qbits, const double* __restrict__ logB, const T* __restrict__ lbs,
+        const double* __restrict__ cmax, const uint32_t* __restrict__ masks, const T* __restrict__ Gam,
+        const T* __restrict__ F, const int* __restrict__ err, unsigned long long* __restrict__ acc,
+        double* __restrict__ post, double* __restrict__ log_PD, size_t js, uint32_t vsel)
+{
+    // an endpoint another rank computes (a rank without any: its first block
+    // still writes the zeros and log P(D))
+    const int mine = __popc(vsel & (uint32_t)(((uint64_t)1 << n) - 1));
+    if (!(vsel >> blockIdx.z & 1u) && (mine || blockIdx.x || blockIdx.z)) return;
+    logB = job_ptr(logB, js);
+    lbs = job_ptr(lbs, js);
     cmax = job_ptr(cmax, js);
+    masks = job_ptr(masks, js);
+    Gam = job_ptr(Gam, js);
     F = job_ptr(F, js);
-    err = job_ptr(err, js);
     acc = job_ptr(acc, js);
+    __shared__ unsigned long long Nu[32], Nz;
+    __shared__ int last_s;
+    const int v = blockIdx.z;
+    const int tid = threadIdx.x;
+    if (tid < 32) Nu[tid] = 0ull;
+    if (tid == 0) Nz = 0ull;
+    __syncthreads();
+    const EdgeScale sc = edge_scale(F, n, qbits, cmax[v]);
+    unsigned long long z = 0ull;
+    for (int64_t f = mine ? blockIdx.x * (int64_t)blockDim.x + tid : K; f < K;
+         f += (int64_t)gridDim.x * blockDim.x) {
+        const size_t x = (size_t)v * K + f;
+        const unsigned long long q = edge_weight(sc, logB[x], lbs[x], Gam[x]);
+        if (q) {
+            z += q;
+            for (uint32_t g = masks[x]; g; g &= g - 1) atomicAdd(&Nu[BN_AT(__ffs(g) - 1, 1, 32)], q);
+        }
+    }
+    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(FULL, z, o);
+    if ((tid & 31) == 0) atomicAdd(&Nz, z);
+    __syncthreads();
+    if (tid < n && Nu[tid]) atomicAdd(&acc[(size_t)v * n + tid], Nu[tid]);
+    if (tid == 0) atomicAdd(&acc[(size_t)n * n + v], Nz);
+    __threadfence();                                // this block's sums before its count
+    __syncthreads();
+    if (tid == 0) {
+        last_s = !mine || atomicAdd(&acc[0], 1ull) + 1ull == (unsigned long long)mine * gridDim.x;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last_s) return;
+    err = job_ptr(err, js);
     post = job_ptr(post, js);
     log_PD = job_ptr(log_PD, js);
     const bool bad = err && *err;
-    const double qscale = ldexp(1.0, qbits);
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-        const int u = t / n, v = t % n;
-        const unsigned long long num = acc[(size_t)v * n + u];
+    for (int t = tid; t < n * n; t += blockDim.x) {
+        const int u = t / n, w = t % n;
+        const unsigned long long num = __ldcg(acc + (size_t)w * n + u);
         double p = 0.0;
-        if (u != v && num > 0ull)
-            p = use_z ? __ull2double_rn(num) / __ull2double_rn(acc[(size_t)n * n + v])
-                      : __ull2double_rn(num) / qscale;
-        post[t] = bad ? NAN : (vsel >> v & 1u) ? p : 0.0;   // other ranks' endpoints: 0
+        if (u != w && num > 0ull)
+            p = sizeof(T) == 4 ? __ull2double_rn(num) / __ull2double_rn(__ldcg(acc + (size_t)n * n + w))
+                               : __ull2double_rn(num) / ldexp(1.0, qbits);
+        post[t] = bad ? NAN : (vsel >> w & 1u) ? p : 0.0;   // other ranks' endpoints: 0
     }
-    if (threadIdx.x == 0 && log_PD) {
-        double c = 0.0;
-        for (int i = 0; i < n; ++i) c += cmax[i];
-        *log_PD = bad ? NAN : ln_full(F, n) + c;
+    if (tid == 0 && log_PD) *log_PD = bad ? NAN : log_evidence(n, cmax, F);
+    __syncthreads();
+    for (int t = tid; t < n * (n + 1); t += blockDim.x) acc[t] = 0ull;
+}
+
+// Steps 4 and 5 for n < 14 in one launch, a block per endpoint v: the whole
+// down-zeta of v fits one tile in shared memory (no phase 2), its families'
+// Gamma come straight out of it, and the block divides its own column.  It
+// replaces six launches (the FP32 offsets, two phases, three of step 5), about
+// 45 of the 150 us of an n = 12 job.
+__device__ __forceinline__ void tail_input(float& y, const float* F, const float* Rc, uint32_t S, uint32_t bv,
+                                           size_t full, const float* off, int sh)
+{
+    y = F[BN_AT(S, 1, full)] + Rc[BN_AT(S | bv, 1, full)];
+    y += off[BN_AT(__popc(S >> sh), 1, 32)];
+}
+__device__ __forceinline__ void tail_input(double& y, const double* F, const double* Rc, uint32_t S, uint32_t bv,
+                                           size_t full, const float*, int)
+{
+    y = F[BN_AT(S, 1, full)] + Rc[BN_AT(S | bv, 1, full)];
+}
+template <int FB>
+__device__ __forceinline__ void tail_input(XValue<FB>& y, const XValue<FB>* F, const XValue<FB>* Rc, uint32_t S,
+                                           uint32_t bv, size_t full, const float*, int)
+{
+    y = x_mul(F[BN_AT(S, 1, full)], Rc[BN_AT(S | bv, 1, full)]);
+}
+__device__ __forceinline__ void apply_weight(float& a, float w) { a += w; }
+__device__ __forceinline__ void apply_weight(double& a, double w) { a += w; }
+template <int FB> __device__ __forceinline__ void apply_weight(XValue<FB>& a, XValue<FB> w) { a = x_mul(a, w); }
+
+template <typename T>
+__global__ void __launch_bounds__(1024)
+k_tail(int n, int d, int64_t K, int qbits, const T* __restrict__ F, const T* __restrict__ Rc,
+       const T* __restrict__ lq, const double* __restrict__ logB, const T* __restrict__ lbs,
+       const double* __restrict__ cmax, const uint32_t* __restrict__ masks,
+       const uint32_t* __restrict__ cmasks, T* __restrict__ Gam, const int* __restrict__ err,
+       double* __restrict__ post, double* __restrict__ log_PD, size_t js, uint32_t vsel)
+{
+    const int v = blockIdx.x;
+    F = job_ptr(F, js);
+    Rc = job_ptr(Rc, js);
+    logB = job_ptr(logB, js);
+    lbs = job_ptr(lbs, js);
+    cmax = job_ptr(cmax, js);
+    masks = job_ptr(masks, js);
+    cmasks = job_ptr(cmasks, js);
+    Gam = job_ptr(Gam, js);
+    err = job_ptr(err, js);
+    post = job_ptr(post, js);
+    const int tid = threadIdx.x;
+    const bool bad = err && *err;
+    if (!(vsel >> v & 1u)) {                        // an endpoint another rank computes
+        if (tid < n) post[(size_t)tid * n + v] = bad ? NAN : 0.0;
+        if (tid == 0 && v == 0 && log_PD && !(vsel & (uint32_t)(((uint64_t)1 << n) - 1)))
+            *job_ptr(log_PD, js) = bad ? NAN : log_evidence(n, cmax, F);
+        return;
     }
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* vals = reinterpret_cast<T*>(smem_raw);
+    __shared__ unsigned long long Nu[32], Nz;
+    __shared__ float off_s[32];
+    __shared__ int sh_s;
+    __shared__ float fvrel_s;
+    if (tid < 32) {
+        Nu[tid] = 0ull;
+        if (tid == 0) Nz = 0ull;
+        if constexpr (sizeof(T) == 4) {             // FP32: the level bases of F and R'
+            off_s[tid] = 0.f;
+            __syncwarp();
+            gamma_offsets(n, v, reinterpret_cast<const float*>(F), reinterpret_cast<const float*>(Rc), off_s, &sh_s,
+                          &fvrel_s);
+        }
+    }
+    __syncthreads();
+    const uint32_t N = 1u << (n - 1);
+    const size_t full = (size_t)1 << n;
+    const int sh = sizeof(T) == 4 ? sh_s : 0;
+    for (uint32_t t = tid; t < N; t += blockDim.x) {
+        const uint32_t S = expand(t, v);
+        T y;
+        tail_input(y, F, Rc, S, 1u << v, full, off_s, sh);
+        if (lq) apply_weight(y, lq[v * n + __popc(S)]);     // q_v(S) of Eq. 12
+        vals[t] = y;
+    }
+    __syncthreads();
+    for (int j = 0; j < n - 1; ++j) {
+        const uint32_t jm = (1u << j) - 1u;
+        for (uint32_t p = tid; p < (N >> 1); p += blockDim.x) {
+            const uint32_t lo = ((p & ~jm) << 1) | (p & jm);
+            if (__popc(lo & jm) <= d) vals[lo] = p2_add(vals[lo], vals[lo | (1u << j)]);
+        }
+        __syncthreads();
+    }
+    const EdgeScale sc = edge_scale(F, n, qbits, cmax[v]);
+    unsigned long long z = 0ull;
+    const int64_t rounds = (K + blockDim.x - 1) / blockDim.x;
+    for (int64_t r = 0; r < rounds; ++r) {
+        const int64_t f = r * blockDim.x + tid;
+        if (f >= K) continue;
+        const size_t x = (size_t)v * K + f;
+        const T g = vals[BN_AT(cmasks[x], 1, N)];
+        Gam[x] = g;
+        const unsigned long long q = edge_weight(sc, logB[x], lbs[x], g);
+        if (q) {
+            z += q;
+            for (uint32_t y = masks[x]; y; y &= y - 1) atomicAdd(&Nu[BN_AT(__ffs(y) - 1, 1, 32)], q);
+        }
+    }
+    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(FULL, z, o);
+    if ((tid & 31) == 0) atomicAdd(&Nz, z);
+    __syncthreads();
+    if (tid < n) {
+        double p = 0.0;
+        if (tid != v && Nu[tid] > 0ull)
+            p = sizeof(T) == 4 ? __ull2double_rn(Nu[tid]) / __ull2double_rn(Nz)
+                               : __ull2double_rn(Nu[tid]) / ldexp(1.0, qbits);
+        post[(size_t)tid * n + v] = bad ? NAN : p;
+    }
+    // one block writes log P(D): that of the first endpoint computed
+    if (tid == 0 && log_PD && (vsel & ((1u << v) - 1u)) == 0u)
+        *job_ptr(log_PD, js) = bad ? NAN : log_evidence(n, cmax, F);
 }
 
 // ===========================================================================
 // Priors beyond the defaults and single features (Eqs. 4-9).
 // ===========================================================================
-
-__device__ __forceinline__ void apply_weight(float& a, float w) { a += w; }
-__device__ __forceinline__ void apply_weight(double& a, double w) { a += w; }
-template <int FB> __device__ __forceinline__ void apply_weight(XValue<FB>& a, XValue<FB> w) { a = x_mul(a, w); }
 
 // A_i(S) += log q_i(S), q_i a function of |S| (Eq. 7): lq[i * n + |S|] in
 // the working precision and log base; A is [i * 2^(n-1) + c], c = S with
@@ -666,8 +823,8 @@ __global__ void k_apply_q(int n, const T* __restrict__ lq, T* __restrict__ A, in
 }
 
 // ===========================================================================
-// The linear FP64 form (XValue, bn_device.cuh) of steps 2 (n < 14),
-// 4 and 5.
+// The linear FP64 form (XValue, bn_device.cuh) of steps 2 (n < 14)
+// and 4.
 // ===========================================================================
 
 // Step 2 for n < 14: one block per node, every family in its slot of the
@@ -697,40 +854,6 @@ k_upzeta_x(int n, int64_t K, const uint32_t* __restrict__ cmasks, const X64S* __
         __syncthreads();
     }
     for (uint32_t t = threadIdx.x; t < N; t += blockDim.x) A[BN_AT((size_t)i * N + t, 1, (size_t)n * N)] = v[t];
-}
-
-// Step 4 phase 1 for n < 14 (k_gamma_p1): one tile per endpoint.
-__global__ void __launch_bounds__(256)
-k_gamma_p1_x(int n, int d, int b, uint32_t nlow, const X64S* __restrict__ F, const X64S* __restrict__ Rc,
-             X64S* __restrict__ W, size_t js, const X64S* __restrict__ lq, uint32_t vsel)
-{
-    const int v = blockIdx.z;
-    if (!(vsel >> v & 1u)) return;
-    F = job_ptr(F, js);
-    Rc = job_ptr(Rc, js);
-    W = job_ptr(W, js) + (size_t)endpoint_slot(vsel, v) * gridDim.x * nlow;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    X64S* vals = reinterpret_cast<X64S*>(smem_raw);
-    const uint32_t tileN = 1u << b;
-    const uint32_t H = blockIdx.x;
-    for (uint32_t t = threadIdx.x; t < tileN; t += blockDim.x) {
-        const uint32_t S = expand((H << b) | t, v);
-        X64S y = x_mul(F[BN_AT(S, 1, (size_t)1 << n)], Rc[BN_AT(S | (1u << v), 1, (size_t)1 << n)]);
-        if (lq) y = x_mul(y, lq[v * n + __popc(S)]);
-        vals[t] = y;
-    }
-    __syncthreads();
-    for (int j = 0; j < b; ++j) {
-        const uint32_t jm = (1u << j) - 1u;
-        for (uint32_t p = threadIdx.x; p < (tileN >> 1); p += blockDim.x) {
-            const uint32_t lo = ((p & ~jm) << 1) | (p & jm);
-            if (__popc(lo & jm) <= d) vals[lo] = x_add(vals[lo], vals[lo | (1u << j)]);
-        }
-        __syncthreads();
-    }
-    X64S* row = W + (size_t)H * nlow;
-    for (uint32_t t = threadIdx.x; t < tileN; t += blockDim.x)
-        if (__popc(t) <= d) row[BN_AT(small_subset_rank(t, b), 1, nlow)] = vals[t];
 }
 
 // Warp-wide sum of the lanes' LazySums, in a fixed tree order.
@@ -800,47 +923,6 @@ k_gamma_p2s_x(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const 
         const X x = warp_sum_x(sb[q]);
         if (lane == 0) Gam[BN_AT(family_index(g | (1u << (b + 5 + q)), n), 1, K)] = x;
     }
-}
-
-// Step 5: e(G) = B_v(G) Gamma_v(G) / F(V) in fixed point (k_edges_acc), from
-// the shifted scores themselves.
-template <typename X>
-__global__ void __launch_bounds__(256)
-k_edges_acc_x(int n, int64_t K, int qbits, const X* __restrict__ lbs, const uint32_t* __restrict__ masks,
-              const X* __restrict__ Gam, const X* __restrict__ F, unsigned long long* __restrict__ acc,
-              size_t js, uint32_t vsel)
-{
-    if (!(vsel >> blockIdx.z & 1u)) return;
-    lbs = job_ptr(lbs, js);
-    masks = job_ptr(masks, js);
-    Gam = job_ptr(Gam, js);
-    F = job_ptr(F, js);
-    acc = job_ptr(acc, js);
-    __shared__ unsigned long long Nu[32], Nz;
-    const int v = blockIdx.z;
-    const int tid = threadIdx.x;
-    if (tid < 32) Nu[tid] = 0ull;
-    if (tid == 0) Nz = 0ull;
-    __syncthreads();
-    const X fv = F[(uint32_t)(((uint64_t)1 << n) - 1)];
-    const double inv = 1.0 / x_mant(fv);
-    const int eq = qbits - x_exp(fv);
-    unsigned long long z = 0ull;
-    for (int64_t f = blockIdx.x * (int64_t)blockDim.x + tid; f < K;
-         f += (int64_t)gridDim.x * blockDim.x) {
-        const size_t x = (size_t)v * K + f;
-        const X b = lbs[x], g = Gam[x];
-        const int e = x_exp(b) + x_exp(g) + eq;      // the term is at most 2^qbits
-        const unsigned long long q =
-            e < -8 ? 0ull : __double2ull_rn(x_mant(b) * x_mant(g) * inv * pow2d(min(e, 64)));
-        z += q;
-        for (uint32_t y = masks[x]; y; y &= y - 1) atomicAdd(&Nu[BN_AT(__ffs(y) - 1, 1, 32)], q);
-    }
-    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(FULL, z, o);
-    if ((tid & 31) == 0) atomicAdd(&Nz, z);
-    __syncthreads();
-    if (tid < n && Nu[tid]) atomicAdd(&acc[(size_t)v * n + tid], Nu[tid]);
-    if (tid == 0) atomicAdd(&acc[(size_t)n * n + v], Nz);
 }
 
 // out = lbs + lf: the shifted scores of B_i(G) f_i(G) (Eq. 6 with a feature).
@@ -1058,6 +1140,7 @@ cudaError_t launch_gamma_table(const Plan& P, const void* F, const void* Rc, cud
 cudaError_t launch_gamma_p1(const Plan& P, const void* F, const void* Rc, const uint16_t* rk13,
                             void* W, cudaStream_t s, const void* lq, const void* A)
 {
+    if (use_tail(P)) return cudaSuccess;            // launch_edges does steps 4 and 5
     if (use_tile13_gamma(P)) return launch_gamma13_p1(P, F, Rc, rk13, W, s, lq, A);
     if (P.prec != 0) {
         const cudaError_t e = launch_gamma_table(P, F, Rc, s);
@@ -1066,10 +1149,7 @@ cudaError_t launch_gamma_p1(const Plan& P, const void* F, const void* Rc, const 
     const int h = P.n - 1 - P.b_g;
     const size_t sm1 = gamma_p1_smem_bytes(P);
     const dim3 grid(1u << h, P.nj, P.n);
-    if (P.lin)
-        launch_or_record(KID_GAMMA_P1_XS, k_gamma_p1_x, grid, 256, sm1, s, P.n, P.d, P.b_g, P.nlow_g, (const X64S*)F,
-                         (const X64S*)Rc, (X64S*)W, P.js, (const X64S*)lq, P.vsel);
-    else if (P.prec == 0)
+    if (P.prec == 0)
         launch_or_record(KID_GAMMA_P1_D, k_gamma_p1<double>, grid, 256, sm1, s, P.n, P.d, P.b_g, P.nlow_g,
                                                   (const double*)F, (const double*)Rc,
                                                   (double*)W, P.js, (const double*)lq, P.vsel);
@@ -1094,20 +1174,19 @@ uint32_t gamma_p2_split(const Plan& P)
 
 int gamma_launches(const Plan& P)
 {
+    if (use_tail(P)) return 0;
     const uint32_t c0 = gamma_p2_split(P);
     return 1 + (P.prec != 0 ? 1 : 0) + (c0 > 0 ? 1 : 0) + (c0 < P.nlow_g ? 1 : 0);
 }
 
 cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_t s)
 {
+    if (use_tail(P)) return cudaSuccess;
     const uint32_t c0 = gamma_p2_split(P);
     if (c0 > 0) {
         const size_t sm2 = gamma_p2_smem_bytes(P);
         const dim3 grid(c0, P.nj, P.n);
-        if (P.lin == 2)
-            launch_or_record(KID_GAMMA_P2_XS, k_gamma_p2<X64S>, grid, 256, sm2, s, P.n, P.d, P.b_g, P.hc_g, P.nlow_g,
-                             P.K, (const X64S*)W, (X64S*)Gam, P.js, P.vsel);
-        else if (P.lin)
+        if (P.lin)
             launch_or_record(KID_GAMMA_P2_X, k_gamma_p2<X64>, grid, 256, sm2, s, P.n, P.d, P.b_g, P.hc_g, P.nlow_g,
                              P.K, (const X64*)W, (X64*)Gam, P.js, P.vsel);
         else if (P.prec == 0)
@@ -1121,10 +1200,7 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_
     }
     if (c0 < P.nlow_g) {
         const dim3 grid((P.nlow_g - c0 + 7) / 8, P.nj, P.n);
-        if (P.lin == 2)
-            launch_or_record(KID_GAMMA_P2S_XS, k_gamma_p2s_x<X64S>, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0,
-                             P.K, (const X64S*)W, (X64S*)Gam, P.js, P.vsel);
-        else if (P.lin)
+        if (P.lin)
             launch_or_record(KID_GAMMA_P2S_X, k_gamma_p2s_x<X64>, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
                              (const X64*)W, (X64*)Gam, P.js, P.vsel);
         else if (P.prec == 0)
@@ -1137,44 +1213,48 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t launch_edges(const Plan& P, const double* logB, const void* lbs, const double* cmax,
-                         const uint32_t* masks, const void* Gam, const void* F, const int* err,
-                         unsigned long long* acc, double* post, double* log_PD, cudaStream_t s)
+// The one-launch form of steps 4 and 5 (k_tail).
+bool use_tail(const Plan& P) { return P.n < 14; }
+
+template <typename T>
+static cudaError_t edges(const Plan& P, int kid, int kid_tail, const double* logB, const void* lbs,
+                         const double* cmax, const uint32_t* masks, const uint32_t* cmasks, void* Gam,
+                         const void* F, const void* Rc, const void* lq, const int* err, unsigned long long* acc,
+                         double* post, double* log_PD, cudaStream_t s)
 {
-    launch_or_record(KID_EDGES_ZERO, k_edges_zero, dim3(1, P.nj), 256, 0, s, P.n, acc, P.js);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    // (the linear forms have one of the two: X64 from n = 14, X64S below)
+    if constexpr (!std::is_same<T, X64>::value) if (use_tail(P)) {
+        // a thread per pair of values, at most 1024
+        const unsigned tb = rec_block((unsigned)std::min(1024, std::max(128, 1 << (P.n - 2))));
+        return launch_or_record(kid_tail, k_tail<T>, dim3(P.n, P.nj), tb, sizeof(T) << (P.n - 1), s, P.n, P.d, P.K,
+                                fixed_bits(P.K), (const T*)F, (const T*)Rc, (const T*)lq, logB, (const T*)lbs, cmax,
+                                masks, cmasks, (T*)Gam, err, post, log_PD, P.js, P.vsel);
+    }
+    if constexpr (std::is_same<T, X64S>::value) return cudaErrorInvalidValue;
+    else {
     const unsigned chunks = (unsigned)std::min<int64_t>((P.K + 1023) / 1024, 64);
-    const dim3 grid(chunks, P.nj, P.n);
+    return launch_or_record(kid, k_edges<T>, dim3(chunks, P.nj, P.n), 256, 0, s, P.n, P.K, fixed_bits(P.K), logB,
+                            (const T*)lbs, cmax, masks, (const T*)Gam, (const T*)F, err, acc, post, log_PD, P.js,
+                            P.vsel);
+    }
+}
+
+cudaError_t launch_edges(const Plan& P, const double* logB, const void* lbs, const double* cmax,
+                         const uint32_t* masks, const uint32_t* cmasks, void* Gam, const void* F, const void* Rc,
+                         const void* lq, const int* err, unsigned long long* acc, double* post, double* log_PD,
+                         cudaStream_t s)
+{
     if (P.lin == 2)
-        launch_or_record(KID_EDGES_ACC_XS, k_edges_acc_x<X64S>, grid, 256, 0, s, P.n, P.K, fixed_bits(P.K),
-                         (const X64S*)lbs, masks, (const X64S*)Gam, (const X64S*)F, acc, P.js, P.vsel);
-    else if (P.lin)
-        launch_or_record(KID_EDGES_ACC_X, k_edges_acc_x<X64>, grid, 256, 0, s, P.n, P.K, fixed_bits(P.K), (const X64*)lbs,
-                         masks, (const X64*)Gam, (const X64*)F, acc, P.js, P.vsel);
-    else if (P.prec == 0)
-        launch_or_record(KID_EDGES_ACC_D, k_edges_acc<double>, grid, 256, 0, s, P.n, P.K, fixed_bits(P.K), logB, cmax, masks,
-                                                 (const double*)Gam, (const double*)F, acc, P.js, P.vsel);
-    else
-        launch_or_record(KID_EDGES_ACC_F, k_edges_acc<float>, grid, 256, 0, s, P.n, P.K, fixed_bits(P.K), logB, cmax, masks,
-                                                (const float*)Gam, (const float*)F, acc, P.js, P.vsel);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (P.lin == 2)
-        launch_or_record(KID_EDGES_FIN_XS, k_edges_fin<X64S>, dim3(1, P.nj), rec_block(1024), 0, s, P.n, 0,
-                         fixed_bits(P.K), cmax, (const X64S*)F, err, acc, post, log_PD, P.js, P.vsel);
-    else if (P.lin)
-        launch_or_record(KID_EDGES_FIN_X, k_edges_fin<X64>, dim3(1, P.nj), rec_block(1024), 0, s, P.n, 0,
-                         fixed_bits(P.K), cmax, (const X64*)F, err, acc, post, log_PD, P.js, P.vsel);
-    else if (P.prec == 0)
-        launch_or_record(KID_EDGES_FIN_D, k_edges_fin<double>, dim3(1, P.nj), rec_block(1024), 0, s, P.n, 0, fixed_bits(P.K), cmax,
-                                                           (const double*)F, err, acc, post,
-                                                           log_PD, P.js, P.vsel);
-    else
-        launch_or_record(KID_EDGES_FIN_F, k_edges_fin<float>, dim3(1, P.nj), rec_block(1024), 0, s, P.n, 1, fixed_bits(P.K), cmax,
-                                                          (const float*)F, err, acc, post,
-                                                          log_PD, P.js, P.vsel);
-    return cudaGetLastError();
+        return edges<X64S>(P, KID_NONE, KID_TAIL_XS, logB, lbs, cmax, masks, cmasks, Gam, F, Rc, lq, err, acc,
+                           post, log_PD, s);
+    if (P.lin)
+        return edges<X64>(P, KID_EDGES_X, KID_NONE, logB, lbs, cmax, masks, cmasks, Gam, F, Rc, lq, err, acc, post,
+                          log_PD, s);
+    if (P.prec == 0)
+        return edges<double>(P, KID_EDGES_D, KID_TAIL_D, logB, lbs, cmax, masks, cmasks, Gam, F, Rc, lq, err, acc,
+                             post, log_PD, s);
+    return edges<float>(P, KID_EDGES_F, KID_TAIL_F, logB, lbs, cmax, masks, cmasks, Gam, F, Rc, lq, err, acc, post,
+                        log_PD, s);
 }
 
 cudaError_t launch_explog_check(const double* x, int64_t count, double* out, cudaStream_t s)
@@ -1204,9 +1284,10 @@ cudaError_t set_kernel_attributes()
     SETA(k_gamma_p2<double>)
     SETA(k_gamma_p2<float>)
     SETA(k_upzeta_x)
-    SETA(k_gamma_p1_x)
     SETA(k_gamma_p2<X64>)
-    SETA(k_gamma_p2<X64S>)
+    SETA(k_tail<float>)
+    SETA(k_tail<double>)
+    SETA(k_tail<X64S>)
 #undef SETA
     e = set_scores_attributes();
     if (e != cudaSuccess) return e;

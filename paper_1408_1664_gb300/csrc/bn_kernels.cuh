@@ -28,18 +28,17 @@ enum KernelId : int32_t {
     KID_ADD_FEATURE_D, KID_ADD_FEATURE_F, KID_SHIFT_D, KID_SHIFT_F,
     KID_UPZETA_D, KID_UPZETA_F, KID_FWD_LEVEL_D, KID_FWD_LEVEL_F, KID_BWD_LEVEL_D,
     KID_BWD_LEVEL_F, KID_GAMMA_TABLE, KID_GAMMA_P1_D, KID_GAMMA_P1_F, KID_GAMMA_P2_D,
-    KID_GAMMA_P2_F, KID_GAMMA_P2S_D, KID_GAMMA_P2S_F, KID_EDGES_ZERO, KID_EDGES_ACC_D,
-    KID_EDGES_ACC_F, KID_EDGES_FIN_D, KID_EDGES_FIN_F, KID_REORDER_D,
+    KID_GAMMA_P2_F, KID_GAMMA_P2S_D, KID_GAMMA_P2S_F, KID_EDGES_D, KID_EDGES_F, KID_REORDER_D,
     KID_REORDER_F, KID_COLB8, KID_COLB4, KID_COLB2, KID_COLW_D, KID_COLW_F, KID_COLS_D,
     KID_COLS_F, KID_UP13_D, KID_UP13_F_TLO, KID_UP13_F, KID_G13_D_Q, KID_G13_D, KID_G13_F_Q,
     KID_G13_F, KID_FROWS_D, KID_FROWS_F_TLO, KID_FROWS_F, KID_BROWS_D, KID_BROWS_F_TLO,
     KID_BROWS_F, KID_COLB4_D, KID_COLB2_D, KID_COLB1_D, KID_COLB1,
     // the linear FP64 form
     KID_SHIFT_XS, KID_APPLY_Q_XS, KID_ADD_FEATURE_XS, KID_UPZETA_XS, KID_FROWS_XS, KID_BROWS_XS,
-    KID_GAMMA_P1_XS, KID_GAMMA_P2_XS, KID_GAMMA_P2S_XS, KID_EDGES_ACC_XS, KID_EDGES_FIN_XS,
+    KID_TAIL_F, KID_TAIL_D, KID_TAIL_XS,
     KID_SHIFT_X, KID_APPLY_Q_X, KID_ADD_FEATURE_X, KID_REORDER_X, KID_COLB4_X, KID_COLB2_X,
     KID_COLB1_X, KID_COLW_X, KID_UP13_X, KID_FROWS_X, KID_BROWS_X, KID_G13_X_Q, KID_G13_X,
-    KID_GAMMA_P2_X, KID_GAMMA_P2S_X, KID_EDGES_ACC_X, KID_EDGES_FIN_X, KID_COUNT
+    KID_GAMMA_P2_X, KID_GAMMA_P2S_X, KID_EDGES_X, KID_COUNT
 };
 
 // Arguments as one trivially copyable structure whose members have the
@@ -240,7 +239,7 @@ inline bool data_below_arity(const uint8_t* data, int m, int n, const uint8_t* a
 // Scratch of step 1: H(X) per set and, for binary data, the all-ones counts
 // (score_sets(P) entries each), and the nodes' encoded maxima (n entries).
 // They lie in arrays the later steps fill: H in F and R', the counts in lbs,
-// the maxima in the edge accumulators.
+// the maxima in Gamma.
 struct SetScratch {
     long long* H;
     uint32_t* cnt;
@@ -249,10 +248,11 @@ struct SetScratch {
 uint32_t score_sets(const Plan& P);       // sets of at most d + 1 variables
 // Bit planes, the lgamma table T (rows x (m+1) int64: lgamma(alpha + N) -
 // lgamma(alpha) in fixed point, scaled by 2^fxs; the scores sum it exactly),
-// the 13-bit rank tables, the maxima and the error word (each when given).
+// the 13-bit rank tables, the maxima, the error word and step 5's
+// accumulators (each when given).
 cudaError_t launch_step1_prep(const Plan& P, const uint8_t* data, uint64_t* planes,
                               const double* alpha, void* T, uint16_t* rank13,
-                              unsigned long long* enc, int* err, cudaStream_t s,
+                              unsigned long long* enc, int* err, unsigned long long* acc, cudaStream_t s,
                               const int* mj = nullptr, const double* fxj = nullptr);
 cudaError_t launch_check_data(const uint8_t* data, const uint8_t* arity, int n, int m,
                               int* err, cudaStream_t s);
@@ -358,10 +358,13 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_
 // FP32: the per-endpoint offsets of the down-zeta input (one small launch,
 // made by launch_gamma_p1 itself; stored after the level words of Rc).
 cudaError_t launch_gamma_table(const Plan& P, const void* F, const void* Rc, cudaStream_t s);
-// Step 5 (three launches); acc: n * (n + 1) scratch words.
+// Step 5 (one launch); acc: n * (n + 1) scratch words, zero before and
+// after.  For n < 14 (use_tail) it is step 4 too: from F and R' (and the order
+// prior lq) to Gam, post and log P(D).
+bool use_tail(const Plan& P);
 cudaError_t launch_edges(const Plan& P, const double* logB, const void* lbs, const double* cmax,
-                         const uint32_t* masks, const void* Gam, const void* F,
-                         const int* err, unsigned long long* acc, double* post, double* log_PD,
+                         const uint32_t* masks, const uint32_t* cmasks, void* Gam, const void* F, const void* Rc,
+                         const void* lq, const int* err, unsigned long long* acc, double* post, double* log_PD,
                          cudaStream_t s);
 
 size_t upzeta_smem_bytes(const Plan& P);

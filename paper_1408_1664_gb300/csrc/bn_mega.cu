@@ -108,7 +108,6 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
     case KID_SET_HIST_BLOCK: run(k_set_hist<256>, a); return true;
     case KID_SET_ANY: run(k_set_any, a); return true;
     case KID_FAMILIES: run(k_family_scores, a); return true;
-    case KID_EDGES_ZERO: run(k_edges_zero, a); return true;
     default: break;
     }
     if constexpr (PREC == 1) {
@@ -121,8 +120,8 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
         case KID_GAMMA_P1_F: run(k_gamma_p1<float>, a); return true;
         case KID_GAMMA_P2_F: run(k_gamma_p2<float>, a); return true;
         case KID_GAMMA_P2S_F: run(k_gamma_p2s<float>, a); return true;
-        case KID_EDGES_ACC_F: run(k_edges_acc<float>, a); return true;
-        case KID_EDGES_FIN_F: run(k_edges_fin<float>, a); return true;
+        case KID_EDGES_F: run(k_edges<float>, a); return true;
+        case KID_TAIL_F: run(k_tail<float>, a); return true;
         case KID_REORDER_F: run(k_reorder_up<float>, a); return true;
         case KID_COLB8: run(k_upzeta13_colb<float, 8>, a); return true;
         case KID_COLB4: run(k_upzeta13_colb<float, 4>, a); return true;
@@ -146,11 +145,7 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
         case KID_UPZETA_XS: run(k_upzeta_x, a); return true;
         case KID_FROWS_XS: run(k_forward_rows<X64S, false>, a); return true;
         case KID_BROWS_XS: run(k_backward_rows<X64S, false>, a); return true;
-        case KID_GAMMA_P1_XS: run(k_gamma_p1_x, a); return true;
-        case KID_GAMMA_P2_XS: run(k_gamma_p2<X64S>, a); return true;
-        case KID_GAMMA_P2S_XS: run(k_gamma_p2s_x<X64S>, a); return true;
-        case KID_EDGES_ACC_XS: run(k_edges_acc_x<X64S>, a); return true;
-        case KID_EDGES_FIN_XS: run(k_edges_fin<X64S>, a); return true;
+        case KID_TAIL_XS: run(k_tail<X64S>, a); return true;
         case KID_REORDER_X: run(k_reorder_up<X64>, a); return true;
         case KID_COLB4_X: run(k_colb_x<4>, a); return true;
         case KID_COLB2_X: run(k_colb_x<2>, a); return true;
@@ -162,8 +157,7 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
         case KID_G13_X: run(k_g13_x<false>, a); return true;
         case KID_GAMMA_P2_X: run(k_gamma_p2<X64>, a); return true;
         case KID_GAMMA_P2S_X: run(k_gamma_p2s_x<X64>, a); return true;
-        case KID_EDGES_ACC_X: run(k_edges_acc_x<X64>, a); return true;
-        case KID_EDGES_FIN_X: run(k_edges_fin<X64>, a); return true;
+        case KID_EDGES_X: run(k_edges<X64>, a); return true;
         case KID_SHIFT_D: run(k_shift_scores<double>, a); return true;
         case KID_UPZETA_D: run(k_upzeta<double>, a); return true;
         case KID_FWD_LEVEL_D: run(k_forward_level<double>, a); return true;
@@ -171,8 +165,8 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
         case KID_GAMMA_P1_D: run(k_gamma_p1<double>, a); return true;
         case KID_GAMMA_P2_D: run(k_gamma_p2<double>, a); return true;
         case KID_GAMMA_P2S_D: run(k_gamma_p2s<double>, a); return true;
-        case KID_EDGES_ACC_D: run(k_edges_acc<double>, a); return true;
-        case KID_EDGES_FIN_D: run(k_edges_fin<double>, a); return true;
+        case KID_EDGES_D: run(k_edges<double>, a); return true;
+        case KID_TAIL_D: run(k_tail<double>, a); return true;
         case KID_REORDER_D: run(k_reorder_up<double>, a); return true;
         case KID_COLW_D: run(k_upzeta13_colw<double>, a); return true;
         case KID_COLB4_D: run(k_upzeta13_colb<double, 4>, a); return true;
@@ -294,25 +288,22 @@ bool persistent_runs(int prec, int kid)
     switch (kid) {
     case KID_STEP1_PREP: case KID_CHECK_DATA: case KID_SET_ONES: case KID_SET_MOEBIUS:
     case KID_SET_HIST_WARP: case KID_SET_HIST_BLOCK: case KID_SET_ANY: case KID_FAMILIES:
-    case KID_EDGES_ZERO:
         return true;
     case KID_SHIFT_F: case KID_UPZETA_F: case KID_FWD_LEVEL_F: case KID_BWD_LEVEL_F:
     case KID_GAMMA_TABLE: case KID_GAMMA_P1_F: case KID_GAMMA_P2_F: case KID_GAMMA_P2S_F:
-    case KID_EDGES_ACC_F: case KID_EDGES_FIN_F: case KID_REORDER_F: case KID_COLB8: case KID_COLB4:
+    case KID_EDGES_F: case KID_TAIL_F: case KID_REORDER_F: case KID_COLB8: case KID_COLB4:
     case KID_COLB2: case KID_COLB1: case KID_COLW_F: case KID_COLS_F: case KID_UP13_F_TLO: case KID_UP13_F:
     case KID_G13_F: case KID_FROWS_F_TLO: case KID_FROWS_F: case KID_BROWS_F_TLO: case KID_BROWS_F:
         return prec == 1;
     case KID_SHIFT_D: case KID_UPZETA_D: case KID_FWD_LEVEL_D: case KID_BWD_LEVEL_D:
-    case KID_GAMMA_P1_D: case KID_GAMMA_P2_D: case KID_GAMMA_P2S_D: case KID_EDGES_ACC_D:
-    case KID_EDGES_FIN_D: case KID_REORDER_D: case KID_COLW_D: case KID_COLS_D: case KID_UP13_D:
+    case KID_GAMMA_P1_D: case KID_GAMMA_P2_D: case KID_GAMMA_P2S_D: case KID_EDGES_D: case KID_TAIL_D: case KID_REORDER_D: case KID_COLW_D: case KID_COLS_D: case KID_UP13_D:
     case KID_COLB4_D: case KID_COLB2_D: case KID_COLB1_D:
     case KID_G13_D: case KID_FROWS_D: case KID_BROWS_D:
-    case KID_SHIFT_XS: case KID_UPZETA_XS: case KID_FROWS_XS: case KID_BROWS_XS: case KID_GAMMA_P1_XS:
-    case KID_GAMMA_P2_XS: case KID_GAMMA_P2S_XS: case KID_EDGES_ACC_XS: case KID_EDGES_FIN_XS:
+    case KID_SHIFT_XS: case KID_UPZETA_XS: case KID_FROWS_XS: case KID_BROWS_XS: case KID_TAIL_XS:
     case KID_SHIFT_X: case KID_REORDER_X: case KID_COLB4_X: case KID_COLB2_X:
     case KID_COLB1_X: case KID_COLW_X: case KID_UP13_X: case KID_FROWS_X: case KID_BROWS_X:
     case KID_G13_X: case KID_GAMMA_P2_X: case KID_GAMMA_P2S_X:
-    case KID_EDGES_ACC_X: case KID_EDGES_FIN_X:
+    case KID_EDGES_X:
         return prec == 0;
     default:
         return false;

@@ -243,11 +243,11 @@ try {
     double* cmax = reinterpret_cast<double*>(base + o_cmax);
     uint16_t* rk13 = reinterpret_cast<uint16_t*>(base + o_rk);
     // step 1's scratch in arrays the later steps fill (8 bytes per set in F
-    // and R', 4 in lbs, the maxima in the edge accumulators)
+    // and R', 4 in lbs, the maxima in Gamma)
     const bn::SetScratch x{reinterpret_cast<long long*>(base + o_F), reinterpret_cast<uint32_t*>(base + o_lbs),
-                           reinterpret_cast<unsigned long long*>(base + o_ea)};
+                           reinterpret_cast<unsigned long long*>(base + o_G)};
     CKS(bn::launch_step1_prep(P, data_dev, planes, alpha, lgT, bn::needs_rank13(P) ? rk13 : nullptr, x.enc,
-                              err, s));
+                              err, reinterpret_cast<unsigned long long*>(base + o_ea), s));
     if (j->data_on_device) CKS(bn::launch_check_data(data_dev, ar, P.n, P.m, err, s));
     CKS(bn::launch_scores(P, data_dev, ar, planes, Dvals, lgT,
                           j->log_rho ? reinterpret_cast<const double*>(base + o_lr) : nullptr, nullptr, x,
@@ -263,7 +263,7 @@ try {
     }
     CKS(bn::launch_gamma_p1(P, base + o_F, base + o_Rc, rk13, base + o_W, s, nullptr, base + o_A));
     CKS(bn::launch_gamma_p2(P, base + o_W, base + o_G, s));
-    CKS(bn::launch_edges(P, logB, base + o_lbs, cmax, masks, base + o_G, base + o_F, err,
+    CKS(bn::launch_edges(P, logB, base + o_lbs, cmax, masks, cm, base + o_G, base + o_F, base + o_Rc, nullptr, err,
                          reinterpret_cast<unsigned long long*>(base + o_ea), post_dev,
                          log_PD_dev, s));
 #undef CKS

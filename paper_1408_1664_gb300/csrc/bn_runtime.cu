@@ -350,10 +350,10 @@ struct Bufs {
     void* A() const { return A_ext ? (void*)A_ext : (void*)(base + L.A); }
     // Step 1's scratch in arrays the later steps fill: 8 bytes per set fit
     // F and R' (at most 2^n sets), 4 per set lbs (n*K values, at least the
-    // nonempty sets' number)
+    // nonempty sets' number), the maxima Gamma
     bn::SetScratch set_scratch() const
     {
-        return {at<long long>(L.F), at<uint32_t>(L.lbs), at<unsigned long long>(L.eacc)};
+        return {at<long long>(L.F), at<uint32_t>(L.lbs), at<unsigned long long>(L.Gam)};
     }
 };
 
@@ -436,7 +436,8 @@ int enqueue_step1(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, cud
     const uint8_t* ar = B.at<uint8_t>(L.arity);
     const bn::SetScratch x = B.set_scratch();
     CK(bn::launch_step1_prep(P, data_dev, B.at<uint64_t>(L.planes), B.at<double>(L.alpha), B.at<void>(L.lgT),
-                             bn::needs_rank13(P) ? B.at<uint16_t>(L.rk13) : nullptr, x.enc, err, s)); ++*nl;
+                             bn::needs_rank13(P) ? B.at<uint16_t>(L.rk13) : nullptr, x.enc, err,
+                             B.at<unsigned long long>(L.eacc), s)); ++*nl;
     if (hj.data_on_device) { CK(bn::launch_check_data(data_dev, ar, P.n, P.m, err, s)); ++*nl; }
     CK(bn::launch_scores(P, data_dev, ar, B.at<uint64_t>(L.planes), B.at<double>(L.Dvals), B.at<void>(L.lgT),
                          hj.log_rho.empty() ? nullptr : B.at<double>(L.log_rho),
@@ -526,9 +527,10 @@ int enqueue_kernels(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, d
         nl += bn::gamma_launches(P);
     }
     CK(bn::launch_edges(P, B.at<double>(L.logB), B.at<void>(L.lbs), B.at<double>(L.cmax), B.at<uint32_t>(L.masks),
-                        B.at<void>(L.Gam), B.at<void>(L.F), err,
+                        B.at<uint32_t>(L.cmasks), B.at<void>(L.Gam), B.at<void>(L.F), B.at<void>(L.Rc),
+                        P.hasq ? B.at<void>(L.logq) : nullptr, err,
                         B.at<unsigned long long>(L.eacc), post_dev, logPD_dev, s));
-    nl += 3;
+    ++nl;
     if (ev) CK(cudaEventRecord(ev->ev[kEvEdges], s));
     if (launches) *launches = nl;
     if (ev) {
@@ -1080,7 +1082,7 @@ try {
     CK(cudaMemcpyAsync(B.at<char>(L.alpha), alpha.data(), alpha.size() * 8, cudaMemcpyHostToDevice, s));
     const uint8_t* ar = B.at<uint8_t>(L.arity);
     CK(bn::launch_step1_prep(P, data_dev, B.at<uint64_t>(L.planes), B.at<double>(L.alpha), B.at<void>(L.lgT),
-                             nullptr, nullptr, B.at<int>(L.err), s));
+                             nullptr, nullptr, B.at<int>(L.err), nullptr, s));
     if (hj.data_on_device) CK(bn::launch_check_data(data_dev, ar, P.n, P.m, B.at<int>(L.err), s));
     // the weights and the sets' scratch sit past logB in the layout
     double* w = nullptr;
@@ -1252,7 +1254,7 @@ try {
     CK(cudaMemcpyAsync(B.at<char>(L.Dvals), hj.Dvals.data(), hj.Dvals.size() * 8, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(B.at<char>(L.alpha), alpha.data(), alpha.size() * 8, cudaMemcpyHostToDevice, s));
     CK(bn::launch_step1_prep(P, data_dev, B.at<uint64_t>(L.planes), B.at<double>(L.alpha), B.at<void>(L.lgT),
-                             nullptr, nullptr, nullptr, s));
+                             nullptr, nullptr, nullptr, nullptr, s));
     CK(bn::launch_set_scores(P, data_dev, B.at<uint8_t>(L.arity), B.at<uint64_t>(L.planes),
                              B.at<double>(L.Dvals), B.at<void>(L.lgT), B.set_scratch(), s, nullptr,
                              B.at<int64_t>(L.dbg), rank));
@@ -1420,14 +1422,14 @@ int enqueue_steps(const Plan& G, const Layout& L, char* base, cudaStream_t s, un
         // words past a job's m are empty and count nothing, rows past its
         // own are never looked up
         const bn::SetScratch x{reinterpret_cast<long long*>(at(L.F)), reinterpret_cast<uint32_t*>(at(L.lbs)),
-                               reinterpret_cast<unsigned long long*>(at(L.eacc))};
+                               reinterpret_cast<unsigned long long*>(at(L.Gam))};
         const uint8_t* data = reinterpret_cast<const uint8_t*>(at(L.data));
         const int* mj = reinterpret_cast<const int*>(at(L.mj));
         const double* fx = reinterpret_cast<const double*>(at(L.fx));
         uint64_t* planes = reinterpret_cast<uint64_t*>(at(L.planes));
         CK(bn::launch_step1_prep(G, data, planes, reinterpret_cast<const double*>(at(L.alpha)), at(L.lgT),
                                  bn::tile13_gamma_fits(G) ? reinterpret_cast<uint16_t*>(at(L.rk13)) : nullptr,
-                                 x.enc, nullptr, s, mj, fx));
+                                 x.enc, nullptr, reinterpret_cast<unsigned long long*>(at(L.eacc)), s, mj, fx));
         CK(bn::launch_scores(G, data, reinterpret_cast<const uint8_t*>(at(L.arity)), planes,
                              reinterpret_cast<const double*>(at(L.Dvals)), at(L.lgT),
                              reinterpret_cast<const double*>(at(L.log_rho)), nullptr, x,
@@ -1465,7 +1467,8 @@ int enqueue_steps(const Plan& G, const Layout& L, char* base, cudaStream_t s, un
     if (stages & 16u)
         CK(bn::launch_edges(G, reinterpret_cast<const double*>(at(L.logB)), at(L.lbs),
                             reinterpret_cast<const double*>(at(L.cmax)),
-                            reinterpret_cast<const uint32_t*>(at(L.masks)), at(L.Gam), at(L.F),
+                            reinterpret_cast<const uint32_t*>(at(L.masks)),
+                            reinterpret_cast<const uint32_t*>(at(L.cmasks)), at(L.Gam), at(L.F), at(L.Rc), nullptr,
                             reinterpret_cast<const int*>(at(L.err)),
                             reinterpret_cast<unsigned long long*>(at(L.eacc)),
                             reinterpret_cast<double*>(at(L.post)),
@@ -1575,10 +1578,9 @@ int record_groups(bn_batch* b)
                 switch (x.kid) {                   // kernels that loop grid-stride in x
                 case bn::KID_STEP1_PREP: case bn::KID_CHECK_DATA: case bn::KID_SET_HIST_WARP:
                 case bn::KID_SET_HIST_BLOCK: case bn::KID_SET_ANY: case bn::KID_FAMILIES:
-                case bn::KID_SHIFT_F: case bn::KID_SHIFT_D: case bn::KID_SHIFT_X: case bn::KID_EDGES_ACC_X:
-                case bn::KID_SHIFT_XS: case bn::KID_EDGES_ACC_XS:
-                case bn::KID_REORDER_X: case bn::KID_COLW_X: case bn::KID_EDGES_ACC_F:
-                case bn::KID_EDGES_ACC_D: case bn::KID_REORDER_F: case bn::KID_REORDER_D:
+                case bn::KID_SHIFT_F: case bn::KID_SHIFT_D: case bn::KID_SHIFT_X: case bn::KID_EDGES_X:
+                case bn::KID_SHIFT_XS:
+                case bn::KID_REORDER_X: case bn::KID_COLW_X: case bn::KID_EDGES_F: case bn::KID_EDGES_D: case bn::KID_REORDER_F: case bn::KID_REORDER_D:
                 case bn::KID_COLW_F: case bn::KID_COLW_D:
                     x.pad[0] |= bn::kRecStrideX;
                     break;
@@ -2520,7 +2522,8 @@ try {
                            P.slab ? nullptr : B.at<void>(L.A)));
     CK(bn::launch_gamma_p2(P, B.at<void>(L.W), B.at<void>(L.Gam), s));
     CK(bn::launch_edges(P, B.at<double>(L.logB), B.at<void>(L.lbs), B.at<double>(L.cmax), B.at<uint32_t>(L.masks),
-                        B.at<void>(L.Gam), B.at<void>(L.F), B.at<int>(L.err),
+                        B.at<uint32_t>(L.cmasks), B.at<void>(L.Gam), B.at<void>(L.F), B.at<void>(L.Rc),
+                        P.hasq ? B.at<void>(L.logq) : nullptr, B.at<int>(L.err),
                         B.at<unsigned long long>(L.eacc), post_dev,
                         log_PD_dev ? log_PD_dev : B.at<double>(L.logPD), s));
     return BN_OK;

@@ -96,8 +96,8 @@ __device__ __forceinline__ long long warp_sum(long long x)
 //  * T[row*(m+1) + N] = [lgamma(alpha_row + N) - lgamma(alpha_row)] * scale
 //    rounded to an integer (scale = 2^S): the fixed-point table;
 //  * the rank tables of the 13-bit patterns (rank13 may be null);
-//  * the per-node maxima, started at the lowest encoding (enc may be null),
-//    and the job's error word (err may be null).
+//  * the per-node maxima, started at the lowest encoding, the job's error word
+//    and step 5's accumulators (enc, err and acc may be null).
 // In a batch group mj holds each job's own sample count and fxj its
 // (scale, 1/scale): entries past the job's m stay 0 (no count reaches them).
 __global__ void __launch_bounds__(256)
@@ -105,7 +105,8 @@ k_step1_prep(const uint8_t* __restrict__ data, int n, int m, int rmax, int W,
              uint64_t* __restrict__ planes, const int* __restrict__ mj,
              const double* __restrict__ alpha, int rows, long long* __restrict__ T, double scale,
              const double* __restrict__ fxj, uint16_t* __restrict__ rank13,
-             unsigned long long* __restrict__ enc, int* __restrict__ err, size_t js)
+             unsigned long long* __restrict__ enc, int* __restrict__ err,
+             unsigned long long* __restrict__ acc, size_t js)
 {
     data = job_ptr(data, js);
     planes = job_ptr(planes, js);
@@ -148,6 +149,8 @@ k_step1_prep(const uint8_t* __restrict__ data, int n, int m, int rmax, int W,
             rk[8192 + r] = (uint16_t)L;
         } else {
             if (enc && lane < n) job_ptr(enc, js)[lane] = 0ull;
+            if (acc)
+                for (int t = lane; t < n * (n + 1); t += 32) job_ptr(acc, js)[t] = 0ull;
             // the error word and the counters of k_sweeps after it (256 bytes)
             if (err) reinterpret_cast<int2*>(job_ptr(err, js))[lane] = make_int2(0, 0);
         }
@@ -712,14 +715,14 @@ uint32_t score_sets(const Plan& P) { return sets_before(P.n, std::min(P.d + 1, P
 
 cudaError_t launch_step1_prep(const Plan& P, const uint8_t* data, uint64_t* planes,
                               const double* alpha, void* T, uint16_t* rank13,
-                              unsigned long long* enc, int* err, cudaStream_t s, const int* mj,
-                              const double* fxj)
+                              unsigned long long* enc, int* err, unsigned long long* acc, cudaStream_t s,
+                              const int* mj, const double* fxj)
 {
     const int64_t items = (int64_t)P.n * 2 * P.W + ((int64_t)P.rows * (P.m + 1) + 31) / 32 +
                           (rank13 ? 256 : 0) + 1;
     return launch_or_record(KID_STEP1_PREP, k_step1_prep, dim3(grid_for(items, 8), P.nj), 256, 0, s, data,
                             P.n, P.m, P.rmax, P.W, planes, mj, alpha, P.rows, (long long*)T,
-                            std::ldexp(1.0, P.fxs), fxj, rank13, enc, err, P.js);
+                            std::ldexp(1.0, P.fxs), fxj, rank13, enc, err, acc, P.js);
 }
 
 cudaError_t launch_check_data(const uint8_t* data, const uint8_t* arity, int n, int m,
