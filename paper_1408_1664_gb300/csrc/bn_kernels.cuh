@@ -156,6 +156,7 @@ struct Plan {
     int up13 = 0;         // step 2 by the 13-dimension tiles (n >= 14)
     int g13 = 0;          // step 4 phase 1 by the 13-dimension tiles (n >= 14)
     int frows = 0;        // FP32 step 3 by the 16-subset row kernels
+    int busy = 0;         // a served job admitted beside others (see use_sweeps)
     int frc = 0;          // FP32 step 3 of a batch group by k_sweeps (one launch)
     // Batch groups: nj jobs with equal plans, their arrays js bytes apart;
     // the launches of steps 2-5 cover all of them (gridDim.y = nj).

@@ -29,10 +29,16 @@ namespace {
 constexpr int LB = 4;             // low bits of an FP32 tile
 constexpr int LB64 = 3;           // low bits of an FP64 tile
 constexpr int BT = 29;            // binomial table rows (n - B < 29: n <= 32 in FP32)
-// k_sweeps: single jobs up to this n (FP32; linear FP64); levels that fill
-// more than kSweepGrid blocks run on the whole GPU; polls before a block gives up a wait (about 1 us each).
+// k_sweeps: single jobs up to this n (FP32; linear FP64; a launch per level is
+// faster from n = 22: FP32 330 us either way, FP64 621 against 729), vectors
+// from kSweepVecN, up to kSweepBusyN while other served jobs run (the whole-GPU
+// form of a wider job would hold every SM: 64 served jobs of n = 19 to 22 took
+// 20.0 ms with it, 15.3 ms without); levels that fill more than kSweepGrid
+// blocks run on the whole GPU; polls before a block gives up a wait (about 1 us each).
 constexpr int kSweepMaxN = 21;
-constexpr int kSweepMaxNX = 20;
+constexpr int kSweepMaxNX = 21;
+constexpr int kSweepVecN = 20;
+constexpr int kSweepBusyN = 18;
 constexpr uint64_t kSweepGrid = 12;
 constexpr uint32_t kSweepSpinCap = 1u << 22;
 
@@ -436,8 +442,8 @@ k_backward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __re
 // separated by a barrier of the blocks that share it, instead of a launch per
 // level.  A level launch of a job up to n of about 20 took 9 to 12 us, nearly
 // all of it latency: the launch itself and one thread walking a tile's terms,
-// each a dependent pair of row loads.  Here a tile's 16 (FP64: 8) subsets take as many lanes
-// (one value each), a lane issues the loads of up to eight (four) terms together,
+// each a dependent pair of row loads.  Here a tile's 16 (FP64: 8) subsets take several lanes
+// (one value each, or a short vector), a lane issues the loads of up to eight (four) terms together,
 // and the first tile's index and A values for the next level are fetched
 // between arriving at the barrier and waiting on it.  The sums run in the
 // order of forward_tile / backward_tile, so the results are the same bits.
@@ -456,22 +462,68 @@ k_backward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __re
 // arrivals of F / R', sync[8] / sync[24] the blocks done (the last resets
 // both); they start at zero (k_step1_prep).
 enum { SYNC_BLOCK = 0, SYNC_CLUSTER = 1, SYNC_GRID = 2 };
-constexpr int kSweepThreads = 512;
 
-template <typename T, bool TLO, int SYNC>
-__global__ void __launch_bounds__(kSweepThreads, 2)
+// N consecutive values (N * sizeof(T) bytes, aligned to them) by load mode;
+// rev: in reverse order.
+template <typename T, int N>
+__device__ __forceinline__ void load_vals(const T* p, T (&v)[N], int mode, bool rev)
+{
+    if constexpr (N == 1) {
+        v[0] = load_one(p, mode);
+    } else if constexpr (sizeof(T) * N == 8) {      // two floats
+        const float2* q = reinterpret_cast<const float2*>(p);
+        const float2 x = mode == LD_STREAM ? __ldcs(q) : mode == LD_L2 ? __ldcg(q) : *q;
+        v[0] = x.x;
+        v[1] = x.y;
+    } else {
+        load_row(p, v, mode);
+    }
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+        const T lo = v[k], hi = v[N - 1 - k];
+        v[k] = rev ? hi : lo;
+        v[N - 1 - k] = rev ? lo : hi;
+    }
+}
+template <typename T, int N>
+__device__ __forceinline__ void store_vals(T* p, const T (&v)[N], bool rev)
+{
+    T w[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) w[k] = rev ? v[N - 1 - k] : v[k];
+    if constexpr (N == 1) *p = w[0];
+    else store_row(p, w);
+}
+
+// VB: a lane holds the 2^VB values whose VB lowest bits vary (0: one value;
+// 2, a 16-byte vector, in FP32).  One value per lane has the shortest chain,
+// the faster form while latency bounds a level; vectors share the addresses,
+// the index walk and half of the in-tile steps, the faster form once the
+// levels are wide: n = 19 103 us (one value) and 117 (vectors), n = 20 145 and
+// 135, n = 21 240 and 199.  (FP64 pairs were slower throughout: n = 20 232 us
+// and 287.)
+template <int VB> struct SweepShape {
+    static constexpr int threads = VB ? 256 : 512;
+    static constexpr int blocks = VB ? 3 : 2;       // resident per SM
+};
+
+template <typename T, bool TLO, int SYNC, int VB>
+__global__ void __launch_bounds__(SweepShape<VB>::threads, SweepShape<VB>::blocks)
 k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restrict__ Rc, size_t js,
          unsigned* __restrict__ sync, int* __restrict__ err, uint32_t cap)
 {
     constexpr int B = sizeof(T) == 4 ? LB : LB64;
-    constexpr int LN = 1 << B;                      // lanes per tile
-    constexpr int CH = sizeof(T) == 4 ? 8 : 4;      // terms loaded together (64 registers)
+    constexpr int NV = 1 << VB, LNB = B - VB, LN = 1 << LNB;   // values per lane, lanes per tile
+    constexpr int CH = sizeof(T) == 4 && VB == 0 ? 8 : 4;      // terms loaded together
     constexpr bool kBases = sizeof(T) == 4;
     constexpr int XMODE = SYNC == SYNC_BLOCK ? LD_PLAIN : LD_L2;
     __shared__ uint32_t bt[BT][BT];
-    __shared__ int wm[kSweepThreads / 32];
+    __shared__ int wm[SweepShape<VB>::threads / 32];
     __shared__ int ok_s;
+    __shared__ uint16_t place[TLO ? 512 : 1];
     fill_table(bt);
+    if (TLO)
+        for (int x = threadIdx.x; x < 512; x += blockDim.x) place[x] = g_place.p9[x];
     __syncthreads();
     const int it = (int)(blockIdx.x / (unsigned)nb);
     const uint32_t rank = blockIdx.x % (unsigned)nb;
@@ -482,38 +534,53 @@ k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restric
     const int nh = n - B;
     const uint32_t hmask = (1u << nh) - 1u;
     const size_t half = (size_t)1 << (n - 1), full = (size_t)1 << n;
+    // the lane's subsets: in-tile bits (l << VB) | r; value e has the in-lane
+    // elements e (R': the missing ones, so the values sit in reverse order)
     const int l = threadIdx.x & (LN - 1);
-    const uint32_t own = fwd ? (uint32_t)l : (uint32_t)l ^ (LN - 1);   // the lane's in-tile elements
+    const uint32_t own = fwd ? (uint32_t)l : (uint32_t)l ^ (LN - 1);   // the lane's elements
     const int size = __popc(own);
-    const unsigned tmask = ((1u << LN) - 1u) << (threadIdx.x & 31 & ~(LN - 1));   // the tile's lanes
+    const unsigned tmask = (LN == 32 ? ~0u : (1u << LN) - 1u) << (threadIdx.x & 31 & ~(LN - 1));   // the tile's lanes
     // the groups of LN lanes number across the blocks: a narrow level spreads over them
-    const uint32_t hw = (threadIdx.x >> B) * (uint32_t)nb + rank;
-    const uint32_t nhw = (blockDim.x >> B) * (uint32_t)nb;
+    const uint32_t hw = (threadIdx.x >> LNB) * (uint32_t)nb + rank;
+    const uint32_t nhw = (blockDim.x >> LNB) * (uint32_t)nb;
     int* lw = kBases ? level_words(reinterpret_cast<float*>(X), n) : nullptr;
     unsigned* arr = SYNC == SYNC_GRID ? sync + (fwd ? 0 : 16) : nullptr;
 
-    // place of element l of row S-without-j of A_{B + j}, and of the row of
-    // A_i (i < B) that the tile's in-tile terms read
-    auto a_at = [&](uint32_t H, int j) {
-        const uint32_t R = squeeze(H, j);
-        return BN_AT((size_t)(B + j) * half + ((size_t)(TLO ? tlo_row(R, 9) : R) << B) + l, 1, n * half);
+    // Places are 32-bit (n <= kSweepMaxN).  That of the lane's values in the row
+    // S-without-j of A_{B + j}, u = 1 << j: H with bit j squeezed out is
+    // (H >> 1) with the bits below j taken from H.
+    auto a_at = [&](uint32_t H, uint32_t u) {
+        const uint32_t up = H >> 1, R = up ^ ((up ^ H) & (u - 1u));
+        const uint32_t row = TLO ? (R & ~511u) | place[R & 511u] : R;
+        return BN_AT(((uint32_t)(B + 31 - __clz(u)) << (n - 1)) + (row << B) + (l << VB), NV, n * half);
     };
+    // the row of A_i (i < B) that the tile's in-tile terms read: for an in-lane
+    // element i NV / 2 values, for a lane element NV
     auto in_at = [&](uint32_t H, int i) {
-        return BN_AT((size_t)i * half + ((size_t)(TLO ? tlo_row(H, 10) : H) << (B - 1)) + squeeze4(l, i), 1,
-                     n * half);
+        const int at = i < VB ? l << (VB - 1) : squeeze4(l, i - VB) << VB;
+        return BN_AT(((uint32_t)i << (n - 1)) + ((TLO ? tlo_row(H, 10) : H) << (B - 1)) + at,
+                     i < VB ? (NV + 1) / 2 : NV, n * half);
     };
     // a group's run of tiles in step st: consecutive in colex order, so
     // only the first is unranked.  Its bits, the A values of its first terms
     // and of its in-tile terms are fetched ahead of the step.
     uint32_t bits = 0, g0 = 0, g1 = 0;
-    T pa[CH], pi[B];
-    auto load_a = [&](uint32_t H, uint32_t& rest, int st, T (&a)[CH]) {
+    constexpr bool kAhead = VB == 0;                // (vectors: more registers, one block fewer)
+    T pa[kAhead ? CH : 1][NV], pin[VB ? VB : 1][NV > 1 ? NV / 2 : 1], plane[LNB][NV];
+    auto load_a = [&](uint32_t H, uint32_t& rest, int st, T (&a)[CH][NV]) {
 #pragma unroll
         for (int q = 0; q < CH; ++q) {
             if (q < st) {
-                a[q] = load_one(A + a_at(H, __ffs(rest) - 1), LD_STREAM);
+                load_vals(A + a_at(H, rest & (0u - rest)), a[q], LD_STREAM, !fwd);
                 rest &= rest - 1;
             }
+        }
+    };
+    auto load_in = [&](uint32_t H) {
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            if (i < VB) load_vals(A + in_at(H, i), pin[i < VB ? i : 0], LD_STREAM, !fwd);
+            else load_vals(A + in_at(H, i), plane[i < VB ? 0 : i - VB], LD_STREAM, !fwd);
         }
     };
     auto ahead = [&](int st) {
@@ -522,11 +589,12 @@ k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restric
         g1 = min(nt, g0 + run);
         if (g0 >= g1) return;
         bits = tile_of(g0, st, nh, bt);
-        const uint32_t H = fwd ? bits : hmask ^ bits;
-        uint32_t rest = bits;
-        load_a(H, rest, st, pa);
-#pragma unroll
-        for (int i = 0; i < B; ++i) pi[i] = load_one(A + in_at(H, i), LD_STREAM);
+        if constexpr (kAhead) {
+            const uint32_t H = fwd ? bits : hmask ^ bits;
+            uint32_t rest = bits;
+            load_a(H, rest, st, pa);
+            load_in(H);
+        }
     };
     ahead(0);
     for (int st = 0; st <= nh; ++st) {
@@ -541,49 +609,75 @@ k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restric
         for (uint32_t g = g0; g < g1; ++g) {
             const uint32_t H = fwd ? bits : hmask ^ bits;
             uint32_t ra = bits, rf = bits;
-            TileSum<T> s;
+            TileSum<T> s[NV];
             for (int c0 = 0; c0 < st; c0 += CH) {
-                T a[CH], f[CH];
+                T a[CH][NV], f[CH][NV];
 #pragma unroll
                 for (int q = 0; q < CH; ++q) {
-                    f[q] = T{};
+#pragma unroll
+                    for (int e = 0; e < NV; ++e) f[q][e] = T{};
                     if (c0 + q < st) {
-                        const T* p = X + BN_AT(((size_t)(H ^ (rf & (0u - rf))) << B) + l, 1, full);
+                        load_vals(X + BN_AT(((H ^ (rf & (0u - rf))) << B) + (l << VB), NV, full), f[q], XMODE,
+                                  !fwd);
                         rf &= rf - 1;
-                        f[q] = load_one(p, XMODE);
                     }
                 }
-                if (g == g0 && c0 == 0) {
+                if (kAhead && g == g0 && c0 == 0) {
 #pragma unroll
                     for (int q = 0; q < CH; ++q) {
-                        a[q] = pa[q];
+#pragma unroll
+                        for (int e = 0; e < NV; ++e) a[q][e] = pa[kAhead ? q : 0][e];
                         ra &= ra - 1;
                     }
                 } else {
                     load_a(H, ra, st - c0, a);
                 }
 #pragma unroll
-                for (int q = 0; q < CH; ++q) s.add(a[q], f[q], c0 + q < st);
-            }
-            s.rebase(rebase);
-            T ai[B];
+                for (int q = 0; q < CH; ++q)
 #pragma unroll
-            for (int i = 0; i < B; ++i) ai[i] = g == g0 ? pi[i] : load_one(A + in_at(H, i), LD_STREAM);
+                    for (int e = 0; e < NV; ++e) s[e].add(a[q][e], f[q][e], c0 + q < st);
+            }
+            if (!kAhead || g != g0) load_in(H);
             // the in-tile terms, in popcount order of the lane's elements: in
-            // round k the lanes with k elements add theirs (the others a left-out
-            // term, so the lanes of a warp stay together)
-            T v = st == 0 ? unit<T>() : s.value();
+            // round k the lanes with k elements add theirs.  One value per lane:
+            // the others add a left-out term, so a warp's lanes stay together
+            T v[NV];
 #pragma unroll
-            for (int k = 1; k <= B; ++k) {
-#pragma unroll
-                for (int i = 0; i < B; ++i) {
-                    const T y = shfl_one(tmask, v, 1 << i);
-                    s.add(ai[i], y, size == k && (own >> i & 1));
-                }
-                if (size == k) v = s.value();
+            for (int e = 0; e < NV; ++e) {
+                s[e].rebase(rebase);
+                v[e] = unit<T>();
             }
-            X[BN_AT(((size_t)H << B) + l, 1, full)] = v;
-            if constexpr (kBases) mx = v > mx ? v : mx;
+#pragma unroll
+            for (int k = 0; k <= LNB; ++k) {
+                T y[LNB][NV];
+                if (k > 0) {
+#pragma unroll
+                    for (int i = 0; i < LNB; ++i)
+#pragma unroll
+                        for (int e = 0; e < NV; ++e) {
+                            y[i][e] = shfl_one(tmask, v[e], 1 << i);
+                            if (VB == 0) s[e].add(plane[i][e], y[i][e], size == k && (own >> i & 1));
+                        }
+                }
+                if (size == k) {
+#pragma unroll
+                    for (int e = 0; e < NV; ++e) {
+#pragma unroll
+                        for (int i = 0; i < VB; ++i)
+                            if (e >> i & 1) s[e].add(pin[i][squeeze4(e, i)], v[e ^ (1 << i)]);
+                        if (VB > 0 && k > 0) {
+#pragma unroll
+                            for (int i = 0; i < LNB; ++i) s[e].add(plane[i][e], y[i][e], own >> i & 1);
+                        }
+                        if (k > 0 || e > 0 || st > 0) v[e] = s[e].value();
+                    }
+                }
+            }
+            store_vals(X + BN_AT((H << B) + (l << VB), NV, full), v, !fwd);
+            if constexpr (kBases) {
+#pragma unroll
+                for (int e = 0; e < NV; ++e) mx = v[e] > mx ? v[e] : mx;
+            }
             if (g + 1 < g1) {                       // the next tile of the run
                 const uint32_t u = bits & (0u - bits), w = bits + u;
                 bits = w | (((w ^ bits) >> 2) >> (__ffs(u) - 1));
@@ -596,7 +690,7 @@ k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restric
                 // the one tile of the first level: its lanes' maximum
                 if (hw == 0) {
                     for (int o = LN / 2; o; o >>= 1) {
-                        const float y = __shfl_xor_sync(0xffffu, mx, o);
+                        const float y = __shfl_xor_sync(tmask, mx, o);
                         mx = y > mx ? y : mx;
                     }
                     if (l == 0) level_words_start(lw, lv, mx);
@@ -950,13 +1044,13 @@ cudaError_t launch_backward_rows(const Plan& P, const void* A, void* Rc, cudaStr
 // widest level has its own lanes.  Clusters (at most 8 blocks, the portable
 // size) serve the small jobs and every batch group; past kSweepGrid blocks
 // the whole GPU shares the two sweeps of a single job (err given).
-static int sweep_blocks(const Plan& P, const int* err)
+static int sweep_blocks(const Plan& P, uint64_t tiles, int per_sm, const int* err)
 {
     const int B = P.prec == 0 ? LB64 : LB;
-    const uint64_t widest = choose(P.n - B, (P.n - B) / 2), per = kSweepThreads >> B;
+    const uint64_t widest = choose(P.n - B, (P.n - B) / 2);
     // the whole-GPU form needs the counters beside the job's error word
-    const uint64_t most = err && widest > kSweepGrid * per ? 152 : 8;
-    return (int)std::max<uint64_t>(1, std::min<uint64_t>((widest + per - 1) / per, most));
+    const uint64_t most = err && widest > kSweepGrid * tiles ? 76 * per_sm : 8;
+    return (int)std::max<uint64_t>(1, std::min<uint64_t>((widest + tiles - 1) / tiles, most));
 }
 
 bool sweeps_fit(const Plan& P)
@@ -966,34 +1060,44 @@ bool sweeps_fit(const Plan& P)
 
 bool use_sweeps(const Plan& P, const int* err)
 {
-    return sweeps_fit(P) && P.n <= (P.lin ? kSweepMaxNX : kSweepMaxN) && err && !recording();
+    const int most = P.busy ? kSweepBusyN : P.lin ? kSweepMaxNX : kSweepMaxN;
+    return sweeps_fit(P) && P.n <= most && err && !recording();
 }
 
-template <typename T, bool TLO>
-static cudaError_t sweeps(const Plan& P, const T* A, T* F, T* Rc, int items, cudaStream_t s, int* err)
+template <typename T, bool TLO, int VB>
+static cudaError_t sweeps_vb(const Plan& P, const T* A, T* F, T* Rc, int items, cudaStream_t s, int* err)
 {
-    const int nb = sweep_blocks(P, err);
+    constexpr int B = sizeof(T) == 4 ? LB : LB64, threads = SweepShape<VB>::threads;
+    const int nb = sweep_blocks(P, threads >> (B - VB), SweepShape<VB>::blocks, err);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(items * nb), 1, 1);
-    cfg.blockDim = dim3(kSweepThreads, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     cfg.attrs = attr;
     cfg.numAttrs = nb > 1 ? 1 : 0;
     unsigned* sync = err ? reinterpret_cast<unsigned*>(err) + 16 : nullptr;
     if (nb == 1)
-        return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_BLOCK>, P.n, nb, A, F, Rc, P.js, sync, err, 0u);
+        return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_BLOCK, VB>, P.n, nb, A, F, Rc, P.js, sync, err, 0u);
     if (nb <= 8) {
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = nb;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
-        return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_CLUSTER>, P.n, nb, A, F, Rc, P.js, sync, err, 0u);
+        return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_CLUSTER, VB>, P.n, nb, A, F, Rc, P.js, sync, err, 0u);
     }
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
-    return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_GRID>, P.n, nb, A, F, Rc, P.js, sync, err,
+    return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_GRID, VB>, P.n, nb, A, F, Rc, P.js, sync, err,
                               kSweepSpinCap);
+}
+
+template <typename T, bool TLO>
+static cudaError_t sweeps(const Plan& P, const T* A, T* F, T* Rc, int items, cudaStream_t s, int* err)
+{
+    if constexpr (sizeof(T) == 4)
+        if (P.n >= kSweepVecN) return sweeps_vb<T, TLO, 2>(P, A, F, Rc, items, s, err);
+    return sweeps_vb<T, TLO, 0>(P, A, F, Rc, items, s, err);
 }
 
 cudaError_t launch_sweeps(const Plan& P, const void* A, void* F, void* Rc, cudaStream_t s, int* err,

@@ -2672,6 +2672,8 @@ void pump(bn_ctx* c)
         void* dev = nullptr;
         if (!rc) rc = dev_alloc(c, &dev, sj.bytes, sl.stream);
         if (!rc) {
+            // whether other jobs share the GPU (the same results either way)
+            sj.hj.P.busy = c->reserved > 0 || c->queue.size() > 1;
             Layout L = make_layout(P, 0);
             Bufs B{(char*)dev, L};
             rc = enqueue(sj.hj, B, B.at<double>(L.post), B.at<double>(L.logPD), sl.stream, &sl.ev,
