@@ -1225,7 +1225,7 @@ static cudaError_t edges(const Plan& P, int kid, int kid_tail, const double* log
     // (the linear forms have one of the two: X64 from n = 14, X64S below)
     if constexpr (!std::is_same<T, X64>::value) if (use_tail(P)) {
         // a thread per pair of values, at most 1024
-        const unsigned tb = rec_block((unsigned)std::min(1024, std::max(128, 1 << (P.n - 2))));
+        const unsigned tb = rec_block((unsigned)std::min(1024, std::max(128, (1 << (P.n - 1)) >> 1)));
         return launch_or_record(kid_tail, k_tail<T>, dim3(P.n, P.nj), tb, sizeof(T) << (P.n - 1), s, P.n, P.d, P.K,
                                 fixed_bits(P.K), (const T*)F, (const T*)Rc, (const T*)lq, logB, (const T*)lbs, cmax,
                                 masks, cmasks, (T*)Gam, err, post, log_PD, P.js, P.vsel);
