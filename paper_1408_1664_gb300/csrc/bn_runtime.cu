@@ -154,11 +154,16 @@ constexpr double kLogZero = -1e7;
 int log_weights(const double* src, size_t count, std::vector<double>& dst)
 {
     dst.assign(src, src + count);
+    // no early exit and integer comparisons for +inf and NaN: the compiler
+    // vectorises the loop
+    uint64_t bad = 0;
     for (double& x : dst) {
-        if (std::isnan(x) || x == INFINITY) return BN_EINVAL;
-        if (x < kLogZero) x = kLogZero;
+        uint64_t b;
+        std::memcpy(&b, &x, 8);
+        bad |= (uint64_t)(b - 0x7ff0000000000000ull < 0x0010000000000000ull) | (uint64_t)(b > 0xfff0000000000000ull);
+        x = x < kLogZero ? kLogZero : x;
     }
-    return BN_OK;
+    return bad ? BN_EINVAL : BN_OK;
 }
 
 // exp(x) of a natural log as an XValue (bn_device.cuh), and back (host).
@@ -217,6 +222,8 @@ double largest_log(const std::vector<double>& v)
 void plan_lin(HostJob& hj, double more)
 {
     Plan& P = hj.P;
+    P.lin = 0;
+    if (P.prec != 0) return;
     const double logs = largest_log(hj.log_rho) + largest_log(hj.log_q) + largest_log(hj.log_w) + more;
     P.lin = bn::lin_tiles_fit(P) ? bn::lin_range(P, hj.arity.data(), hj.ess, logs) : 0;
     if (P.hasw)
@@ -376,17 +383,49 @@ int upload_priors(const HostJob& hj, const Bufs& B, cudaStream_t s)
     return BN_OK;
 }
 
+// Host data up to this size goes through pinned staging.
+constexpr size_t kStageData = (size_t)512 << 10;
+// Bytes of the staging image of a job's inputs: the layout's data, small
+// tables and what lies between them.
+size_t stage_image(const Plan& P, const Layout& L)
+{
+    return (size_t)P.m * P.n <= kStageData ? L.lgT - L.data : 0;
+}
+
 // Enqueue steps 1-5 on stream s.  Small host arrays go through `stage`
-// (pinned, >= stage_bytes) when given, else through pageable copies.
+// (pinned, >= stage_bytes) when given, else through pageable copies.  With
+// stage_data (a caller that waits for the job before it uses `stage` again)
+// host data goes there too: data and tables in one copy.
 int enqueue(const HostJob& hj, const Bufs& B, double* post_dev, double* logPD_dev,
             cudaStream_t s, Events* ev, int* launches, char* stage, size_t stage_bytes,
-            bool upload_tables = true, const Side* side = nullptr)
+            bool upload_tables = true, const Side* side = nullptr, bool stage_data = false)
 {
     const Plan& P = hj.P;
     const Layout& L = B.L;
     if (ev) CK(cudaEventRecord(ev->ev[0], s));
     // inputs
     const uint8_t* data_dev = B.at<uint8_t>(L.data);
+    const size_t image = stage_image(P, L);
+    if (stage_data && !hj.data_on_device && image && stage_bytes >= image) {
+        auto at = [&](size_t off) { return stage + (off - L.data); };
+        if (P.m > 0) std::memcpy(stage, hj.data, (size_t)P.m * P.n);
+        if (upload_tables) {
+            std::memcpy(at(L.arity), hj.arity.data(), P.n);
+            double* lr = reinterpret_cast<double*>(at(L.log_rho));
+            double* dv = reinterpret_cast<double*>(at(L.Dvals));
+            double* al_ = reinterpret_cast<double*>(at(L.alpha));
+            for (int t = 0; t <= P.d; ++t) lr[t] = (size_t)t < hj.log_rho.size() ? hj.log_rho[t] : 0.0;
+            for (int q = 0; q < P.rows; ++q) {
+                dv[q] = hj.Dvals[q];
+                al_[q] = hj.ess / hj.Dvals[q];
+            }
+        }
+        const size_t bytes = upload_tables ? image : (size_t)P.m * P.n;
+        if (bytes) CK(cudaMemcpyAsync(B.at<char>(L.data), stage, bytes, cudaMemcpyHostToDevice, s));
+        const int rc = upload_priors(hj, B, s);
+        if (rc) return rc;
+        return enqueue_kernels(hj, B, data_dev, post_dev, logPD_dev, s, ev, launches, side);
+    }
     if (P.m > 0) {
         if (hj.data_on_device) {
             data_dev = hj.data;
@@ -617,6 +656,8 @@ struct bn_ctx {
     size_t spill_bytes = 0, spill_dev = 0;
     char* pin = nullptr;
     size_t pin_bytes = 0;
+    size_t pin_out = 0;          // a blocking call's results in it
+    bool pin_idle = true;        // no copy from or to it in flight
     static constexpr int kRing = 32;
     Events ring[kRing];
     int ring_pos = 0;            // next set to use
@@ -804,7 +845,7 @@ int ensure_spill(bn_ctx* c, size_t a_bytes, size_t dev_part, cudaStream_t s)
 }
 
 int run_direct(bn_ctx* c, const bn_job_desc* job, HostJob& hj, double* post_dev,
-               double* logPD_dev, cudaStream_t s)
+               double* logPD_dev, cudaStream_t s, bool blocking = false)
 {
     Layout L = make_layout(hj.P, 0);
     size_t a_bytes = 0, dev_part = 0;
@@ -829,8 +870,14 @@ int run_direct(bn_ctx* c, const bn_job_desc* job, HostJob& hj, double* post_dev,
         rc = ensure_spill(c, a_bytes, dev_part, s);
         if (rc) return rc;
     }
-    rc = ensure_pin(&c->pin, &c->pin_bytes, small_bytes(hj.P) + 64);
+    // pinned: the inputs' staging, then (a blocking call) the results
+    const size_t in_bytes = std::max(small_bytes(hj.P) + 64, blocking ? stage_image(hj.P, L) : 0);
+    const size_t out_bytes = blocking ? L.logPD - L.post + 8 + 8 : 0;
+    if (blocking && !c->pin_idle) CK(cudaStreamSynchronize(s));
+    rc = ensure_pin(&c->pin, &c->pin_bytes, al(in_bytes) + out_bytes);
     if (rc) return rc;
+    c->pin_out = al(in_bytes);
+    c->pin_idle = false;
     Events& ev = c->ring[c->ring_pos % bn_ctx::kRing];
     if (!ev.ok && (rc = ev.create())) return rc;
     Bufs B{c->ws, L, a_bytes ? c->spill : nullptr};
@@ -855,7 +902,7 @@ int run_direct(bn_ctx* c, const bn_job_desc* job, HostJob& hj, double* post_dev,
     c->tables_sig.clear();
     rc = enqueue(hj, B, post_dev ? post_dev : B.at<double>(L.post),
                  logPD_dev ? logPD_dev : B.at<double>(L.logPD), s, &ev, &c->last_launches,
-                 c->pin, c->pin_bytes, upload, &c->side);
+                 c->pin, al(in_bytes), upload, &c->side, blocking);
     if (rc == BN_OK) {
         c->tables_sig = sig;
         c->ring_pos = (c->ring_pos + 1) % bn_ctx::kRing;
@@ -1026,18 +1073,23 @@ try {
     int rc = validate_and_plan(job, hj);
     if (rc) return rc;
     if (cudaSetDevice(c->device) != cudaSuccess) return BN_ECUDA;
-    rc = run_direct(c, job, hj, nullptr, nullptr, c->stream);
+    rc = run_direct(c, job, hj, nullptr, nullptr, c->stream, true);
     if (rc) return rc;
     const Layout& L = c->last_layout;
     const Plan& P = hj.P;
-    int err = 0;
-    CK(cudaMemcpyAsync(post, c->ws + L.post, (size_t)P.n * P.n * 8, cudaMemcpyDeviceToHost, c->stream));
-    double lpd = 0;
-    CK(cudaMemcpyAsync(&lpd, c->ws + L.logPD, 8, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(&err, c->ws + L.err, 4, cudaMemcpyDeviceToHost, c->stream));
+    // posteriors and log P(D) lie together: one copy, and one of the error
+    // word, into pinned memory
+    char* out = c->pin + c->pin_out;
+    const size_t o_lpd = L.logPD - L.post;
+    CK(cudaMemcpyAsync(out, c->ws + L.post, o_lpd + 8, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(out + o_lpd + 8, c->ws + L.err, 4, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    c->pin_idle = true;
+    int err = 0;
+    std::memcpy(&err, out + o_lpd + 8, 4);
     if (err) return err_word_status(err);
-    if (log_PD) *log_PD = lpd;
+    std::memcpy(post, out, (size_t)P.n * P.n * 8);
+    if (log_PD) std::memcpy(log_PD, out + o_lpd, 8);
     Events& ev = c->ring[(c->ring_pos + bn_ctx::kRing - 1) % bn_ctx::kRing];
     fill_stats(P, ev, c->last_launches, &c->last_stats);
     return BN_OK;
@@ -2647,9 +2699,10 @@ void pump(bn_ctx* c)
         const Plan& P = sj.hj.P;
         cudaStreamSynchronize(sl.stream);
         int err = 0;
-        std::memcpy(&err, sl.pin + (size_t)P.n * P.n * 8 + 8, 4);
+        const size_t o_lpd = al((size_t)P.n * P.n * 8);     // as in the layout
+        std::memcpy(&err, sl.pin + o_lpd + 8, 4);
         sj.post.assign((double*)sl.pin, (double*)sl.pin + (size_t)P.n * P.n);
-        std::memcpy(&sj.logPD, sl.pin + (size_t)P.n * P.n * 8, 8);
+        std::memcpy(&sj.logPD, sl.pin + o_lpd, 8);
         fill_stats(P, sl.ev, sl.launches, &sj.stats);
         sj.rc = err ? err_word_status(err) : sj.rc;
         sj.state = Q_DONE;
@@ -2667,22 +2720,23 @@ void pump(bn_ctx* c)
         if (c->reserved + sj.bytes > c->budget) { ++it; continue; }
         Slot& sl = c->slots[free_slot];
         const Plan& P = sj.hj.P;
-        const size_t out_bytes = (size_t)P.n * P.n * 8 + 16;
-        int rc = ensure_pin(&sl.pin, &sl.pin_bytes, out_bytes + small_bytes(P) + 64);
+        const Layout L = make_layout(P, 0);
+        const size_t out_bytes = L.logPD - L.post + 16;     // posteriors, log P(D), error word
+        int rc = ensure_pin(&sl.pin, &sl.pin_bytes,
+                            al(out_bytes) + std::max(small_bytes(P) + 64, stage_image(P, L)));
         void* dev = nullptr;
         if (!rc) rc = dev_alloc(c, &dev, sj.bytes, sl.stream);
         if (!rc) {
             // whether other jobs share the GPU (the same results either way)
             sj.hj.P.busy = c->reserved > 0 || c->queue.size() > 1;
-            Layout L = make_layout(P, 0);
             Bufs B{(char*)dev, L};
             rc = enqueue(sj.hj, B, B.at<double>(L.post), B.at<double>(L.logPD), sl.stream, &sl.ev,
                          &sl.launches, sl.pin + al(out_bytes), sl.pin_bytes - al(out_bytes), true,
-                         &sl.side);
+                         &sl.side, true);
             if (!rc) {
-                if (cudaMemcpyAsync(sl.pin, B.at<char>(L.post), (size_t)P.n * P.n * 8, cudaMemcpyDeviceToHost, sl.stream) != cudaSuccess ||
-                    cudaMemcpyAsync(sl.pin + (size_t)P.n * P.n * 8, B.at<char>(L.logPD), 8, cudaMemcpyDeviceToHost, sl.stream) != cudaSuccess ||
-                    cudaMemcpyAsync(sl.pin + (size_t)P.n * P.n * 8 + 8, B.at<char>(L.err), 4, cudaMemcpyDeviceToHost, sl.stream) != cudaSuccess ||
+                const size_t o_lpd = L.logPD - L.post;
+                if (cudaMemcpyAsync(sl.pin, B.at<char>(L.post), o_lpd + 8, cudaMemcpyDeviceToHost, sl.stream) != cudaSuccess ||
+                    cudaMemcpyAsync(sl.pin + o_lpd + 8, B.at<char>(L.err), 4, cudaMemcpyDeviceToHost, sl.stream) != cudaSuccess ||
                     cudaEventRecord(sl.done, sl.stream) != cudaSuccess)
                     rc = BN_ECUDA;
             }
