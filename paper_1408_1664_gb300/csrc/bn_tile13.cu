@@ -1365,8 +1365,11 @@ k_gamma13_p1(int n, int d, uint32_t nlow, const T* __restrict__ F,
         const T M = ord_dec(tmax_s) + T(TB);
         T L = Lg::ninf();                           // relevance cut (see above)
         if (Aup) {
-            const T at = job_ptr(Aup, js)[BN_AT(((size_t)v << (n - 1)) + (((size_t)H << TB) | (TN - 1)), 1,
-                                                (size_t)n << (n - 1))];
+            T at = job_ptr(Aup, js)[BN_AT(((size_t)v << (n - 1)) + (((size_t)H << TB) | (TN - 1)), 1,
+                                          (size_t)n << (n - 1))];
+            // the bound is the sum of B_v: A_v without its factor q_v (a zero
+            // factor is held as -1e7 nats, where FP32 counts in units of 1)
+            if (Q) at += (sizeof(T) == 4 ? T(4) : T(1e-6)) - lq_s[__popc(H) + TB];
             // log P(D) in the units of s (FP32: relative to the integer Z)
             const T fv = kBases ? (T)fvrel_s : F[((size_t)1 << n) - 1];
             L = fv - margin - at;
@@ -1687,7 +1690,10 @@ k_g13_x(int n, int d, uint32_t nlow, const X64* __restrict__ F, const X64* __res
     if (Aup) {
         const X64 at = job_ptr(Aup, js)[BN_AT(((size_t)v << (n - 1)) + (((size_t)H << TB) | (TN - 1)), 1,
                                               (size_t)n << (n - 1))];
-        L = max(L, x_exp(F[((size_t)1 << n) - 1]) - x_exp(at) - 1 - margin);
+        // the bound is the sum of B_v: A_v without its factor q_v (unknown when
+        // that is zero)
+        const X64 q = Q ? lq[v * n + __popc(H) + TB] : x_one<X64>();
+        if (at.u && q.u) L = max(L, x_exp(F[((size_t)1 << n) - 1]) - x_exp(at) + x_exp(q) - 2 - margin);
     }
     // s of the full tile set, the smallest output, is a load of its own: the
     // first reference puts the smallest output that matters at 2^kXKeep, and
