@@ -416,6 +416,161 @@ k_gamma_p2(int n, int d, int b, int hc, uint32_t nlow, int64_t K, const T* __res
     }
 }
 
+// Phase 2 for the columns with at least two high elements left, a block per
+// endpoint and run of CPB consecutive columns: the 2^h values of each column
+// sit in shared memory (one column after another, the columns' starts four
+// banks apart), the downward steps run three dimensions at a time in registers
+// (eight values per thread) and the outputs with at most d - |g| high elements
+// go to their families.  A run of columns reads whole sectors of W's rows and
+// a step touches shared memory once per three dimensions; a block per column
+// with a step per dimension (k_gamma_p2, kept for columns past 64 KB) took
+// 2.15 ms at n = 25, d = 8.
+//
+// The steps are additions relative to one scale (an exponential per input, a
+// logarithm per output resolved), in one or a few passes like the tiles': a
+// pass resolves the outputs of at least 2^low in its scale, the next moves
+// down by the range.  A column's outputs lie between W at the full high set
+// and the largest input times 2^h, and those below L = log2 F(V) - margin -
+// log2 (sum of B_v) move no posterior (the cut of phase 1 with the largest
+// set): the passes end at max(W(full), L).  Columns that would take more than
+// kP2Passes passes sum logarithms instead.
+template <bool LIN>
+__device__ __forceinline__ void p2_steps(float* v, uint32_t H2, uint32_t HS, int h, int cpb)
+{
+    for (int j0 = 0; j0 < h; j0 += 3) {
+        const int nb = min(3, h - j0);
+        const uint32_t lowm = (1u << j0) - 1u;
+        const uint32_t np = H2 >> nb;
+        for (uint32_t g = threadIdx.x; g < np * cpb; g += blockDim.x) {
+            const uint32_t cc = g >> (h - nb), p = g & (np - 1u);
+            const uint32_t base = cc * HS + (((p & ~lowm) << nb) | (p & lowm));
+            float x[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q < (1 << nb)) x[q] = v[base + ((uint32_t)q << j0)];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                if (k >= nb) continue;
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (q < (1 << nb) && !(q >> k & 1)) {
+                        if constexpr (LIN) x[q] = x[q] + x[q | (1 << k)];
+                        else x[q] = p2_add(x[q], x[q | (1 << k)]);
+                    }
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q < (1 << nb)) v[base + ((uint32_t)q << j0)] = x[q];
+        }
+        __syncthreads();
+    }
+}
+
+__device__ __forceinline__ int p2_mag(float w) { return w > -2.0e9f ? (int)floorf(w) : -2000000000; }
+// Largest sum and smallest exact output of a pass, in bits above its
+// reference (Window<float> of bn_tile13.cu).
+constexpr int kP2Top = 126, kP2Low = -80;
+constexpr float kP2Keep = 8.271806125530277e-25f;  // 2^-80
+constexpr int kP2Passes = 4;
+
+template <int CPB>
+__global__ void __launch_bounds__(256)
+k_gamma_p2r(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const float* __restrict__ W,
+            float* __restrict__ Gam, const float* __restrict__ Aup, const float* __restrict__ lq, int margin, size_t js, uint32_t vsel)
+{
+    const int v = blockIdx.z;
+    if (!(vsel >> v & 1u)) return;
+    const int h = n - 1 - b;
+    const uint32_t H2 = 1u << h, HS = H2 + 4;
+    W = job_ptr(W, js) + ((size_t)endpoint_slot(vsel, v) << h) * nlow;
+    Gam = job_ptr(Gam, js) + (size_t)v * K;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* vals = reinterpret_cast<float*>(smem_raw);
+    __shared__ uint32_t hb[18][20];                 // C(b + bit, t)
+    __shared__ int mag_s[CPB], ref_s[CPB], span_s;
+    __shared__ uint32_t base_s[CPB], soff[20];
+    __shared__ int kg_s[CPB];
+    const int tid = threadIdx.x;
+    const uint32_t cb = blockIdx.x * CPB;
+    const int cols = min((uint32_t)CPB, c0 - cb);
+    for (int x = tid; x < 18 * 20; x += blockDim.x) hb[x / 20][x % 20] = binom(b + x / 20, x % 20);
+    if (tid < CPB) {
+        mag_s[tid] = -2000000000;
+        int kg = 0;
+        uint32_t r = cb + min(tid, cols - 1);
+        while (r >= binom(b, kg)) { r -= binom(b, kg); ++kg; }
+        kg_s[tid] = kg;
+        base_s[tid] = r;                            // its rank among the kg-subsets
+    }
+    if (tid < 20) {
+        uint32_t o = 0;
+        for (int s = 0; s < tid; ++s) o += binom(n - 1, s);
+        soff[tid] = o;
+    }
+    if (tid == 0) span_s = 0;
+    __syncthreads();
+    // blockDim.x is a multiple of CPB: a thread's column is fixed in these loops
+    const int mycol = tid % CPB;
+    const float* Wc = W + cb + min(mycol, cols - 1);
+    int mag = -2000000000;
+    for (uint32_t H = tid / CPB; H < H2; H += blockDim.x / CPB)
+        mag = max(mag, p2_mag(Wc[BN_AT((size_t)H * nlow, 1, (size_t)nlow << h)]));
+    atomicMax(&mag_s[mycol], mag);
+    __syncthreads();
+    if (tid < CPB) {
+        int L = -2000000000;
+        if (Aup) {
+            // log2 F(V), in [0, 1) relative to the integer Z, and the sum of B_v
+            // over all parent sets: A_v(V - {v}) without its factor q_v (a zero
+            // factor is held as -1.4e7, in units of 1)
+            const float at = job_ptr(Aup, js)[BN_AT(((size_t)(v + 1) << (n - 1)) - 1, 1, (size_t)n << (n - 1))];
+            const int av = p2_mag(at) - (lq ? p2_mag(lq[v * n + n - 1]) - 4 : 0);
+            L = -av - 2 - margin;
+        }
+        const int top = mag_s[tid] + h + 2;         // every output is below 2^top
+        const int low = max(L, p2_mag(Wc[BN_AT((size_t)(H2 - 1) * nlow, 1, (size_t)nlow << h)]));
+        ref_s[tid] = top - kP2Top;
+        atomicMax(&span_s, top - low);
+    }
+    __syncthreads();
+    constexpr int range = kP2Top - kP2Low;
+    const int span = span_s;
+    const int passes = span <= range ? 1 : span <= kP2Passes * range ? (span + range - 1) / range : 0;
+    unsigned long long done = 0ull;                 // bit i: the thread's i-th output is written
+    for (int pass = 0; pass < max(passes, 1); ++pass) {
+        const int down = pass * range;
+        const bool last = pass + 1 >= passes;
+        for (uint32_t H = tid / CPB; H < H2; H += blockDim.x / CPB) {
+            const float w = Wc[BN_AT((size_t)H * nlow, 1, (size_t)nlow << h)];
+            vals[mycol * HS + H] = passes ? ex2_approx(w - (float)(ref_s[mycol] - down)) : w;
+        }
+        __syncthreads();
+        if (passes) p2_steps<true>(vals, H2, HS, h, cols);
+        else p2_steps<false>(vals, H2, HS, h, cols);
+        int i = 0;
+        for (uint32_t e = tid; e < H2 * cols; e += blockDim.x, ++i) {
+            const uint32_t cc = e >> h, t = e & (H2 - 1u);
+            const int kg = kg_s[cc], k = kg + __popc(t);
+            if (k > d || (done >> (i & 63) & 1ull)) continue;
+            float o = vals[cc * HS + t];
+            if (passes) {
+                if (!last && o < kP2Keep) continue;
+                // a sum flushed in the last pass is irrelevant: kept finite
+                const int ref = ref_s[cc] - down;
+                o = fmaxf((float)ref + lg2_approx(o), (float)(ref - 126));
+                done |= 1ull << (i & 63);
+            }
+            // family index of g with the high part t: sizes below k, then the
+            // colex rank (the low part's, then one entry per high bit)
+            uint32_t f = base_s[cc] + soff[k];
+            int pos = kg + 1;
+            for (uint32_t x = t; x; x &= x - 1, ++pos) f += hb[__ffs(x) - 1][pos];
+            Gam[BN_AT(f, 1, K)] = o;
+        }
+        __syncthreads();                            // the values are reused
+    }
+}
+
 // Family index of the mask cm over the n-1 bits of V - {v}: by size, then
 // colexicographic rank (the canonical order of the scores).
 __device__ __forceinline__ uint32_t family_index(uint32_t cm, int n)
@@ -520,6 +675,134 @@ k_gamma_p2s(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const T*
         if (5 + q >= h) break;
         const T x = warp_lse(mb[q], sb[q]);
         if (lane == 0) Gam[BN_AT(family_index(g | (1u << (b + 5 + q)), n), 1, K)] = x;
+    }
+}
+
+// The same columns in FP32 for h >= 8, a block per eight consecutive columns.
+// A warp's load takes eight columns of four rows: four whole sectors, where a
+// lane per row touched 32 (the L1 was 96 % busy with them).  Lane 8 r + c takes
+// column c and the rows whose two lowest bits are r, warp w those whose three
+// highest bits are w; the bits between are the loop's, the same for the whole
+// warp, so eight rows at a time are summed over their three lowest loop bits
+// and enter the other sums as one term.  A lane's sums share one scale: one
+// exponential per row (one per sum before).  The scale lies 90 to 102 bits
+// below the lane's largest value, which uses the upper part of the exponent
+// range too: a sum 178 bits below the largest (2^-88 in its scale, where the
+// terms flushed are below 2^-108 together) is still exact, as strongly
+// dependent data need; one below that is formed again in logarithms by a warp.
+__global__ void __launch_bounds__(256)
+k_gamma_p2w(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const float* __restrict__ W,
+            float* __restrict__ Gam, size_t js, uint32_t vsel)
+{
+    constexpr int MB = 13;                          // loop bits (h <= 18)
+    using L = LogOps<float>;
+    const int v = blockIdx.z;
+    if (!(vsel >> v & 1u)) return;
+    W = job_ptr(W, js) + ((size_t)endpoint_slot(vsel, v) << (n - 1 - b)) * nlow;
+    Gam = job_ptr(Gam, js) + (size_t)v * K;
+    __shared__ float2 part[8][8][20];               // [warp][column][sum]: (scale, sum)
+    __shared__ uint32_t g_s[8];
+    __shared__ int redo_s[8];                       // per column: sums to form again
+    const int h = n - 1 - b, hi = h - 5;            // hi: loop bits, 2 .. h - 4
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = lane & 7, r = lane >> 3;
+    const uint32_t cb = c0 + blockIdx.x * 8;
+    const int cols = min(8u, nlow - cb);
+    const size_t wsize = (size_t)nlow << h;
+    if (threadIdx.x < 8) {
+        int kg = 0;
+        uint32_t x = cb + min((int)threadIdx.x, cols - 1);
+        while (x >= binom(b, kg)) { x -= binom(b, kg); ++kg; }
+        g_s[threadIdx.x] = colex_unrank(x, kg, b);
+        redo_s[threadIdx.x] = 0;
+    }
+    __syncthreads();
+    // the last column's values stand in for those past the end
+    const float* Wc = W + cb + min(c, cols - 1);
+    const uint32_t base = ((uint32_t)warp << (h - 3)) | (uint32_t)r;
+    float m = L::ninf(), s = 0.0f, sb[MB];
+#pragma unroll
+    for (int q = 0; q < MB; ++q) sb[q] = 0.0f;
+    for (uint32_t k = 0; k < (1u << hi); k += 8) {
+        float w[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) w[q] = Wc[BN_AT((size_t)(base + ((k + q) << 2)) * nlow, 1, wsize)];
+        float top = w[0];
+#pragma unroll
+        for (int q = 1; q < 8; ++q) top = fmaxf(top, w[q]);
+        if (top - m > 102.0f) {                     // +inf while empty
+            const float sc = L::ex(0.5f * (m - (top - 90.0f)));
+            s = s * sc * sc;
+#pragma unroll
+            for (int q = 0; q < MB; ++q) sb[q] = sb[q] * sc * sc;
+            m = top - 90.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) w[q] = L::ex(w[q] - m);
+        const float p1 = w[2] + w[3], p2 = w[4] + w[5], p3 = w[6] + w[7];
+        const float t = (w[0] + w[1]) + p1 + (p2 + p3);
+        s += t;
+        sb[0] += (w[1] + w[3]) + (w[5] + w[7]);
+        sb[1] += p1 + p3;
+        sb[2] += p2 + p3;
+#pragma unroll
+        for (int q = 3; q < MB; ++q)
+            if (k >> q & 1u) sb[q] += t;
+    }
+    // over the four row phases: the largest scale, every sum relative to it
+    float top = fmaxf(m, __shfl_xor_sync(FULL, m, 8));
+    top = fmaxf(top, __shfl_xor_sync(FULL, top, 16));
+    const float sc = L::ex(0.5f * (m - top));       // in halves: the sums are up to 2^102
+    s = s * sc * sc;
+    const float s1 = s + __shfl_xor_sync(FULL, s, 16);      // phases r and r ^ 2
+    const float s2 = s + __shfl_xor_sync(FULL, s, 8);       // phases r and r ^ 1
+    const float all = s1 + __shfl_xor_sync(FULL, s1, 8);
+    if (r == 3) {                                   // phases 1, 3 and 2, 3: bits 0 and 1
+        part[warp][c][0] = make_float2(top, all);
+        part[warp][c][1] = make_float2(top, s1);
+        part[warp][c][2] = make_float2(top, s2);
+    }
+#pragma unroll
+    for (int q = 0; q < MB; ++q) {
+        if (q >= hi) break;
+        float x = sb[q] * sc * sc;
+        x += __shfl_xor_sync(FULL, x, 16);
+        x += __shfl_xor_sync(FULL, x, 8);
+        if (r == 0) part[warp][c][3 + q] = make_float2(top, x);
+    }
+    __syncthreads();
+    // output o of column c: 0 every row, 1 + j the rows with high bit j
+    auto store = [&](int col, int o, float x) {
+        const uint32_t cm = g_s[col] | (o ? 1u << (b + o - 1) : 0u);
+        Gam[BN_AT(family_index(cm, n), 1, K)] = x;
+    };
+    for (int x = threadIdx.x; x < 8 * (h + 1); x += blockDim.x) {
+        const int col = x & 7, o = x >> 3;
+        if (col >= cols || (o && d - __popc(g_s[col]) != 1)) continue;
+        const int j = o - 1;                        // the high bit
+        const int at = j < h - 3 ? o : 0;           // warp bits: sums of the warps with the bit
+        float t = L::ninf();
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t = fmaxf(t, part[w][col][0].x);
+        float sum = 0.0f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const float2 p = part[w][col][at];
+            const float e = L::ex(0.5f * (p.x - t));
+            if (j < h - 3 || (w >> (j - (h - 3)) & 1)) sum += p.y * e * e;
+        }
+        if (sum > 3.2311742677852644e-27f) store(col, o, t + L::lg(sum));     // 2^-88
+        else atomicOr(&redo_s[col], 1 << o);
+    }
+    __syncthreads();
+    for (int x = warp; x < 8 * (h + 1); x += 8) {
+        const int col = x & 7, o = x >> 3;
+        if (!(redo_s[col] >> o & 1)) continue;
+        float mm = L::ninf(), ss = 0.0f;
+        for (uint32_t H = lane; H < (1u << h); H += 32)
+            if (H >> (o - 1) & 1u) lse_lazy_k(mm, ss, W[BN_AT((size_t)H * nlow + cb + col, 1, wsize)]);
+        const float y = warp_lse(mm, ss);
+        if (lane == 0) store(col, o, y);
     }
 }
 
@@ -1179,14 +1462,49 @@ int gamma_launches(const Plan& P)
     return 1 + (P.prec != 0 ? 1 : 0) + (c0 > 0 ? 1 : 0) + (c0 < P.nlow_g ? 1 : 0);
 }
 
-cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_t s)
+// Columns per block of k_gamma_p2r: 64 KB of values (at most 64 outputs per
+// thread), at most 8 columns; 0: k_gamma_p2.  Its full transform beats the
+// guarded one of k_gamma_p2 on short columns (h <= 9; n = 22, d = 8: phase 2
+// 0.73 -> 0.34 ms) and where most high parts are outputs (d >= 7; n = 25, d =
+// 8: 2.15 -> 1.87 ms), not on long columns with few outputs (n = 25, d = 6:
+// 0.54 against 0.56 ms).  FP32: the linear FP64 form gained nothing (n = 23).
+static int p2r_columns(const Plan& P)
+{
+    const int h = P.n - 1 - P.b_g;
+    if (P.prec == 0 || P.d > 18 || (h > 9 && P.d < 7)) return 0;
+    const size_t fit = (size_t)64 * 1024 / ((size_t)4 << h);
+    int c = 8;
+    while ((size_t)c > fit) c /= 2;
+    return c;
+}
+
+template <int CPB>
+static cudaError_t gamma_p2r(const Plan& P, int kid, uint32_t c0, const void* W, void* Gam, const void* A,
+                             const void* lq, cudaStream_t s)
+{
+    const int h = P.n - 1 - P.b_g;
+    // the K outputs of an endpoint move no posterior by more than 2^-24 together
+    const int margin = 24 + (int)std::ceil(std::log2((double)P.K));
+    return launch_or_record(kid, k_gamma_p2r<CPB>, dim3((c0 + CPB - 1) / CPB, P.nj, P.n), 256,
+                            (((size_t)1 << h) + 4) * CPB * sizeof(float), s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
+                            (const float*)W, (float*)Gam, (const float*)A, (const float*)lq, margin, P.js, P.vsel);
+}
+
+cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, const void* A, const void* lq,
+                            cudaStream_t s)
 {
     if (use_tail(P)) return cudaSuccess;
     const uint32_t c0 = gamma_p2_split(P);
     if (c0 > 0) {
+        const int cpb = p2r_columns(P);
+        cudaError_t e = cudaSuccess;
         const size_t sm2 = gamma_p2_smem_bytes(P);
         const dim3 grid(c0, P.nj, P.n);
-        if (P.lin)
+        if (cpb == 8) e = gamma_p2r<8>(P, KID_P2R8, c0, W, Gam, A, lq, s);
+        else if (cpb == 4) e = gamma_p2r<4>(P, KID_P2R4, c0, W, Gam, A, lq, s);
+        else if (cpb == 2) e = gamma_p2r<2>(P, KID_P2R2, c0, W, Gam, A, lq, s);
+        else if (cpb == 1) e = gamma_p2r<1>(P, KID_P2R1, c0, W, Gam, A, lq, s);
+        else if (P.lin)
             launch_or_record(KID_GAMMA_P2_X, k_gamma_p2<X64>, grid, 256, sm2, s, P.n, P.d, P.b_g, P.hc_g, P.nlow_g,
                              P.K, (const X64*)W, (X64*)Gam, P.js, P.vsel);
         else if (P.prec == 0)
@@ -1195,14 +1513,18 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_
         else
             launch_or_record(KID_GAMMA_P2_F, k_gamma_p2<float>, grid, 256, sm2, s, P.n, P.d, P.b_g, P.hc_g, P.nlow_g, P.K,
                                                      (const float*)W, (float*)Gam, P.js, P.vsel);
-        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     if (c0 < P.nlow_g) {
+        const int h2 = P.n - 1 - P.b_g;             // high bits
         const dim3 grid((P.nlow_g - c0 + 7) / 8, P.nj, P.n);
         if (P.lin)
             launch_or_record(KID_GAMMA_P2S_X, k_gamma_p2s_x<X64>, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
                              (const X64*)W, (X64*)Gam, P.js, P.vsel);
+        else if (P.prec != 0 && h2 >= 8)
+            launch_or_record(KID_GAMMA_P2W, k_gamma_p2w, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
+                             (const float*)W, (float*)Gam, P.js, P.vsel);
         else if (P.prec == 0)
             launch_or_record(KID_GAMMA_P2S_D, k_gamma_p2s<double>, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
                                                      (const double*)W, (double*)Gam, P.js, P.vsel);
@@ -1285,6 +1607,10 @@ cudaError_t set_kernel_attributes()
     SETA(k_gamma_p2<float>)
     SETA(k_upzeta_x)
     SETA(k_gamma_p2<X64>)
+    SETA(k_gamma_p2r<8>)
+    SETA(k_gamma_p2r<4>)
+    SETA(k_gamma_p2r<2>)
+    SETA(k_gamma_p2r<1>)
     SETA(k_tail<float>)
     SETA(k_tail<double>)
     SETA(k_tail<X64S>)

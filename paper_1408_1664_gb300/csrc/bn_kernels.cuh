@@ -38,7 +38,8 @@ enum KernelId : int32_t {
     KID_TAIL_F, KID_TAIL_D, KID_TAIL_XS,
     KID_SHIFT_X, KID_APPLY_Q_X, KID_ADD_FEATURE_X, KID_REORDER_X, KID_COLB4_X, KID_COLB2_X,
     KID_COLB1_X, KID_COLW_X, KID_UP13_X, KID_FROWS_X, KID_BROWS_X, KID_G13_X_Q, KID_G13_X,
-    KID_GAMMA_P2_X, KID_GAMMA_P2S_X, KID_EDGES_X, KID_COUNT
+    KID_GAMMA_P2_X, KID_GAMMA_P2S_X, KID_EDGES_X,
+    KID_P2R8, KID_P2R4, KID_P2R2, KID_P2R1, KID_GAMMA_P2W, KID_COUNT
 };
 
 // Arguments as one trivially copyable structure whose members have the
@@ -355,7 +356,8 @@ cudaError_t launch_backward(const Plan& P, const void* A, void* Rc, cudaStream_t
 cudaError_t launch_gamma_p1(const Plan& P, const void* F, const void* Rc, const uint16_t* rk13,
                             void* W, cudaStream_t s, const void* lq = nullptr,
                             const void* A = nullptr);
-cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, cudaStream_t s);
+cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, const void* A, const void* lq,
+                            cudaStream_t s);
 // FP32: the per-endpoint offsets of the down-zeta input (one small launch,
 // made by launch_gamma_p1 itself; stored after the level words of Rc).
 cudaError_t launch_gamma_table(const Plan& P, const void* F, const void* Rc, cudaStream_t s);

@@ -262,7 +262,7 @@ try {
         CKS(bn::launch_backward(P, base + o_A, base + o_Rc, s, nullptr));
     }
     CKS(bn::launch_gamma_p1(P, base + o_F, base + o_Rc, rk13, base + o_W, s, nullptr, base + o_A));
-    CKS(bn::launch_gamma_p2(P, base + o_W, base + o_G, s));
+    CKS(bn::launch_gamma_p2(P, base + o_W, base + o_G, base + o_A, nullptr, s));
     CKS(bn::launch_edges(P, logB, base + o_lbs, cmax, masks, cm, base + o_G, base + o_F, base + o_Rc, nullptr, err,
                          reinterpret_cast<unsigned long long*>(base + o_ea), post_dev,
                          log_PD_dev, s));

@@ -553,7 +553,8 @@ int enqueue_kernels(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, d
             CK(bn::launch_gamma_p1(Q, B.at<void>(L.F), B.at<void>(L.Rc), B.at<uint16_t>(L.rk13),
                                    B.at<void>(L.W), s, P.hasq ? B.at<void>(L.logq) : nullptr, B.A()));
             if (ev && v0 + P.vgroup >= P.n) CK(cudaEventRecord(ev->ev[5], s));
-            CK(bn::launch_gamma_p2(Q, B.at<void>(L.W), B.at<void>(L.Gam), s));
+            CK(bn::launch_gamma_p2(Q, B.at<void>(L.W), B.at<void>(L.Gam), B.A(),
+                                   P.hasq ? B.at<void>(L.logq) : nullptr, s));
             nl += bn::gamma_launches(Q);
         }
         if (ev) CK(cudaEventRecord(ev->ev[6], s));
@@ -561,7 +562,8 @@ int enqueue_kernels(const HostJob& hj, const Bufs& B, const uint8_t* data_dev, d
         CK(bn::launch_gamma_p1(P, B.at<void>(L.F), B.at<void>(L.Rc), B.at<uint16_t>(L.rk13),
                                B.at<void>(L.W), s, P.hasq ? B.at<void>(L.logq) : nullptr, B.A()));
         if (ev) CK(cudaEventRecord(ev->ev[5], s));
-        CK(bn::launch_gamma_p2(P, B.at<void>(L.W), B.at<void>(L.Gam), s));
+        CK(bn::launch_gamma_p2(P, B.at<void>(L.W), B.at<void>(L.Gam), B.A(),
+                                   P.hasq ? B.at<void>(L.logq) : nullptr, s));
         if (ev) CK(cudaEventRecord(ev->ev[6], s));
         nl += bn::gamma_launches(P);
     }
@@ -1514,7 +1516,7 @@ int enqueue_steps(const Plan& G, const Layout& L, char* base, cudaStream_t s, un
     if (stages & 8u) {
         CK(bn::launch_gamma_p1(G, at(L.F), at(L.Rc), reinterpret_cast<const uint16_t*>(at(L.rk13)),
                                at(L.W), s, nullptr, at(L.A)));
-        CK(bn::launch_gamma_p2(G, at(L.W), at(L.Gam), s));
+        CK(bn::launch_gamma_p2(G, at(L.W), at(L.Gam), at(L.A), nullptr, s));
     }
     if (stages & 16u)
         CK(bn::launch_edges(G, reinterpret_cast<const double*>(at(L.logB)), at(L.lbs),
@@ -2572,7 +2574,8 @@ try {
     CK(bn::launch_gamma_p1(P, B.at<void>(L.F), B.at<void>(L.Rc), B.at<uint16_t>(L.rk13),
                            B.at<void>(L.W), s, P.hasq ? B.at<void>(L.logq) : nullptr,
                            P.slab ? nullptr : B.at<void>(L.A)));
-    CK(bn::launch_gamma_p2(P, B.at<void>(L.W), B.at<void>(L.Gam), s));
+    CK(bn::launch_gamma_p2(P, B.at<void>(L.W), B.at<void>(L.Gam),
+                           P.slab ? nullptr : B.at<void>(L.A), P.hasq ? B.at<void>(L.logq) : nullptr, s));
     CK(bn::launch_edges(P, B.at<double>(L.logB), B.at<void>(L.lbs), B.at<double>(L.cmax), B.at<uint32_t>(L.masks),
                         B.at<uint32_t>(L.cmasks), B.at<void>(L.Gam), B.at<void>(L.F), B.at<void>(L.Rc),
                         P.hasq ? B.at<void>(L.logq) : nullptr, B.at<int>(L.err),

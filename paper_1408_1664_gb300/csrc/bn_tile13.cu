@@ -644,7 +644,7 @@ __device__ __forceinline__ void colb_steps(T* v, uint32_t H2, int h, int CPB)
         const uint32_t lowm = (1u << j0) - 1u;
         const uint32_t np = H2 >> nb;
         for (uint32_t g = threadIdx.x; g < np * CPB; g += blockDim.x) {
-            const uint32_t cc = g / np, p = g % np;
+            const uint32_t cc = g >> (h - nb), p = g & (np - 1u);
             const uint32_t base = cc * H2 + (((p & ~lowm) << nb) | (p & lowm));
             T x[8];
 #pragma unroll
@@ -770,7 +770,7 @@ k_upzeta13_colb(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
     __syncthreads();
     const bool lin = lin_s != 0;
     if (lin) {
-        for (uint32_t e = threadIdx.x; e < H2 * CPB; e += blockDim.x) v[e] = Lg::ex(v[e] - scale_s[e / H2]);
+        for (uint32_t e = threadIdx.x; e < H2 * CPB; e += blockDim.x) v[e] = Lg::ex(v[e] - scale_s[e >> hl]);
         __syncthreads();
         colb_steps<true>(v, H2, hl, CPB);
     } else {
@@ -1478,7 +1478,7 @@ __device__ __forceinline__ void colb_steps_x(X64* v, uint32_t H2, int h, int CPB
     for (int j = 0; j < h; ++j) {
         const uint32_t lowm = (1u << j) - 1u, np = H2 >> 1;
         for (uint32_t g = threadIdx.x; g < np * CPB; g += blockDim.x) {
-            const uint32_t cc = g / np, p = g % np;
+            const uint32_t cc = g >> (h - 1), p = g & (np - 1u);
             const uint32_t lo = cc * H2 + (((p & ~lowm) << 1) | (p & lowm)), hi = lo | (1u << j);
             v[hi] = x_add(v[hi], v[lo]);
         }
@@ -1582,7 +1582,7 @@ k_colb_x(int n, int d, int64_t K, const X64* __restrict__ tab, X64* __restrict__
     __syncthreads();
     const bool lin = lin_s != 0;
     if (lin) {
-        for (uint32_t e = threadIdx.x; e < H2 * CPB; e += blockDim.x) vd[e] = x_scaled(v[e], ref_s[e / H2]);
+        for (uint32_t e = threadIdx.x; e < H2 * CPB; e += blockDim.x) vd[e] = x_scaled(v[e], ref_s[e >> hl]);
         __syncthreads();
         colb_steps<true>(vd, H2, hl, CPB);
     } else {

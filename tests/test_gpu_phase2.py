@@ -1,5 +1,8 @@
-"""The down-zeta's relevance cut under an order prior with zero factors at
-large sets, against the oracle."""
+"""The down-zeta's second phase and its relevance cuts at their edges, FP32
+against the FP64 path (other kernels) within the FP32 tolerance of 1e-4: the
+wide column sums (from n = 22), the register transform of short and of many
+columns, strongly dependent data (sums hundreds of bits below their column's
+largest), and an order prior with zero factors at large sets."""
 import numpy as np
 import pytest
 
@@ -17,6 +20,28 @@ def ctx():
         pytest.skip("no CUDA device")
     with B.Context(0) as c:
         yield c
+
+
+def _both(ctx, data, arity, d, **kw):
+    p = {f: B.bn_edge_posteriors(ctx.h, B.Job(data, arity, d, precision=f, **kw))[0] for f in ("fp32", "fp64")}
+    assert np.all(np.isfinite(p["fp32"])) and np.all(np.isfinite(p["fp64"]))
+    np.testing.assert_allclose(p["fp32"], p["fp64"], atol=1e-4, rtol=0)
+
+
+@pytest.mark.parametrize("n,d", [(22, 0), (22, 1), (22, 3), (23, 2), (17, 8), (19, 7), (14, 3), (15, 14)])
+def test_fp32_against_fp64(ctx, n, d):
+    ds = datagen.random_dag_data(n, 300, 2, 3, 1.0, seed=300 + n)
+    _both(ctx, ds.data, ds.arity, d)
+
+
+@pytest.mark.parametrize("n,d", [(22, 2), (18, 4), (16, 8)])
+def test_strongly_dependent_data(ctx, n, d):
+    ds = datagen.random_dag_data(n, 2000, 2, 2, 1.0, seed=400 + n)
+    data = ds.data.copy()
+    data[:, n - 1] = data[:, 0]
+    data[:, n - 2] = data[:, 5]
+    data[:, 1] = data[:, 6]
+    _both(ctx, data, ds.arity, d)
 
 
 @pytest.mark.parametrize("n,size", [(15, 13), (15, 14), (16, 13), (14, 13)])
