@@ -635,38 +635,114 @@ k_upzeta13_cols(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
 // output; exact as in the tiles); otherwise every step is a log-sum-exp.
 // The blocks after those copy the columns from ncb on, whose sums have a
 // single row (the empty high set), a warp per tile.
-template <bool LIN, typename T>
-__device__ __forceinline__ void colb_steps(T* v, uint32_t H2, int h, int CPB)
+//
+// Value e = (column << hl) | H sits at colb_pos(e): bits 5..7 of e go into
+// the bank bits so that the steps over dims 0..2 (lanes differ in bits 3..7),
+// 3..5 (bits 0..2, 6, 7) and above (bits 0..4) have no bank conflict (8 and 4
+// lanes per bank without it; 64 bits: bits 4..6, over the 16 bank pairs of
+// half a warp), and the column goes there too: rows are read and outputs
+// written by lanes with the column fastest, 32 / CPB rows a request.  The map
+// is linear over XOR, so a thread finds its eight places with seven XORs.
+// A thread per row, 4 to 8 scattered columns each, was bound by its requests
+// of 32 sectors.  FP32 sums, us before -> after (the swizzle alone): n = 26
+// d = 4 305 -> 213 (264), n = 25 d = 6 1257 -> 612 (1126), d = 8 2945 -> 1353
+// (2627).  512 threads measured 573 and 1288 at d = 6 and 8, but 19 against 14
+// at n = 20 and 91 against 63 in FP64 at n = 23.
+constexpr int kColbThreads = 256;
+
+template <int BYTES, int CPB>
+__device__ __forceinline__ uint32_t colb_pos(uint32_t e, int hl)
 {
-    using Lg = LogOps<T>;
+    constexpr int lanes = BYTES == 4 ? 32 : 16;
+    const uint32_t p = e ^ ((e >> hl) * (lanes / CPB));
+    if constexpr (BYTES == 4) return p ^ ((e >> 5) & 7u) ^ (((e >> 6) & 3u) << 3);
+    else return p ^ ((e >> 4) & 7u) ^ (((e >> 6) & 1u) << 3);
+}
+
+// The upward zeta of CPB columns of 2^h values each, three dimensions at a
+// time; `first` maps a value as it is first read, `op` adds two (column last).
+template <int CPB, typename T, typename FIRST, typename OP>
+__device__ __forceinline__ void colb_steps(T* v, int h, FIRST first, OP op)
+{
     for (int j0 = 0; j0 < h; j0 += 3) {
         const int nb = min(3, h - j0);
         const uint32_t lowm = (1u << j0) - 1u;
-        const uint32_t np = H2 >> nb;
-        for (uint32_t g = threadIdx.x; g < np * CPB; g += blockDim.x) {
-            const uint32_t cc = g >> (h - nb), p = g & (np - 1u);
-            const uint32_t base = cc * H2 + (((p & ~lowm) << nb) | (p & lowm));
+        const uint32_t groups = (uint32_t)CPB << (h - nb);
+        const uint32_t s1 = colb_pos<sizeof(T), CPB>(1u << j0, h), s2 = colb_pos<sizeof(T), CPB>(2u << j0, h),
+                       s4 = colb_pos<sizeof(T), CPB>(4u << j0, h);
+        for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x) {
+            const uint32_t cc = g >> (h - nb);
+            const uint32_t base = colb_pos<sizeof(T), CPB>(((g & ~lowm) << nb) | (g & lowm), h);
             T x[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                if (q < (1 << nb)) x[q] = v[base + ((uint32_t)q << j0)];
+                if (q < (1 << nb)) x[q] = v[base ^ (q & 1 ? s1 : 0u) ^ (q & 2 ? s2 : 0u) ^ (q & 4 ? s4 : 0u)];
+            if (j0 == 0) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (q < (1 << nb)) x[q] = first(x[q], cc);
+            }
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 if (k >= nb) continue;
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
-                    if (q < (1 << nb) && (q >> k & 1)) x[q] = LIN ? x[q] + x[q ^ (1 << k)] : Lg::lse(x[q], x[q ^ (1 << k)]);
+                    if (q < (1 << nb) && (q >> k & 1)) x[q] = op(x[q], x[q ^ (1 << k)], cc);
             }
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                if (q < (1 << nb)) v[base + ((uint32_t)q << j0)] = x[q];
+                if (q < (1 << nb)) v[base ^ (q & 1 ? s1 : 0u) ^ (q & 2 ? s2 : 0u) ^ (q & 4 ? s4 : 0u)] = x[q];
         }
         __syncthreads();
     }
 }
 
+// The chunks of a column (hc > 0): a cluster's 2^hc blocks hold one chunk of
+// the top hc high bits each; the steps over those bits read the peers' values
+// for the same low bits H, in the butterflies' order (so the sums equal the
+// unchunked ones bit for bit).
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+template <typename T> __device__ __forceinline__ T peer_ld(const T* p, uint32_t rank)
+{
+    const uint32_t own = (uint32_t)__cvta_generic_to_shared(p);
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(own), "r"(rank));
+    if constexpr (sizeof(T) == 4) {
+        uint32_t u;
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(u) : "r"(at));
+        return __builtin_bit_cast(T, u);
+    } else {
+        unsigned long long u;
+        asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(u) : "r"(at));
+        return __builtin_bit_cast(T, u);
+    }
+}
+template <typename T, typename OP>
+__device__ __forceinline__ T chunk_sum(const T* p, uint32_t chunk, uint32_t cc, OP op)
+{
+    T x[8];
+#pragma unroll
+    for (uint32_t q = 0; q < 8; ++q)
+        if ((q & ~chunk) == 0) x[q] = peer_ld(p, q);
+#pragma unroll
+    for (uint32_t b = 0; b < 3; ++b) {
+        if (!(chunk >> b & 1)) continue;
+#pragma unroll
+        for (uint32_t q = 0; q < 8; ++q)
+            if ((q >> b & 1) && (q & ~chunk) == 0) x[q] = op(x[q], x[q ^ (1u << b)], cc);
+    }
+    T y = x[0];
+#pragma unroll
+    for (uint32_t q = 1; q < 8; ++q)
+        if (q == chunk) y = x[q];
+    return y;
+}
+
 template <typename T, int CPB>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kColbThreads)
 k_upzeta13_colb(int n, int d, int64_t K, const T* __restrict__ tab, T* __restrict__ A,
                 size_t js, int nodes, uint32_t ncb, int hc)
 {
@@ -677,14 +753,15 @@ k_upzeta13_colb(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
     __shared__ SBinom sb;
     __shared__ uint32_t off13[16];
     __shared__ uint32_t rowoff_k[32];
-    __shared__ T wred[8][CPB];                       // the warps' column maxima
+    __shared__ T wred[kColbThreads / 32][CPB];                       // the warps' column maxima
+    __shared__ T cmax_s[CPB], f0_s[CPB];             // a column's largest and H = {} value
     __shared__ T scale_s[CPB];                       // a column's linear scale
-    __shared__ int lin_s;
+    __shared__ int lin_s[CPB], all_lin;              // columns within one window
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* v = reinterpret_cast<T*>(smem_raw);           // [column of the run][H]
     const int h = n - 1 - TB;
-    // hc > 0: the top hc high bits are this block's chunk, fixed; the steps
-    // run over the other hl bits and k_upzeta13_colt adds the chunks after
+    // hc > 0: the top hc high bits are this block's chunk, fixed, and the
+    // block's rank in its cluster
     const int hl = h - hc;
     const uint32_t H2 = 1u << hl;
     const uint32_t ncol = num_small_subsets(TB, d);
@@ -718,122 +795,84 @@ k_upzeta13_colb(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
     const uint32_t c0 = ((blockIdx.x >> hc) % nrun) * CPB;
     const uint32_t Hc = chunk << hl;                 // the chunk's high bits
     const T* tb = tab + (size_t)i * K;
-    int kl[CPB];                                     // low elements of each column (-1: none)
-    T mx[CPB];
-#pragma unroll
-    for (int cc = 0; cc < CPB; ++cc) {
-        const uint32_t c = c0 + cc;
-        int k = 0;
-        while (k < TB && off13[k + 1] <= c) ++k;
-        kl[cc] = c < ncb ? k : -1;
-        mx[cc] = Lg::ninf();
-    }
-    for (uint32_t H = threadIdx.x; H < H2; H += blockDim.x) {
-        const uint32_t Hf = Hc | H;
-        const int kh = __popc(Hf);
-        uint32_t r = 0;                              // colex rank of Hf among kh-subsets
-        int t = 1;
-        for (uint32_t x = Hf; x; x &= x - 1, ++t) r += sb_binom(sb, __ffs(x) - 1, t);
-        // the row of G_H in the node's table (only formed where some column reads it)
-        const uint32_t row = kh <= d ? rowoff_k[kh] + r * off13[min(d - kh, TB) + 1] : 0u;
-#pragma unroll
-        for (int cc = 0; cc < CPB; ++cc) {
-            const bool in = kl[cc] >= 0 && kh <= d - kl[cc];
-            const T val = in ? tb[BN_AT(row + c0 + cc, 1, K)] : Lg::ninf();
-            v[cc * H2 + H] = val;
-            mx[cc] = val > mx[cc] ? val : mx[cc];
-        }
-    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int cc = 0; cc < CPB; ++cc) {
-        for (int o = 16; o; o >>= 1) {
-            const T y = __shfl_xor_sync(FULLMASK, mx[cc], o);
-            mx[cc] = y > mx[cc] ? y : mx[cc];
+    const uint32_t cc = lane & (CPB - 1), c = c0 + cc;   // this lane's column
+    int kl = 0;                                      // its low elements (-1: none)
+    while (kl < TB && off13[kl + 1] <= c) ++kl;
+    if (c >= ncb) kl = -1;
+    const int kl0 = __shfl_sync(FULLMASK, kl, 0);
+    T mx = Lg::ninf();
+    for (uint32_t Hb = warp * 32; Hb < H2; Hb += blockDim.x) {
+        const uint32_t Hf = Hc | Hb | lane;
+        const int kh = __popc(Hf);
+        uint32_t row = 0;                            // the row of G_H in the node's table
+        if (kh <= d - kl0) {                         // some column reads it
+            int t = 1;                               // colex rank of Hf among kh-subsets
+            for (uint32_t x = Hf; x; x &= x - 1, ++t) row += sb_binom(sb, __ffs(x) - 1, t);
+            row = rowoff_k[kh] + row * off13[min(d - kh, TB) + 1];
         }
-        if (lane == 0) wred[warp][cc] = mx[cc];
+#pragma unroll
+        for (int j = 0; j < CPB; ++j) {
+            const uint32_t src = j * (32 / CPB) + lane / CPB, H = Hb | src;
+            const uint32_t rj = __shfl_sync(FULLMASK, row, src);
+            const bool in = kl >= 0 && __popc(Hc | H) <= d - kl;
+            const T val = in ? tb[BN_AT(rj + c, 1, K)] : Lg::ninf();
+            v[colb_pos<sizeof(T), CPB>((cc << hl) | H, hl)] = val;
+            mx = val > mx ? val : mx;
+        }
     }
+    for (int o = 16; o >= CPB; o >>= 1) {
+        const T y = __shfl_xor_sync(FULLMASK, mx, o);
+        mx = y > mx ? y : mx;
+    }
+    if (lane < CPB) wred[warp][lane] = mx;
     __syncthreads();
+    if (threadIdx.x < CPB) {
+        T m = wred[0][threadIdx.x];
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = wred[w][threadIdx.x] > m ? wred[w][threadIdx.x] : m;
+        cmax_s[threadIdx.x] = m;
+        f0_s[threadIdx.x] = v[colb_pos<sizeof(T), CPB>(threadIdx.x << hl, hl)];
+    }
+    if (hc) cluster_sync();
+    else __syncthreads();
     if (threadIdx.x == 0) {
         // a column's outputs lie in [f(G_L), its largest input + log 2^h]
-        const T hb = sizeof(T) == 4 ? T(hl) : T(hl) * T(0.69314718055994530942);
-        int lin = 1;
-        for (int cc = 0; cc < CPB; ++cc) {
-            T m = wred[0][cc];
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = wred[w][cc] > m ? wred[w][cc] : m;
+        const T hb = sizeof(T) == 4 ? T(h) : T(h) * T(0.69314718055994530942);
+        int all = 1;
+        for (uint32_t q = 0; q < CPB; ++q) {
+            T m = cmax_s[q], f = f0_s[q];
+            if (hc) {
+                f = peer_ld(f0_s + q, 0);
+                for (uint32_t p = 0; p < (1u << hc); ++p) {
+                    const T x = peer_ld(cmax_s + q, p);
+                    m = x > m ? x : m;
+                }
+            }
             const T top = m + hb;
-            scale_s[cc] = top - Wn::top;
-            if (kl[cc] >= 0 && !(top - v[cc * H2] < Wn::win)) lin = 0;
+            scale_s[q] = top - Wn::top;
+            lin_s[q] = c0 + q >= ncb || top - f < Wn::win;
+            all &= lin_s[q];
         }
-        lin_s = lin;
+        all_lin = all;
     }
     __syncthreads();
-    const bool lin = lin_s != 0;
-    if (lin) {
-        for (uint32_t e = threadIdx.x; e < H2 * CPB; e += blockDim.x) v[e] = Lg::ex(v[e] - scale_s[e >> hl]);
-        __syncthreads();
-        colb_steps<true>(v, H2, hl, CPB);
-    } else {
-        colb_steps<false>(v, H2, hl, CPB);
-    }
+    if (all_lin)
+        colb_steps<CPB>(v, hl, [&](T x, uint32_t cc) { return Lg::ex(x - scale_s[cc]); },
+                   [](T a, T b, uint32_t) { return a + b; });
+    else
+        colb_steps<CPB>(v, hl, [&](T x, uint32_t cc) { return lin_s[cc] ? Lg::ex(x - scale_s[cc]) : x; },
+                   [&](T a, T b, uint32_t cc) { return lin_s[cc] ? a + b : Lg::lse(a, b); });
+    if (hc) cluster_sync();                          // the peers' steps are done
     T* Ai = A + ((size_t)i << (n - 1));
-    for (uint32_t H = threadIdx.x; H < H2; H += blockDim.x) {
-        T* o = Ai + BN_AT(((size_t)(Hc | H) << TB) + c0, CPB, (size_t)1 << (n - 1));
-        T y[CPB];
-#pragma unroll
-        for (int cc = 0; cc < CPB; ++cc) {
-            const T x = v[cc * H2 + H];
-            y[cc] = lin ? scale_s[cc] + Lg::lg(x) : x;
+    if (c < ncb) {
+        for (uint32_t H = warp * (32 / CPB) + lane / CPB; H < H2; H += (32 / CPB) * (blockDim.x >> 5)) {
+            const T* at = v + colb_pos<sizeof(T), CPB>((cc << hl) | H, hl);
+            const T x = hc ? chunk_sum(at, chunk, cc, [&](T a, T b, uint32_t q) { return lin_s[q] ? a + b : Lg::lse(a, b); })
+                           : *at;
+            Ai[BN_AT(((size_t)(Hc | H) << TB) + c, 1, (size_t)1 << (n - 1))] = lin_s[cc] ? scale_s[cc] + Lg::lg(x) : x;
         }
-        if constexpr (sizeof(T) == 4 && CPB == 4) {
-            if (c0 + 4 <= ncb) {
-                *reinterpret_cast<float4*>(o) = make_float4(y[0], y[1], y[2], y[3]);
-                continue;
-            }
-        }
-#pragma unroll
-        for (int cc = 0; cc < CPB; ++cc)
-            if (c0 + cc < ncb) o[cc] = y[cc];
     }
-}
-
-// The chunks of the column butterflies (k_upzeta13_colb with hc > 0): slot c
-// of tile (i, (q << hl) | L) holds the sum over the rows inside chunk q
-// alone; the upward zeta over the hc chunk bits, a thread per (i, L, c) with
-// c fastest (coalesced), leaves the full column sums.
-__device__ __forceinline__ float sum_of(float a, float b) { return LogOps<float>::lse(a, b); }
-__device__ __forceinline__ double sum_of(double a, double b) { return LogOps<double>::lse(a, b); }
-__device__ __forceinline__ X64 sum_of(X64 a, X64 b) { return x_add(a, b); }
-
-template <typename T>
-__global__ void __launch_bounds__(256)
-k_upzeta13_colt(int n, T* __restrict__ A, int nodes, uint32_t ncb, int hc)
-{
-    const int h = n - 1 - TB, hl = h - hc;
-    const uint64_t total = ((uint64_t)nodes << hl) * ncb;
-    const size_t asize = (size_t)nodes << (n - 1);
-    for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < total;
-         x += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t c = (uint32_t)(x % ncb);
-        const uint64_t y = x / ncb;
-        const uint32_t L = (uint32_t)(y & ((1u << hl) - 1u));
-        const int i = (int)(y >> hl);
-        T* Ai = A + ((size_t)i << (n - 1));
-        T q[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (k < (1 << hc)) q[k] = Ai[BN_AT((((size_t)k << hl) | L) << TB | c, 1, asize)];
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            if (b >= hc) continue;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (k < (1 << hc) && (k >> b & 1)) q[k] = sum_of(q[k], q[k ^ (1 << b)]);
-        }
-#pragma unroll
-        for (int k = 1; k < 8; ++k)
-            if (k < (1 << hc)) Ai[BN_AT((((size_t)k << hl) | L) << TB | c, 1, asize)] = q[k];
-    }
+    if (hc) cluster_sync();                          // no peer reads this block's values any more
 }
 
 template <typename T>
@@ -1473,21 +1512,8 @@ __device__ __forceinline__ int block_max(int e, int* red, int t)
 }
 
 // Column sums by butterflies over the high dimensions (k_upzeta13_colb).
-__device__ __forceinline__ void colb_steps_x(X64* v, uint32_t H2, int h, int CPB)
-{
-    for (int j = 0; j < h; ++j) {
-        const uint32_t lowm = (1u << j) - 1u, np = H2 >> 1;
-        for (uint32_t g = threadIdx.x; g < np * CPB; g += blockDim.x) {
-            const uint32_t cc = g >> (h - 1), p = g & (np - 1u);
-            const uint32_t lo = cc * H2 + (((p & ~lowm) << 1) | (p & lowm)), hi = lo | (1u << j);
-            v[hi] = x_add(v[hi], v[lo]);
-        }
-        __syncthreads();
-    }
-}
-
 template <int CPB>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kColbThreads)
 k_colb_x(int n, int d, int64_t K, const X64* __restrict__ tab, X64* __restrict__ A, size_t js, int nodes,
          uint32_t ncb, int hc)
 {
@@ -1496,12 +1522,12 @@ k_colb_x(int n, int d, int64_t K, const X64* __restrict__ tab, X64* __restrict__
     __shared__ SBinom sb;
     __shared__ uint32_t off13[16];
     __shared__ uint32_t rowoff_k[32];
-    __shared__ int wred[8][CPB];                     // the warps' column maxima (exponents)
+    __shared__ int wred[kColbThreads / 32][CPB];                     // the warps' column maxima (exponents)
+    __shared__ int cmax_s[CPB], f0_s[CPB];
     __shared__ int ref_s[CPB];                       // a column's reference exponent
-    __shared__ int lin_s;
+    __shared__ int lin_s[CPB], all_lin;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    X64* v = reinterpret_cast<X64*>(smem_raw);       // [column of the run][H]
-    double* vd = reinterpret_cast<double*>(smem_raw);
+    X64* v = reinterpret_cast<X64*>(smem_raw);       // [column of the run][H]; doubles while linear
     const int h = n - 1 - TB;
     const int hl = h - hc;                           // hc: chunk bits (see k_upzeta13_colb)
     const uint32_t H2 = 1u << hl;
@@ -1536,65 +1562,87 @@ k_colb_x(int n, int d, int64_t K, const X64* __restrict__ tab, X64* __restrict__
     const uint32_t c0 = ((blockIdx.x >> hc) % nrun) * CPB;
     const uint32_t Hc = chunk << hl;
     const X64* tb = tab + (size_t)i * K;
-    int kl[CPB], mx[CPB];
-#pragma unroll
-    for (int cc = 0; cc < CPB; ++cc) {
-        const uint32_t c = c0 + cc;
-        int k = 0;
-        while (k < TB && off13[k + 1] <= c) ++k;
-        kl[cc] = c < ncb ? k : -1;
-        mx[cc] = -kXBias;
-    }
-    for (uint32_t H = threadIdx.x; H < H2; H += blockDim.x) {
-        const uint32_t Hf = Hc | H;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t cc = lane & (CPB - 1), c = c0 + cc;   // this lane's column
+    int kl = 0;                                      // its low elements (-1: none)
+    while (kl < TB && off13[kl + 1] <= c) ++kl;
+    if (c >= ncb) kl = -1;
+    const int kl0 = __shfl_sync(FULLMASK, kl, 0);
+    int mx = -kXBias;
+    for (uint32_t Hb = warp * 32; Hb < H2; Hb += blockDim.x) {
+        const uint32_t Hf = Hc | Hb | lane;
         const int kh = __popc(Hf);
-        uint32_t r = 0;
-        int t = 1;
-        for (uint32_t x = Hf; x; x &= x - 1, ++t) r += sb_binom(sb, __ffs(x) - 1, t);
-        const uint32_t row = kh <= d ? rowoff_k[kh] + r * off13[min(d - kh, TB) + 1] : 0u;
+        uint32_t row = 0;                            // the row of G_H in the node's table
+        if (kh <= d - kl0) {                         // some column reads it
+            int t = 1;                               // colex rank of Hf among kh-subsets
+            for (uint32_t x = Hf; x; x &= x - 1, ++t) row += sb_binom(sb, __ffs(x) - 1, t);
+            row = rowoff_k[kh] + row * off13[min(d - kh, TB) + 1];
+        }
 #pragma unroll
-        for (int cc = 0; cc < CPB; ++cc) {
-            const bool in = kl[cc] >= 0 && kh <= d - kl[cc];
-            const X64 val = in ? tb[BN_AT(row + c0 + cc, 1, K)] : X64{0ull};
-            v[cc * H2 + H] = val;
-            mx[cc] = max(mx[cc], x_exp(val));
+        for (int j = 0; j < CPB; ++j) {
+            const uint32_t src = j * (32 / CPB) + lane / CPB, H = Hb | src;
+            const uint32_t rj = __shfl_sync(FULLMASK, row, src);
+            const bool in = kl >= 0 && __popc(Hc | H) <= d - kl;
+            const X64 val = in ? tb[BN_AT(rj + c, 1, K)] : X64{0ull};
+            v[colb_pos<8, CPB>((cc << hl) | H, hl)] = val;
+            mx = max(mx, x_exp(val));
         }
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int cc = 0; cc < CPB; ++cc) {
-        mx[cc] = __reduce_max_sync(FULLMASK, mx[cc]);
-        if (lane == 0) wred[warp][cc] = mx[cc];
+    for (int o = 16; o >= CPB; o >>= 1) {
+        mx = max(mx, __shfl_xor_sync(FULLMASK, mx, o));
     }
+    if (lane < CPB) wred[warp][lane] = mx;
     __syncthreads();
+    if (threadIdx.x < CPB) {
+        int m = wred[0][threadIdx.x];
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max(m, wred[w][threadIdx.x]);
+        cmax_s[threadIdx.x] = m;
+        f0_s[threadIdx.x] = x_exp(v[colb_pos<8, CPB>(threadIdx.x << hl, hl)]);
+    }
+    if (hc) cluster_sync();
+    else __syncthreads();
     if (threadIdx.x == 0) {
         // a column's outputs lie between its H = {} value and its largest
         // input times 2^h: one pass when both fit
-        int lin = 1;
-        for (int cc = 0; cc < CPB; ++cc) {
-            int m = wred[0][cc];
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max(m, wred[w][cc]);
-            ref_s[cc] = m + hl + 1 - kXTop;
-            if (kl[cc] >= 0 && x_exp(v[cc * H2]) - ref_s[cc] < kXKeep) lin = 0;
+        int all = 1;
+        for (uint32_t q = 0; q < CPB; ++q) {
+            int m = cmax_s[q];
+            int f = f0_s[q];
+            if (hc) {
+                f = peer_ld(f0_s + q, 0);
+                for (uint32_t p = 0; p < (1u << hc); ++p) m = max(m, peer_ld(cmax_s + q, p));
+            }
+            ref_s[q] = m + h + 1 - kXTop;
+            lin_s[q] = c0 + q >= ncb || f - ref_s[q] >= kXKeep;
+            all &= lin_s[q];
         }
-        lin_s = lin;
+        all_lin = all;
     }
     __syncthreads();
-    const bool lin = lin_s != 0;
-    if (lin) {
-        for (uint32_t e = threadIdx.x; e < H2 * CPB; e += blockDim.x) vd[e] = x_scaled(v[e], ref_s[e >> hl]);
-        __syncthreads();
-        colb_steps<true>(vd, H2, hl, CPB);
-    } else {
-        colb_steps_x(v, H2, hl, CPB);
-    }
+    const auto scaled = [&](X64 x, uint32_t cc) {
+        return lin_s[cc] ? X64{(uint64_t)__double_as_longlong(x_scaled(x, ref_s[cc]))} : x;
+    };
+    const auto plus = [](X64 a, X64 b) {
+        return X64{(uint64_t)__double_as_longlong(__longlong_as_double((long long)a.u) +
+                                                  __longlong_as_double((long long)b.u))};
+    };
+    if (all_lin)
+        colb_steps<CPB>(v, hl, scaled, [&](X64 a, X64 b, uint32_t) { return plus(a, b); });
+    else
+        colb_steps<CPB>(v, hl, scaled, [&](X64 a, X64 b, uint32_t cc) { return lin_s[cc] ? plus(a, b) : x_add(a, b); });
+    if (hc) cluster_sync();                          // the peers' steps are done
     X64* Ai = A + ((size_t)i << (n - 1));
-    for (uint32_t H = threadIdx.x; H < H2; H += blockDim.x) {
-        X64* o = Ai + BN_AT(((size_t)(Hc | H) << TB) + c0, CPB, (size_t)1 << (n - 1));
-#pragma unroll
-        for (int cc = 0; cc < CPB; ++cc)
-            if (c0 + cc < ncb) o[cc] = lin ? x_pack<X64>(vd[cc * H2 + H], ref_s[cc]) : v[cc * H2 + H];
+    if (c < ncb) {
+        for (uint32_t H = warp * (32 / CPB) + lane / CPB; H < H2; H += (32 / CPB) * (blockDim.x >> 5)) {
+            const X64* at = v + colb_pos<8, CPB>((cc << hl) | H, hl);
+            const X64 x = hc ? chunk_sum(at, chunk, cc, [&](X64 a, X64 b, uint32_t q) {
+                return lin_s[q] ? plus(a, b) : x_add(a, b);
+            }) : *at;
+            Ai[BN_AT(((size_t)(Hc | H) << TB) + c, 1, (size_t)1 << (n - 1))] =
+                lin_s[cc] ? x_pack<X64>(__longlong_as_double((long long)x.u), ref_s[cc]) : x;
+        }
     }
+    if (hc) cluster_sync();                          // no peer reads this block's values any more
 }
 
 // Up-zeta tile (k_upzeta13): the tile's column sums are staged in shared
@@ -1797,16 +1845,19 @@ static uint32_t colb_columns(const Plan& P)
     return (uint32_t)c;
 }
 
-// High bits beyond one 128 KB column in shared memory: the column
-// butterflies then run per chunk of those bits, added by k_upzeta13_colt
-// (single jobs launched directly, with A in device memory, only; 4 for the
-// others, which then keep the per-tile sums).
+// High bits whose chunks of a column lie in the blocks of a cluster: beyond
+// h = 12, so that a block holds 4 columns (FP32; 2 in FP64) in 64 KB and three
+// share an SM; at most 3 bits, the 8 blocks of a portable cluster.  Recorded
+// launches have no clusters: a block holds whole columns of up to 128 KB
+// there (4, more than is taken, past that).  n = 29 (h = 15), FP32: one
+// column of 128 KB a block 13.4 ms, chunks in clusters of 8 blocks 4.9 ms.
 static int colb_chunk_bits(const Plan& P)
 {
     const int h = P.n - 1 - TB;
     const int hmax = P.prec == 0 ? 14 : 15;          // 2^h values of 8 or 4 bytes in 128 KB
-    if (h <= hmax) return 0;
-    return recording() || P.nj != 1 || P.spill ? 4 : h - hmax;
+    if (recording() || (P.spill && h > hmax)) return h <= hmax ? 0 : 4;
+    const int hc = std::min(3, std::max(0, h - 12));
+    return h - hc <= hmax ? hc : 4;
 }
 
 // Column sums by butterflies over the h high dimensions when they take at
@@ -1924,6 +1975,31 @@ bool lin_tiles_fit(const Plan& P)
     return colw_fits(P) && up13_x_smem(P) <= 220 * 1024;
 }
 
+// A column-sum launch: plain (or recorded), or in clusters of 2^hc blocks.
+struct ColbLaunch {
+    dim3 grid;
+    unsigned threads;
+    size_t smem;
+    int hc;
+    cudaStream_t s;
+    template <typename... P, typename... A> cudaError_t operator()(int kid, void (*k)(P...), A... a) const
+    {
+        if (!hc) return launch_or_record(kid, k, grid, threads, smem, s, a...);
+        cudaLaunchAttribute attr = {};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 1u << hc;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, k, static_cast<P>(a)...);
+    }
+};
+
 cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unrank13, void* A,
                             cudaStream_t s, cudaEvent_t sums_done, int* err)
 {
@@ -1934,66 +2010,42 @@ cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unra
     uint64_t nrow = 0;
     for (int k = 0; k <= P.d && k <= h; ++k) nrow += binom_host(h, k);
     if (use_colb(P)) {                                // butterflies over the high dims
-        // columns per block: as many as fit 64 KB, at most 8 (FP32) or 4 (FP64)
+        // columns per block: as many chunks as fit 64 KB, at most 8 (FP32) or
+        // 4 (FP64), one where a chunk is 128 KB
         const size_t es = P.prec == 0 ? 8 : 4;
-        // (one column of up to 128 KB from h = 14 in FP32, 13 in FP64)
-        const int cpb = (int)std::max<size_t>(1, std::min<size_t>((size_t)(64 * 1024) / (es << h), P.prec == 0 ? 4 : 8));
+        const int hc = colb_chunk_bits(P);
+        const int cpb = (int)std::max<size_t>(1, std::min<size_t>((size_t)(64 * 1024) / (es << (h - hc)), P.prec == 0 ? 4 : 8));
         uint64_t ncol = 0;
         for (int k = 0; k <= P.d && k <= TB; ++k) ncol += binom_host(TB, k);
         const uint32_t ncb = colb_columns(P);
         const uint64_t ntiles = (uint64_t)nodes << h;
         // the copy blocks follow the butterfly blocks (none when the tile
-        // kernel stages those columns from the table itself)
+        // kernel stages those columns from the table itself), in whole clusters
         const bool copies = ncb < ncol && !upzeta_table_copies(P, tab, err);
-        const int hc = colb_chunk_bits(P);
-        const unsigned nblk = (unsigned)(((uint64_t)nodes * ((ncb + cpb - 1) / cpb) << hc) +
-                                         (copies ? (ntiles + 7) / 8 : 0));
+        const unsigned threads = rec_block(kColbThreads), wpb = threads / 32;
+        const unsigned ncopy = copies ? (unsigned)(((ntiles + wpb - 1) / wpb + ((1u << hc) - 1)) >> hc << hc) : 0;
+        const unsigned nblk = (unsigned)((uint64_t)nodes * ((ncb + cpb - 1) / cpb) << hc) + ncopy;
         const size_t smb = ((size_t)cpb << (h - hc)) * es;
-        const dim3 gb(nblk, P.nj);
+        const ColbLaunch L{dim3(nblk, P.nj), threads, smb, hc, s};
         if (P.lin) {
-            if (cpb >= 4)
-                launch_or_record(KID_COLB4_X, k_colb_x<4>, gb, 256, smb, s, P.n, P.d, P.K, (const X64*)tab,
-                                 (X64*)A, P.js, nodes, ncb, hc);
-            else if (cpb == 2)
-                launch_or_record(KID_COLB2_X, k_colb_x<2>, gb, 256, smb, s, P.n, P.d, P.K, (const X64*)tab,
-                                 (X64*)A, P.js, nodes, ncb, hc);
-            else
-                launch_or_record(KID_COLB1_X, k_colb_x<1>, gb, 256, smb, s, P.n, P.d, P.K, (const X64*)tab,
-                                 (X64*)A, P.js, nodes, ncb, hc);
+            const X64* tx = (const X64*)tab;
+            X64* Ax = (X64*)A;
+            if (cpb >= 4) L(KID_COLB4_X, k_colb_x<4>, P.n, P.d, P.K, tx, Ax, P.js, nodes, ncb, hc);
+            else if (cpb == 2) L(KID_COLB2_X, k_colb_x<2>, P.n, P.d, P.K, tx, Ax, P.js, nodes, ncb, hc);
+            else L(KID_COLB1_X, k_colb_x<1>, P.n, P.d, P.K, tx, Ax, P.js, nodes, ncb, hc);
         } else if (P.prec == 0) {
-            if (cpb >= 4)
-                launch_or_record(KID_COLB4_D, k_upzeta13_colb<double, 4>, gb, 256, smb, s, P.n, P.d, P.K,
-                                 (const double*)tab, (double*)A, P.js, nodes, ncb, hc);
-            else if (cpb == 2)
-                launch_or_record(KID_COLB2_D, k_upzeta13_colb<double, 2>, gb, 256, smb, s, P.n, P.d, P.K,
-                                 (const double*)tab, (double*)A, P.js, nodes, ncb, hc);
-            else
-                launch_or_record(KID_COLB1_D, k_upzeta13_colb<double, 1>, gb, 256, smb, s, P.n, P.d, P.K,
-                                 (const double*)tab, (double*)A, P.js, nodes, ncb, hc);
-        } else if (cpb == 8) {
-            launch_or_record(KID_COLB8, k_upzeta13_colb<float, 8>, gb, 256, smb, s, P.n, P.d, P.K,
-                             (const float*)tab, (float*)A, P.js, nodes, ncb, hc);
-        } else if (cpb >= 4) {
-            launch_or_record(KID_COLB4, k_upzeta13_colb<float, 4>, gb, 256, smb, s, P.n, P.d, P.K,
-                             (const float*)tab, (float*)A, P.js, nodes, ncb, hc);
-        } else if (cpb == 2) {
-            launch_or_record(KID_COLB2, k_upzeta13_colb<float, 2>, gb, 256, smb, s, P.n, P.d, P.K,
-                             (const float*)tab, (float*)A, P.js, nodes, ncb, hc);
+            const double* td = (const double*)tab;
+            double* Ad = (double*)A;
+            if (cpb >= 4) L(KID_COLB4_D, k_upzeta13_colb<double, 4>, P.n, P.d, P.K, td, Ad, P.js, nodes, ncb, hc);
+            else if (cpb == 2) L(KID_COLB2_D, k_upzeta13_colb<double, 2>, P.n, P.d, P.K, td, Ad, P.js, nodes, ncb, hc);
+            else L(KID_COLB1_D, k_upzeta13_colb<double, 1>, P.n, P.d, P.K, td, Ad, P.js, nodes, ncb, hc);
         } else {
-            launch_or_record(KID_COLB1, k_upzeta13_colb<float, 1>, gb, 256, smb, s, P.n, P.d, P.K,
-                             (const float*)tab, (float*)A, P.js, nodes, ncb, hc);
-        }
-        if (hc > 0) {                                 // add the chunks (never recorded)
-            const cudaError_t ec = cudaGetLastError();
-            if (ec != cudaSuccess) return ec;
-            const uint64_t total = ((uint64_t)nodes << (h - hc)) * ncb;
-            const unsigned gt = (unsigned)std::min<uint64_t>((total + 255) / 256, 152 * 64);
-            if (P.lin)
-                k_upzeta13_colt<X64><<<gt, 256, 0, s>>>(P.n, (X64*)A, nodes, ncb, hc);
-            else if (P.prec == 0)
-                k_upzeta13_colt<double><<<gt, 256, 0, s>>>(P.n, (double*)A, nodes, ncb, hc);
-            else
-                k_upzeta13_colt<float><<<gt, 256, 0, s>>>(P.n, (float*)A, nodes, ncb, hc);
+            const float* tf = (const float*)tab;
+            float* Af = (float*)A;
+            if (cpb == 8) L(KID_COLB8, k_upzeta13_colb<float, 8>, P.n, P.d, P.K, tf, Af, P.js, nodes, ncb, hc);
+            else if (cpb >= 4) L(KID_COLB4, k_upzeta13_colb<float, 4>, P.n, P.d, P.K, tf, Af, P.js, nodes, ncb, hc);
+            else if (cpb == 2) L(KID_COLB2, k_upzeta13_colb<float, 2>, P.n, P.d, P.K, tf, Af, P.js, nodes, ncb, hc);
+            else L(KID_COLB1, k_upzeta13_colb<float, 1>, P.n, P.d, P.K, tf, Af, P.js, nodes, ncb, hc);
         }
     } else if (colw_fits(P)) {                        // warp per tile, 8 tiles per block
         const uint64_t ntiles = (uint64_t)nodes << h;
