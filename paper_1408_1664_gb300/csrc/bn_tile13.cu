@@ -1121,12 +1121,23 @@ k_upzeta13(int n, int d, const uint16_t* __restrict__ unrank13, T* __restrict__ 
 // blockIdx.x, blockIdx.x + gridDim.x, ...  Thread 0 keeps the next tile's
 // column sums in flight while the block transforms the current one (one bulk
 // copy into shared memory, counted by an mbarrier), and every finished tile
-// leaves as one 32 KB bulk store from a shared-memory staging block, so the
-// block's threads issue neither the loads nor the stores.  The arithmetic
-// and the outputs are those of k_upzeta13, bit for bit.  Shared memory: A0
-// (exchanges), A1 (inputs), the warps' maxima, the mbarrier and a flag, the
-// staged column sums (ncol floats rounded up to 16 bytes, and 48 bytes more)
-// and the output block.  With ncb < ncol the columns from ncb on (d low
+// leaves as one 32 KB bulk store from shared memory, so the block's threads
+// issue neither the loads nor the stores.  The arithmetic and the outputs are
+// those of k_upzeta13, bit for bit.  Shared memory: two blocks of 32 KB, the
+// warps' maxima, the mbarrier and a flag, and the staged column sums (ncol
+// floats rounded up to 16 bytes, and 48 bytes more).
+//
+// What bounds it: 27 instructions an output at 16 warps per SM waited at the
+// barriers (47 % issue with a block each for inputs, exchanges and outputs: two
+// blocks per SM, one at d = 8).  A one-window tile now stays in one 32 KB
+// block from its inputs to its outputs (a thread exchanges into the places it
+// read) while the last tile's store leaves the other; of two windows the first
+// exchanges in the other block, where the outputs then gather.  Three blocks
+// per SM where kUp13ThreeM says so, two to d = 8.  Tiles, us, before -> now:
+// n = 23, m = 500 146 -> 137, n = 29 11480 -> 10690, n = 25 d = 8 (one block
+// per SM before) 1250 -> 865, n = 26, m = 2000 2264 -> 2222.
+//
+// With ncb < ncol the columns from ncb on (d low
 // elements: the sum of one row, the empty high set) were not written by the
 // column-sum kernel; they are the first ncol entries of node i's reordered
 // score table `tab` (K entries per node, K a multiple of 4), and a second
@@ -1135,29 +1146,26 @@ k_upzeta13(int n, int d, const uint16_t* __restrict__ unrank13, T* __restrict__ 
 // kErrDeviceTimeout in *err and the block returns after one more bounded
 // wait for it.  `hold` (a test hook, 0 otherwise) withholds the block's
 // first copies, so that its wait runs out.
-template <bool TLO>
-__global__ void __launch_bounds__(TT, 2)
+template <bool TLO, int NB>
+__global__ void __launch_bounds__(TT, NB)
 k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restrict__ A, uint32_t ntiles,
             int* __restrict__ err, uint32_t cap, int hold, const float* __restrict__ tab, int64_t K,
             uint32_t ncb)
 {
     using Lg = LogOps<float>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    float* A0 = reinterpret_cast<float*>(smem_raw);
-    float* A1 = A0 + TN;
-    float* wmax = A1 + TN;                               // TT / 32 floats
+    float* const AA = reinterpret_cast<float*>(smem_raw);  // the two blocks
+    float* wmax = AA + 2 * TN;                           // TT / 32 floats
     uint64_t* bar = reinterpret_cast<uint64_t*>(wmax + TT / 32);
     int* gave_up = reinterpret_cast<int*>(bar + 1);
     float* S = reinterpret_cast<float*>(bar + 2);       // staged column sums
     const uint32_t ncol = num_small_subsets(TB, d);
-    float* OUT = S + ((ncol * 4u + 15u) & ~15u) / 4 + 12; // the finished tile
     const int h = n - 1 - TB;
     const size_t asize = (size_t)ntiles << TB;
     // the tile's columns (before ncb) and, from the table, the rest
     const uint32_t ncb4 = ncb & ~3u;
     const uint32_t sbytes = (ncb * 4u + 15u) & ~15u;
     const uint32_t tbytes = ncb < ncol ? ((ncol - ncb4) * 4u + 15u) & ~15u : 0u;
-    float* S2 = S + sbytes / 4;
     const int t = threadIdx.x, lane = t & 31;
     const int pt = __popc(t);
     // thread 0: the copies of tile `tl` on the barrier
@@ -1165,13 +1173,16 @@ k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restri
         mbar_expect(bar, sbytes + tbytes);
         bulk_copy_in(S, A + BN_AT((size_t)tl << TB, TN, asize), sbytes, bar);
         if (tbytes)
-            bulk_copy_in(S2, tab + BN_AT((size_t)(tl >> h) * K + ncb4, 4, (size_t)(ntiles >> h) * K), tbytes, bar);
+            bulk_copy_in(S + sbytes / 4, tab + BN_AT((size_t)(tl >> h) * K + ncb4, 4, (size_t)(ntiles >> h) * K), tbytes, bar);
     };
     if (t == 0) mbar_init(bar, 1);
     __syncthreads();
     uint32_t tile = blockIdx.x;
     if (t == 0 && tile < ntiles && !hold) stage(tile);
+    uint32_t side = 0;                                   // the block the next tile's inputs go to
     for (uint32_t parity = 0; tile < ntiles; tile += gridDim.x, parity ^= 1u) {
+        float* const A1 = AA + side * TN;                // inputs
+        float* const A0 = AA + (side ^ 1u) * TN;         // the last tile's outputs, if one-window
         const int i = (int)(tile >> h);
         float* out = A + BN_AT((size_t)tile << TB, TN, asize);
         const int lw = i < 4 ? 3 : 4;
@@ -1182,7 +1193,7 @@ k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restri
             return ((lw == 4 ? g_place.p9[r] : g_place.p10[r]) << lw) | (e & lmask);
         };
         if (t == 0) {
-            bulk_wait_read();                            // the last tile's store has read OUT
+            bulk_wait_read_but1();                       // the store before the last has read A1
             *gave_up = mbar_wait_bounded(bar, parity, cap) ? 0 : 1;
         }
         __syncthreads();
@@ -1198,7 +1209,7 @@ k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restri
         // elements are no column (no input)
         float tm = Lg::ninf();
         for (uint32_t c = t; c < ncol; c += TT) {
-            const float v = c < ncb ? S[c] : S2[c - ncb4];
+            const float v = c < ncb ? S[c] : S[sbytes / 4 + c - ncb4];
             A1[swz(BN_AT(unrank13[c], 1, TN))] = v;
             tm = v > tm ? v : tm;
         }
@@ -1221,6 +1232,16 @@ k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restri
         const int npass = span < Wn::win ? 1
                           : span < float(Wn::max_pass) * Wn::win ? (int)ceilf(span / Wn::win)
                                                                  : Wn::max_pass + 1;
+        // outputs 8q .. 8q + 7 (a run stays inside one row: lw >= 3); half the
+        // threads store the upper half first (bank conflicts)
+        const int flip = (t >> 2) & 1;
+        auto put8 = [&](float4* o, const float (&x)[TR], int q) {
+            const float4 lo = make_float4(x[8 * q], x[8 * q + 1], x[8 * q + 2], x[8 * q + 3]);
+            const float4 hi = make_float4(x[8 * q + 4], x[8 * q + 5], x[8 * q + 6], x[8 * q + 7]);
+            o[flip] = flip ? hi : lo;
+            o[!flip] = flip ? lo : hi;
+        };
+        float* out_s = A0;                               // where the finished tile lies
         if (npass == 1) {
             const float sp = M - Wn::top;
             float x[TR];
@@ -1228,56 +1249,88 @@ k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restri
 #pragma unroll
             for (int r = 0; r < TR; ++r) x[r] = (__popc(r) + pt <= d) ? Lg::ex(x[r] - sp) : 0.0f;
             bfly_plain<true>(x, 0, 5);
-            st1(A0, x, t);
+            st1(A1, x, t);
             __syncthreads();
-            ld2(A0, x, t);
+            ld2(A1, x, t);
             bfly_plain<true>(x, 0, 5);
-            st2(A0, x, t);
+            st2(A1, x, t);
             __syncthreads();
-            ld3(A0, x, t);
+            ld3(A1, x, t);
             bfly_plain<true>(x, 0, 3);
 #pragma unroll
             for (int r = 0; r < TR; ++r) x[r] = sp + Lg::lg(x[r]);
-            // a run of 8 consecutive elements stays inside one row (lw >= 3)
+            out_s = A1;
+            side ^= 1u;
+            __syncthreads();                             // A1 is read: the outputs may land
 #pragma unroll
-            for (int q = 0; q < TR / 8; ++q) {
-                float4* p = reinterpret_cast<float4*>(OUT + BN_AT(opos(el3(8 * q, t)), 8, TN));
-                p[0] = make_float4(x[8 * q], x[8 * q + 1], x[8 * q + 2], x[8 * q + 3]);
-                p[1] = make_float4(x[8 * q + 4], x[8 * q + 5], x[8 * q + 6], x[8 * q + 7]);
-            }
+            for (int q = 0; q < TR / 8; ++q)
+                put8(reinterpret_cast<float4*>(A1 + BN_AT(opos(el3(8 * q, t)), 8, TN)), x, q);
         } else if (npass <= Wn::max_pass) {
+            // the first window exchanges in A0 and keeps the inputs, the
+            // second in A1; the outputs gather in A0
+            static_assert(Wn::max_pass == 2, "two windows");
             uint32_t done = 0u;                          // bit r: output el3(r, t) written
             uint32_t run3[TR / 8];
 #pragma unroll
             for (int q = 0; q < TR / 8; ++q) run3[q] = BN_AT(opos(el3(8 * q, t)), 8, TN);
+            if (t == 0) bulk_wait_read();                // A0 is free
+            __syncthreads();
             float sp = M - Wn::top;
-            for (int p = 0; p < npass; ++p, sp -= Wn::win) {
-                const bool last = p + 1 == npass;
+            for (int p = 0; p < 2; ++p, sp -= Wn::win) {
+                float* const E = p ? A1 : A0;
                 float x[TR];
                 ld1(A1, x, t);
 #pragma unroll
                 for (int r = 0; r < TR; ++r) x[r] = (__popc(r) + pt <= d) ? Lg::ex(x[r] - sp) : 0.0f;
                 bfly_plain<true>(x, 0, 5);
-                st1(A0, x, t);
+                st1(E, x, t);
                 __syncthreads();
-                ld2(A0, x, t);
+                ld2(E, x, t);
                 bfly_plain<true>(x, 0, 5);
-                st2(A0, x, t);
+                st2(E, x, t);
                 __syncthreads();
-                ld3(A0, x, t);
+                ld3(E, x, t);
                 bfly_plain<true>(x, 0, 3);
+                int all = 1;
+                if (p == 0) {
 #pragma unroll
-                for (int r = 0; r < TR; ++r) {
-                    const float lx = Lg::lg(x[r]);
-                    if (!(done >> r & 1u) && (last || lx >= Wn::lo)) {
-                        OUT[run3[r >> 3] + (r & 7)] = sp + lx;
-                        done |= 1u << r;
+                    for (int r = 0; r < TR; ++r) {
+                        x[r] = Lg::lg(x[r]);
+                        done |= (uint32_t)(x[r] >= Wn::lo) << r;
                     }
+#pragma unroll
+                    for (int r = 0; r < TR; ++r) x[r] += sp;
+                    all = __syncthreads_and(done == 0xffffffffu);    // A0 is read
+                } else {
+#pragma unroll
+                    for (int r = 0; r < TR; ++r) x[r] = sp + Lg::lg(x[r]);
                 }
-                if (last) break;
-                if (__syncthreads_and(done == 0xffffffffu)) break;   // also guards A0 reuse
+                // 8 consecutive outputs as two 16-byte stores, the upper first in
+                // half the threads (bank conflicts); the second window keeps the
+                // outputs of the first
+#pragma unroll
+                for (int q = 0; q < TR / 8; ++q) {
+                    float4* o = reinterpret_cast<float4*>(A0 + run3[q]);
+                    if (p) {
+                        const float4 a = o[flip], b = o[!flip];
+                        const float4 lo = flip ? b : a, hi = flip ? a : b;
+                        const uint32_t dq = done >> (8 * q);
+                        if (dq & 1u) x[8 * q] = lo.x;
+                        if (dq & 2u) x[8 * q + 1] = lo.y;
+                        if (dq & 4u) x[8 * q + 2] = lo.z;
+                        if (dq & 8u) x[8 * q + 3] = lo.w;
+                        if (dq & 16u) x[8 * q + 4] = hi.x;
+                        if (dq & 32u) x[8 * q + 5] = hi.y;
+                        if (dq & 64u) x[8 * q + 6] = hi.z;
+                        if (dq & 128u) x[8 * q + 7] = hi.w;
+                    }
+                    put8(o, x, q);
+                }
+                if (all) break;
             }
         } else {
+            if (t == 0) bulk_wait_read();                // A0 is free
+            __syncthreads();
             // max-plus pass, then the exact sum pass (k_upzeta13)
 #pragma unroll
             for (int r = 0; r < TR; ++r) {
@@ -1298,12 +1351,13 @@ k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restri
             bfly_max<true>(v, 0, 3);
             float sc[TR];
             sum_pass<true>(v, sc, A1, A0, t, d);
+            __syncthreads();                             // A0 is read: the outputs may land
 #pragma unroll
-            for (int r = 0; r < TR; ++r) OUT[BN_AT(opos(el1(r, t)), 1, TN)] = scaled_log(v[r], sc[r]);
+            for (int r = 0; r < TR; ++r) A0[BN_AT(opos(el1(r, t)), 1, TN)] = scaled_log(v[r], sc[r]);
         }
-        fence_async_shared();                            // OUT is written: the store may read it
+        fence_async_shared();                            // written: the store may read it
         __syncthreads();
-        if (t == 0) bulk_store(out, OUT, TN * 4u);
+        if (t == 0) bulk_store(out, out_s, TN * 4u);
     }
     if (t == 0) bulk_wait();
 }
@@ -1929,12 +1983,10 @@ cudaError_t launch_reorder_up(const Plan& P, const void* lbs, void* tab, cudaStr
 
 size_t upzeta13p_smem_bytes(const Plan& P)
 {
-    uint64_t ncol = 0;
-    for (int k = 0; k <= P.d && k <= TB; ++k) ncol += binom_host(TB, k);
-    // A0, A1, the warps' maxima, the mbarrier and a flag, the staged column
-    // sums (16-byte multiple, and 48 bytes for the two copies' rounding),
-    // the output block
-    return (size_t)TN * 4 * 2 + (TT / 32) * 4 + 16 + ((ncol * 4 + 15) & ~(uint64_t)15) + 48 + (size_t)TN * 4;
+    // two blocks of 32 KB, the warps' maxima, the mbarrier and a flag, the
+    // staged column sums (16-byte multiple, and 48 bytes for the two copies'
+    // rounding)
+    return (size_t)TN * 4 * 2 + (TT / 32) * 4 + 16 + (((size_t)num_small_subsets_host(P.d) * 4 + 15) & ~(size_t)15) + 48;
 }
 
 // The persistent FP32 tile kernel runs single jobs whose A is in device
@@ -1944,6 +1996,15 @@ static bool use_upzeta13p(const Plan& P, const int* err)
 {
     return err && P.prec != 0 && P.nj == 1 && !P.spill && !recording();
 }
+
+// Three blocks per SM (80 registers; the exact path spills) for the sample
+// counts whose tiles mostly take one window, two (128 registers) for the
+// others and where the staged sums leave no room for three.  us, d = 4,
+// binary, column sums included, two / three blocks: n = 22, m = 500 100 / 93,
+// 1000 110 / 106, 1500 129 / 137; n = 24 393 / 375, 498 / 529, 544 / 592; n =
+// 26 1468 / 1340, 1818 / 1786, 2089 / 2132, m = 2000 2436 / 2695; n = 29, m =
+// 500 16588 / 15536.
+constexpr int kUp13ThreeM = 700;
 
 // The persistent tile kernel stages the columns with d low elements straight
 // from the reordered score table when the column sums come from the column
@@ -2075,23 +2136,23 @@ cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unra
     if (use_upzeta13p(P, err)) {
         const uint32_t ntiles = (uint32_t)nodes << h;
         const size_t smp = upzeta13p_smem_bytes(P);
-        int dev = 0, nsm = 0, per_sm = 0;
-        e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-            e = use_tlo(P) ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_upzeta13p<true>, TT, smp)
-                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_upzeta13p<false>, TT, smp);
-        if (e != cudaSuccess) return e;
-        const unsigned blocks = (unsigned)std::min<uint64_t>(ntiles, (uint64_t)std::max(per_sm, 1) * nsm);
-        const uint32_t ncol = num_small_subsets_host(P.d);
-        const uint32_t ncb = upzeta_table_copies(P, tab, err) ? colb_columns(P) : ncol;
-        if (use_tlo(P))
-            k_upzeta13p<true><<<blocks, TT, smp, s>>>(P.n, P.d, unrank13, (float*)A, ntiles, err, kCopySpinCap, 0,
-                                                      (const float*)tab, P.K, ncb);
-        else
-            k_upzeta13p<false><<<blocks, TT, smp, s>>>(P.n, P.d, unrank13, (float*)A, ntiles, err, kCopySpinCap, 0,
-                                                       (const float*)tab, P.K, ncb);
-        return cudaGetLastError();
+        const auto launch = [&](auto kernel) {
+            int dev = 0, nsm = 0, per_sm = 0;
+            e = cudaGetDevice(&dev);
+            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, TT, smp);
+            if (e != cudaSuccess) return;
+            const unsigned blocks = (unsigned)std::min<uint64_t>(ntiles, (uint64_t)std::max(per_sm, 1) * nsm);
+            const uint32_t ncol = num_small_subsets_host(P.d);
+            const uint32_t ncb = upzeta_table_copies(P, tab, err) ? colb_columns(P) : ncol;
+            kernel<<<blocks, TT, smp, s>>>(P.n, P.d, unrank13, (float*)A, ntiles, err, kCopySpinCap, 0,
+                                           (const float*)tab, P.K, ncb);
+            e = cudaGetLastError();
+        };
+        const bool three = P.m <= kUp13ThreeM && P.d <= 5;
+        if (use_tlo(P)) three ? launch(k_upzeta13p<true, 3>) : launch(k_upzeta13p<true, 2>);
+        else three ? launch(k_upzeta13p<false, 3>) : launch(k_upzeta13p<false, 2>);
+        return e;
     }
     if (P.lin)
         return launch_or_record(KID_UP13_X, k_up13_x, grid, TT, up13_x_smem(P), s, P.n, P.d, unrank13 - TN,
@@ -2112,14 +2173,14 @@ cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unra
 cudaError_t launch_upzeta13p_withheld(float* A, uint16_t* rank13, uint16_t* unrank13, int* err,
                                       uint32_t polls, cudaStream_t s)
 {
-    cudaError_t e = allow_max_dynamic_smem(k_upzeta13p<false>);
+    cudaError_t e = allow_max_dynamic_smem(k_upzeta13p<false, 3>);
     if (e != cudaSuccess) return e;
     k_rank13_tables<<<TN / 256, 256, 0, s>>>(rank13, unrank13, 0);
     Plan P{};
     P.n = 14;
     P.d = 4;
     P.prec = 1;
-    k_upzeta13p<false><<<1, TT, upzeta13p_smem_bytes(P), s>>>(14, 4, unrank13, A, 1u, err, polls, 1, nullptr,
+    k_upzeta13p<false, 3><<<1, TT, upzeta13p_smem_bytes(P), s>>>(14, 4, unrank13, A, 1u, err, polls, 1, nullptr,
                                                              int64_t(0), num_small_subsets_host(4));
     return cudaGetLastError();
 }
@@ -2190,8 +2251,10 @@ cudaError_t set_tile13_attributes()
     SETA((k_upzeta13<double, false>))
     SETA((k_upzeta13<float, false>))
     SETA((k_upzeta13<float, true>))
-    SETA(k_upzeta13p<false>)
-    SETA(k_upzeta13p<true>)
+    SETA((k_upzeta13p<false, 2>))
+    SETA((k_upzeta13p<true, 2>))
+    SETA((k_upzeta13p<false, 3>))
+    SETA((k_upzeta13p<true, 3>))
     SETA((k_gamma13_p1<double, false>))
     SETA((k_gamma13_p1<float, false>))
     SETA((k_gamma13_p1<double, true>))
