@@ -198,8 +198,8 @@ k_set_ones(int n, int m, int W, uint32_t nsets, int lq, const uint64_t* __restri
 // cnt over the supersets of s inside X: one subtraction per state and
 // variable (a downward Moebius transform of 2^k values), then a table lookup
 // per state.  The samples are not touched, so the cost does not depend on m
-// (n = 25, d = 8, m = 500: the scores 33.3 ms -> see the table of the design
-// notes).  Sets of at most 5 variables take a thread (32 registers; the
+// (n = 25, d = 8, m = 500: the scores 33.3 -> 4.8 ms, and with
+// k_set_pairs 3.7).  Sets of at most 5 variables take a thread (32 registers; the
 // states of a missing variable count 0 and add T[0] = 0), the first ns5 of
 // them; larger ones (up to 10) a warp: the five lowest variables are the lane
 // bits, the others 2^(k-5) registers.  What bounds it: the gathers of cnt and
@@ -364,6 +364,171 @@ k_set_moebius(int n, int m, int kmax, uint32_t nsets, uint32_t ns5, uint32_t nal
         }
     }
     (void)kmax;
+}
+
+// The sets of b, b + 1 and b + 2 variables (b = kmax - 2, 5 .. 8) from their
+// bases: a warp takes the base Y (b variables, bits as in moebius_warp), then
+// each variable c below all of Y, then each pair c0 < c1 below all of Y, so
+// every set comes up once.  With v the counts of Y's joint states among the
+// samples whose added variables are 1 (2^b counts gathered and transformed),
+// the states with an added variable 0 are differences of such counts:
+//   Y + c:        v_c, v - v_c
+//   Y + c0 + c1:  v_01, v_1 - v_01, v_0 - v_01, v - v_0 - v_1 + v_01.
+// That takes a quarter of the gathers and shuffles of 2^(b+2) counts; the
+// table lookups, one per state, are the same.  The v_c stay in shared memory
+// (16 bits: m < 65536).  Bases with many variables below them go first.  What
+// bounds it: the L1 requests of the gathers (cnt: a line per lane; T: one per
+// distinct count).  Scores, us, set by set -> from bases: n = 25, m = 500,
+// d = 6 656 -> 427, d = 8 4826 -> 3699.  Four pairs at once measured 427
+// against 519 with bases of 5 but 4998 against 4303 with bases of 7.
+template <int RB>
+__device__ __forceinline__ void pairs_warp(uint32_t Y, int b, int lane, const uint32_t* __restrict__ soff,
+                                           const uint32_t* __restrict__ cnt, uint32_t nsets,
+                                           const long long* __restrict__ T0, const long long* __restrict__ T1,
+                                           const long long* __restrict__ T2, uint16_t* __restrict__ vc,
+                                           long long* __restrict__ H, int64_t* __restrict__ dbg, uint32_t dbg_set)
+{
+    constexpr int R = 1 << RB;
+    const int p0 = __popc(lane);
+    // off[s][r]: index of this lane's subset of Y with s smaller variables
+    // added, less the ranks of those
+    uint32_t off[3][R];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        uint32_t low = 0, rest = Y, rr[R];
+        int pos = 1 + s;
+#pragma unroll
+        for (int e = 0; e < 5; ++e) {
+            const int c = __ffs(rest) - 1;
+            rest &= rest - 1;
+            if (lane >> e & 1) low += gbinom(c, pos++);
+        }
+        rr[0] = 0;
+        off[s][0] = soff[p0 + s] + low;
+#pragma unroll
+        for (int e = 0; e < RB; ++e) {
+            const int c = __ffs(rest) - 1;
+            rest &= rest - 1;
+#pragma unroll
+            for (int r = 0; r < (1 << e); ++r) {
+                int pc = 0;
+#pragma unroll
+                for (int q = 0; q < RB; ++q) pc += r >> q & 1;
+                rr[r | 1 << e] = rr[r] + gbinom(c, p0 + pc + 1 + s);
+                off[s][r | 1 << e] = soff[p0 + pc + 1 + s] + low + rr[r | 1 << e];
+            }
+        }
+    }
+    auto counts = [&](uint32_t (&v)[R], const uint32_t (&o)[R], uint32_t add) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = cnt[BN_AT(o[r] + add, 1, nsets)];
+#pragma unroll
+        for (int q = 0; q < RB; ++q)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (!(r >> q & 1)) v[r] -= v[r | (1 << q)];
+#pragma unroll
+        for (int w = 1; w < 32; w <<= 1)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const uint32_t y = __shfl_xor_sync(WARPMASK, v[r], w);
+                v[r] -= (lane & w) ? 0u : y;
+            }
+    };
+    auto leave = [&](uint32_t idx, long long acc) {
+        acc = warp_sum(acc);
+        if (lane == 0) H[BN_AT(idx, 1, nsets)] = acc;
+    };
+    const uint32_t i0 = __shfl_sync(WARPMASK, off[0][R - 1], 31), i1 = __shfl_sync(WARPMASK, off[1][R - 1], 31),
+                   i2 = __shfl_sync(WARPMASK, off[2][R - 1], 31);
+    const int nc = __ffs(Y) - 1;                    // the variables below Y
+    uint32_t v[R];
+    counts(v, off[0], 0u);
+    long long acc = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        acc += T0[v[r]];
+        if (dbg && i0 == dbg_set) dbg[lane | r << 5] = v[r];
+    }
+    leave(i0, acc);
+    for (int c1 = 0; c1 < nc; ++c1) {
+        uint32_t v1[R];
+        counts(v1, off[1], (uint32_t)c1);
+        acc = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            vc[(c1 * R + r) * 32 + lane] = (uint16_t)v1[r];
+            acc += T1[v1[r]] + T1[v[r] - v1[r]];
+            if (dbg && i1 + c1 == dbg_set) {
+                dbg[(lane | r << 5) << 1 | 1] = v1[r];
+                dbg[(lane | r << 5) << 1] = v[r] - v1[r];
+            }
+        }
+        leave(i1 + c1, acc);
+        const uint32_t rank1 = (uint32_t)c1 * (uint32_t)(c1 - 1) / 2;   // C(c1, 2)
+        // several pairs at once while they cost few registers
+        constexpr int U = R == 1 ? 4 : 1;
+        for (int c = 0; c < c1; c += U) {
+            uint32_t w[U][R];
+#pragma unroll
+            for (int u = 0; u < U; ++u) counts(w[u], off[2], rank1 + min(c + u, c1 - 1));
+            long long a[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int c0 = min(c + u, c1 - 1);
+                a[u] = 0;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const uint32_t v0 = vc[(c0 * R + r) * 32 + lane];     // this lane's own
+                    const uint32_t n10 = v1[r] - w[u][r], n01 = v0 - w[u][r], n00 = v[r] - v1[r] - n01;
+                    a[u] += T2[w[u][r]] + T2[n10] + T2[n01] + T2[n00];
+                    if (dbg && i2 + rank1 + c0 == dbg_set) {
+                        int64_t* o = dbg + ((lane | r << 5) << 2);
+                        o[0] = n00;
+                        o[1] = n01;
+                        o[2] = n10;
+                        o[3] = w[u][r];
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) a[u] = warp_sum(a[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (lane == 0 && c + u < c1) H[BN_AT(i2 + rank1 + c + u, 1, nsets)] = a[u];
+        }
+    }
+}
+
+constexpr int kPairsMin = 7;                        // kmax from which bases take over
+template <int RB>
+__global__ void __launch_bounds__(256, RB < 3 ? 3 : 2)
+k_set_pairs(int n, int m, int b, uint32_t nsets, uint32_t nbase, const uint32_t* __restrict__ cnt,
+            const double* __restrict__ Dvals, int rows, const long long* __restrict__ T,
+            long long* __restrict__ H, int64_t* __restrict__ dbg, uint32_t dbg_set, size_t js)
+{
+    cnt = job_ptr(cnt, js);
+    Dvals = job_ptr(Dvals, js);
+    T = job_ptr(T, js);
+    H = job_ptr(H, js);
+    __shared__ uint32_t soff[16];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (threadIdx.x < 16) {
+        uint32_t o = 0;
+        for (int k = 0; k < (int)threadIdx.x && k <= n; ++k) o += gbinom(n, k);
+        soff[threadIdx.x] = o;
+    }
+    __syncthreads();
+    const uint32_t warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (warp >= nbase) return;
+    int k;
+    const uint32_t Y = set_of(soff[b] + (nbase - 1 - warp), n, &k);
+    const int lane = threadIdx.x & 31;
+    uint16_t* vc = reinterpret_cast<uint16_t*>(smem_raw) + ((size_t)(threadIdx.x >> 5) * (n - b) << b);
+    const long long* T0 = T + (size_t)find_row(Dvals, rows, 1u << b) * (m + 1);
+    const long long* T1 = T + (size_t)find_row(Dvals, rows, 2u << b) * (m + 1);
+    const long long* T2 = T + (size_t)find_row(Dvals, rows, 4u << b) * (m + 1);
+    pairs_warp<RB>(Y, b, lane, soff, cnt, nsets, T0, T1, T2, vc, H, dbg, dbg_set);
 }
 
 // Data of any arity: H(X) from a histogram of the samples' joint states in
@@ -684,6 +849,7 @@ uint32_t sets_before(int n, int k)
 // at most 16384 (64 KB), beside the staged data; at most 192 KB in all.
 struct SetSplit {
     int moebius, warp, block, end;
+    int pairs;                                      // size of k_set_pairs' bases (0: not used)
     int mw;                                         // words of a staged column
     uint32_t wstates, bstates;
 };
@@ -698,6 +864,7 @@ SetSplit split_sets(const Plan& P)
     x.end = std::min(P.d + 1, P.n) + 1;
     x.mw = ((P.m + 3) / 4) | 1;                     // odd: columns start in different banks
     x.moebius = P.allbin ? std::min(x.end, kMoebiusMax + 1) : 0;
+    x.pairs = x.moebius - 1 >= kPairsMin && P.m < 65536 ? x.moebius - 3 : 0;
     x.warp = x.moebius;
     while (x.warp < x.end && P.states[x.warp] <= kWarpStates &&
            hist_bytes(P, x.mw, 8 * P.states[x.warp]) <= kSetSmem)
@@ -762,11 +929,27 @@ cudaError_t launch_set_scores(const Plan& P, const uint8_t* data, const uint8_t*
                              dim3((unsigned)((((int64_t)nsets << lq) + 255) / 256), P.nj), 256, 0, s, P.n,
                              P.m, P.W, nsets, lq, planes, mj, x.cnt, P.js);
         if (e != cudaSuccess) return e;
-        const uint32_t warps = (nsets - ns5 + kMoebiusRun - 1) / kMoebiusRun;
-        e = launch_or_record(KID_SET_MOEBIUS, k_set_moebius, dim3((ns5 + 255) / 256 + (warps + 7) / 8, P.nj),
-                             256, 0, s, P.n, P.m, z.moebius - 1, nsets, ns5, nsets, x.cnt, Dvals, P.rows, T,
+        // the sizes up to `own` set by set, the last three from their bases
+        const int b = z.pairs;
+        const uint32_t own = b ? sets_before(P.n, b) : nsets, own5 = std::min(ns5, own);
+        const uint32_t warps = (own - own5 + kMoebiusRun - 1) / kMoebiusRun;
+        e = launch_or_record(KID_SET_MOEBIUS, k_set_moebius, dim3((own5 + 255) / 256 + (warps + 7) / 8, P.nj),
+                             256, 0, s, P.n, P.m, z.moebius - 1, own, own5, nsets, x.cnt, Dvals, P.rows, T,
                              x.H, dbg, dbg_set, P.js);
         if (e != cudaSuccess) return e;
+        if (b) {
+            const uint32_t nbase = (uint32_t)choose(P.n, b);
+            const auto launch = [&](int kid, auto kernel) {
+                return launch_or_record(kid, kernel, dim3((nbase + 7) / 8, P.nj), 256,
+                                        ((size_t)(P.n - b) * 8 << b) * 2, s, P.n, P.m, b, nsets, nbase, x.cnt,
+                                        Dvals, P.rows, T, x.H, dbg, dbg_set, P.js);
+            };
+            e = b == 5   ? launch(KID_SET_PAIRS5, k_set_pairs<0>)
+                : b == 6 ? launch(KID_SET_PAIRS6, k_set_pairs<1>)
+                : b == 7 ? launch(KID_SET_PAIRS7, k_set_pairs<2>)
+                         : launch(KID_SET_PAIRS8, k_set_pairs<3>);
+            if (e != cudaSuccess) return e;
+        }
     }
     if (z.warp > z.moebius) {
         const uint32_t s0 = sets_before(P.n, z.moebius), s1 = sets_before(P.n, z.warp);
@@ -812,7 +995,7 @@ cudaError_t launch_scores(const Plan& P, const uint8_t* data, const uint8_t* ari
 int scores_launches(const Plan& P)
 {
     const SetSplit z = split_sets(P);
-    return (z.moebius > 0 ? 2 : 0) + (z.warp > z.moebius) + (z.block > z.warp) + (z.end > z.block) + 1;
+    return (z.moebius > 0 ? 2 : 0) + (z.pairs > 0) + (z.warp > z.moebius) + (z.block > z.warp) + (z.end > z.block) + 1;
 }
 
 cudaError_t launch_shift_scores(const Plan& P, const double* logB, const unsigned long long* enc,
@@ -835,6 +1018,10 @@ cudaError_t launch_shift_scores(const Plan& P, const double* logB, const unsigne
 cudaError_t set_scores_attributes()
 {
     cudaError_t e = allow_max_dynamic_smem(k_set_hist<32>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_pairs<0>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_pairs<1>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_pairs<2>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_pairs<3>);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_hist<256>);
     return e;
 }
