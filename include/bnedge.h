@@ -65,7 +65,9 @@ enum {
 };
 
 enum {
-    BN_FP64 = 0,         /* every DP array in FP64, natural-log domain        */
+    BN_FP64 = 0,         /* every DP value in 64 bits: an exponent and a fraction
+                            of at least 46 bits where the scores' range allows
+                            (n >= 5), else natural logs in FP64             */
     BN_FP32_SHIFTED = 1  /* DP arrays in FP32 log2 domain, each node's scores
                             shifted by their FP64 maximum; scores, P(D) and the
                             final division stay FP64                          */
@@ -85,8 +87,8 @@ typedef struct bn_ctx_opts {
 
 /* bn_ctx_opts.flags: BN_CTX_NO_AUTOTUNE, batches keep the default schedule
  * (and a persistent launch keeps clusters of 8 blocks) instead of timing the
- * alternatives; BN_CTX_CLUSTER_STEP3, every FP32 batch group with n >= 5
- * runs step 3 in the persistent cluster kernel whatever the timing says;
+ * alternatives; BN_CTX_CLUSTER_STEP3, every batch group whose step 3 has
+ * row tiles runs all its levels in one launch whatever the timing says;
  * BN_CTX_GRAPH_BATCH, batches run as a graph of launches instead of one
  * persistent launch (see bn_batch_create; CLUSTER_STEP3 implies it). */
 #define BN_CTX_NO_AUTOTUNE 1
