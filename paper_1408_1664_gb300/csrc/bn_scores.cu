@@ -939,9 +939,15 @@ cudaError_t launch_set_scores(const Plan& P, const uint8_t* data, const uint8_t*
         if (e != cudaSuccess) return e;
         if (b) {
             const uint32_t nbase = (uint32_t)choose(P.n, b);
+            // neighbouring bases differ widely in work (the variables below them),
+            // and a block holds its place until its slowest warp ends: two warps
+            // a block (with 8, 13 of the 24 warps an SM has room for were at work).
+            // Whole job, m = 500: n = 25, d = 8 10.95 -> 10.52 ms, n = 20 1.052 ->
+            // 1.026 ms; d = 6 4.67 -> 4.65.  A recorded launch has blocks of 256 threads.
+            const unsigned threads = recording() ? 256 : 64, per = threads / 32;
             const auto launch = [&](int kid, auto kernel) {
-                return launch_or_record(kid, kernel, dim3((nbase + 7) / 8, P.nj), 256,
-                                        ((size_t)(P.n - b) * 8 << b) * 2, s, P.n, P.m, b, nsets, nbase, x.cnt,
+                return launch_or_record(kid, kernel, dim3((nbase + per - 1) / per, P.nj), threads,
+                                        ((size_t)(P.n - b) * per << b) * 2, s, P.n, P.m, b, nsets, nbase, x.cnt,
                                         Dvals, P.rows, T, x.H, dbg, dbg_set, P.js);
             };
             e = b == 5   ? launch(KID_SET_PAIRS5, k_set_pairs<0>)
