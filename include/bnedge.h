@@ -88,7 +88,8 @@ typedef struct bn_ctx_opts {
 /* bn_ctx_opts.flags: BN_CTX_NO_AUTOTUNE, batches keep the default schedule
  * (and a persistent launch keeps clusters of 8 blocks) instead of timing the
  * alternatives; BN_CTX_CLUSTER_STEP3, every batch group whose step 3 has
- * row tiles runs all its levels in one launch whatever the timing says;
+ * row tiles (and n <= 28) runs all its levels in one launch whatever the
+ * timing says;
  * BN_CTX_GRAPH_BATCH, batches run as a graph of launches instead of one
  * persistent launch (see bn_batch_create; CLUSTER_STEP3 implies it). */
 #define BN_CTX_NO_AUTOTUNE 1
@@ -456,6 +457,15 @@ int bn_debug_bounds(int32_t* line, int32_t* unit);
  * host doubles x: out (4 * count host doubles) receives, per x, the
  * library's exp, CUDA's exp, the library's log, CUDA's log. */
 int bn_debug_explog(const double* x, int64_t count, double* out);
+/* What the host planned for a job (no GPU needed): `count` values, the first
+ * of the enumeration below, go to out.  BN_EINVAL for an invalid job or a
+ * count beyond it. */
+enum {
+    BN_PLAN_SWEEPS = 0,  /* 1: F and R' of a batch group of such jobs may run in
+                            one launch                                       */
+    BN_PLAN_COUNT = 1
+};
+int bn_debug_plan(const bn_job_desc* job, int32_t* out, int32_t count);
 #endif /* BN_TESTING */
 
 #ifdef __cplusplus

@@ -69,7 +69,8 @@ EXPORTS = ["bn_ctx_create", "bn_ctx_destroy", "bn_num_families", "bn_scores",
 
 # Test hooks: exported only by the testing build (BN_TESTING).
 TEST_EXPORTS = ["bn_debug_stage", "bn_debug_counts", "bn_debug_batch_drop", "bn_debug_bounds",
-                "bn_debug_explog", "bn_debug_copy_wait"]
+                "bn_debug_explog", "bn_debug_copy_wait", "bn_debug_plan"]
+BN_PLAN_SWEEPS, BN_PLAN_COUNT = range(2)
 
 
 def testing_build() -> bool:
@@ -148,6 +149,7 @@ def load(build_if_missing: bool = False) -> C.CDLL:
         "bn_debug_bounds": (C.c_int, [C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
         "bn_debug_explog": (C.c_int, [P, C.c_int64, P]),
         "bn_debug_copy_wait": (C.c_int, [C.c_uint32, C.POINTER(C.c_int32)]),
+        "bn_debug_plan": (C.c_int, [C.POINTER(bn_job_desc), C.POINTER(C.c_int32), C.c_int32]),
         "bn_shard_create": (C.c_int, [P, C.POINTER(bn_job_desc), C.c_int32, C.c_int32, C.c_int32,
                                       C.POINTER(P)]),
         "bn_shard_bytes": (C.c_int, [P, C.POINTER(C.c_uint64)]),
@@ -361,6 +363,15 @@ def bn_debug_bounds() -> tuple[int, int]:
     if rc:
         raise BnError(rc, "bn_debug_bounds")
     return int(line.value), int(unit.value)
+
+
+def bn_debug_plan(job: Job) -> list[int]:
+    """What the host planned for a job, by BN_PLAN_* (no GPU needed)."""
+    out = (C.c_int32 * BN_PLAN_COUNT)()
+    rc = load().bn_debug_plan(C.byref(job.desc), out, BN_PLAN_COUNT)
+    if rc:
+        raise BnError(rc, "bn_debug_plan")
+    return list(out)
 
 
 def bn_debug_counts(ctx: int, job: Job, i: int, mask: int, cells: int) -> np.ndarray:

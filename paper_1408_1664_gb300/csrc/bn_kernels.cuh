@@ -337,7 +337,7 @@ cudaError_t launch_top_slabs(const Plan& V, int k, const void* Av, void* Atop, c
 cudaError_t launch_level_rows(const Plan& P, uint32_t r, int hl, void* X, void* buf, int dir,
                               cudaStream_t s);
 // F and R' in one launch (k_sweeps): FP32 plans with the row schedule and
-// linear FP64 plans, whole jobs with A in device memory.  use_sweeps: whether a single job's direct
+// linear FP64 plans up to n = 28, whole jobs with A in device memory.  use_sweeps: whether a single job's direct
 // launches take it; err is the job's error word, the first of 256 bytes that
 // also hold the sweeps' counters.  Rc null: F alone.
 bool sweeps_fit(const Plan& P);

@@ -37,6 +37,11 @@ constexpr int BT = 29;            // binomial table rows (n - B < 29: n <= 32 in
 // blocks run on the whole GPU; polls before a block gives up a wait (about 1 us each).
 constexpr int kSweepMaxN = 21;
 constexpr int kSweepMaxNX = 21;
+// Largest n of any k_sweeps launch: the kernel's places among the n 2^(n-1)
+// values of A are 32-bit numbers, and 28 2^27 is the last such size below 2^32
+// (from n = 29 they wrap to other nodes' rows).  A batch group may come up to
+// here; a level of a larger job fills the GPU by itself anyway.
+constexpr int kSweepPlacesN = 28;
 constexpr int kSweepVecN = 20;
 constexpr int kSweepBusyN = 18;
 constexpr uint64_t kSweepGrid = 12;
@@ -546,7 +551,7 @@ k_sweeps(int n, int nb, const T* __restrict__ A, T* __restrict__ F, T* __restric
     int* lw = kBases ? level_words(reinterpret_cast<float*>(X), n) : nullptr;
     unsigned* arr = SYNC == SYNC_GRID ? sync + (fwd ? 0 : 16) : nullptr;
 
-    // Places are 32-bit (n <= kSweepMaxN).  That of the lane's values in the row
+    // Places are 32-bit (n <= kSweepPlacesN).  That of the lane's values in the row
     // S-without-j of A_{B + j}, u = 1 << j: H with bit j squeezed out is
     // (H >> 1) with the bits below j taken from H.
     auto a_at = [&](uint32_t H, uint32_t u) {
@@ -1055,7 +1060,8 @@ static int sweep_blocks(const Plan& P, uint64_t tiles, int per_sm, const int* er
 
 bool sweeps_fit(const Plan& P)
 {
-    return ((rows_levels_fit(P) && P.frows) || P.lin) && P.shard_k == 0 && !P.slab && !P.spill;
+    return ((rows_levels_fit(P) && P.frows) || P.lin) && P.n <= kSweepPlacesN && P.shard_k == 0 && !P.slab &&
+           !P.spill;
 }
 
 bool use_sweeps(const Plan& P, const int* err)
@@ -1103,6 +1109,7 @@ static cudaError_t sweeps(const Plan& P, const T* A, T* F, T* Rc, int items, cud
 cudaError_t launch_sweeps(const Plan& P, const void* A, void* F, void* Rc, cudaStream_t s, int* err,
                           int* launches)
 {
+    if (P.n > kSweepPlacesN) return cudaErrorInvalidValue;
     const int items = Rc ? 2 * P.nj : 1;            // a feature's job: F alone
     const cudaError_t e = P.lin == 2 ? sweeps<X64S, false>(P, (const X64S*)A, (X64S*)F, (X64S*)Rc, items, s, err)
                           : P.lin ? sweeps<X64, false>(P, (const X64*)A, (X64*)F, (X64*)Rc, items, s, err)

@@ -2325,6 +2325,21 @@ try {
     return exception_code();
 }
 
+// Test hook: what the host planned for a job.
+int bn_debug_plan(const bn_job_desc* job, int32_t* out, int32_t count)
+try {
+    if (!out || count < 0 || count > BN_PLAN_COUNT) return BN_EINVAL;
+    HostJob hj;
+    const int rc = validate_and_plan(job, hj);
+    if (rc) return rc;
+    int32_t v[BN_PLAN_COUNT] = {};
+    v[BN_PLAN_SWEEPS] = bn::sweeps_fit(hj.P);
+    std::copy(v, v + count, out);
+    return BN_OK;
+} catch (...) {
+    return exception_code();
+}
+
 // Test hook: the first failing index check of the BN_CHECK_BOUNDS build.
 int bn_debug_bounds(int32_t* line, int32_t* unit)
 try {
