@@ -1125,7 +1125,8 @@ k_upzeta13(int n, int d, const uint16_t* __restrict__ unrank13, T* __restrict__ 
 // issue neither the loads nor the stores.  The arithmetic and the outputs are
 // those of k_upzeta13, bit for bit.  Shared memory: two blocks of 32 KB, the
 // warps' maxima, the mbarrier and a flag, and the staged column sums (ncol
-// floats rounded up to 16 bytes, and 48 bytes more).
+// floats rounded up to 16 bytes, and 48 bytes more).  The word after the flag
+// keeps the tile's smallest output until the next tile's first barrier.
 //
 // What bounds it: 27 instructions an output at 16 warps per SM waited at the
 // barriers (47 % issue with a block each for inputs, exchanges and outputs: two
@@ -1158,6 +1159,7 @@ k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restri
     float* wmax = AA + 2 * TN;                           // TT / 32 floats
     uint64_t* bar = reinterpret_cast<uint64_t*>(wmax + TT / 32);
     int* gave_up = reinterpret_cast<int*>(bar + 1);
+    float* lowest = reinterpret_cast<float*>(gave_up + 1);   // the tile's smallest output
     float* S = reinterpret_cast<float*>(bar + 2);       // staged column sums
     const uint32_t ncol = num_small_subsets(TB, d);
     const int h = n - 1 - TB;
@@ -1218,6 +1220,9 @@ k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restri
             tm = o2 > tm ? o2 : tm;
         }
         if (lane == 0) wmax[t >> 5] = tm;
+        // C(empty), in a word of its own: its place in A1 is thread 0's first
+        // exchange below, before slower warps have read it
+        if (t == 0) *lowest = S[0];
         fence_async_shared();                            // S is read: the next copy may land
         __syncthreads();
         if (t == 0 && tile + gridDim.x < ntiles) stage(tile + gridDim.x);
@@ -1228,7 +1233,7 @@ k_upzeta13p(int n, int d, const uint16_t* __restrict__ unrank13, float* __restri
         // single-scale passes as in k_upzeta13
         using Wn = Window<float>;
         const float M = tmx + float(TB);
-        const float span = M - A1[0];
+        const float span = M - *lowest;
         const int npass = span < Wn::win ? 1
                           : span < float(Wn::max_pass) * Wn::win ? (int)ceilf(span / Wn::win)
                                                                  : Wn::max_pass + 1;
