@@ -65,9 +65,10 @@ enum {
 };
 
 enum {
-    BN_FP64 = 0,         /* every DP value in 64 bits: an exponent and a fraction
-                            of at least 46 bits where the scores' range allows
-                            (n >= 5), else natural logs in FP64             */
+    BN_FP64 = 0,         /* every DP value in 64 bits: a fraction of 52 bits from
+                            2^-1024 up, of 46 bits and a wider exponent below,
+                            where the scores' range allows (n >= 5), else
+                            natural logs in FP64; sums in double            */
     BN_FP32_SHIFTED = 1  /* DP arrays in FP32 log2 domain, each node's scores
                             shifted by their FP64 maximum; scores, P(D) and the
                             final division stay FP64                          */

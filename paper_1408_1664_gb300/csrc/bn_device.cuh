@@ -464,88 +464,100 @@ template <typename T> struct LseAcc {
 
 // ---------------------------------------------------------------------------
 // The linear FP64 form (Plan::lin).  A value v >= 0 of the FP64 path is kept
-// itself, not its logarithm: 64 bits hold an exponent of 64 - FB bits and a
-// fraction of FB bits.  Every sum over logarithms costs an FP64 exponential
+// itself, not its logarithm.  Every sum over logarithms costs an FP64 exponential
 // per term and a logarithm per result, on a pipe that retires two lanes per
 // clock and SM; here a term costs one multiplication and one fused
-// multiply-add there and integer operations on the exponents.  Values compare
-// like their bits; 0 is all zeros; anything below the smallest kept exponent
-// is 0.  Sums run in double, relative to an integer exponent.
-//   X64: FB = 46, values in 2^+-131072 (90000 nats), rounding 2^-47 = 7e-15.
-//     Used from n = 14: a stored logarithm of a few hundred nats is no more
-//     exact (its unit in the last place is 6e-14 from 256 nats on).
-//   X64S: FB = 49, values in 2^+-16384, rounding 2^-50.  Used below n = 14,
-//     where logarithms stay short and the wider fraction is needed to lose
-//     nothing against them.
-// The planner keeps the logarithms when the job's values could leave the
-// range (lin_range in bn_kernels.cuh).
+// multiply-add there and integer operations on the exponents.  Sums run in
+// double, relative to an integer exponent.
+//
+// A double's 11 exponent bits are too few (F(V) of a large job lies thousands
+// of bits below 1), and a wider exponent at a fixed width would take its bits
+// from every fraction.  So the width follows the value, as that of a logarithm
+// does.  The top 12 bits hold E, the others a fraction of 52 bits:
+//   E >= 2048:  the value's exponent e = E - 3072, in [-1024, 1024)
+//   E < 2048:   e = 64 E + (the fraction's lowest 6 bits) - 132096
+// Below 2^-1024 the lowest bits of the fraction are given, and the others are
+// chosen so that the whole is nearest: 46 bits.  A logarithm of at least 1 nat
+// rounds by 2^-53 or more, one of 710 nats (2^1024) by 2^-44: no value is held
+// to fewer bits than by its logarithm.  The fraction is read the same way on
+// both sides, the exponent by a select.  0 is all zeros (it reads as
+// 2^-132096, far below every sum it enters); anything below 2^kXMin is 0.  The
+// planner keeps the logarithms when the job's values could leave the range
+// (lin_range in bn_kernels.cuh).
 // ---------------------------------------------------------------------------
-template <int FB> struct XValue {
-    static constexpr int frac = FB;
-    static constexpr int bias = 1 << (63 - FB);
-    static constexpr int min = (FB == 46 ? 4096 : 2048) - bias;   // smallest exponent kept
+struct X64 {
     unsigned long long u;
 };
-using X64 = XValue<46>;
-using X64S = XValue<49>;
-constexpr int kXBias = X64::bias, kXMin = X64::min;
+constexpr int kXBias = 1024 + (1 << 17);            // the exponent of 0 is -kXBias
+constexpr int kXNear = 3072;
+constexpr int kXMin = 4096 - kXBias;                // smallest exponent kept
+constexpr int kXMax = 1023;                         // and the largest
 
-template <typename X> __host__ __device__ __forceinline__ X x_one() { return X{(unsigned long long)X::bias << X::frac}; }
-// The exponent (that of 0 is -bias: far below every sum it enters) and the
-// fraction with its leading one, in [1, 2).
-template <int FB> __device__ __forceinline__ int x_exp(XValue<FB> x) { return (int)(x.u >> FB) - XValue<FB>::bias; }
-template <int FB> __device__ __forceinline__ double x_mant(XValue<FB> x)
+__host__ __device__ __forceinline__ X64 x_one() { return X64{(unsigned long long)kXNear << 52}; }
+// The exponent and the fraction with its leading one, in [1, 2).
+__host__ __device__ __forceinline__ int x_exp(X64 x)
 {
-    return __longlong_as_double((long long)(((x.u << (52 - FB)) & 0x000fffffffffffffull) | 0x3ff0000000000000ull));
+    const unsigned hi = (unsigned)(x.u >> 32);
+    int e = (int)(((hi >> 14) & ~63u) | ((unsigned)x.u & 63u)) - kXBias;
+    if ((int)hi < 0) e = (int)(hi >> 20) - kXNear;
+    return e;
+}
+__device__ __forceinline__ double x_mant(X64 x)
+{
+    return __longlong_as_double((long long)((x.u & 0x000fffffffffffffull) | 0x3ff0000000000000ull));
 }
 // x * 2^-ref as a double: 0 below 2^-1000, +inf above 2^1010.
-template <int FB> __device__ __forceinline__ double x_scaled(XValue<FB> x, int ref)
+__device__ __forceinline__ double x_scaled(X64 x, int ref)
 {
     const int e = x_exp(x) - ref;
     const unsigned long long b =
-        ((x.u << (52 - FB)) & 0x000fffffffffffffull) | ((unsigned long long)(unsigned)(e + 1023) << 52);
+        (x.u & 0x000fffffffffffffull) | ((unsigned long long)(unsigned)(e + 1023) << 52);
     return __longlong_as_double(e < -1000 ? 0ll : e > 1010 ? 0x7ff0000000000000ll : (long long)b);
 }
-// s * 2^ref (s >= 0, finite) rounded to the nearest stored value.
-template <typename X> __device__ __forceinline__ X x_pack(double s, int ref)
+// The code of the value (1 + f 2^-52) 2^e, kXMin <= e <= kXMax, f < 2^52.
+__host__ __device__ __forceinline__ unsigned long long x_code(int e, unsigned long long f)
 {
-    constexpr int drop = 52 - X::frac;
-    const unsigned long long b = (unsigned long long)__double_as_longlong(s) + (1ull << (drop - 1));
+    if (e >= -1024) return ((unsigned long long)(unsigned)(e + kXNear) << 52) | f;
+    // the nearest fraction with these lowest bits (at the ends of the low word
+    // the nearest in it)
+    const unsigned x = (unsigned)(e + kXBias), low = x & 63u, lo = (unsigned)f;
+    const unsigned r = low > 32u ? (lo < low - 32u ? 0u : lo - (low - 32u))
+                                 : (lo + (32u - low) < lo ? ~0u : lo + (32u - low));
+    return ((unsigned long long)(x >> 6) << 52) | (f & 0x000fffff00000000ull) | (r & ~63u) | low;
+}
+// s * 2^ref (s >= 0, finite) as the nearest stored value.
+__device__ __forceinline__ X64 x_pack(double s, int ref)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(s);
     const int ex = (int)(b >> 52);
     const int e = ex - 1023 + ref;
-    if (ex == 0 || e < X::min) return X{0ull};
-    return X{((unsigned long long)(unsigned)(e + X::bias) << X::frac) | ((b & 0x000fffffffffffffull) >> drop)};
+    return X64{ex == 0 || e < kXMin ? 0ull : x_code(e, b & 0x000fffffffffffffull)};
 }
-// 2^e for an integer e <= 1023 (0 below 2^-1022).
-__device__ __forceinline__ double pow2d(int e)
+// 2^e for an integer e <= 1024 (0 below 2^-1022, +inf at 1024).
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((max(e, -1023) + 1023) << 20, 0); }
+__device__ __forceinline__ X64 x_mul(X64 a, X64 b) { return x_pack(x_mant(a) * x_mant(b), x_exp(a) + x_exp(b)); }
+__device__ __forceinline__ X64 x_add(X64 a, X64 b)
 {
-    return __longlong_as_double(e < -1022 ? 0ll : (long long)(e + 1023) << 52);
-}
-template <int FB> __device__ __forceinline__ XValue<FB> x_mul(XValue<FB> a, XValue<FB> b)
-{
-    return x_pack<XValue<FB>>(x_mant(a) * x_mant(b), x_exp(a) + x_exp(b));
-}
-template <int FB> __device__ __forceinline__ XValue<FB> x_add(XValue<FB> a, XValue<FB> b)
-{
-    const XValue<FB> hi = a.u > b.u ? a : b, lo = a.u > b.u ? b : a;
-    const int e = x_exp(hi);
-    return x_pack<XValue<FB>>(fma(x_mant(lo), pow2d(x_exp(lo) - e), x_mant(hi)), e);
+    const int ea = x_exp(a), eb = x_exp(b);
+    const X64 hi = ea > eb ? a : b, lo = ea > eb ? b : a;
+    const int e = max(ea, eb);
+    return x_pack(fma(x_mant(lo), pow2d(min(ea, eb) - e), x_mant(hi)), e);
 }
 // exp(x) for a natural logarithm x: x = k ln 2 + r in two parts, so that the
 // fraction is as exact as x.
-template <typename X> __device__ __forceinline__ X x_from_ln(double x)
+__device__ __forceinline__ X64 x_from_ln(double x)
 {
-    if (!(x > -91000.0)) return X{0ull};
+    if (!(x > -91000.0)) return X64{0ull};
     const double k = rint(x * 1.4426950408889634074);
     double r = fma(-k, explog::kLn2Hi, x);
     r = fma(-k, explog::kLn2Lo, r);
-    return x_pack<X>(exp_t(r), (int)k);
+    return x_pack(exp_t(r), (int)k);
 }
 
 // A lazy sum: add() takes one term, value() gives the result in the array's
 // own form.  float / double: (m, s) stands for m + log(s), s rescaled only
 // when a term exceeds m by more than 64 log units, so a term costs one
-// exponential (the values are finite).  XValue: s 2^e, rescaled only when a term
+// exponential (the values are finite).  X64: s 2^e, rescaled only when a term
 // exceeds 2^e by more than 2^500.
 template <typename T> struct LazySum {
     T m, s;
@@ -561,8 +573,7 @@ template <typename T> struct LazySum {
     }
     __device__ __forceinline__ T value() const { return m + LogOps<T>::lg(s); }
 };
-template <int FB> struct LazySum<XValue<FB>> {
-    using X = XValue<FB>;
+template <> struct LazySum<X64> {
     int e;
     double s;
     __device__ __forceinline__ LazySum() : e(-(1 << 28)), s(0.0) {}
@@ -574,8 +585,8 @@ template <int FB> struct LazySum<XValue<FB>> {
         s = fma(big ? s : p, pow2d(big ? -d : d), big ? p : s);
         e = big ? ep : e;
     }
-    __device__ __forceinline__ void add(X x) { add(x_mant(x), x_exp(x)); }
-    __device__ __forceinline__ X value() const { return x_pack<X>(s, e); }
+    __device__ __forceinline__ void add(X64 x) { add(x_mant(x), x_exp(x)); }
+    __device__ __forceinline__ X64 value() const { return x_pack(s, e); }
 };
 
 // Order-preserving integer encodings for atomicMax on shared memory.

@@ -349,10 +349,10 @@ __global__ void k_gamma_table(int n, const float* __restrict__ F, float* __restr
 
 __device__ __forceinline__ float p2_add(float a, float b) { return LogOps<float>::lse(a, b); }
 __device__ __forceinline__ double p2_add(double a, double b) { return LogOps<double>::lse(a, b); }
-template <int FB> __device__ __forceinline__ XValue<FB> p2_add(XValue<FB> a, XValue<FB> b) { return x_add(a, b); }
+__device__ __forceinline__ X64 p2_add(X64 a, X64 b) { return x_add(a, b); }
 __device__ __forceinline__ void p2_zero(float& a) { a = LogOps<float>::ninf(); }
 __device__ __forceinline__ void p2_zero(double& a) { a = LogOps<double>::ninf(); }
-template <int FB> __device__ __forceinline__ void p2_zero(XValue<FB>& a) { a.u = 0ull; }
+__device__ __forceinline__ void p2_zero(X64& a) { a.u = 0ull; }
 
 template <typename T>
 __global__ void __launch_bounds__(256)
@@ -825,9 +825,9 @@ k_gamma_p2w(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const fl
 // The weight e(G) 2^qbits of family x, rounded: 0 without an exponential when
 // it is certainly below one half.
 struct EdgeScale {
-    double cv, lnfv, qscale, inv;                   // logs: c_v, ln F(V), 2^qbits; XValue: 1 / F(V)'s fraction
+    double cv, lnfv, qscale, inv;                   // logs: c_v, ln F(V), 2^qbits; X64: 1 / F(V)'s fraction
     float cut;                                      // FP32: log2 of a weight that rounds to 0
-    int eq;                                         // XValue: qbits - F(V)'s exponent
+    int eq;                                         // X64: qbits - F(V)'s exponent
 };
 __device__ __forceinline__ EdgeScale edge_scale(const float* F, int n, int qbits, double cv)
 {
@@ -842,9 +842,9 @@ __device__ __forceinline__ EdgeScale edge_scale(const double* F, int n, int qbit
     const double fv = F[(uint32_t)(((uint64_t)1 << n) - 1)];
     return {cv, fv, ldexp(1.0, qbits), 0.0, -0.69314718f * (float)(qbits + 3), 0};
 }
-template <int FB> __device__ __forceinline__ EdgeScale edge_scale(const XValue<FB>* F, int n, int qbits, double)
+__device__ __forceinline__ EdgeScale edge_scale(const X64* F, int n, int qbits, double)
 {
-    const XValue<FB> fv = F[(uint32_t)(((uint64_t)1 << n) - 1)];
+    const X64 fv = F[(uint32_t)(((uint64_t)1 << n) - 1)];
     return {0.0, 0.0, 0.0, 1.0 / x_mant(fv), 0.f, qbits - x_exp(fv)};
 }
 __device__ __forceinline__ unsigned long long edge_weight(const EdgeScale& s, double logB, float lb, float g)
@@ -859,8 +859,7 @@ __device__ __forceinline__ unsigned long long edge_weight(const EdgeScale& s, do
     if (x < (double)s.cut) return 0ull;
     return __double2ull_rn(exp(x) * s.qscale);
 }
-template <int FB>
-__device__ __forceinline__ unsigned long long edge_weight(const EdgeScale& s, double, XValue<FB> b, XValue<FB> g)
+__device__ __forceinline__ unsigned long long edge_weight(const EdgeScale& s, double, X64 b, X64 g)
 {
     const int e = x_exp(b) + x_exp(g) + s.eq;       // the weight is at most 2^qbits
     return e < -8 ? 0ull : __double2ull_rn(x_mant(b) * x_mant(g) * s.inv * pow2d(min(e, 64)));
@@ -874,9 +873,9 @@ __device__ __forceinline__ double ln_full(const float* F, int n)
                                 level_base_fwd(level_words(F, n), n - kLevelShift));
 }
 __device__ __forceinline__ double ln_full(const double* F, int n) { return F[((size_t)1 << n) - 1]; }
-template <int FB> __device__ __forceinline__ double ln_full(const XValue<FB>* F, int n)
+__device__ __forceinline__ double ln_full(const X64* F, int n)
 {
-    const XValue<FB> f = F[((size_t)1 << n) - 1];
+    const X64 f = F[((size_t)1 << n) - 1];
     return f.u ? (double)x_exp(f) * 0.69314718055994530942 + log(x_mant(f)) : -INFINITY;
 }
 template <typename T>
@@ -972,15 +971,14 @@ __device__ __forceinline__ void tail_input(double& y, const double* F, const dou
 {
     y = F[BN_AT(S, 1, full)] + Rc[BN_AT(S | bv, 1, full)];
 }
-template <int FB>
-__device__ __forceinline__ void tail_input(XValue<FB>& y, const XValue<FB>* F, const XValue<FB>* Rc, uint32_t S,
+__device__ __forceinline__ void tail_input(X64& y, const X64* F, const X64* Rc, uint32_t S,
                                            uint32_t bv, size_t full, const float*, int)
 {
     y = x_mul(F[BN_AT(S, 1, full)], Rc[BN_AT(S | bv, 1, full)]);
 }
 __device__ __forceinline__ void apply_weight(float& a, float w) { a += w; }
 __device__ __forceinline__ void apply_weight(double& a, double w) { a += w; }
-template <int FB> __device__ __forceinline__ void apply_weight(XValue<FB>& a, XValue<FB> w) { a = x_mul(a, w); }
+__device__ __forceinline__ void apply_weight(X64& a, X64 w) { a = x_mul(a, w); }
 
 template <typename T>
 __global__ void __launch_bounds__(1024)
@@ -1106,24 +1104,23 @@ __global__ void k_apply_q(int n, const T* __restrict__ lq, T* __restrict__ A, in
 }
 
 // ===========================================================================
-// The linear FP64 form (XValue, bn_device.cuh) of steps 2 (n < 14)
-// and 4.
+// The linear FP64 form (X64, bn_device.cuh) of steps 2 (n < 14) and 4.
 // ===========================================================================
 
 // Step 2 for n < 14: one block per node, every family in its slot of the
 // 2^(n-1) values in shared memory, then the butterflies of Algorithm 2.
 __global__ void __launch_bounds__(256)
-k_upzeta_x(int n, int64_t K, const uint32_t* __restrict__ cmasks, const X64S* __restrict__ lbs,
-           X64S* __restrict__ A, size_t js)
+k_upzeta_x(int n, int64_t K, const uint32_t* __restrict__ cmasks, const X64* __restrict__ lbs,
+           X64* __restrict__ A, size_t js)
 {
     cmasks = job_ptr(cmasks, js);
     lbs = job_ptr(lbs, js);
     A = job_ptr(A, js);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    X64S* v = reinterpret_cast<X64S*>(smem_raw);
+    X64* v = reinterpret_cast<X64*>(smem_raw);
     const uint32_t N = 1u << (n - 1);
     const int i = (int)blockIdx.x;
-    for (uint32_t t = threadIdx.x; t < N; t += blockDim.x) v[t] = X64S{0ull};
+    for (uint32_t t = threadIdx.x; t < N; t += blockDim.x) v[t] = X64{0ull};
     __syncthreads();
     for (int64_t f = threadIdx.x; f < K; f += blockDim.x)
         v[BN_AT(cmasks[(size_t)i * K + f], 1, N)] = lbs[(size_t)i * K + f];
@@ -1140,7 +1137,7 @@ k_upzeta_x(int n, int64_t K, const uint32_t* __restrict__ cmasks, const X64S* __
 }
 
 // Warp-wide sum of the lanes' LazySums, in a fixed tree order.
-template <typename X> __device__ __forceinline__ X warp_sum_x(LazySum<X> a)
+__device__ __forceinline__ X64 warp_sum_x(LazySum<X64> a)
 {
     for (int o = 16; o; o >>= 1) {
         const int e2 = __shfl_xor_sync(FULL, a.e, o);
@@ -1155,10 +1152,9 @@ template <typename X> __device__ __forceinline__ X warp_sum_x(LazySum<X> a)
 
 // Phase 2 for the columns with at most one high element left (k_gamma_p2s).
 // One unpacking per value of W; each sum it enters costs an aligned addition.
-template <typename X>
 __global__ void __launch_bounds__(256)
-k_gamma_p2s_x(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const X* __restrict__ W,
-              X* __restrict__ Gam, size_t js, uint32_t vsel)
+k_gamma_p2s_x(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const X64* __restrict__ W,
+              X64* __restrict__ Gam, size_t js, uint32_t vsel)
 {
     constexpr int MB = 14;                          // high bits from 5 up (h <= 18)
     const int v = blockIdx.z;
@@ -1174,11 +1170,11 @@ k_gamma_p2s_x(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const 
     while (r >= binom(b, kg)) { r -= binom(b, kg); ++kg; }
     const uint32_t g = colex_unrank(r, kg, b);
     const bool one = d - kg == 1;
-    LazySum<X> s0, sb[MB];
+    LazySum<X64> s0, sb[MB];
     const uint32_t nH = 1u << h;
     const size_t wsize = (size_t)nlow << h;
-    X wa = lane < nH ? W[BN_AT((size_t)lane * nlow + col, 1, wsize)] : X{0ull};
-    X wb = lane + 32 < nH ? W[BN_AT((size_t)(lane + 32) * nlow + col, 1, wsize)] : X{0ull};
+    X64 wa = lane < nH ? W[BN_AT((size_t)lane * nlow + col, 1, wsize)] : X64{0ull};
+    X64 wb = lane + 32 < nH ? W[BN_AT((size_t)(lane + 32) * nlow + col, 1, wsize)] : X64{0ull};
     for (uint32_t H = lane; H < nH; H += 32) {
         const double p = x_mant(wa);
         const int e = x_exp(wa);
@@ -1191,19 +1187,19 @@ k_gamma_p2s_x(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const 
                 if (5 + q < h && (H >> (5 + q) & 1u)) sb[q].add(p, e);
         }
     }
-    const X all = warp_sum_x(s0);
+    const X64 all = warp_sum_x(s0);
     if (lane == 0) Gam[BN_AT(family_index(g, n), 1, K)] = all;
     if (!one) return;
     for (int bb = 0; bb < h && bb < 5; ++bb) {
-        LazySum<X> s = s0;
-        if (!(lane >> bb & 1)) s = LazySum<X>();
-        const X x = warp_sum_x(s);
+        LazySum<X64> s = s0;
+        if (!(lane >> bb & 1)) s = LazySum<X64>();
+        const X64 x = warp_sum_x(s);
         if (lane == 0) Gam[BN_AT(family_index(g | (1u << (b + bb)), n), 1, K)] = x;
     }
 #pragma unroll
     for (int q = 0; q < MB; ++q) {
         if (5 + q >= h) break;
-        const X x = warp_sum_x(sb[q]);
+        const X64 x = warp_sum_x(sb[q]);
         if (lane == 0) Gam[BN_AT(family_index(g | (1u << (b + 5 + q)), n), 1, K)] = x;
     }
 }
@@ -1268,9 +1264,7 @@ cudaError_t launch_apply_q(const Plan& P, const void* lq, void* A, cudaStream_t 
 {
     const int64_t total = (int64_t)P.n << (P.n - 1);
     const int grid = grid_for(total, 256, 152 * 16);
-    if (P.lin == 2)
-        launch_or_record(KID_APPLY_Q_XS, k_apply_q<X64S>, grid, 256, 0, s, P.n, (const X64S*)lq, (X64S*)A, 0);
-    else if (P.lin)
+    if (P.lin)
         launch_or_record(KID_APPLY_Q_X, k_apply_q<X64>, grid, 256, 0, s, P.n, (const X64*)lq, (X64*)A, 0);
     else if (P.prec == 0)
         launch_or_record(KID_APPLY_Q_D, k_apply_q<double>, grid, 256, 0, s, P.n, (const double*)lq, (double*)A, 0);
@@ -1284,10 +1278,7 @@ cudaError_t launch_add_feature(const Plan& P, const void* lbs, const void* lf, v
                                cudaStream_t s)
 {
     const int64_t nK = (int64_t)P.n * P.K;
-    if (P.lin == 2)
-        launch_or_record(KID_ADD_FEATURE_XS, k_add_feature<X64S>, grid_for(nK, 256), 256, 0, s,
-            (const X64S*)lbs, (const X64S*)lf, (X64S*)out, nK);
-    else if (P.lin)
+    if (P.lin)
         launch_or_record(KID_ADD_FEATURE_X, k_add_feature<X64>, grid_for(nK, 256), 256, 0, s,
             (const X64*)lbs, (const X64*)lf, (X64*)out, nK);
     else if (P.prec == 0)
@@ -1325,8 +1316,8 @@ cudaError_t launch_upzeta(const Plan& P, const uint32_t* cmasks, const void* lbs
         return launch_upzeta13(P, tab, rk13 + 8192, A, s, sums_done, err);
     }
     if (P.lin)                                      // n < 14: a node per block
-        return launch_or_record(KID_UPZETA_XS, k_upzeta_x, dim3(P.n, P.nj), 256, (size_t)8 << (P.n - 1), s, P.n,
-                                P.K, cmasks, (const X64S*)lbs, (X64S*)A, P.js);
+        return launch_or_record(KID_UPZETA_X, k_upzeta_x, dim3(P.n, P.nj), 256, (size_t)8 << (P.n - 1), s, P.n,
+                                P.K, cmasks, (const X64*)lbs, (X64*)A, P.js);
     const int h = P.n - 1 - P.b_up;
     const dim3 grid((unsigned)P.n << h, P.nj);
     const size_t sm = upzeta_smem_bytes(P);
@@ -1520,7 +1511,7 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, const void*
         const int h2 = P.n - 1 - P.b_g;             // high bits
         const dim3 grid((P.nlow_g - c0 + 7) / 8, P.nj, P.n);
         if (P.lin)
-            launch_or_record(KID_GAMMA_P2S_X, k_gamma_p2s_x<X64>, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
+            launch_or_record(KID_GAMMA_P2S_X, k_gamma_p2s_x, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
                              (const X64*)W, (X64*)Gam, P.js, P.vsel);
         else if (P.prec != 0 && h2 >= 8)
             launch_or_record(KID_GAMMA_P2W, k_gamma_p2w, grid, 256, 0, s, P.n, P.d, P.b_g, P.nlow_g, c0, P.K,
@@ -1544,21 +1535,17 @@ static cudaError_t edges(const Plan& P, int kid, int kid_tail, const double* log
                          const void* F, const void* Rc, const void* lq, const int* err, unsigned long long* acc,
                          double* post, double* log_PD, cudaStream_t s)
 {
-    // (the linear forms have one of the two: X64 from n = 14, X64S below)
-    if constexpr (!std::is_same<T, X64>::value) if (use_tail(P)) {
+    if (use_tail(P)) {
         // a thread per pair of values, at most 1024
         const unsigned tb = rec_block((unsigned)std::min(1024, std::max(128, (1 << (P.n - 1)) >> 1)));
         return launch_or_record(kid_tail, k_tail<T>, dim3(P.n, P.nj), tb, sizeof(T) << (P.n - 1), s, P.n, P.d, P.K,
                                 fixed_bits(P.K), (const T*)F, (const T*)Rc, (const T*)lq, logB, (const T*)lbs, cmax,
                                 masks, cmasks, (T*)Gam, err, post, log_PD, P.js, P.vsel);
     }
-    if constexpr (std::is_same<T, X64S>::value) return cudaErrorInvalidValue;
-    else {
     const unsigned chunks = (unsigned)std::min<int64_t>((P.K + 1023) / 1024, 64);
     return launch_or_record(kid, k_edges<T>, dim3(chunks, P.nj, P.n), 256, 0, s, P.n, P.K, fixed_bits(P.K), logB,
                             (const T*)lbs, cmax, masks, (const T*)Gam, (const T*)F, err, acc, post, log_PD, P.js,
                             P.vsel);
-    }
 }
 
 cudaError_t launch_edges(const Plan& P, const double* logB, const void* lbs, const double* cmax,
@@ -1566,11 +1553,8 @@ cudaError_t launch_edges(const Plan& P, const double* logB, const void* lbs, con
                          const void* lq, const int* err, unsigned long long* acc, double* post, double* log_PD,
                          cudaStream_t s)
 {
-    if (P.lin == 2)
-        return edges<X64S>(P, KID_NONE, KID_TAIL_XS, logB, lbs, cmax, masks, cmasks, Gam, F, Rc, lq, err, acc,
-                           post, log_PD, s);
     if (P.lin)
-        return edges<X64>(P, KID_EDGES_X, KID_NONE, logB, lbs, cmax, masks, cmasks, Gam, F, Rc, lq, err, acc, post,
+        return edges<X64>(P, KID_EDGES_X, KID_TAIL_X, logB, lbs, cmax, masks, cmasks, Gam, F, Rc, lq, err, acc, post,
                           log_PD, s);
     if (P.prec == 0)
         return edges<double>(P, KID_EDGES_D, KID_TAIL_D, logB, lbs, cmax, masks, cmasks, Gam, F, Rc, lq, err, acc,
@@ -1613,7 +1597,7 @@ cudaError_t set_kernel_attributes()
     SETA(k_gamma_p2r<1>)
     SETA(k_tail<float>)
     SETA(k_tail<double>)
-    SETA(k_tail<X64S>)
+    SETA(k_tail<X64>)
 #undef SETA
     e = set_scores_attributes();
     if (e != cudaSuccess) return e;

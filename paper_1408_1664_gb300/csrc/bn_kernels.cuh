@@ -34,8 +34,7 @@ enum KernelId : int32_t {
     KID_G13_F, KID_FROWS_D, KID_FROWS_F_TLO, KID_FROWS_F, KID_BROWS_D, KID_BROWS_F_TLO,
     KID_BROWS_F, KID_COLB4_D, KID_COLB2_D, KID_COLB1_D, KID_COLB1,
     // the linear FP64 form
-    KID_SHIFT_XS, KID_APPLY_Q_XS, KID_ADD_FEATURE_XS, KID_UPZETA_XS, KID_FROWS_XS, KID_BROWS_XS,
-    KID_TAIL_F, KID_TAIL_D, KID_TAIL_XS,
+    KID_UPZETA_X, KID_TAIL_F, KID_TAIL_D, KID_TAIL_X,
     KID_SHIFT_X, KID_APPLY_Q_X, KID_ADD_FEATURE_X, KID_REORDER_X, KID_COLB4_X, KID_COLB2_X,
     KID_COLB1_X, KID_COLW_X, KID_UP13_X, KID_FROWS_X, KID_BROWS_X, KID_G13_X_Q, KID_G13_X,
     KID_GAMMA_P2_X, KID_GAMMA_P2S_X, KID_EDGES_X,
@@ -199,16 +198,17 @@ inline void set_states(Plan& P, const uint32_t* sorted)
     }
 }
 
-// Whether an FP64 job may keep its values linear (Plan::lin): 1 in X64 (n >=
-// 14), 2 in X64S (n < 14), 0 as logarithms.  With the nodes' scores shifted
+// Whether an FP64 job may keep its values linear (Plan::lin).  With the nodes' scores shifted
 // by their maxima the values lie below 2^1000, and only those within reach of
 // F(V) matter; F(V) is at least the weight of the empty parent sets, Prod_i
 // B_i(empty) / c_i, and that is bounded per node by m log2 r + r log2(r (1 +
 // m / ess)) bits of score and by `logs`, the largest magnitude of the job's own
-// (finite) log weights per node in nats.  118000 (12500) bits leave 9000
-// (1800) for the products beside F(V).  Lattices whose tiles do not fit keep
+// (finite) log weights per node in nats.  118000 bits leave 10000 of the range
+// for the products beside F(V).  Above, no value exceeds n! K^n (every order,
+// every A_i at most K) times e^up, `up` the sum over the nodes of their largest
+// order-prior and feature weights above 1, in nats.  Lattices whose tiles do not fit keep
 // the logarithms.
-inline int lin_range(const Plan& P, const uint8_t* arity, double ess, double logs)
+inline int lin_range(const Plan& P, const uint8_t* arity, double ess, double logs, double up)
 {
     if (P.prec != 0 || P.n < 5 || P.n > 31) return 0;
     if (P.n >= 14 && !(P.up13 && P.g13)) return 0;
@@ -217,8 +217,8 @@ inline int lin_range(const Plan& P, const uint8_t* arity, double ess, double log
         const double r = arity[i];
         bits += P.m * std::log2(r) + r * std::log2(r * (1.0 + P.m / ess) + 2.0) + 2.8854 * logs;
     }
-    if (P.n >= 14) return bits < 118000.0 ? 1 : 0;
-    return bits < 12500.0 ? 2 : 0;
+    const double above = P.n * std::log2((double)P.K) + 1.4427 * (std::lgamma(P.n + 1.0) + up);
+    return bits < 118000.0 && above < 1000.0;
 }
 
 // Host check of m x n row-major data: every value below its variable's

@@ -69,7 +69,7 @@ __device__ __forceinline__ void lazy_add(double& m, double& s, double x)
 
 // The sum of one subset's terms A * F: (m, s) as above for logarithms (an
 // empty sum has m far below any value, finite so that a left-out term of -inf
-// changes nothing), LazySum for XValue.  add() takes a term or leaves it out.
+// changes nothing), LazySum for X64.  add() takes a term or leaves it out.
 template <typename T> struct TileSum {
     T m = (T)-3.0e38f, s = T(0);
     __device__ __forceinline__ void add(T a, T f, bool take = true)
@@ -79,20 +79,18 @@ template <typename T> struct TileSum {
     __device__ __forceinline__ void rebase(T r) { m -= r; }
     __device__ __forceinline__ T value() const { return m + LogOps<T>::lg(s); }
 };
-template <int FB> struct TileSum<XValue<FB>> {
-    using X = XValue<FB>;
-    LazySum<X> v;
-    __device__ __forceinline__ void add(X a, X f, bool take = true)
+template <> struct TileSum<X64> {
+    LazySum<X64> v;
+    __device__ __forceinline__ void add(X64 a, X64 f, bool take = true)
     {
         const double p = x_mant(a) * x_mant(f);
         v.add(take ? p : 0.0, take ? x_exp(a) + x_exp(f) : -(1 << 28));
     }
-    __device__ __forceinline__ void rebase(X) {}
-    __device__ __forceinline__ X value() const { return v.value(); }
+    __device__ __forceinline__ void rebase(X64) {}
+    __device__ __forceinline__ X64 value() const { return v.value(); }
 };
 template <typename T> __device__ __forceinline__ T unit() { return T(0); }         // log 1
-template <> __device__ __forceinline__ X64 unit<X64>() { return x_one<X64>(); }
-template <> __device__ __forceinline__ X64S unit<X64S>() { return x_one<X64S>(); }
+template <> __device__ __forceinline__ X64 unit<X64>() { return x_one(); }
 
 // x with bit i (i < B) removed: an index among the 2^(B-1) B-bit patterns
 // without bit i.
@@ -132,8 +130,8 @@ __device__ __forceinline__ void load_row(const double* p, double (&v)[N], int mo
     }
 }
 
-template <int N, int FB>
-__device__ __forceinline__ void load_row(const XValue<FB>* p, XValue<FB> (&v)[N], int mode)
+template <int N>
+__device__ __forceinline__ void load_row(const X64* p, X64 (&v)[N], int mode)
 {
     const ulonglong2* q = reinterpret_cast<const ulonglong2*>(p);
 #pragma unroll
@@ -149,15 +147,15 @@ __device__ __forceinline__ float load_one(const float* p, int mode)
 {
     return mode == LD_STREAM ? __ldcs(p) : mode == LD_L2 ? __ldcg(p) : *p;
 }
-template <int FB> __device__ __forceinline__ XValue<FB> load_one(const XValue<FB>* p, int mode)
+__device__ __forceinline__ X64 load_one(const X64* p, int mode)
 {
     const unsigned long long* q = &p->u;
-    return XValue<FB>{mode == LD_STREAM ? __ldcs(q) : mode == LD_L2 ? __ldcg(q) : *q};
+    return X64{mode == LD_STREAM ? __ldcs(q) : mode == LD_L2 ? __ldcg(q) : *q};
 }
 __device__ __forceinline__ float shfl_one(unsigned mask, float v, int o) { return __shfl_xor_sync(mask, v, o); }
-template <int FB> __device__ __forceinline__ XValue<FB> shfl_one(unsigned mask, XValue<FB> v, int o)
+__device__ __forceinline__ X64 shfl_one(unsigned mask, X64 v, int o)
 {
-    return XValue<FB>{__shfl_xor_sync(mask, v.u, o)};
+    return X64{__shfl_xor_sync(mask, v.u, o)};
 }
 
 template <int N>
@@ -176,8 +174,8 @@ __device__ __forceinline__ void store_row(double* p, const double (&v)[N])
     for (int k = 0; k < N / 2; ++k) q[k] = make_double2(v[2 * k], v[2 * k + 1]);
 }
 
-template <int N, int FB>
-__device__ __forceinline__ void store_row(XValue<FB>* p, const XValue<FB> (&v)[N])
+template <int N>
+__device__ __forceinline__ void store_row(X64* p, const X64 (&v)[N])
 {
     ulonglong2* q = reinterpret_cast<ulonglong2*>(p);
 #pragma unroll
@@ -941,7 +939,6 @@ static cudaError_t rows_level(const Plan& P, int sweep, int hl, uint32_t nt, uns
         return cudaGetLastError();
     }
     const int kid = std::is_same<T, X64>::value ? (sweep == 0 ? KID_FROWS_X : KID_BROWS_X)
-                    : std::is_same<T, X64S>::value ? (sweep == 0 ? KID_FROWS_XS : KID_BROWS_XS)
                     : sizeof(T) == 8 ? (sweep == 0 ? KID_FROWS_D : KID_BROWS_D)
                     : TLO ? (sweep == 0 ? KID_FROWS_F_TLO : KID_BROWS_F_TLO)
                           : (sweep == 0 ? KID_FROWS_F : KID_BROWS_F);
@@ -959,7 +956,6 @@ cudaError_t launch_rows_level(const Plan& P, int sweep, int hl, const void* A, v
     if (nt == 0) return cudaSuccess;
     const unsigned tb = rec_block(level_block(nt));
     const dim3 grid((nt + tb - 1) / tb, P.nj);
-    if (P.lin == 2) return rows_level<X64S, false>(P, sweep, hl, nt, tb, grid, A, X, Atop, s);
     if (P.lin) return rows_level<X64, false>(P, sweep, hl, nt, tb, grid, A, X, Atop, s);
     if (P.prec == 0) return rows_level<double, false>(P, sweep, hl, nt, tb, grid, A, X, Atop, s);
     if (use_tlo(P)) return rows_level<float, true>(P, sweep, hl, nt, tb, grid, A, X, Atop, s);
@@ -1111,8 +1107,7 @@ cudaError_t launch_sweeps(const Plan& P, const void* A, void* F, void* Rc, cudaS
 {
     if (P.n > kSweepPlacesN) return cudaErrorInvalidValue;
     const int items = Rc ? 2 * P.nj : 1;            // a feature's job: F alone
-    const cudaError_t e = P.lin == 2 ? sweeps<X64S, false>(P, (const X64S*)A, (X64S*)F, (X64S*)Rc, items, s, err)
-                          : P.lin ? sweeps<X64, false>(P, (const X64*)A, (X64*)F, (X64*)Rc, items, s, err)
+    const cudaError_t e = P.lin ? sweeps<X64, false>(P, (const X64*)A, (X64*)F, (X64*)Rc, items, s, err)
                           : use_tlo(P) ? sweeps<float, true>(P, (const float*)A, (float*)F, (float*)Rc, items, s, err)
                                      : sweeps<float, false>(P, (const float*)A, (float*)F, (float*)Rc, items, s, err);
     if (e == cudaSuccess && launches) ++*launches;

@@ -150,11 +150,8 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
     } else {
         switch (kid) {
         case KID_SHIFT_X: run(k_shift_scores<X64>, a); return true;
-        case KID_SHIFT_XS: run(k_shift_scores<X64S>, a); return true;
-        case KID_UPZETA_XS: run(k_upzeta_x, a); return true;
-        case KID_FROWS_XS: run(k_forward_rows<X64S, false>, a); return true;
-        case KID_BROWS_XS: run(k_backward_rows<X64S, false>, a); return true;
-        case KID_TAIL_XS: run(k_tail<X64S>, a); return true;
+        case KID_UPZETA_X: run(k_upzeta_x, a); return true;
+        case KID_TAIL_X: run(k_tail<X64>, a); return true;
         case KID_REORDER_X: run(k_reorder_up<X64>, a); return true;
         case KID_COLB4_X: run(k_colb_x<4>, a); return true;
         case KID_COLB2_X: run(k_colb_x<2>, a); return true;
@@ -165,7 +162,7 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
         case KID_BROWS_X: run(k_backward_rows<X64, false>, a); return true;
         case KID_G13_X: run(k_g13_x<false>, a); return true;
         case KID_GAMMA_P2_X: run(k_gamma_p2<X64>, a); return true;
-        case KID_GAMMA_P2S_X: run(k_gamma_p2s_x<X64>, a); return true;
+        case KID_GAMMA_P2S_X: run(k_gamma_p2s_x, a); return true;
         case KID_EDGES_X: run(k_edges<X64>, a); return true;
         case KID_SHIFT_D: run(k_shift_scores<double>, a); return true;
         case KID_UPZETA_D: run(k_upzeta<double>, a); return true;
@@ -309,7 +306,7 @@ bool persistent_runs(int prec, int kid)
     case KID_GAMMA_P1_D: case KID_GAMMA_P2_D: case KID_GAMMA_P2S_D: case KID_EDGES_D: case KID_TAIL_D: case KID_REORDER_D: case KID_COLW_D: case KID_COLS_D: case KID_UP13_D:
     case KID_COLB4_D: case KID_COLB2_D: case KID_COLB1_D:
     case KID_G13_D: case KID_FROWS_D: case KID_BROWS_D:
-    case KID_SHIFT_XS: case KID_UPZETA_XS: case KID_FROWS_XS: case KID_BROWS_XS: case KID_TAIL_XS:
+    case KID_UPZETA_X: case KID_TAIL_X:
     case KID_SHIFT_X: case KID_REORDER_X: case KID_COLB4_X: case KID_COLB2_X:
     case KID_COLB1_X: case KID_COLW_X: case KID_UP13_X: case KID_FROWS_X: case KID_BROWS_X:
     case KID_G13_X: case KID_GAMMA_P2_X: case KID_GAMMA_P2S_X:

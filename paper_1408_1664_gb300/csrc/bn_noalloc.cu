@@ -194,7 +194,7 @@ try {
     bn::default_schedule(P);
     double rho_max = 0.0;
     for (int k = 0; k <= P.d; ++k) rho_max = std::fmax(rho_max, std::fabs(log_rho[k]));
-    P.lin = bn::lin_tiles_fit(P) ? bn::lin_range(P, arity, j->ess, rho_max) : 0;
+    P.lin = bn::lin_tiles_fit(P) ? bn::lin_range(P, arity, j->ess, rho_max, 0.0) : 0;
 
     // layout inside the static array
     const size_t es = P.prec == 0 ? 8 : 4;

@@ -166,29 +166,22 @@ int log_weights(const double* src, size_t count, std::vector<double>& dst)
     return bad ? BN_EINVAL : BN_OK;
 }
 
-// exp(x) of a natural log as an XValue (bn_device.cuh), and back (host).
-template <typename X> unsigned long long x_from_ln(double x)
+// exp(x) of a natural log as an X64 (bn_device.cuh), and back (host).
+unsigned long long x_from_ln(double x)
 {
     if (!(x > -91000.0)) return 0ull;
     int e = (int)std::lround(x * 1.4426950408889634074);
-    const double r = (x - e * bn::explog::kLn2Hi) - e * bn::explog::kLn2Lo;
+    const double r = std::fma((double)-e, bn::explog::kLn2Lo, std::fma((double)-e, bn::explog::kLn2Hi, x));
     int e2 = 0;
     const double m = std::frexp(std::exp(r), &e2) * 2.0;    // [1, 2)
     e += e2 - 1;
-    unsigned long long f = (unsigned long long)std::llround(std::ldexp(m, X::frac));
-    if (f >> (X::frac + 1)) { f >>= 1; ++e; }
-    if (e < X::min) return 0ull;
-    return ((unsigned long long)(e + X::bias) << X::frac) | (f & ((1ull << X::frac) - 1));
+    return e < bn::kXMin ? 0ull : bn::x_code(e, (unsigned long long)std::ldexp(m - 1.0, 52));
 }
-template <typename X> double x_to_ln(unsigned long long u)
+double x_to_ln(unsigned long long u)
 {
     if (!u) return -INFINITY;
-    const double m = 1.0 + std::ldexp((double)(u & ((1ull << X::frac) - 1)), -X::frac);
-    return ((double)((int)(u >> X::frac) - X::bias)) * 0.69314718055994530942 + std::log(m);
-}
-double lin_to_ln(const Plan& P, unsigned long long u)
-{
-    return P.lin == 2 ? x_to_ln<bn::X64S>(u) : x_to_ln<bn::X64>(u);
+    const double f = std::ldexp((double)(u & ((1ull << 52) - 1)), -52);
+    return (double)bn::x_exp(bn::X64{u}) * 0.69314718055994530942 + std::log1p(f);
 }
 
 // In the form of the plan's values: FP32 base-2 logs, FP64 natural logs or
@@ -198,7 +191,7 @@ std::vector<char> working_logs(const std::vector<double>& v, const Plan& P)
     std::vector<char> out(v.size() * (P.prec == 0 ? 8 : 4));
     if (P.lin) {
         unsigned long long* u = reinterpret_cast<unsigned long long*>(out.data());
-        for (size_t t = 0; t < v.size(); ++t) u[t] = P.lin == 2 ? x_from_ln<bn::X64S>(v[t]) : x_from_ln<bn::X64>(v[t]);
+        for (size_t t = 0; t < v.size(); ++t) u[t] = x_from_ln(v[t]);
     } else if (P.prec == 0) {
         std::memcpy(out.data(), v.data(), out.size());
     } else {
@@ -217,15 +210,26 @@ double largest_log(const std::vector<double>& v)
     return x;
 }
 
-// Whether the job's values stay linear (FP64; more: a feature's log weights).
+// The sum over the nodes of their largest log weight above 0.
+double sum_above(const std::vector<double>& v, int n)
+{
+    const size_t per = v.size() / n;
+    double x = 0.0;
+    for (int i = 0; per && i < n; ++i)
+        x += std::max(0.0, *std::max_element(v.begin() + i * per, v.begin() + (i + 1) * per));
+    return x;
+}
+
+// Whether the job's values stay linear (FP64; lf: a feature's log weights).
 // A zero weight on an empty parent set leaves F(V) without its lower bound.
-void plan_lin(HostJob& hj, double more)
+void plan_lin(HostJob& hj, const std::vector<double>& lf)
 {
     Plan& P = hj.P;
     P.lin = 0;
     if (P.prec != 0) return;
-    const double logs = largest_log(hj.log_rho) + largest_log(hj.log_q) + largest_log(hj.log_w) + more;
-    P.lin = bn::lin_tiles_fit(P) ? bn::lin_range(P, hj.arity.data(), hj.ess, logs) : 0;
+    const double logs = largest_log(hj.log_rho) + largest_log(hj.log_q) + largest_log(hj.log_w) + largest_log(lf);
+    const double up = sum_above(hj.log_q, P.n) + sum_above(lf, P.n);
+    P.lin = bn::lin_tiles_fit(P) ? bn::lin_range(P, hj.arity.data(), hj.ess, logs, up) : 0;
     if (P.hasw)
         for (int i = 0; i < P.n; ++i)
             if (hj.log_w[(size_t)i * P.K] < 0.5 * kLogZero) P.lin = 0;
@@ -289,7 +293,7 @@ int validate_and_plan(const bn_job_desc* j, HostJob& hj)
     P.nlow_g = (uint32_t)nl;
     P.wb = std::min(P.n, 5);
     bn::default_schedule(P);
-    plan_lin(hj, 0.0);
+    plan_lin(hj, {});
     return BN_OK;
 }
 
@@ -1171,7 +1175,7 @@ try {
     const Plan& P = hj.P;
     std::vector<double> lf;
     if (log_weights(log_f, (size_t)P.n * P.K, lf)) return BN_EINVAL;
-    plan_lin(hj, largest_log(lf));
+    plan_lin(hj, lf);
     if (cudaSetDevice(c->device) != cudaSuccess) return BN_ECUDA;
     const Layout L = make_layout(P, 0, true);
     rc = ensure_ws(c, L.total);
@@ -1243,7 +1247,7 @@ try {
         if (P.lin) {
             unsigned long long u;
             std::memcpy(&u, raw[k], 8);
-            fv[k] = lin_to_ln(P, u);
+            fv[k] = x_to_ln(u);
         } else if (P.prec == 0) {
             std::memcpy(&fv[k], raw[k], 8);
         } else {
@@ -1416,7 +1420,7 @@ try {
         for (size_t t = 0; t < want / 8; ++t) {
             unsigned long long u;
             std::memcpy(&u, x + t, 8);
-            x[t] = lin_to_ln(P, u);
+            x[t] = x_to_ln(u);
         }
     }
     if (P.prec != 0 && (stage == BN_STAGE_F || stage == BN_STAGE_RC || stage == BN_STAGE_GAMMA))
@@ -1633,7 +1637,6 @@ int record_groups(bn_batch* b)
                 case bn::KID_STEP1_PREP: case bn::KID_CHECK_DATA: case bn::KID_SET_HIST_WARP:
                 case bn::KID_SET_HIST_BLOCK: case bn::KID_SET_ANY: case bn::KID_FAMILIES:
                 case bn::KID_SHIFT_F: case bn::KID_SHIFT_D: case bn::KID_SHIFT_X: case bn::KID_EDGES_X:
-                case bn::KID_SHIFT_XS:
                 case bn::KID_REORDER_X: case bn::KID_COLW_X: case bn::KID_EDGES_F: case bn::KID_EDGES_D: case bn::KID_REORDER_F: case bn::KID_REORDER_D:
                 case bn::KID_COLW_F: case bn::KID_COLW_D:
                     x.pad[0] |= bn::kRecStrideX;
@@ -1644,11 +1647,11 @@ int record_groups(bn_batch* b)
                 pp.smem = std::max<size_t>(pp.smem, x.smem);
                 const bool f = x.kid == bn::KID_FROWS_F || x.kid == bn::KID_FROWS_F_TLO ||
                                x.kid == bn::KID_FROWS_D || x.kid == bn::KID_FROWS_X ||
-                               x.kid == bn::KID_FROWS_XS || x.kid == bn::KID_FWD_LEVEL_F ||
+                               x.kid == bn::KID_FWD_LEVEL_F ||
                                x.kid == bn::KID_FWD_LEVEL_D;
                 const bool r = x.kid == bn::KID_BROWS_F || x.kid == bn::KID_BROWS_F_TLO ||
                                x.kid == bn::KID_BROWS_D || x.kid == bn::KID_BROWS_X ||
-                               x.kid == bn::KID_BROWS_XS || x.kid == bn::KID_BWD_LEVEL_F ||
+                               x.kid == bn::KID_BWD_LEVEL_F ||
                                x.kid == bn::KID_BWD_LEVEL_D;
                 if (f || r) {
                     if (level_at == SIZE_MAX) level_at = stages.size();

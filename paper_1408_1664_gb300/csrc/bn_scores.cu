@@ -758,10 +758,10 @@ k_family_scores(int n, int64_t K, const long long* __restrict__ H, uint32_t nset
 
 __device__ __forceinline__ void from_ln(double x, float& y) { y = (float)LogOps<float>::from_ln(x); }
 __device__ __forceinline__ void from_ln(double x, double& y) { y = x; }
-template <int FB> __device__ __forceinline__ void from_ln(double x, XValue<FB>& y) { y = x_from_ln<XValue<FB>>(x); }
+__device__ __forceinline__ void from_ln(double x, X64& y) { y = x_from_ln(x); }
 
 // The shifted scores lbs = log B - c_i in the working precision and base
-// (XValue: B / exp(c_i)),
+// (X64: B / exp(c_i)),
 // the shifts cmax themselves (from their encodings), and, for the
 // 13-dimension up-zeta tiles (tab not null), the same scores reordered by
 // high and low part of the parent set (see k_reorder_up).
@@ -1008,9 +1008,6 @@ cudaError_t launch_shift_scores(const Plan& P, const double* logB, const unsigne
                                 const uint32_t* cmasks, double* cmax, void* lbs, void* tab, cudaStream_t s)
 {
     const dim3 grid(grid_for((int64_t)P.n * P.K, 256, 152 * 16), P.nj);
-    if (P.lin == 2)
-        return launch_or_record(KID_SHIFT_XS, k_shift_scores<X64S>, grid, 256, 0, s, P.n, P.d, P.K, logB, enc,
-                                cmasks, cmax, (X64S*)lbs, (X64S*)nullptr, P.js);
     if (P.lin)
         return launch_or_record(KID_SHIFT_X, k_shift_scores<X64>, grid, 256, 0, s, P.n, P.d, P.K, logB, enc,
                                 cmasks, cmax, (X64*)lbs, (X64*)tab, P.js);

@@ -1698,7 +1698,7 @@ k_colb_x(int n, int d, int64_t K, const X64* __restrict__ tab, X64* __restrict__
                 return lin_s[q] ? plus(a, b) : x_add(a, b);
             }) : *at;
             Ai[BN_AT(((size_t)(Hc | H) << TB) + c, 1, (size_t)1 << (n - 1))] =
-                lin_s[cc] ? x_pack<X64>(__longlong_as_double((long long)x.u), ref_s[cc]) : x;
+                lin_s[cc] ? x_pack(__longlong_as_double((long long)x.u), ref_s[cc]) : x;
         }
     }
     if (hc) cluster_sync();                          // no peer reads this block's values any more
@@ -1754,14 +1754,14 @@ k_up13_x(int n, int d, const uint16_t* __restrict__ rank13, X64* __restrict__ A,
                 ulonglong2* p = reinterpret_cast<ulonglong2*>(out + el3(8 * q, t));
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    p[k] = make_ulonglong2(x_pack<X64>(x[8 * q + 2 * k], ref).u, x_pack<X64>(x[8 * q + 2 * k + 1], ref).u);
+                    p[k] = make_ulonglong2(x_pack(x[8 * q + 2 * k], ref).u, x_pack(x[8 * q + 2 * k + 1], ref).u);
             }
             return;
         }
 #pragma unroll
         for (int r = 0; r < TR; ++r)
             if (!(done >> r & 1u) && (last || x[r] >= pow2d(kXKeep))) {
-                out[el3(r, t)] = x_pack<X64>(x[r], ref);
+                out[el3(r, t)] = x_pack(x[r], ref);
                 done |= 1u << r;
             }
         if (last) return;
@@ -1799,7 +1799,7 @@ k_g13_x(int n, int d, uint32_t nlow, const X64* __restrict__ F, const X64* __res
                                               (size_t)n << (n - 1))];
         // the bound is the sum of B_v: A_v without its factor q_v (unknown when
         // that is zero)
-        const X64 q = Q ? lq[v * n + __popc(H) + TB] : x_one<X64>();
+        const X64 q = Q ? lq[v * n + __popc(H) + TB] : x_one();
         if (at.u && q.u) L = max(L, x_exp(F[((size_t)1 << n) - 1]) - x_exp(at) + x_exp(q) - 2 - margin);
     }
     // s of the full tile set, the smallest output, is a load of its own: the
@@ -1827,8 +1827,7 @@ k_g13_x(int n, int d, uint32_t nlow, const X64* __restrict__ F, const X64* __res
                 e += x_exp(q);
             }
             mx = max(mx, e);
-            const int k = e - ref;
-            x[r] = k > 1000 ? __longlong_as_double(0x7ff0000000000000ll) : k < -1000 ? 0.0 : p * pow2d(k);
+            x[r] = p * pow2d(min(e - ref, 1024));    // 0 or +inf outside a double's range
             // sixteen values' loads in flight: more would spill
             if ((r & 15) == 15) asm volatile("" ::: "memory");
         }
@@ -1863,7 +1862,7 @@ k_g13_x(int n, int d, uint32_t nlow, const X64* __restrict__ F, const X64* __res
         for (uint32_t c = t; c < nlow; c += TT, ++k) {
             const double o = A0[swz(BN_AT(unrank13[c], 1, TN))];
             if (!(done >> k & 1u) && (last || o >= pow2d(kXKeep))) {
-                row[BN_AT(c, 1, nlow)] = x_pack<X64>(o, ref);
+                row[BN_AT(c, 1, nlow)] = x_pack(o, ref);
                 done |= 1u << k;
             }
         }
