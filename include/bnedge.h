@@ -458,6 +458,13 @@ int bn_debug_bounds(int32_t* line, int32_t* unit);
  * host doubles x: out (4 * count host doubles) receives, per x, the
  * library's exp, CUDA's exp, the library's log, CUDA's log. */
 int bn_debug_explog(const double* x, int64_t count, double* out);
+/* Phase 2 of an FP32 job's down-zeta (n >= 14) on given inputs: W, n endpoints
+ * of 2^(n-14) rows (the sets of the top n-14 bits) of the sums over the low 13
+ * bits (the sets of at most d of them, by size, then colexicographically),
+ * host floats (log2); Gamma, n*K host floats, receives the log2 of the sums
+ * over the rows that contain a family's high part.  The job gives n, d and
+ * the samples' shape only. */
+int bn_debug_phase2(const bn_job_desc* job, const float* W, float* Gamma);
 /* What the host planned for a job (no GPU needed): `count` values, the first
  * of the enumeration below, go to out.  BN_EINVAL for an invalid job or a
  * count beyond it. */

@@ -69,7 +69,7 @@ EXPORTS = ["bn_ctx_create", "bn_ctx_destroy", "bn_num_families", "bn_scores",
 
 # Test hooks: exported only by the testing build (BN_TESTING).
 TEST_EXPORTS = ["bn_debug_stage", "bn_debug_counts", "bn_debug_batch_drop", "bn_debug_bounds",
-                "bn_debug_explog", "bn_debug_copy_wait", "bn_debug_plan"]
+                "bn_debug_explog", "bn_debug_copy_wait", "bn_debug_plan", "bn_debug_phase2"]
 BN_PLAN_SWEEPS, BN_PLAN_COUNT = range(2)
 
 
@@ -149,6 +149,7 @@ def load(build_if_missing: bool = False) -> C.CDLL:
         "bn_debug_bounds": (C.c_int, [C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
         "bn_debug_explog": (C.c_int, [P, C.c_int64, P]),
         "bn_debug_copy_wait": (C.c_int, [C.c_uint32, C.POINTER(C.c_int32)]),
+        "bn_debug_phase2": (C.c_int, [C.POINTER(bn_job_desc), P, P]),
         "bn_debug_plan": (C.c_int, [C.POINTER(bn_job_desc), C.POINTER(C.c_int32), C.c_int32]),
         "bn_shard_create": (C.c_int, [P, C.POINTER(bn_job_desc), C.c_int32, C.c_int32, C.c_int32,
                                       C.POINTER(P)]),
@@ -363,6 +364,16 @@ def bn_debug_bounds() -> tuple[int, int]:
     if rc:
         raise BnError(rc, "bn_debug_bounds")
     return int(line.value), int(unit.value)
+
+
+def bn_debug_phase2(job: Job, W: np.ndarray) -> np.ndarray:
+    """Phase 2 of the down-zeta on given inputs, FP32: n x K log2 sums."""
+    W = np.ascontiguousarray(W, np.float32)
+    out = np.zeros((job.n, bn_num_families(job.n, job.d)), np.float32)
+    rc = load().bn_debug_phase2(C.byref(job.desc), _ptr(W), _ptr(out))
+    if rc:
+        raise BnError(rc, "bn_debug_phase2")
+    return out
 
 
 def bn_debug_plan(job: Job) -> list[int]:

@@ -466,7 +466,42 @@ __device__ __forceinline__ void p2_steps(float* v, uint32_t H2, uint32_t HS, int
     }
 }
 
+// Logarithms and sums in the scale of an integer (2^ref, as the sums of a
+// pass).  The integer part of a logarithm goes straight into the exponent and
+// back: w - ref itself is rounded to the bits of a number of up to 126 (2^-18)
+// where w may have more, and so is the logarithm of a sum of up to 2^126.
 __device__ __forceinline__ int p2_mag(float w) { return w > -2.0e9f ? (int)floorf(w) : -2000000000; }
+__device__ __forceinline__ float p2_pow2(int k)    // 2^k; 0 below 2^-126, +inf above 2^127
+{
+    return __uint_as_float((unsigned)(min(max(k, -127), 128) + 127) << 23);
+}
+struct P2Scale {
+    // w - ref is exact from |ref| = 2^21 on; below, the integer part of w comes
+    // from an addition that rounds to it (1.5 2^23: the low bits hold it)
+    float base, low;
+    int bias;
+    __device__ __forceinline__ explicit P2Scale(int ref)
+    {
+        const bool wide = abs(ref) > (1 << 21);
+        base = wide ? (float)ref : 0.0f;
+        const int i = wide ? 0 : ref;
+        low = (float)(i - 127);
+        bias = 127 - i;
+    }
+    // 2^(w - ref): 0 below 2^-126, +inf above 2^127 (TOP: w may lie there)
+    template <bool TOP> __device__ __forceinline__ float value(float w) const
+    {
+        w = fmaxf(w - base, low);
+        if (TOP) w = fminf(w, low + 255.0f);
+        const float t = w + 12582912.0f;
+        return ex2_approx(w - (t - 12582912.0f)) * __uint_as_float((unsigned)(__float_as_int(t) + bias) << 23);
+    }
+};
+__device__ __forceinline__ float p2_log(float s, int ref)      // s at least 2^-126
+{
+    const int b = __float_as_int(s);
+    return (float)(ref + (b >> 23) - 127) + lg2_approx(__int_as_float((b & 0x7fffff) | 0x3f800000));
+}
 // Largest sum and smallest exact output of a pass, in bits above its
 // reference (Window<float> of bn_tile13.cu).
 constexpr int kP2Top = 126, kP2Low = -80;
@@ -540,9 +575,10 @@ k_gamma_p2r(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const fl
     for (int pass = 0; pass < max(passes, 1); ++pass) {
         const int down = pass * range;
         const bool last = pass + 1 >= passes;
+        const P2Scale sc(ref_s[mycol] - down);
         for (uint32_t H = tid / CPB; H < H2; H += blockDim.x / CPB) {
             const float w = Wc[BN_AT((size_t)H * nlow, 1, (size_t)nlow << h)];
-            vals[mycol * HS + H] = passes ? ex2_approx(w - (float)(ref_s[mycol] - down)) : w;
+            vals[mycol * HS + H] = passes ? sc.value<true>(w) : w;
         }
         __syncthreads();
         if (passes) p2_steps<true>(vals, H2, HS, h, cols);
@@ -557,7 +593,7 @@ k_gamma_p2r(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const fl
                 if (!last && o < kP2Keep) continue;
                 // a sum flushed in the last pass is irrelevant: kept finite
                 const int ref = ref_s[cc] - down;
-                o = fmaxf((float)ref + lg2_approx(o), (float)(ref - 126));
+                o = o < 1.1754943508222875e-38f ? (float)(ref - 126) : p2_log(o, ref);
                 done |= 1ull << (i & 63);
             }
             // family index of g with the high part t: sizes below k, then the
@@ -700,7 +736,8 @@ k_gamma_p2w(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const fl
     if (!(vsel >> v & 1u)) return;
     W = job_ptr(W, js) + ((size_t)endpoint_slot(vsel, v) << (n - 1 - b)) * nlow;
     Gam = job_ptr(Gam, js) + (size_t)v * K;
-    __shared__ float2 part[8][8][20];               // [warp][column][sum]: (scale, sum)
+    __shared__ float part[8][8][20];                // [warp][column][sum]
+    __shared__ int scale_s[8][8];                   // [warp][column]
     __shared__ uint32_t g_s[8];
     __shared__ int redo_s[8];                       // per column: sums to form again
     const int h = n - 1 - b, hi = h - 5;            // hi: loop bits, 2 .. h - 4
@@ -720,7 +757,9 @@ k_gamma_p2w(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const fl
     // the last column's values stand in for those past the end
     const float* Wc = W + cb + min(c, cols - 1);
     const uint32_t base = ((uint32_t)warp << (h - 3)) | (uint32_t)r;
-    float m = L::ninf(), s = 0.0f, sb[MB];
+    int m = -(1 << 30);                             // the scale
+    P2Scale sc(m);
+    float s = 0.0f, sb[MB];
 #pragma unroll
     for (int q = 0; q < MB; ++q) sb[q] = 0.0f;
     for (uint32_t k = 0; k < (1u << hi); k += 8) {
@@ -730,15 +769,17 @@ k_gamma_p2w(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const fl
         float top = w[0];
 #pragma unroll
         for (int q = 1; q < 8; ++q) top = fmaxf(top, w[q]);
-        if (top - m > 102.0f) {                     // +inf while empty
-            const float sc = L::ex(0.5f * (m - (top - 90.0f)));
-            s = s * sc * sc;
+        const int mt = p2_mag(top);
+        if (mt - m > 102) {
+            const float r0 = p2_pow2((m - (mt - 90)) >> 1), r1 = p2_pow2((m - (mt - 90) + 1) >> 1);
+            s = s * r0 * r1;
 #pragma unroll
-            for (int q = 0; q < MB; ++q) sb[q] = sb[q] * sc * sc;
-            m = top - 90.0f;
+            for (int q = 0; q < MB; ++q) sb[q] = sb[q] * r0 * r1;
+            m = mt - 90;
+            sc = P2Scale(m);
         }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) w[q] = L::ex(w[q] - m);
+        for (int q = 0; q < 8; ++q) w[q] = sc.value<false>(w[q]);
         const float p1 = w[2] + w[3], p2 = w[4] + w[5], p3 = w[6] + w[7];
         const float t = (w[0] + w[1]) + p1 + (p2 + p3);
         s += t;
@@ -750,25 +791,27 @@ k_gamma_p2w(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const fl
             if (k >> q & 1u) sb[q] += t;
     }
     // over the four row phases: the largest scale, every sum relative to it
-    float top = fmaxf(m, __shfl_xor_sync(FULL, m, 8));
-    top = fmaxf(top, __shfl_xor_sync(FULL, top, 16));
-    const float sc = L::ex(0.5f * (m - top));       // in halves: the sums are up to 2^102
-    s = s * sc * sc;
+    int top = max(m, __shfl_xor_sync(FULL, m, 8));
+    top = max(top, __shfl_xor_sync(FULL, top, 16));
+    // in halves: the sums are up to 2^102
+    const float r0 = p2_pow2((m - top) >> 1), r1 = p2_pow2((m - top + 1) >> 1);
+    s = s * r0 * r1;
     const float s1 = s + __shfl_xor_sync(FULL, s, 16);      // phases r and r ^ 2
     const float s2 = s + __shfl_xor_sync(FULL, s, 8);       // phases r and r ^ 1
     const float all = s1 + __shfl_xor_sync(FULL, s1, 8);
     if (r == 3) {                                   // phases 1, 3 and 2, 3: bits 0 and 1
-        part[warp][c][0] = make_float2(top, all);
-        part[warp][c][1] = make_float2(top, s1);
-        part[warp][c][2] = make_float2(top, s2);
+        scale_s[warp][c] = top;
+        part[warp][c][0] = all;
+        part[warp][c][1] = s1;
+        part[warp][c][2] = s2;
     }
 #pragma unroll
     for (int q = 0; q < MB; ++q) {
         if (q >= hi) break;
-        float x = sb[q] * sc * sc;
+        float x = sb[q] * r0 * r1;
         x += __shfl_xor_sync(FULL, x, 16);
         x += __shfl_xor_sync(FULL, x, 8);
-        if (r == 0) part[warp][c][3 + q] = make_float2(top, x);
+        if (r == 0) part[warp][c][3 + q] = x;
     }
     __syncthreads();
     // output o of column c: 0 every row, 1 + j the rows with high bit j
@@ -781,17 +824,16 @@ k_gamma_p2w(int n, int d, int b, uint32_t nlow, uint32_t c0, int64_t K, const fl
         if (col >= cols || (o && d - __popc(g_s[col]) != 1)) continue;
         const int j = o - 1;                        // the high bit
         const int at = j < h - 3 ? o : 0;           // warp bits: sums of the warps with the bit
-        float t = L::ninf();
+        int t = scale_s[0][col];
 #pragma unroll
-        for (int w = 0; w < 8; ++w) t = fmaxf(t, part[w][col][0].x);
+        for (int w = 1; w < 8; ++w) t = max(t, scale_s[w][col]);
         float sum = 0.0f;
 #pragma unroll
         for (int w = 0; w < 8; ++w) {
-            const float2 p = part[w][col][at];
-            const float e = L::ex(0.5f * (p.x - t));
-            if (j < h - 3 || (w >> (j - (h - 3)) & 1)) sum += p.y * e * e;
+            const int k = scale_s[w][col] - t;
+            if (j < h - 3 || (w >> (j - (h - 3)) & 1)) sum += part[w][col][at] * p2_pow2(k >> 1) * p2_pow2((k + 1) >> 1);
         }
-        if (sum > 3.2311742677852644e-27f) store(col, o, t + L::lg(sum));     // 2^-88
+        if (sum > 3.2311742677852644e-27f) store(col, o, p2_log(sum, t));     // 2^-88
         else atomicOr(&redo_s[col], 1 << o);
     }
     __syncthreads();

@@ -2328,6 +2328,28 @@ try {
     return exception_code();
 }
 
+// Test hook: phase 2 of the down-zeta on given inputs.
+int bn_debug_phase2(const bn_job_desc* job, const float* W, float* Gamma)
+try {
+    if (!W || !Gamma) return BN_EINVAL;
+    HostJob hj;
+    const int rc = validate_and_plan(job, hj);
+    if (rc) return rc;
+    const Plan& P = hj.P;
+    if (P.prec == 0 || P.n < 14) return BN_EINVAL;
+    CK(bn::set_kernel_attributes());
+    const size_t wbytes = ((size_t)P.n << (P.n - 14)) * P.nlow_g * 4, gbytes = (size_t)P.n * P.K * 4;
+    char* buf = nullptr;
+    CK(cudaMalloc(&buf, al(wbytes) + gbytes));
+    cudaError_t e = cudaMemcpy(buf, W, wbytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = bn::launch_gamma_p2(P, buf, buf + al(wbytes), nullptr, nullptr, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpy(Gamma, buf + al(wbytes), gbytes, cudaMemcpyDeviceToHost);
+    cudaFree(buf);
+    return e == cudaSuccess ? BN_OK : BN_ECUDA;
+} catch (...) {
+    return exception_code();
+}
+
 // Test hook: what the host planned for a job.
 int bn_debug_plan(const bn_job_desc* job, int32_t* out, int32_t count)
 try {
