@@ -471,7 +471,8 @@ int bn_debug_phase2(const bn_job_desc* job, const float* W, float* Gamma);
 enum {
     BN_PLAN_SWEEPS = 0,  /* 1: F and R' of a batch group of such jobs may run in
                             one launch                                       */
-    BN_PLAN_COUNT = 1
+    BN_PLAN_ANY_SETS = 1,/* set sizes whose states are counted one by one      */
+    BN_PLAN_COUNT = 2
 };
 int bn_debug_plan(const bn_job_desc* job, int32_t* out, int32_t count);
 #endif /* BN_TESTING */

@@ -70,7 +70,7 @@ EXPORTS = ["bn_ctx_create", "bn_ctx_destroy", "bn_num_families", "bn_scores",
 # Test hooks: exported only by the testing build (BN_TESTING).
 TEST_EXPORTS = ["bn_debug_stage", "bn_debug_counts", "bn_debug_batch_drop", "bn_debug_bounds",
                 "bn_debug_explog", "bn_debug_copy_wait", "bn_debug_plan", "bn_debug_phase2"]
-BN_PLAN_SWEEPS, BN_PLAN_COUNT = range(2)
+BN_PLAN_SWEEPS, BN_PLAN_ANY_SETS, BN_PLAN_COUNT = range(3)
 
 
 def testing_build() -> bool:

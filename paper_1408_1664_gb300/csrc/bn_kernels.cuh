@@ -39,7 +39,7 @@ enum KernelId : int32_t {
     KID_COLB1_X, KID_COLW_X, KID_UP13_X, KID_FROWS_X, KID_BROWS_X, KID_G13_X_Q, KID_G13_X,
     KID_GAMMA_P2_X, KID_GAMMA_P2S_X, KID_EDGES_X,
     KID_P2R8, KID_P2R4, KID_P2R2, KID_P2R1, KID_GAMMA_P2W,
-    KID_SET_PAIRS5, KID_SET_PAIRS6, KID_SET_PAIRS7, KID_SET_PAIRS8, KID_COUNT
+    KID_SET_HISTC_WARP, KID_SET_HISTC_BLOCK, KID_SET_PAIRS5, KID_SET_PAIRS6, KID_SET_PAIRS7, KID_SET_PAIRS8, KID_COUNT
 };
 
 // Arguments as one trivially copyable structure whose members have the
@@ -274,6 +274,8 @@ cudaError_t launch_scores(const Plan& P, const uint8_t* data, const uint8_t* ari
                           const int* mj = nullptr, const double* fxj = nullptr);
 // Kernels one launch_scores call starts.
 int scores_launches(const Plan& P);
+// Set sizes that k_set_any counts (more than 16384 joint states).
+int any_set_sizes(const Plan& P);
 // lbs = log B - c_i, the shifts c_i from enc to cmax, and the reordered table
 // of the 13-dimension tiles (tab, may be null).
 cudaError_t launch_shift_scores(const Plan& P, const double* logB, const unsigned long long* enc,

@@ -109,6 +109,8 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
     case KID_SET_PAIRS7: run(k_set_pairs<2>, a); return true;
     case KID_SET_PAIRS8: run(k_set_pairs<3>, a); return true;
     case KID_SET_HIST_WARP: run(k_set_hist<32>, a); return true;
+    case KID_SET_HISTC_WARP: run(k_set_hist_chunks<32>, a); return true;
+    case KID_SET_HISTC_BLOCK: run(k_set_hist_chunks<256>, a); return true;
     case KID_SET_HIST_BLOCK: run(k_set_hist<256>, a); return true;
     case KID_SET_ANY: run(k_set_any, a); return true;
     case KID_FAMILIES: run(k_family_scores, a); return true;
@@ -294,7 +296,8 @@ bool persistent_runs(int prec, int kid)
     switch (kid) {
     case KID_STEP1_PREP: case KID_CHECK_DATA: case KID_SET_ONES: case KID_SET_MOEBIUS:
     case KID_SET_PAIRS5: case KID_SET_PAIRS6: case KID_SET_PAIRS7: case KID_SET_PAIRS8:
-    case KID_SET_HIST_WARP: case KID_SET_HIST_BLOCK: case KID_SET_ANY: case KID_FAMILIES:
+    case KID_SET_HIST_WARP: case KID_SET_HIST_BLOCK: case KID_SET_HISTC_WARP: case KID_SET_HISTC_BLOCK:
+    case KID_SET_ANY: case KID_FAMILIES:
         return true;
     case KID_SHIFT_F: case KID_UPZETA_F: case KID_FWD_LEVEL_F: case KID_BWD_LEVEL_F:
     case KID_GAMMA_TABLE: case KID_GAMMA_P1_F: case KID_GAMMA_P2_F: case KID_GAMMA_P2S_F:

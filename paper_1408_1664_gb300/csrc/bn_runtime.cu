@@ -1635,7 +1635,7 @@ int record_groups(bn_batch* b)
                     return BN_EINVAL;
                 switch (x.kid) {                   // kernels that loop grid-stride in x
                 case bn::KID_STEP1_PREP: case bn::KID_CHECK_DATA: case bn::KID_SET_HIST_WARP:
-                case bn::KID_SET_HIST_BLOCK: case bn::KID_SET_ANY: case bn::KID_FAMILIES:
+                case bn::KID_SET_HISTC_WARP: case bn::KID_SET_HISTC_BLOCK: case bn::KID_SET_HIST_BLOCK: case bn::KID_SET_ANY: case bn::KID_FAMILIES:
                 case bn::KID_SHIFT_F: case bn::KID_SHIFT_D: case bn::KID_SHIFT_X: case bn::KID_EDGES_X:
                 case bn::KID_REORDER_X: case bn::KID_COLW_X: case bn::KID_EDGES_F: case bn::KID_EDGES_D: case bn::KID_REORDER_F: case bn::KID_REORDER_D:
                 case bn::KID_COLW_F: case bn::KID_COLW_D:
@@ -2359,6 +2359,7 @@ try {
     if (rc) return rc;
     int32_t v[BN_PLAN_COUNT] = {};
     v[BN_PLAN_SWEEPS] = bn::sweeps_fit(hj.P);
+    v[BN_PLAN_ANY_SETS] = bn::any_set_sizes(hj.P);
     std::copy(v, v + count, out);
     return BN_OK;
 } catch (...) {

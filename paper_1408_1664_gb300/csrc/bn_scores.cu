@@ -531,6 +531,41 @@ k_set_pairs(int n, int m, int b, uint32_t nsets, uint32_t nbase, const uint32_t*
     pairs_warp<RB>(Y, b, lane, soff, cnt, nsets, T0, T1, T2, vc, H, dbg, dbg_set);
 }
 
+// One set's counts over the staged words [0, words) of every column, the
+// samples from 4 * from on and below upto: lane gl of G.
+template <int G>
+__device__ __forceinline__ void count_states(const uint32_t* col, int mw, int from, int words, int upto,
+                                             const uint32_t* ar, uint32_t X, uint32_t* h, int gl, uint32_t states)
+{
+    uint32_t q = 1;
+    for (int w0 = gl; w0 < words; w0 += 4 * G) {
+        uint32_t lo[4] = {0, 0, 0, 0}, hi[4] = {0, 0, 0, 0};
+        q = 1;
+        for (uint32_t x = X; x; x &= x - 1) {
+            const int v = __ffs(x) - 1;
+            const uint32_t* cv = col + v * mw;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int w = w0 + u * G;
+                const uint32_t y = w < words ? cv[w] : 0u;
+                lo[u] += (y & 0x00ff00ffu) * q;
+                hi[u] += ((y >> 8) & 0x00ff00ffu) * q;
+            }
+            q *= ar[v];
+        }
+        // key < q unless a value is not below its arity (device data, which
+        // k_check_data reports): such a sample is left out
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int s = 4 * (from + w0 + u * G);
+            const uint32_t key[4] = {lo[u] & 0xffffu, hi[u] & 0xffffu, lo[u] >> 16, hi[u] >> 16};
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                if (s + b < upto && key[b] < q) atomicAdd(&h[BN_AT(key[b], 1, states)], 1u);
+        }
+    }
+}
+
 // Data of any arity: H(X) from a histogram of the samples' joint states in
 // shared memory.  A block stages the whole data set once, transposed to
 // columns of bytes (four samples per 32-bit word), and its groups of G
@@ -578,34 +613,8 @@ k_set_hist(int n, int m, int mw, uint32_t s0, uint32_t s1, uint32_t states,
     for (uint32_t idx = s0 + grp; idx < s1; idx += ngrp) {
         int k;
         const uint32_t X = set_of(idx, n, &k);
+        count_states<G>(col, mw, 0, words, mown, ar, X, h, gl, states);
         uint32_t q = 1;
-        for (int w0 = gl; w0 < words; w0 += 4 * G) {
-            uint32_t lo[4] = {0, 0, 0, 0}, hi[4] = {0, 0, 0, 0};
-            q = 1;
-            for (uint32_t x = X; x; x &= x - 1) {
-                const int v = __ffs(x) - 1;
-                const uint32_t* cv = col + v * mw;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int w = w0 + u * G;
-                    const uint32_t y = w < words ? cv[w] : 0u;
-                    lo[u] += (y & 0x00ff00ffu) * q;
-                    hi[u] += ((y >> 8) & 0x00ff00ffu) * q;
-                }
-                q *= ar[v];
-            }
-            // key < q unless a value is not below its arity (device data, which
-            // k_check_data reports): such a sample is left out
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int s = 4 * (w0 + u * G);
-                const uint32_t key[4] = {lo[u] & 0xffffu, hi[u] & 0xffffu, lo[u] >> 16, hi[u] >> 16};
-#pragma unroll
-                for (int b = 0; b < 4; ++b)
-                    if (s + b < mown && key[b] < q) atomicAdd(&h[BN_AT(key[b], 1, states)], 1u);
-            }
-        }
-        q = 1;                                      // groups without samples need it too
         for (uint32_t x = X; x; x &= x - 1) q *= ar[__ffs(x) - 1];
         if (G == 32) __syncwarp(); else __syncthreads();
         const long long* Tk = T + (size_t)find_row(Dvals, rows, q) * (m + 1);
@@ -630,9 +639,83 @@ k_set_hist(int n, int m, int mw, uint32_t s0, uint32_t s1, uint32_t states,
     }
 }
 
+// The same for data that do not fit: they pass by in chunks of 4 cw samples, once
+// for every round of R sets per group, while the groups' R histograms add up.
+// Walking the states with the bit planes instead, as k_set_any does, takes
+// states * m / 64 words of k ANDs, each with a division for its digit.  Scores,
+// n = 20, arity 3, d = 4, m = 10000: walked 5.57 ms, in chunks 0.52; n = 22, d = 5
+// 94 and 4.1.
+template <int G>
+__global__ void __launch_bounds__(256)
+k_set_hist_chunks(int n, int m, int mw, int cw, int R, uint32_t s0, uint32_t s1, uint32_t states,
+                  const uint8_t* __restrict__ data, const uint8_t* __restrict__ arity,
+                  const int* __restrict__ mj, const double* __restrict__ Dvals, int rows,
+                  const long long* __restrict__ T, long long* __restrict__ H, int64_t* __restrict__ dbg,
+                  uint32_t dbg_set, size_t js)
+{
+    data = job_ptr(data, js);
+    arity = job_ptr(arity, js);
+    Dvals = job_ptr(Dvals, js);
+    T = job_ptr(T, js);
+    H = job_ptr(H, js);
+    const int mown = mj ? *job_ptr(mj, js) : m;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    uint32_t* col = reinterpret_cast<uint32_t*>(smem_raw);      // [n][mw]
+    uint32_t* ar = col + (size_t)n * mw;
+    __shared__ long long part[8];
+    const int all = (mown + 3) >> 2;
+    if (threadIdx.x < n) ar[threadIdx.x] = arity[threadIdx.x];
+    const int gl = threadIdx.x % G;
+    uint32_t* h = ar + 32 + (size_t)(threadIdx.x / G) * R * states;     // this group's histograms
+    for (uint32_t c = gl; c < R * states; c += G) h[c] = 0u;
+    const uint32_t per = blockDim.x / G * R;
+    for (uint32_t b0 = s0 + blockIdx.x * per; b0 < s1; b0 += gridDim.x * per) {
+        const uint32_t i0 = b0 + threadIdx.x / G * R, i1 = min(s1, i0 + R);
+        int k;
+        for (int from = 0; from < all; from += cw) {
+            const int words = min(all - from, cw);
+            __syncthreads();                        // the last chunk is counted, its histograms are read
+            for (int t = threadIdx.x; t < n * words; t += blockDim.x) {
+                const int v = t % n, w = t / n, s = 4 * (from + w);
+                uint32_t x = 0;
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (s + b < mown) x |= (uint32_t)data[(size_t)(s + b) * n + v] << (8 * b);
+                col[v * mw + w] = x;
+            }
+            __syncthreads();
+            for (uint32_t idx = i0; idx < i1; ++idx)
+                count_states<G>(col, mw, from, words, min(mown, 4 * (from + words)), ar, set_of(idx, n, &k),
+                                h + (idx - i0) * states, gl, states);
+        }
+        __syncthreads();
+        for (uint32_t idx = i0; idx < i1; ++idx) {
+            uint32_t q = 1;
+            for (uint32_t x = set_of(idx, n, &k); x; x &= x - 1) q *= ar[__ffs(x) - 1];
+            const long long* Tk = T + (size_t)find_row(Dvals, rows, q) * (m + 1);
+            uint32_t* hs = h + (idx - i0) * states;
+            long long acc = 0;
+            for (uint32_t c = gl; c < q; c += G) {
+                const uint32_t N = hs[c];
+                acc += Tk[N];
+                if (dbg && idx == dbg_set) dbg[c] = N;
+                hs[c] = 0u;
+            }
+            acc = warp_sum(acc);
+            if (G > 32) {
+                if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+                __syncthreads();
+                acc = 0;
+                for (int w = 0; w < (int)(blockDim.x >> 5); ++w) acc += part[w];
+                __syncthreads();                    // part is reused
+            }
+            if (gl == 0) H[BN_AT(idx, 1, s1)] = acc;
+        }
+    }
+}
+
 // Any set: a warp walks the joint states and counts each with the AND of its
-// bit planes, lanes over the words.  For sets whose histogram or data do not
-// fit shared memory.
+// bit planes, lanes over the words.  For sets of more than kBlockStates states.
 __global__ void __launch_bounds__(256)
 k_set_any(int n, int m, int W, int rmax, uint32_t s0, uint32_t s1,
           const uint8_t* __restrict__ arity, const uint64_t* __restrict__ planes,
@@ -844,17 +927,20 @@ uint32_t sets_before(int n, int k)
 }
 
 // The kernels of a plan's sets: sizes [0, moebius), [moebius, warp) and
-// [warp, block) by warp and block histograms, [block, end) by k_set_any.
-// A warp's histogram holds at most 1024 states (32 KB per block), a block's
-// at most 16384 (64 KB), beside the staged data; at most 192 KB in all.
+// [warp, block) by warp and block histograms over the whole data, [block,
+// cwarp) and [cwarp, cblock) by the same over chunks of it, [cblock, end) by
+// k_set_any.  A warp's histogram holds at most 1024 states (32 KB per block),
+// a block's at most 16384 (64 KB), beside the staged data; at most 192 KB in
+// all.  Chunks and the histograms of a round (R sets per group, as many as 32
+// and 64 KB hold, at most 8) take 96 KB, two blocks per SM.
 struct SetSplit {
-    int moebius, warp, block, end;
+    int moebius, warp, block, cwarp, cblock, end;
     int pairs;                                      // size of k_set_pairs' bases (0: not used)
     int mw;                                         // words of a staged column
-    uint32_t wstates, bstates;
+    uint32_t wstates, bstates, cwstates, cbstates;
 };
 constexpr uint32_t kWarpStates = 1024, kBlockStates = 16384;
-constexpr size_t kSetSmem = 192 * 1024;
+constexpr size_t kSetSmem = 192 * 1024, kChunkSmem = 96 * 1024;
 
 size_t hist_bytes(const Plan& P, int mw, uint32_t states) { return 4 * ((size_t)P.n * mw + 32 + states); }
 
@@ -873,8 +959,27 @@ SetSplit split_sets(const Plan& P)
     while (x.block < x.end && P.states[x.block] <= kBlockStates &&
            hist_bytes(P, x.mw, P.states[x.block]) <= kSetSmem)
         x.bstates = P.states[x.block++];
+    x.cwarp = x.block;
+    while (x.cwarp < x.end && P.states[x.cwarp] <= kWarpStates) x.cwstates = P.states[x.cwarp++];
+    x.cblock = x.cwarp;
+    while (x.cblock < x.end && P.states[x.cblock] <= kBlockStates) x.cbstates = P.states[x.cblock++];
     return x;
 }
+
+// The shape of a chunked launch: `groups` per block, sets of at most `states`.
+struct ChunkShape {
+    int R, cw, mw;                                  // sets per group and round; words of a chunk, of a column
+    size_t bytes;
+    ChunkShape(const Plan& P, int groups, uint32_t states)
+    {
+        const uint32_t most = groups > 1 ? kWarpStates : kBlockStates;
+        R = (int)std::min<uint32_t>(8, std::max<uint32_t>(1, most / states));
+        const size_t h = 4 * ((size_t)groups * R * states + 32);
+        cw = (int)((kChunkSmem - h) / (4 * (size_t)P.n)) - 1;      // at least 255 words (n <= 32)
+        mw = cw | 1;
+        bytes = h + 4 * (size_t)P.n * mw;
+    }
+};
 
 }  // namespace
 
@@ -976,8 +1081,28 @@ cudaError_t launch_set_scores(const Plan& P, const uint8_t* data, const uint8_t*
                              arity, mj, Dvals, P.rows, T, x.H, dbg, dbg_set, P.js);
         if (e != cudaSuccess) return e;
     }
-    if (z.end > z.block) {
-        const uint32_t s0 = sets_before(P.n, z.block), s1 = sets_before(P.n, z.end);
+    if (z.cwarp > z.block) {
+        const uint32_t s0 = sets_before(P.n, z.block), s1 = sets_before(P.n, z.cwarp);
+        const ChunkShape c(P, 8, z.cwstates);
+        const unsigned g = (unsigned)std::min<int64_t>(((int64_t)(s1 - s0) + 8 * c.R - 1) / (8 * c.R),
+                                                       std::max(1, 152 * 4 / P.nj));
+        e = launch_or_record(KID_SET_HISTC_WARP, k_set_hist_chunks<32>, dim3(g, P.nj), 256, c.bytes, s, P.n, P.m, c.mw,
+                             c.cw, c.R, s0, s1, z.cwstates, data, arity, mj, Dvals, P.rows, T, x.H, dbg, dbg_set,
+                             P.js);
+        if (e != cudaSuccess) return e;
+    }
+    if (z.cblock > z.cwarp) {
+        const uint32_t s0 = sets_before(P.n, z.cwarp), s1 = sets_before(P.n, z.cblock);
+        const ChunkShape c(P, 1, z.cbstates);
+        const unsigned g = (unsigned)std::min<int64_t>(((int64_t)(s1 - s0) + c.R - 1) / c.R,
+                                                       std::max(1, 152 * 4 / P.nj));
+        e = launch_or_record(KID_SET_HISTC_BLOCK, k_set_hist_chunks<256>, dim3(g, P.nj), 256, c.bytes, s, P.n, P.m, c.mw,
+                             c.cw, c.R, s0, s1, z.cbstates, data, arity, mj, Dvals, P.rows, T, x.H, dbg, dbg_set,
+                             P.js);
+        if (e != cudaSuccess) return e;
+    }
+    if (z.end > z.cblock) {
+        const uint32_t s0 = sets_before(P.n, z.cblock), s1 = sets_before(P.n, z.end);
         e = launch_or_record(KID_SET_ANY, k_set_any, dim3(grid_for((int64_t)(s1 - s0), 8, 152 * 16), P.nj),
                              256, 0, s, P.n, P.m, P.W, P.rmax, s0, s1, arity, planes, mj, Dvals, P.rows, T,
                              x.H, dbg, dbg_set, P.js);
@@ -1001,7 +1126,14 @@ cudaError_t launch_scores(const Plan& P, const uint8_t* data, const uint8_t* ari
 int scores_launches(const Plan& P)
 {
     const SetSplit z = split_sets(P);
-    return (z.moebius > 0 ? 2 : 0) + (z.pairs > 0) + (z.warp > z.moebius) + (z.block > z.warp) + (z.end > z.block) + 1;
+    return (z.moebius > 0 ? 2 : 0) + (z.pairs > 0) + (z.warp > z.moebius) + (z.block > z.warp) +
+           (z.cwarp > z.block) + (z.cblock > z.cwarp) + (z.end > z.cblock) + 1;
+}
+
+int any_set_sizes(const Plan& P)
+{
+    const SetSplit z = split_sets(P);
+    return z.end - z.cblock;
 }
 
 cudaError_t launch_shift_scores(const Plan& P, const double* logB, const unsigned long long* enc,
@@ -1021,6 +1153,8 @@ cudaError_t launch_shift_scores(const Plan& P, const double* logB, const unsigne
 cudaError_t set_scores_attributes()
 {
     cudaError_t e = allow_max_dynamic_smem(k_set_hist<32>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_hist_chunks<32>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_hist_chunks<256>);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_pairs<0>);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_pairs<1>);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_set_pairs<2>);

@@ -22,3 +22,17 @@ def test_one_launch_sweeps_end_with_their_places(precision, first, last):
     of larger jobs may take it, by the flag or by the tuner."""
     for n in range(first, last + 1):
         assert _plan(n, 1, precision=precision)[B.BN_PLAN_SWEEPS] == (n << (n - 1) <= 2 ** 32), n
+
+
+@pytest.mark.parametrize("n,m,arity,d", [(20, 10000, 3, 4), (29, 6400, 3, 3), (12, 100000, 4, 5),
+                                         (20, 9400, [2 + i % 3 for i in range(20)], 5)])
+def test_no_sample_count_takes_the_state_walk(n, m, arity, d):
+    """The joint states of a set are counted by a histogram however many
+    samples there are; only sets of more than 16384 states are walked."""
+    assert _plan(n, d, m=m, arity=arity)[B.BN_PLAN_ANY_SETS] == 0
+
+
+def test_sets_of_many_states_take_the_state_walk():
+    """7^4 = 2401 states fit a histogram, 7^5 = 16807 do not."""
+    assert _plan(8, 3, arity=7)[B.BN_PLAN_ANY_SETS] == 0
+    assert _plan(8, 4, arity=7)[B.BN_PLAN_ANY_SETS] == 1
