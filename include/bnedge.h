@@ -465,6 +465,10 @@ int bn_debug_explog(const double* x, int64_t count, double* out);
  * over the rows that contain a family's high part.  The job gives n, d and
  * the samples' shape only. */
 int bn_debug_phase2(const bn_job_desc* job, const float* W, float* Gamma);
+/* Blocks that would share F (and as many R') of a single job in its
+ * one-launch sweeps on a device of `sms` SMs, at most `per_sm` of them on an SM
+ * at a time (no GPU needed); *blocks = 0: a launch per level. */
+int bn_debug_sweep_blocks(const bn_job_desc* job, int32_t sms, int32_t* blocks, int32_t* per_sm);
 /* What the host planned for a job (no GPU needed): `count` values, the first
  * of the enumeration below, go to out.  BN_EINVAL for an invalid job or a
  * count beyond it. */

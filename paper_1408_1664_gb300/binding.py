@@ -69,7 +69,8 @@ EXPORTS = ["bn_ctx_create", "bn_ctx_destroy", "bn_num_families", "bn_scores",
 
 # Test hooks: exported only by the testing build (BN_TESTING).
 TEST_EXPORTS = ["bn_debug_stage", "bn_debug_counts", "bn_debug_batch_drop", "bn_debug_bounds",
-                "bn_debug_explog", "bn_debug_copy_wait", "bn_debug_plan", "bn_debug_phase2"]
+                "bn_debug_explog", "bn_debug_copy_wait", "bn_debug_plan", "bn_debug_phase2",
+                "bn_debug_sweep_blocks"]
 BN_PLAN_SWEEPS, BN_PLAN_ANY_SETS, BN_PLAN_COUNT = range(3)
 
 
@@ -149,6 +150,8 @@ def load(build_if_missing: bool = False) -> C.CDLL:
         "bn_debug_bounds": (C.c_int, [C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
         "bn_debug_explog": (C.c_int, [P, C.c_int64, P]),
         "bn_debug_copy_wait": (C.c_int, [C.c_uint32, C.POINTER(C.c_int32)]),
+        "bn_debug_sweep_blocks": (C.c_int, [C.POINTER(bn_job_desc), C.c_int32, C.POINTER(C.c_int32),
+                                            C.POINTER(C.c_int32)]),
         "bn_debug_phase2": (C.c_int, [C.POINTER(bn_job_desc), P, P]),
         "bn_debug_plan": (C.c_int, [C.POINTER(bn_job_desc), C.POINTER(C.c_int32), C.c_int32]),
         "bn_shard_create": (C.c_int, [P, C.POINTER(bn_job_desc), C.c_int32, C.c_int32, C.c_int32,
@@ -374,6 +377,16 @@ def bn_debug_phase2(job: Job, W: np.ndarray) -> np.ndarray:
     if rc:
         raise BnError(rc, "bn_debug_phase2")
     return out
+
+
+def bn_debug_sweep_blocks(job: Job, sms: int) -> tuple[int, int]:
+    """(blocks per sweep, blocks per SM) of a single job's one-launch sweeps on
+    a device of ``sms`` SMs (no GPU needed)."""
+    blocks, per_sm = C.c_int32(), C.c_int32()
+    rc = load().bn_debug_sweep_blocks(C.byref(job.desc), sms, C.byref(blocks), C.byref(per_sm))
+    if rc:
+        raise BnError(rc, "bn_debug_sweep_blocks")
+    return int(blocks.value), int(per_sm.value)
 
 
 def bn_debug_plan(job: Job) -> list[int]:

@@ -19,6 +19,7 @@
 // times 32, and every value entering is finite (A and F are logs of
 // positive sums; a zero weight is a finite soft zero).
 #include <algorithm>
+#include <atomic>
 
 #include "bn_device.cuh"
 #include "bn_kernels.cuh"
@@ -1041,17 +1042,70 @@ cudaError_t launch_backward_rows(const Plan& P, const void* A, void* Rc, cudaStr
     return rows_sweep(P, 1, A, Rc, s, launches);
 }
 
+// The instance of k_sweeps that a plan takes.
+template <typename V, bool L, int W> struct SweepForm {
+    using T = V;
+    static constexpr bool TLO = L;
+    static constexpr int VB = W;
+    static constexpr int threads = SweepShape<W>::threads;
+    static constexpr int tiles = threads >> ((sizeof(V) == 4 ? LB : LB64) - W);    // of a block at a time
+};
+template <typename F> static auto with_sweep_form(const Plan& P, F f)
+{
+    const bool vec = P.n >= kSweepVecN;
+    if (P.lin) return f(SweepForm<X64, false, 0>{});
+    if (use_tlo(P)) return vec ? f(SweepForm<float, true, 2>{}) : f(SweepForm<float, true, 0>{});
+    return vec ? f(SweepForm<float, false, 2>{}) : f(SweepForm<float, false, 0>{});
+}
+
+static uint64_t widest_level(const Plan& P)
+{
+    const int nh = P.n - (P.prec == 0 ? LB64 : LB);
+    return choose(nh, nh / 2);
+}
+
+// Whether the whole GPU shares the two sweeps of a single job: levels that
+// fill more than kSweepGrid blocks.
+static bool whole_gpu(const Plan& P, int tiles) { return widest_level(P) > kSweepGrid * tiles; }
+
 // Blocks that share one item of k_sweeps: enough that every tile of the
 // widest level has its own lanes.  Clusters (at most 8 blocks, the portable
-// size) serve the small jobs and every batch group; past kSweepGrid blocks
-// the whole GPU shares the two sweeps of a single job (err given).
-static int sweep_blocks(const Plan& P, uint64_t tiles, int per_sm, const int* err)
+// size) serve the small jobs and every batch group.  The whole-GPU form takes
+// at most `resident` blocks over both items, what the device holds at a time (its
+// blocks wait on one another); 0: too few for it.
+static int sweep_blocks(const Plan& P, int tiles, bool whole, int resident)
 {
-    const int B = P.prec == 0 ? LB64 : LB;
-    const uint64_t widest = choose(P.n - B, (P.n - B) / 2);
-    // the whole-GPU form needs the counters beside the job's error word
-    const uint64_t most = err && widest > kSweepGrid * tiles ? 76 * per_sm : 8;
-    return (int)std::max<uint64_t>(1, std::min<uint64_t>((widest + tiles - 1) / tiles, most));
+    const uint64_t need = (widest_level(P) + tiles - 1) / tiles;
+    if (!whole) return (int)std::max<uint64_t>(1, std::min<uint64_t>(need, 8));
+    return resident / 2 > 8 ? (int)std::min<uint64_t>(need, resident / 2) : 0;
+}
+
+// Blocks of the whole-GPU form that the current device holds at a time, asked
+// once per device; 0 where it has no cooperative launches.
+template <typename Form> static int resident_blocks()
+{
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];        // the answer + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev < kDevices && known[dev].load() > 0) return known[dev].load() - 1;
+    int coop = 0, nsm = 0, per_sm = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &per_sm, k_sweeps<typename Form::T, Form::TLO, SYNC_GRID, Form::VB>, Form::threads, 0) != cudaSuccess)
+        return 0;
+    const int r = coop ? nsm * std::min(per_sm, SweepShape<Form::VB>::blocks) : 0;
+    if (dev < kDevices) known[dev].store(r + 1);
+    return r;
+}
+
+int debug_sweep_blocks(const Plan& P, int sms, int* per_sm)
+{
+    return with_sweep_form(P, [&](auto f) {
+        *per_sm = SweepShape<f.VB>::blocks;
+        return sweep_blocks(P, f.tiles, whole_gpu(P, f.tiles), sms * SweepShape<f.VB>::blocks);
+    });
 }
 
 bool sweeps_fit(const Plan& P)
@@ -1063,14 +1117,24 @@ bool sweeps_fit(const Plan& P)
 bool use_sweeps(const Plan& P, const int* err)
 {
     const int most = P.busy ? kSweepBusyN : P.lin ? kSweepMaxNX : kSweepMaxN;
-    return sweeps_fit(P) && P.n <= most && err && !recording();
+    if (!sweeps_fit(P) || P.n > most || !err || recording()) return false;
+    return with_sweep_form(P, [&](auto f) {
+        return !whole_gpu(P, f.tiles) || sweep_blocks(P, f.tiles, true, resident_blocks<decltype(f)>()) > 0;
+    });
 }
 
-template <typename T, bool TLO, int VB>
-static cudaError_t sweeps_vb(const Plan& P, const T* A, T* F, T* Rc, int items, cudaStream_t s, int* err)
+template <typename Form>
+static cudaError_t sweeps(const Plan& P, const void* Av, void* Fv, void* Rv, int items, cudaStream_t s, int* err)
 {
-    constexpr int B = sizeof(T) == 4 ? LB : LB64, threads = SweepShape<VB>::threads;
-    const int nb = sweep_blocks(P, threads >> (B - VB), SweepShape<VB>::blocks, err);
+    using T = typename Form::T;
+    constexpr bool TLO = Form::TLO;
+    constexpr int VB = Form::VB, threads = Form::threads;
+    const T* A = static_cast<const T*>(Av);
+    T *F = static_cast<T*>(Fv), *Rc = static_cast<T*>(Rv);
+    // the whole-GPU form needs the counters beside the job's error word
+    const bool whole = err && whole_gpu(P, Form::tiles);
+    const int nb = sweep_blocks(P, Form::tiles, whole, whole ? resident_blocks<Form>() : 0);
+    if (nb == 0) return cudaErrorCooperativeLaunchTooLarge;     // (use_sweeps answers no)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(items * nb), 1, 1);
     cfg.blockDim = dim3(threads, 1, 1);
@@ -1081,7 +1145,7 @@ static cudaError_t sweeps_vb(const Plan& P, const T* A, T* F, T* Rc, int items, 
     unsigned* sync = err ? reinterpret_cast<unsigned*>(err) + 16 : nullptr;
     if (nb == 1)
         return cudaLaunchKernelEx(&cfg, k_sweeps<T, TLO, SYNC_BLOCK, VB>, P.n, nb, A, F, Rc, P.js, sync, err, 0u);
-    if (nb <= 8) {
+    if (!whole) {
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = nb;
         attr[0].val.clusterDim.y = 1;
@@ -1094,22 +1158,13 @@ static cudaError_t sweeps_vb(const Plan& P, const T* A, T* F, T* Rc, int items, 
                               kSweepSpinCap);
 }
 
-template <typename T, bool TLO>
-static cudaError_t sweeps(const Plan& P, const T* A, T* F, T* Rc, int items, cudaStream_t s, int* err)
-{
-    if constexpr (sizeof(T) == 4)
-        if (P.n >= kSweepVecN) return sweeps_vb<T, TLO, 2>(P, A, F, Rc, items, s, err);
-    return sweeps_vb<T, TLO, 0>(P, A, F, Rc, items, s, err);
-}
-
 cudaError_t launch_sweeps(const Plan& P, const void* A, void* F, void* Rc, cudaStream_t s, int* err,
                           int* launches)
 {
     if (P.n > kSweepPlacesN) return cudaErrorInvalidValue;
     const int items = Rc ? 2 * P.nj : 1;            // a feature's job: F alone
-    const cudaError_t e = P.lin ? sweeps<X64, false>(P, (const X64*)A, (X64*)F, (X64*)Rc, items, s, err)
-                          : use_tlo(P) ? sweeps<float, true>(P, (const float*)A, (float*)F, (float*)Rc, items, s, err)
-                                     : sweeps<float, false>(P, (const float*)A, (float*)F, (float*)Rc, items, s, err);
+    const cudaError_t e =
+        with_sweep_form(P, [&](auto f) { return sweeps<decltype(f)>(P, A, F, Rc, items, s, err); });
     if (e == cudaSuccess && launches) ++*launches;
     return e;
 }

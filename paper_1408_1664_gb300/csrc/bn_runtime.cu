@@ -2350,6 +2350,20 @@ try {
     return exception_code();
 }
 
+// Test hook: the blocks of a job's one-launch sweeps.
+int bn_debug_sweep_blocks(const bn_job_desc* job, int32_t sms, int32_t* blocks, int32_t* per_sm)
+try {
+    if (!blocks || !per_sm || sms < 1) return BN_EINVAL;
+    HostJob hj;
+    const int rc = validate_and_plan(job, hj);
+    if (rc) return rc;
+    if (!bn::sweeps_fit(hj.P)) return BN_EINVAL;
+    *blocks = bn::debug_sweep_blocks(hj.P, sms, per_sm);
+    return BN_OK;
+} catch (...) {
+    return exception_code();
+}
+
 // Test hook: what the host planned for a job.
 int bn_debug_plan(const bn_job_desc* job, int32_t* out, int32_t count)
 try {

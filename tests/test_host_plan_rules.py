@@ -36,3 +36,21 @@ def test_sets_of_many_states_take_the_state_walk():
     """7^4 = 2401 states fit a histogram, 7^5 = 16807 do not."""
     assert _plan(8, 3, arity=7)[B.BN_PLAN_ANY_SETS] == 0
     assert _plan(8, 4, arity=7)[B.BN_PLAN_ANY_SETS] == 1
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_one_launch_sweeps_fit_the_device(precision):
+    """The blocks of the whole-GPU sweeps wait on one another: F's and R's
+    together never exceed what the device holds at a time, and a device too
+    small for the form keeps a launch per level."""
+    for n in range(5, 22):
+        job = B.Job(np.zeros((2, n), np.uint8), [2] * n, 2, precision=precision)
+        most, _ = B.bn_debug_sweep_blocks(job, 152)
+        assert most > 0
+        for sms in (1, 4, 8, 20, 76, 132, 148, 152):
+            blocks, per_sm = B.bn_debug_sweep_blocks(job, sms)
+            if most <= 8:                               # one block, or a cluster
+                assert blocks == most
+            else:
+                assert 2 * blocks <= sms * per_sm and blocks != 1
+                assert blocks > 8 or (blocks == 0 and sms * per_sm < 18)
