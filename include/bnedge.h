@@ -465,6 +465,11 @@ int bn_debug_explog(const double* x, int64_t count, double* out);
  * over the rows that contain a family's high part.  The job gives n, d and
  * the samples' shape only. */
 int bn_debug_phase2(const bn_job_desc* job, const float* W, float* Gamma);
+/* The bounded wait of the one-launch sweeps' whole-GPU form: F of 16
+ * variables with one of its blocks missing, so the others give up their first
+ * wait after `polls` polls and return; *err_word receives the job error word
+ * they leave (2, as for bn_debug_copy_wait). */
+int bn_debug_sweep_wait(uint32_t polls, int32_t* err_word);
 /* Blocks that would share F (and as many R') of a single job in its
  * one-launch sweeps on a device of `sms` SMs, at most `per_sm` of them on an SM
  * at a time (no GPU needed); *blocks = 0: a launch per level. */

@@ -70,7 +70,7 @@ EXPORTS = ["bn_ctx_create", "bn_ctx_destroy", "bn_num_families", "bn_scores",
 # Test hooks: exported only by the testing build (BN_TESTING).
 TEST_EXPORTS = ["bn_debug_stage", "bn_debug_counts", "bn_debug_batch_drop", "bn_debug_bounds",
                 "bn_debug_explog", "bn_debug_copy_wait", "bn_debug_plan", "bn_debug_phase2",
-                "bn_debug_sweep_blocks"]
+                "bn_debug_sweep_blocks", "bn_debug_sweep_wait"]
 BN_PLAN_SWEEPS, BN_PLAN_ANY_SETS, BN_PLAN_COUNT = range(3)
 
 
@@ -152,6 +152,7 @@ def load(build_if_missing: bool = False) -> C.CDLL:
         "bn_debug_copy_wait": (C.c_int, [C.c_uint32, C.POINTER(C.c_int32)]),
         "bn_debug_sweep_blocks": (C.c_int, [C.POINTER(bn_job_desc), C.c_int32, C.POINTER(C.c_int32),
                                             C.POINTER(C.c_int32)]),
+        "bn_debug_sweep_wait": (C.c_int, [C.c_uint32, C.POINTER(C.c_int32)]),
         "bn_debug_phase2": (C.c_int, [C.POINTER(bn_job_desc), P, P]),
         "bn_debug_plan": (C.c_int, [C.POINTER(bn_job_desc), C.POINTER(C.c_int32), C.c_int32]),
         "bn_shard_create": (C.c_int, [P, C.POINTER(bn_job_desc), C.c_int32, C.c_int32, C.c_int32,

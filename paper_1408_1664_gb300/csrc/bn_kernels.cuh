@@ -344,6 +344,8 @@ cudaError_t launch_level_rows(const Plan& P, uint32_t r, int hl, void* X, void* 
 // also hold the sweeps' counters.  Rc null: F alone.
 bool sweeps_fit(const Plan& P);
 bool use_sweeps(const Plan& P, const int* err);
+constexpr int kWithheldN = 16, kWithheldBlocks = 16;
+cudaError_t launch_sweeps_withheld(const float* A, float* F, int* err, uint32_t polls, cudaStream_t s);
 // Blocks per item that a single job's sweeps would take on a device of `sms`
 // SMs (0: the level launches), and the most of them an SM holds.
 int debug_sweep_blocks(const Plan& P, int sms, int* per_sm);

@@ -1169,6 +1169,15 @@ cudaError_t launch_sweeps(const Plan& P, const void* A, void* F, void* Rc, cudaS
     return e;
 }
 
+// Test hook: F of n = kWithheldN in the whole-GPU form with the last of its
+// blocks missing, so that the others' first wait runs out after `polls` polls.
+cudaError_t launch_sweeps_withheld(const float* A, float* F, int* err, uint32_t polls, cudaStream_t s)
+{
+    k_sweeps<float, false, SYNC_GRID, 0><<<kWithheldBlocks - 1, SweepShape<0>::threads, 0, s>>>(
+        kWithheldN, kWithheldBlocks, A, F, nullptr, 0, reinterpret_cast<unsigned*>(err) + 16, err, polls);
+    return cudaGetLastError();
+}
+
 #endif  // BN_MEGA
 
 }  // namespace bn

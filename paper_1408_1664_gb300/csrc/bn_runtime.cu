@@ -2350,6 +2350,30 @@ try {
     return exception_code();
 }
 
+// Test hook: the one-launch sweeps' bounded wait for a block that never comes.
+int bn_debug_sweep_wait(uint32_t polls, int32_t* err_word)
+try {
+    if (!err_word) return BN_EINVAL;
+    const int n = bn::kWithheldN;
+    const size_t abytes = ((size_t)n << (n - 1)) * 4, fbytes = al(((size_t)1 << n) * 4 + bn::kLevelWords * 4);
+    char* buf = nullptr;
+    CK(cudaMalloc(&buf, abytes + fbytes + 256));
+    int* err = reinterpret_cast<int*>(buf + abytes + fbytes);
+    cudaError_t e = cudaMemset(buf, 0, abytes + fbytes + 256);
+    if (e == cudaSuccess)
+        e = bn::launch_sweeps_withheld(reinterpret_cast<float*>(buf), reinterpret_cast<float*>(buf + abytes), err,
+                                       polls, nullptr);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    int w = 0;
+    if (e == cudaSuccess) e = cudaMemcpy(&w, err, 4, cudaMemcpyDeviceToHost);
+    cudaFree(buf);
+    if (e != cudaSuccess) return BN_ECUDA;
+    *err_word = w;
+    return BN_OK;
+} catch (...) {
+    return exception_code();
+}
+
 // Test hook: the blocks of a job's one-launch sweeps.
 int bn_debug_sweep_blocks(const bn_job_desc* job, int32_t sms, int32_t* blocks, int32_t* per_sm)
 try {
