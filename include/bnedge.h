@@ -122,8 +122,9 @@ typedef struct bn_job_desc {
  * whose exponential, and that of every sum it enters, is exactly 0); NaN or
  * +inf give BN_EINVAL.  Batches and
  * bn_edge_posteriors_static reject a job that sets either (BN_EINVAL).  If
- * every parent set of some node has weight zero, P(D) = 0 and the
- * posteriors are undefined. */
+ * every order, or every network, has a zero factor, P(D) = 0 and the
+ * posteriors are undefined: the results, finite numbers, are those of factors
+ * e^-1e7 in the zeros' place (log P(D) below -5e6). */
 
 typedef struct bn_stats {
     double ms_scores;        /* device time of each stage, CUDA events on the
@@ -481,7 +482,8 @@ enum {
     BN_PLAN_SWEEPS = 0,  /* 1: F and R' of a batch group of such jobs may run in
                             one launch                                       */
     BN_PLAN_ANY_SETS = 1,/* set sizes whose states are counted one by one      */
-    BN_PLAN_COUNT = 2
+    BN_PLAN_LINEAR = 2,  /* 1: FP64 values held themselves, not as logarithms  */
+    BN_PLAN_COUNT = 3
 };
 int bn_debug_plan(const bn_job_desc* job, int32_t* out, int32_t count);
 #endif /* BN_TESTING */

@@ -71,7 +71,7 @@ EXPORTS = ["bn_ctx_create", "bn_ctx_destroy", "bn_num_families", "bn_scores",
 TEST_EXPORTS = ["bn_debug_stage", "bn_debug_counts", "bn_debug_batch_drop", "bn_debug_bounds",
                 "bn_debug_explog", "bn_debug_copy_wait", "bn_debug_plan", "bn_debug_phase2",
                 "bn_debug_sweep_blocks", "bn_debug_sweep_wait"]
-BN_PLAN_SWEEPS, BN_PLAN_ANY_SETS, BN_PLAN_COUNT = range(3)
+BN_PLAN_SWEEPS, BN_PLAN_ANY_SETS, BN_PLAN_LINEAR, BN_PLAN_COUNT = range(4)
 
 
 def testing_build() -> bool:

@@ -198,24 +198,29 @@ inline void set_states(Plan& P, const uint32_t* sorted)
     }
 }
 
-// Whether an FP64 job may keep its values linear (Plan::lin).  With the nodes' scores shifted
-// by their maxima the values lie below 2^1000, and only those within reach of
-// F(V) matter; F(V) is at least the weight of the empty parent sets, Prod_i
-// B_i(empty) / c_i, and that is bounded per node by m log2 r + r log2(r (1 +
-// m / ess)) bits of score and by `logs`, the largest magnitude of the job's own
-// (finite) log weights per node in nats.  118000 bits leave 10000 of the range
-// for the products beside F(V).  Above, no value exceeds n! K^n (every order,
-// every A_i at most K) times e^up, `up` the sum over the nodes of their largest
-// order-prior and feature weights above 1, in nats.  Lattices whose tiles do not fit keep
-// the logarithms.
-inline int lin_range(const Plan& P, const uint8_t* arity, double ess, double logs, double up)
+// Whether an FP64 job may keep its values linear (Plan::lin).  The nodes'
+// scores are shifted by their maxima c_i, and only the values within reach of F(V)
+// matter.  F(V) is at least the weight of one network without zero factors,
+// Prod_i B_i(G_i) / c_i: the empty parent sets, or those that plan_lin found
+// (parents[i] members, q joint states at most).  A node's factor is above 2^-b with
+// b = m log2 r + min(q, m) r log2(r (1 + m q / ess)) bits of score (every parent
+// state its own Dirichlet-multinomial) and twice `logs`, the largest magnitude of
+// the job's own nonzero log weights per node in nats.  118000 bits leave 10000
+// of the range for the products beside F(V).  Above, no value exceeds n! K^n
+// (every order, every A_i at most K) times e^up, `up` the sum over the nodes of
+// their largest order-prior and feature weights above 1, in nats.  Lattices whose
+// tiles do not fit keep the logarithms.
+inline int lin_range(const Plan& P, const uint8_t* arity, double ess, double logs, double up,
+                     const int* parents = nullptr)
 {
     if (P.prec != 0 || P.n < 5 || P.n > 31) return 0;
     if (P.n >= 14 && !(P.up13 && P.g13)) return 0;
     double bits = 0.0;
     for (int i = 0; i < P.n; ++i) {
         const double r = arity[i];
-        bits += P.m * std::log2(r) + r * std::log2(r * (1.0 + P.m / ess) + 2.0) + 2.8854 * logs;
+        const double q = parents ? P.states[parents[i]] : 1.0;
+        bits += P.m * std::log2(r) + std::fmax(1.0, std::fmin(q, P.m)) * r * std::log2(r * (1.0 + P.m * q / ess) + 2.0) +
+                2.8854 * logs;
     }
     const double above = P.n * std::log2((double)P.K) + 1.4427 * (std::lgamma(P.n + 1.0) + up);
     return bits < 118000.0 && above < 1000.0;

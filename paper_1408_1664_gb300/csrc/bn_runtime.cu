@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstring>
 #include <deque>
+#include <functional>
 #include <array>
 #include <map>
 #include <mutex>
@@ -220,19 +221,99 @@ double sum_above(const std::vector<double>& v, int n)
     return x;
 }
 
+bool zero_weight(double x) { return x < 0.5 * kLogZero; }
+
+// Whether some order has no zero factor: the order prior's factors depend on a
+// node and its place alone, so the question is a perfect matching of the nodes
+// with the n places (augmenting paths).
+bool order_exists(const std::vector<double>& log_q, int n)
+{
+    std::vector<int> at(n, -1);                  // the node in each place
+    for (int i = 0; i < n; ++i) {
+        std::vector<char> seen(n, 0);
+        const std::function<bool(int)> place = [&](int v) {
+            for (int k = 0; k < n; ++k) {
+                if (seen[k] || zero_weight(log_q[(size_t)v * n + k])) continue;
+                seen[k] = 1;
+                if (at[k] < 0 || place(at[k])) {
+                    at[k] = v;
+                    return true;
+                }
+            }
+            return false;
+        };
+        if (!place(i)) return false;
+    }
+    return true;
+}
+
+// A network of families without zero weights, when one exists: the nodes are
+// placed one after another, each as soon as the nodes before it hold a parent
+// set for it (which parent sets a node may take only grows with the placed
+// nodes, so the order of trying does not matter).  size[i] is the number of
+// parents of node i's family.  False: none exists, or the search over the
+// families is longer than a few ten thousand per node.
+bool network_exists(const HostJob& hj, const std::vector<double>& lf, std::vector<int>& size)
+{
+    const Plan& P = hj.P;
+    const auto weight = [&](int i, int64_t f, int k) {
+        if (k < (int)hj.log_rho.size() && zero_weight(hj.log_rho[k])) return false;
+        if (!hj.log_w.empty() && zero_weight(hj.log_w[(size_t)i * P.K + f])) return false;
+        return lf.empty() || !zero_weight(lf[(size_t)i * P.K + f]);
+    };
+    size.assign(P.n, -1);
+    uint32_t placed = 0;
+    int64_t left = (int64_t)1 << 22;
+    for (bool more = true; more;) {
+        more = false;
+        for (int i = 0; i < P.n; ++i) {
+            if (size[i] >= 0) continue;
+            const uint32_t low = (1u << i) - 1u;
+            const uint32_t have = (placed & low) | ((placed >> 1) & ~low);   // over the other nodes
+            int64_t f = 0;
+            for (int k = 0; k <= P.d && size[i] < 0; ++k) {
+                const int64_t count = host_binom(P.n - 1, k);
+                uint32_t x = (uint32_t)(((uint64_t)1 << k) - 1u);            // colexicographic
+                for (int64_t c = 0; c < count; ++c, ++f) {
+                    if (!(x & ~have) && weight(i, f, k)) {
+                        size[i] = k;
+                        break;
+                    }
+                    if (--left < 0) return false;
+                    if (x) {
+                        const uint32_t u = x & (0u - x), w = x + u;
+                        x = w | (((w ^ x) >> 2) / u);
+                    }
+                }
+            }
+            if (size[i] < 0) continue;
+            placed |= 1u << i;
+            more = true;
+        }
+    }
+    return placed == (uint32_t)(((uint64_t)1 << P.n) - 1);
+}
+
 // Whether the job's values stay linear (FP64; lf: a feature's log weights).
-// A zero weight on an empty parent set leaves F(V) without its lower bound.
+// lin_range's bound needs an order and a network without zero factors; where
+// neither can be shown, P(D) may be zero, and the logarithms hold it as they hold
+// the zero factors.
 void plan_lin(HostJob& hj, const std::vector<double>& lf)
 {
     Plan& P = hj.P;
     P.lin = 0;
-    if (P.prec != 0) return;
+    if (P.prec != 0 || !bn::lin_tiles_fit(P)) return;
+    const auto any_zero = [](const std::vector<double>& v) { return std::any_of(v.begin(), v.end(), zero_weight); };
+    bool empties = hj.log_rho.empty() || !zero_weight(hj.log_rho[0]);        // every node may have no parents
+    for (int i = 0; i < P.n && empties; ++i)
+        empties = (hj.log_w.empty() || !zero_weight(hj.log_w[(size_t)i * P.K])) &&
+                  (lf.empty() || !zero_weight(lf[(size_t)i * P.K]));
+    std::vector<int> size(P.n, 0);
+    if (any_zero(hj.log_q) && (!empties || !order_exists(hj.log_q, P.n))) return;
+    if (!empties && !network_exists(hj, lf, size)) return;
     const double logs = largest_log(hj.log_rho) + largest_log(hj.log_q) + largest_log(hj.log_w) + largest_log(lf);
     const double up = sum_above(hj.log_q, P.n) + sum_above(lf, P.n);
-    P.lin = bn::lin_tiles_fit(P) ? bn::lin_range(P, hj.arity.data(), hj.ess, logs, up) : 0;
-    if (P.hasw)
-        for (int i = 0; i < P.n; ++i)
-            if (hj.log_w[(size_t)i * P.K] < 0.5 * kLogZero) P.lin = 0;
+    P.lin = bn::lin_range(P, hj.arity.data(), hj.ess, logs, up, size.data());
 }
 
 int validate_and_plan(const bn_job_desc* j, HostJob& hj)
@@ -2397,6 +2478,7 @@ try {
     if (rc) return rc;
     int32_t v[BN_PLAN_COUNT] = {};
     v[BN_PLAN_SWEEPS] = bn::sweeps_fit(hj.P);
+    v[BN_PLAN_LINEAR] = hj.P.lin;
     v[BN_PLAN_ANY_SETS] = bn::any_set_sizes(hj.P);
     std::copy(v, v + count, out);
     return BN_OK;
