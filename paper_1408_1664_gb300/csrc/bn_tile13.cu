@@ -2003,12 +2003,15 @@ static bool use_upzeta13p(const Plan& P, const int* err)
 
 // Three blocks per SM (80 registers; the exact path spills) for the sample
 // counts whose tiles mostly take one window, two (128 registers) for the
-// others and where the staged sums leave no room for three.  us, d = 4,
-// binary, column sums included, two / three blocks: n = 22, m = 500 100 / 93,
-// 1000 110 / 106, 1500 129 / 137; n = 24 393 / 375, 498 / 529, 544 / 592; n =
-// 26 1468 / 1340, 1818 / 1786, 2089 / 2132, m = 2000 2436 / 2695; n = 29, m =
-// 500 16588 / 15536.
-constexpr int kUp13ThreeM = 700;
+// others and where the staged sums leave no room for three.  A tile's span
+// grows with the evidence, so with m; the data decide the rest.  The tiles'
+// time with three blocks over that with two, mean (and range) over eleven
+// shapes, n = 21 to 28, d = 2 to 5, binary and arities 2 to 4: m = 150 0.91
+// (0.90-0.95), 500 0.93 (0.90-0.97), 700 0.95 (0.92-1.02), 800 0.98 (0.92-1.02),
+// 900 1.00 (0.92-1.04), 1000 1.02 (0.96-1.09), 1500 1.07 (0.97-1.15), 2000 1.14
+// (1.05-1.28).  us, two / three: n = 26 d = 4, m = 800 1524 / 1478, m = 900
+// 1759 / 1788; n = 21 d = 3 mixed, m = 700 44.0 / 43.0, m = 800 47.1 / 48.1.
+constexpr int kUp13ThreeM = 800;
 
 // The persistent tile kernel stages the columns with d low elements straight
 // from the reordered score table when the column sums come from the column
