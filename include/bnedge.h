@@ -449,9 +449,9 @@ int bn_debug_copy_wait(uint32_t polls, int32_t* err_word);
  * outputs, the packed levels of a split job -- against their arrays'
  * sizes; a failing access records its source line and goes to offset 0
  * instead (no fault, no trap).  This call waits for the device and returns
- * the first failure since the last call: *unit = 1 (bn_kernels.cu),
- * 2 (bn_tile13.cu), 3 (bn_levels.cu) or 4 (bn_mega.cu) and *line its source
- * line, or both 0 when every check passed.  In the other builds *line = -1
+ * the first failure since the last call: *unit = 1 (bn_scores.cu),
+ * 2 (bn_kernels.cu), 3 (bn_tile13.cu), 4 (bn_levels.cu) or 5 (bn_mega.cu) and
+ * *line its source line, or both 0 when every check passed.  In the other builds *line = -1
  * (no checks compiled). */
 int bn_debug_bounds(int32_t* line, int32_t* unit);
 /* The FP64 path's table-driven exp and log (after Tang's method) beside

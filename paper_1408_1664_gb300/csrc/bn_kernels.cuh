@@ -304,7 +304,7 @@ cudaError_t launch_add_feature(const Plan& P, const void* lbs, const void* lf, v
 // shift wrote it already); smaller n use one shared-memory tile per node
 // slice and ignore `tab`.
 // `rk13` points at the two 8192-entry uint16 subset-rank tables (rank, then
-// inverse) of the 13-dimension tiles, filled by launch_rank13_tables.  `err`
+// inverse) of the 13-dimension tiles, filled by launch_step1_prep.  `err`
 // (the job's error word) lets an FP32 single job use the persistent tile
 // kernel, which reports a bulk copy that never landed there.
 cudaError_t launch_upzeta(const Plan& P, const uint32_t* cmasks, const void* lbs, void* tab,
@@ -388,8 +388,8 @@ size_t upzeta_smem_bytes(const Plan& P);
 cudaError_t launch_reorder_up(const Plan& P, const void* lbs, void* tab, cudaStream_t s);
 cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unrank13, void* A,
                             cudaStream_t s, cudaEvent_t sums_done = nullptr, int* err = nullptr);
-cudaError_t launch_upzeta13p_withheld(float* A, uint16_t* rank13, uint16_t* unrank13, int* err,
-                                      uint32_t polls, cudaStream_t s);
+cudaError_t launch_upzeta13p_withheld(float* A, const uint16_t* unrank13, int* err, uint32_t polls,
+                                      cudaStream_t s);
 cudaError_t launch_gamma13_p1(const Plan& P, const void* F, const void* Rc,
                               const uint16_t* rank13, void* W, cudaStream_t s,
                               const void* lq = nullptr, const void* A = nullptr);

@@ -229,7 +229,7 @@ __device__ __forceinline__ void fill_table(uint32_t (*bt)[BT])
 // the rank's); Atop holds, for each top variable t = nl + q, its slab over
 // the nl low variables.  A term of a low node reads its slab with the top
 // bits of the row index dropped; a term of a top variable reads Atop.
-template <typename T, int FMODE, int B, bool TLO = false, bool SLAB = false>
+template <typename T, int B, bool TLO = false, bool SLAB = false>
 __device__ __forceinline__ T forward_tile(int n, uint32_t Ht, const T* __restrict__ A,
                                           T* __restrict__ F, T rebase = T{}, int nl = 0,
                                           const T* __restrict__ Atop = nullptr)
@@ -256,7 +256,7 @@ __device__ __forceinline__ T forward_tile(int n, uint32_t Ht, const T* __restric
                                (SLAB ? nl : n) * half),
                      a, LD_STREAM);
         }
-        load_row(F + BN_AT((size_t)Hm << B, LN, full), f, FMODE);
+        load_row(F + BN_AT((size_t)Hm << B, LN, full), f, LD_PLAIN);
 #pragma unroll
         for (int l = 0; l < LN; ++l) s[l].add(a[l], f[l]);
     }
@@ -290,7 +290,7 @@ __device__ __forceinline__ T forward_tile(int n, uint32_t Ht, const T* __restric
 
 // The 2^B values of R' in tile Ht (the tiles of the level above written):
 //   R'(T) = sum_{i not in T} A_i(T) R'(T + {i}),  R'(V) = 1
-template <typename T, int FMODE, int B, bool TLO = false, bool SLAB = false>
+template <typename T, int B, bool TLO = false, bool SLAB = false>
 __device__ __forceinline__ T backward_tile(int n, uint32_t Ht, const T* __restrict__ A,
                                            T* __restrict__ Rc, T rebase = T{}, int nl = 0,
                                            const T* __restrict__ Atop = nullptr)
@@ -317,7 +317,7 @@ __device__ __forceinline__ T backward_tile(int n, uint32_t Ht, const T* __restri
                                (SLAB ? nl : n) * half),
                      a, LD_STREAM);
         }
-        load_row(Rc + BN_AT((size_t)(Ht | (1u << j)) << B, LN, full), r, FMODE);
+        load_row(Rc + BN_AT((size_t)(Ht | (1u << j)) << B, LN, full), r, LD_PLAIN);
 #pragma unroll
         for (int l = 0; l < LN; ++l) s[l].add(a[l], r[l]);
     }
@@ -395,8 +395,8 @@ k_forward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __res
         const T rebase = hl > 0 ? (T)level_delta(lw, hl - 1) : T(0);
         T mx = LogOps<T>::ninf();
         if (g < ntiles)
-            mx = forward_tile<T, LD_PLAIN, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, F,
-                                                         rebase, n - kfix, Atop);
+            mx = forward_tile<T, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, F, rebase,
+                                               n - kfix, Atop);
         if (hl == 0) {
             if (g == 0) level_words_start(lw, 0, mx);
         } else {
@@ -404,8 +404,7 @@ k_forward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __res
         }
     } else {
         if (g >= ntiles) return;
-        forward_tile<T, LD_PLAIN, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, F, T{},
-                                                n - kfix, Atop);
+        forward_tile<T, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, F, T{}, n - kfix, Atop);
     }
 }
 
@@ -428,8 +427,8 @@ k_backward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __re
         const T rebase = hl < nh ? (T)level_delta(lw, hl + 1) : T(0);
         T mx = LogOps<T>::ninf();
         if (g < ntiles)
-            mx = backward_tile<T, LD_PLAIN, B, TLO, SLAB>(n, level_tile(g, hl, nh, rfix, kfix, bt), A, Rc,
-                                                          rebase, n - kfix, Atop);
+            mx = backward_tile<T, B, TLO, SLAB>(n, level_tile(g, hl, nh, rfix, kfix, bt), A, Rc, rebase,
+                                                n - kfix, Atop);
         if (hl == nh) {
             if (g == 0) level_words_start(lw, nh, mx);
         } else {
@@ -437,8 +436,7 @@ k_backward_rows(int n, int hl, uint32_t ntiles, const T* __restrict__ A, T* __re
         }
     } else {
         if (g >= ntiles) return;
-        backward_tile<T, LD_PLAIN, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, Rc, T{},
-                                                 n - kfix, Atop);
+        backward_tile<T, B, TLO, SLAB>(n, level_tile(g, hl, n - B, rfix, kfix, bt), A, Rc, T{}, n - kfix, Atop);
     }
 }
 

@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <new>
+#include <numeric>
 #include <stdexcept>
 #include <chrono>
 #include <cmath>
@@ -2391,13 +2392,19 @@ int bn_debug_copy_wait(uint32_t polls, int32_t* err_word)
 try {
     if (!err_word) return BN_EINVAL;
     char* buf = nullptr;
-    const size_t abytes = 8192 * 4, tbytes = 2 * 8192 * 2;
+    // the 13-bit patterns by size, then value
+    std::vector<uint16_t> order(8192);
+    std::iota(order.begin(), order.end(), (uint16_t)0);
+    std::stable_sort(order.begin(), order.end(),
+                     [](uint16_t a, uint16_t b) { return __builtin_popcount(a) < __builtin_popcount(b); });
+    const size_t abytes = 8192 * 4, tbytes = 8192 * 2;
     CK(cudaMalloc(&buf, abytes + tbytes + 16));
     float* A = reinterpret_cast<float*>(buf);
-    uint16_t* rk = reinterpret_cast<uint16_t*>(buf + abytes);
+    uint16_t* unrank = reinterpret_cast<uint16_t*>(buf + abytes);
     int* err = reinterpret_cast<int*>(buf + abytes + tbytes);
     cudaError_t e = cudaMemset(buf, 0, abytes + tbytes + 16);
-    if (e == cudaSuccess) e = bn::launch_upzeta13p_withheld(A, rk, rk + 8192, err, polls, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpy(unrank, order.data(), tbytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = bn::launch_upzeta13p_withheld(A, unrank, err, polls, nullptr);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     int w = 0;
     if (e == cudaSuccess) e = cudaMemcpy(&w, err, 4, cudaMemcpyDeviceToHost);

@@ -205,7 +205,7 @@ k_set_ones(int n, int m, int W, uint32_t nsets, int lq, const uint64_t* __restri
 // bits, the others 2^(k-5) registers.  What bounds it: the gathers of cnt and
 // T (both L2-resident), and for k = 9 the 80 shuffles of the lane bits.
 template <int RB>
-__device__ __forceinline__ long long moebius_warp(uint32_t X, int n, int lane,
+__device__ __forceinline__ long long moebius_warp(uint32_t X, int lane,
                                                   const uint32_t* __restrict__ soff,
                                                   const uint32_t* __restrict__ cnt, uint32_t nsets,
                                                   const long long* __restrict__ Tk, int64_t* dbg)
@@ -263,7 +263,6 @@ __device__ __forceinline__ long long moebius_warp(uint32_t X, int n, int lane,
 #pragma unroll
         for (int r = 0; r < R; ++r) dbg[lane | (r << 5)] = v[r];
     }
-    (void)n;
     return warp_sum(acc);
 }
 
@@ -271,7 +270,7 @@ constexpr int kMoebiusMax = 10;                     // variables of a set a warp
 constexpr int kMoebiusRun = 4;                      // consecutive sets per warp
 
 __global__ void __launch_bounds__(256)
-k_set_moebius(int n, int m, int kmax, uint32_t nsets, uint32_t ns5, uint32_t nall,
+k_set_moebius(int n, int m, uint32_t nsets, uint32_t ns5, uint32_t nall,
               const uint32_t* __restrict__ cnt, const double* __restrict__ Dvals, int rows,
               const long long* __restrict__ T, long long* __restrict__ H, int64_t* __restrict__ dbg,
               uint32_t dbg_set, size_t js)
@@ -346,11 +345,11 @@ k_set_moebius(int n, int m, int kmax, uint32_t nsets, uint32_t ns5, uint32_t nal
         int64_t* db = dbg && idx == dbg_set ? dbg : nullptr;
         long long h;
         switch (k) {
-        case 6: h = moebius_warp<1>(X, n, lane, soff, cnt, nall, Tk, db); break;
-        case 7: h = moebius_warp<2>(X, n, lane, soff, cnt, nall, Tk, db); break;
-        case 8: h = moebius_warp<3>(X, n, lane, soff, cnt, nall, Tk, db); break;
-        case 9: h = moebius_warp<4>(X, n, lane, soff, cnt, nall, Tk, db); break;
-        default: h = moebius_warp<5>(X, n, lane, soff, cnt, nall, Tk, db); break;
+        case 6: h = moebius_warp<1>(X, lane, soff, cnt, nall, Tk, db); break;
+        case 7: h = moebius_warp<2>(X, lane, soff, cnt, nall, Tk, db); break;
+        case 8: h = moebius_warp<3>(X, lane, soff, cnt, nall, Tk, db); break;
+        case 9: h = moebius_warp<4>(X, lane, soff, cnt, nall, Tk, db); break;
+        default: h = moebius_warp<5>(X, lane, soff, cnt, nall, Tk, db); break;
         }
         if (lane == 0) H[BN_AT(idx, 1, nall)] = h;
         if (++idx >= end) break;
@@ -363,10 +362,9 @@ k_set_moebius(int n, int m, int kmax, uint32_t nsets, uint32_t ns5, uint32_t nal
             X = w | (((w ^ X) >> 2) >> (__ffs(u) - 1));
         }
     }
-    (void)kmax;
 }
 
-// The sets of b, b + 1 and b + 2 variables (b = kmax - 2, 5 .. 8) from their
+// The sets of b, b + 1 and b + 2 variables (b + 2 the largest size, b = 5 .. 8) from their
 // bases: a warp takes the base Y (b variables, bits as in moebius_warp), then
 // each variable c below all of Y, then each pair c0 < c1 below all of Y, so
 // every set comes up once.  With v the counts of Y's joint states among the
@@ -500,7 +498,7 @@ __device__ __forceinline__ void pairs_warp(uint32_t Y, int b, int lane, const ui
     }
 }
 
-constexpr int kPairsMin = 7;                        // kmax from which bases take over
+constexpr int kPairsMin = 7;                        // largest size from which bases take over
 template <int RB>
 __global__ void __launch_bounds__(256, RB < 3 ? 3 : 2)
 k_set_pairs(int n, int m, int b, uint32_t nsets, uint32_t nbase, const uint32_t* __restrict__ cnt,
@@ -1039,7 +1037,7 @@ cudaError_t launch_set_scores(const Plan& P, const uint8_t* data, const uint8_t*
         const uint32_t own = b ? sets_before(P.n, b) : nsets, own5 = std::min(ns5, own);
         const uint32_t warps = (own - own5 + kMoebiusRun - 1) / kMoebiusRun;
         e = launch_or_record(KID_SET_MOEBIUS, k_set_moebius, dim3((own5 + 255) / 256 + (warps + 7) / 8, P.nj),
-                             256, 0, s, P.n, P.m, z.moebius - 1, own, own5, nsets, x.cnt, Dvals, P.rows, T,
+                             256, 0, s, P.n, P.m, own, own5, nsets, x.cnt, Dvals, P.rows, T,
                              x.H, dbg, dbg_set, P.js);
         if (e != cudaSuccess) return e;
         if (b) {

@@ -611,12 +611,6 @@ k_upzeta13_cols(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
     for (uint32_t c = ncopy + t; c < ncol; c += TT) out[c] = tb[c];
 }
 
-// Part 1 with one warp per tile: each warp enumerates its tile's rows into
-// its own list and sums the columns lane by lane (consecutive columns:
-// coalesced reads of a row); no block barrier after the tables are filled.
-// Columns with d low elements are copies, those with d - 1 take the 1 + |H|
-// rows of at most one high element, the others every row of size at most
-// d - |G_L|.
 // Column sums by butterflies over the h high dimensions.  Blocks below
 // nodes * ceil(ncb / CPB) take one node i and a run of CPB consecutive low
 // columns c < ncb: the 2^h values B_i(G_H + G_L) of each column (zero where
@@ -630,9 +624,9 @@ k_upzeta13_cols(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
 //
 // Every output of a column lies between its H = {} value f(G_L) and its
 // largest input plus log 2^h, so when that span is under one single-scale
-// window (Window) for every column of the block, the sums run in linear
-// scale (an exponential per input, an addition per step, a logarithm per
-// output; exact as in the tiles); otherwise every step is a log-sum-exp.
+// window (Window), the column's sums run in linear scale (an exponential per
+// input, an addition per step, a logarithm per output; exact as in the
+// tiles); otherwise every step is a log-sum-exp.
 // The blocks after those copy the columns from ncb on, whose sums have a
 // single row (the empty high set), a warp per tile.
 //
@@ -875,6 +869,12 @@ k_upzeta13_colb(int n, int d, int64_t K, const T* __restrict__ tab, T* __restric
     if (hc) cluster_sync();                          // no peer reads this block's values any more
 }
 
+// Part 1 with one warp per tile: each warp enumerates its tile's rows into
+// its own list and sums the columns lane by lane (consecutive columns:
+// coalesced reads of a row); no block barrier after the tables are filled.
+// Columns with d low elements are copies, those with d - 1 take the 1 + |H|
+// rows of at most one high element, the others every row of size at most
+// d - |G_L|.
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_upzeta13_colw(int n, int d, int64_t K, const T* __restrict__ tab, T* __restrict__ A, size_t js,
@@ -1873,20 +1873,6 @@ k_g13_x(int n, int d, uint32_t nlow, const X64* __restrict__ F, const X64* __res
     }
 }
 
-// rank13[L] = position of L among the subsets of 13 bits ordered by size then
-// value; unrank13 is its inverse.
-__global__ void k_rank13_tables(uint16_t* __restrict__ rank13, uint16_t* __restrict__ unrank13,
-                                size_t js)
-{
-    rank13 = job_ptr(rank13, js);
-    unrank13 = job_ptr(unrank13, js);
-    const uint32_t L = blockIdx.x * blockDim.x + threadIdx.x;
-    if (L >= (uint32_t)TN) return;
-    const uint32_t r = small_subset_rank(L, TB);
-    rank13[L] = (uint16_t)r;
-    unrank13[r] = (uint16_t)L;
-}
-
 #ifndef BN_MEGA  // host launchers (bn_mega.cu includes only the device code)
 #ifdef BN_CHECK_BOUNDS
 BN_BOUNDS_READER(bounds_line_tile13)
@@ -2175,14 +2161,12 @@ cudaError_t launch_upzeta13(const Plan& P, const void* tab, const uint16_t* unra
 
 // One block of the persistent tile kernel (n = 14, d = 4: one tile) with its
 // first bulk copy withheld: its wait gives up after `polls` polls and sets
-// kErrDeviceTimeout in *err.  A holds one tile (8192 floats); unrank13 is
-// filled here.
-cudaError_t launch_upzeta13p_withheld(float* A, uint16_t* rank13, uint16_t* unrank13, int* err,
-                                      uint32_t polls, cudaStream_t s)
+// kErrDeviceTimeout in *err.  A holds one tile (8192 floats).
+cudaError_t launch_upzeta13p_withheld(float* A, const uint16_t* unrank13, int* err, uint32_t polls,
+                                      cudaStream_t s)
 {
     cudaError_t e = allow_max_dynamic_smem(k_upzeta13p<false, 3>);
     if (e != cudaSuccess) return e;
-    k_rank13_tables<<<TN / 256, 256, 0, s>>>(rank13, unrank13, 0);
     Plan P{};
     P.n = 14;
     P.d = 4;
