@@ -239,18 +239,16 @@ int bn_edge_posteriors_static(const bn_job_desc* job, double* post_dev,
 /* Batches.  Many independent jobs (typically small n) planned together
  * (Algorithm 1 for each job; the paper has no batch form).
  * bn_batch_create validates every job and copies its host inputs into one
- * device arena.  Jobs with equal n, d, precision and kind of data (every
- * arity 2, or not) form a group: their arrays lie at a fixed stride in a
+ * device arena.  Jobs with equal n, d, precision (FP64: and form of its
+ * values) and kind of data (every arity 2, or not) form a group: their arrays lie at a fixed stride in a
  * layout padded to the group's largest m, arity and lgamma table, and every
  * launch of steps 1-5 covers the whole group.
  * Unless the context has BN_CTX_NO_AUTOTUNE, the schedule of each group --
- * the kernel of the scores (one lane per 64-sample word or one lane per
- * parent configuration, non-binary data), of the up-zeta (13-dimension
- * tiles or shared-memory tiles), of F and R' (16-subset rows or warp tiles,
- * FP32; then one launch per popcount level or one persistent launch of
- * thread-block clusters, each cluster taking F or R' of one job at a time
- * and running all its levels between cluster barriers) and of the down-zeta
- * phase 1 -- is chosen by timing: the groups run at the same time, so the
+ * the kernel of the up-zeta (13-dimension tiles or shared-memory tiles), of
+ * F and R' (16-subset rows or warp tiles, FP32; then a launch per popcount
+ * level, or one launch in which a block or a thread-block cluster of up to 8
+ * takes F or R' of one job and runs all its levels between barriers) and of
+ * the down-zeta phase 1 -- is chosen by timing: the groups run at the same time, so the
  * autotuner times the whole batch on its own data, switching one kernel
  * choice at a time for all groups, the groups with n <= 14 or those with
  * n > 14, and keeps a switch that makes the batch more than 1% faster.  The
@@ -258,7 +256,7 @@ int bn_edge_posteriors_static(const bn_job_desc* job, double* post_dev,
  * all cached takes them without timing.  Every schedule gives the same
  * values up to rounding (within the stated tolerances, 1e-9 FP64 and 1e-4
  * FP32, of the job run alone; equal bit for bit under the default schedule
- * and with the cluster kernel).  The batch then exists in two forms: the
+ * and with the one-launch form).  The batch then exists in two forms: the
  * launches of all groups recorded into one CUDA graph, one branch per
  * group; and, unless the context has BN_CTX_GRAPH_BATCH or
  * BN_CTX_CLUSTER_STEP3, one persistent launch per precision that runs the

@@ -3,11 +3,12 @@
 //
 // Step 2  k_upzeta         truncated upward zeta (Eq. 7, Definition 1)
 // Step 3  k_forward_level, k_backward_level   F (Eq. 9) and R (Eq. 10)
-// Step 4  k_gamma_p1, k_gamma_p2              truncated downward zeta (Eq. 12)
-// Step 5  k_edges          Eq. 11 and the division by P(D)
+// Step 4  k_gamma_p1, k_gamma_p2, ..p2r, ..p2s, ..p2w   truncated downward zeta (Eq. 12)
+// Step 5  k_edges          Eq. 11 and the division by P(D); k_tail: steps 4 and 5 for n < 14
 //
-// Values are logs: natural logs in FP64, base-2 logs in FP32 (see
-// bn_device.cuh).  Every node's scores are shifted by their maximum c_i
+// Values are base-2 logs in FP32 and the numbers themselves with a wide exponent
+// in FP64 (X64), or natural logs where their range is not bounded (see
+// bn_device.cuh, lin_range).  Every node's scores are shifted by their maximum c_i
 // before step 2: replacing B_i by B_i / exp(c_i) scales every order's weight
 // by the same factor prod_i exp(-c_i), which cancels in P(u->v | D), and
 // keeps the log magnitudes of A, F, R and Gamma small.
