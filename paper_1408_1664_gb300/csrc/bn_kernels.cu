@@ -423,9 +423,9 @@ k_gamma_p2(int n, int d, int b, int hc, uint32_t nlow, int64_t K, const T* __res
 // banks apart), the downward steps run three dimensions at a time in registers
 // (eight values per thread) and the outputs with at most d - |g| high elements
 // go to their families.  A run of columns reads whole sectors of W's rows and
-// a step touches shared memory once per three dimensions; a block per column
-// with a step per dimension (k_gamma_p2, kept for columns past 64 KB) took
-// 2.15 ms at n = 25, d = 8.
+// a step touches shared memory once per three dimensions (n = 22, d = 8: phase 2
+// 612 us with a block per column and a step per dimension, k_gamma_p2, and 277
+// here; p2r_columns has the other sizes).
 //
 // The steps are additions relative to one scale (an exponential per input, a
 // logarithm per output resolved), in one or a few passes like the tiles': a
@@ -1497,19 +1497,21 @@ int gamma_launches(const Plan& P)
 }
 
 // Columns per block of k_gamma_p2r: 64 KB of values (at most 64 outputs per
-// thread), at most 8 columns; 0: k_gamma_p2.  Its full transform beats the
-// guarded one of k_gamma_p2 on short columns (h <= 9; n = 22, d = 8: phase 2
-// 0.73 -> 0.34 ms) and where most high parts are outputs (d >= 7; n = 25, d =
-// 8: 2.15 -> 1.87 ms), not on long columns with few outputs (n = 25, d = 6:
-// 0.54 against 0.56 ms).  FP32: the linear FP64 form gained nothing (n = 23).
+// thread), 8 or 4 columns; 0: k_gamma_p2.  The full transform of eight columns
+// at a time beats the guarded one of a column per block where columns are short
+// or enough of their high parts are outputs, and there are columns enough for the
+// GPU.  Phase 2, us, k_gamma_p2 against k_gamma_p2r (m = 500): h = 7, d = 3 29 and
+// 30, d = 4 51 and 48; h = 8, d = 3 25 and 29, d = 4 43 and 40, d = 8 612 and 277;
+// h = 9, d = 4 53 and 58, d = 5 119 and 104; h = 10, d = 5 171 and 174, d = 6 390
+// and 338, d = 8 1240 and 917; h = 11, d = 7 1348 and 1448, d = 8 2334 and 2373;
+// h = 12, d = 7 4135 and 3072, d = 8 5897 and 5210; h = 13, d = 7 7507 and 8588.
+// FP32: the linear FP64 form gained nothing (n = 23).
 static int p2r_columns(const Plan& P)
 {
     const int h = P.n - 1 - P.b_g;
-    if (P.prec == 0 || P.d > 18 || (h > 9 && P.d < 7)) return 0;
-    const size_t fit = (size_t)64 * 1024 / ((size_t)4 << h);
-    int c = 8;
-    while ((size_t)c > fit) c /= 2;
-    return c;
+    if (P.prec == 0 || P.d > 18) return 0;
+    if (h <= 7 || (h <= 10 && P.d >= h - 4)) return 8;
+    return h == 12 && P.d >= 7 ? 4 : 0;
 }
 
 template <int CPB>
@@ -1536,8 +1538,6 @@ cudaError_t launch_gamma_p2(const Plan& P, const void* W, void* Gam, const void*
         const dim3 grid(c0, P.nj, P.n);
         if (cpb == 8) e = gamma_p2r<8>(P, KID_P2R8, c0, W, Gam, A, lq, s);
         else if (cpb == 4) e = gamma_p2r<4>(P, KID_P2R4, c0, W, Gam, A, lq, s);
-        else if (cpb == 2) e = gamma_p2r<2>(P, KID_P2R2, c0, W, Gam, A, lq, s);
-        else if (cpb == 1) e = gamma_p2r<1>(P, KID_P2R1, c0, W, Gam, A, lq, s);
         else if (P.lin)
             launch_or_record(KID_GAMMA_P2_X, k_gamma_p2<X64>, grid, 256, sm2, s, P.n, P.d, P.b_g, P.hc_g, P.nlow_g,
                              P.K, (const X64*)W, (X64*)Gam, P.js, P.vsel);
@@ -1636,8 +1636,6 @@ cudaError_t set_kernel_attributes()
     SETA(k_gamma_p2<X64>)
     SETA(k_gamma_p2r<8>)
     SETA(k_gamma_p2r<4>)
-    SETA(k_gamma_p2r<2>)
-    SETA(k_gamma_p2r<1>)
     SETA(k_tail<float>)
     SETA(k_tail<double>)
     SETA(k_tail<X64>)

@@ -38,7 +38,7 @@ enum KernelId : int32_t {
     KID_SHIFT_X, KID_APPLY_Q_X, KID_ADD_FEATURE_X, KID_REORDER_X, KID_COLB4_X, KID_COLB2_X,
     KID_COLB1_X, KID_COLW_X, KID_UP13_X, KID_FROWS_X, KID_BROWS_X, KID_G13_X_Q, KID_G13_X,
     KID_GAMMA_P2_X, KID_GAMMA_P2S_X, KID_EDGES_X,
-    KID_P2R8, KID_P2R4, KID_P2R2, KID_P2R1, KID_GAMMA_P2W,
+    KID_P2R8, KID_P2R4, KID_GAMMA_P2W,
     KID_SET_HISTC_WARP, KID_SET_HISTC_BLOCK, KID_SET_PAIRS5, KID_SET_PAIRS6, KID_SET_PAIRS7, KID_SET_PAIRS8, KID_COUNT
 };
 

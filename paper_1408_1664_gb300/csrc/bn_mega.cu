@@ -127,8 +127,6 @@ __device__ __forceinline__ bool dispatch(int kid, const unsigned char* a)
         case KID_GAMMA_P2_F: run(k_gamma_p2<float>, a); return true;
         case KID_P2R8: run(k_gamma_p2r<8>, a); return true;
         case KID_P2R4: run(k_gamma_p2r<4>, a); return true;
-        case KID_P2R2: run(k_gamma_p2r<2>, a); return true;
-        case KID_P2R1: run(k_gamma_p2r<1>, a); return true;
         case KID_GAMMA_P2W: run(k_gamma_p2w, a); return true;
         case KID_GAMMA_P2S_F: run(k_gamma_p2s<float>, a); return true;
         case KID_EDGES_F: run(k_edges<float>, a); return true;
@@ -301,7 +299,7 @@ bool persistent_runs(int prec, int kid)
         return true;
     case KID_SHIFT_F: case KID_UPZETA_F: case KID_FWD_LEVEL_F: case KID_BWD_LEVEL_F:
     case KID_GAMMA_TABLE: case KID_GAMMA_P1_F: case KID_GAMMA_P2_F: case KID_GAMMA_P2S_F:
-    case KID_EDGES_F: case KID_TAIL_F: case KID_P2R8: case KID_P2R4: case KID_P2R2: case KID_P2R1: case KID_GAMMA_P2W: case KID_REORDER_F: case KID_COLB8: case KID_COLB4:
+    case KID_EDGES_F: case KID_TAIL_F: case KID_P2R8: case KID_P2R4: case KID_GAMMA_P2W: case KID_REORDER_F: case KID_COLB8: case KID_COLB4:
     case KID_COLB2: case KID_COLB1: case KID_COLW_F: case KID_COLS_F: case KID_UP13_F_TLO: case KID_UP13_F:
     case KID_G13_F: case KID_FROWS_F_TLO: case KID_FROWS_F: case KID_BROWS_F_TLO: case KID_BROWS_F:
         return prec == 1;
