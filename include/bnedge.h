@@ -87,7 +87,7 @@ typedef struct bn_ctx_opts {
 } bn_ctx_opts;
 
 /* bn_ctx_opts.flags: BN_CTX_NO_AUTOTUNE, batches keep the default schedule
- * (and a persistent launch keeps clusters of 8 blocks) instead of timing the
+ * (and a persistent launch takes one block per queue item) instead of timing the
  * alternatives; BN_CTX_CLUSTER_STEP3, every batch group whose step 3 has
  * row tiles (and n <= 28) runs all its levels in one launch whatever the
  * timing says;

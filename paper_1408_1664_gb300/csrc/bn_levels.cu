@@ -1,6 +1,6 @@
 // bn_levels.cu -- F (Eq. 9) and R' (Eq. 10) over the subset lattice, one
-// thread per tile of 2^B subsets: 16 in FP32 (base-2 logs), 8 in FP64
-// (natural logs; a row of 8 doubles is 64 bytes, like 16 floats).
+// thread per tile of 2^B subsets: 16 in FP32 (base-2 logs), 8 in FP64 (X64
+// values, or natural logs; a row of 8 is 64 bytes, like 16 floats).
 //
 // A tile is the 2^B subsets S = (Ht << B) | l that share their high bits Ht
 // (l = the B low bits).  Tiles are launched one popcount level of Ht at a
@@ -13,7 +13,7 @@
 // Every thread of a launch has the same number of terms (same |Ht|), so warps
 // do not diverge, and the index arithmetic is shared by the 2^B subsets.
 //
-// Log-sum-exp is kept lazily: (m, s) stands for m + lg(s) with m the first
+// Sums of logarithms are kept lazily: (m, s) stands for m + lg(s) with m the first
 // term and s rescaled only when a term exceeds m by more than 2^64 (FP32) or
 // e^40 (FP64), so a term costs one exponential.  s stays below that factor
 // times 32, and every value entering is finite (A and F are logs of

@@ -186,8 +186,8 @@ double x_to_ln(unsigned long long u)
     return (double)bn::x_exp(bn::X64{u}) * 0.69314718055994530942 + std::log1p(f);
 }
 
-// In the form of the plan's values: FP32 base-2 logs, FP64 natural logs or
-// the values themselves.
+// In the form of the plan's values: FP32 base-2 logs, FP64 the numbers
+// themselves (X64) or natural logs.
 std::vector<char> working_logs(const std::vector<double>& v, const Plan& P)
 {
     std::vector<char> out(v.size() * (P.prec == 0 ? 8 : 4));
