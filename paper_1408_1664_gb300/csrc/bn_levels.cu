@@ -31,7 +31,7 @@ constexpr int LB = 4;             // low bits of an FP32 tile
 constexpr int LB64 = 3;           // low bits of an FP64 tile
 constexpr int BT = 29;            // binomial table rows (n - B < 29: n <= 32 in FP32)
 // k_sweeps: single jobs up to this n (FP32; linear FP64; a launch per level is
-// faster from n = 22: FP32 330 us either way, FP64 621 against 729), vectors
+// faster from n = 22: FP32 330 us either way, FP64 640 against 748), vectors
 // from kSweepVecN, up to kSweepBusyN while other served jobs run (the whole-GPU
 // form of a wider job would hold every SM: 64 served jobs of n = 19 to 22 took
 // 20.0 ms with it, 15.3 ms without); levels that fill more than kSweepGrid
